@@ -22,8 +22,9 @@
 // Warp roles per CTA (352 threads with the default 8 epilogue warps): warp 0 takes work units from a global
 // counter (runs of column tiles of one row block, so CTAs whose tiles hold
 // many candidates take fewer) and issues TMA; warps 1 and 10 issue the MMAs
-// of the even and odd tiles into their own TMEM accumulator (warp 1 also
-// allocates the 2 x 256 TMEM columns); warps 2-9 drain the accumulators
+// of the even and odd tiles into their own TMEM accumulator when K <= 128
+// (warp 1 alone issues every tile's for deeper K; it also allocates the
+// 2 x 256 TMEM columns); warps 2-9 drain the accumulators
 // (warp w reads TMEM lane quarter w mod 4 and one half of the columns) and
 // release a tile's accumulator as soon as none of their values passes the
 // threshold.  The A panel (128 rows x K) of a unit stays in shared memory;
@@ -419,9 +420,13 @@ k_gemm_topk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   // past d (7 steps instead of 8 for d = 100).
   const int ksteps = args.ksteps;
 
+  // Two MMA issuers share the B stages only when a stage holds a whole tile
+  // (see the issuers below).
+  const int issuers = katoms == spt ? 2 : 1;
+
   if (threadIdx.x == 0) {
     mbar_init(&sh->a_full, 1);
-    mbar_init(&sh->a_empty, 2);   // both MMA issuers
+    mbar_init(&sh->a_empty, issuers);
     mbar_init(&sh->done, 2);
     for (int s = 0; s < nstage; ++s) {
       mbar_init(&sh->b_full[s], 1);
@@ -433,7 +438,7 @@ k_gemm_topk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     }
     for (int k = 0; k < kSched; ++k) {
       mbar_init(&sh->sched_full[k], 1);
-      mbar_init(&sh->sched_empty[k], 3);  // the two MMA issuers and the epilogue
+      mbar_init(&sh->sched_empty[k], issuers + 1);  // the MMA issuers and the epilogue
     }
     sh->abort_flag = 0;
     sh->epi_abort = 0;
@@ -525,7 +530,18 @@ k_gemm_topk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     // them accumulator par: while one thread waits on its barriers the
     // other's MMAs keep the tensor pipe busy (one thread alone spends as
     // long on its waits and commits as on the 7 MMAs of a K = 100 tile).
-    if (lane == 0) {
+    //
+    // A parity wait on a stage's use n is meaningful only once use n - 1 has
+    // completed (before that, the barrier's last completed phase has the
+    // awaited parity and the wait passes at once).  An issuer that skips the
+    // other's tiles does not see their stages fill, so it first waits for its
+    // accumulator: the epilogue drains tiles in order, so a drained tile
+    // it - 2 means that every tile up to it - 2 was loaded and multiplied,
+    // and the stage's previous use is tile it - nstage at the latest (nstage
+    // >= 3 where a stage holds a tile).  Where a tile takes several stages
+    // (K > 128) the previous use may be a slice of tile it - 1: one issuer
+    // then takes every tile and sees every phase in turn.
+    if (lane == 0 && (issuers == 2 || warp == 1)) {
       const int par = warp == 1 ? 0 : 1;
       const int groups = katoms / spt;   // stages per tile
       int s = 0;
@@ -537,7 +553,6 @@ k_gemm_topk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       // Descriptors of the first A slice and the first B stage; a K step of
       // 16 adds 32 bytes (2 in the descriptor's 16-byte address units).
       const uint64_t da0 = desc_sw128(sA), db0 = desc_sw128(sB);
-      const uint32_t d_tmem = tmem_base + (uint32_t)(par * BN);
       while (!quit) {
         if (!mbar_wait(&sh->sched_full[ks], kph, abort_flag)) break;
         const long long u = *((volatile long long*)&sh->sched_unit[ks]);
@@ -551,7 +566,8 @@ k_gemm_topk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         if (!mbar_wait(&sh->a_full, (uint32_t)(panel & 1), abort_flag)) break;
         ++panel;
         for (long long cb = x.c0; cb < x.c1 && !quit; ++cb, ++it) {
-          if ((int)(it & 1) != par) {   // the other issuer's tile: skip its stages
+          const int buf = (int)(it & 1);
+          if (issuers == 2 && buf != par) {   // the other issuer's tile: skip its stages
             for (int g = 0; g < groups; ++g)
               if (++s == nstage) {
                 s = 0;
@@ -560,11 +576,10 @@ k_gemm_topk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             continue;
           }
           for (int k0 = 0; k0 < katoms; k0 += spt) {
-            // B first, then the accumulator: the B wait overlaps the
-            // epilogue's drain of this accumulator.
-            if (!mbar_wait(&sh->b_full[s], phase, abort_flag) ||
-                (k0 == 0 && it >= 2 &&
-                 !mbar_wait(&sh->acc_empty[par], (uint32_t)(((it >> 1) - 1) & 1), abort_flag))) {
+            // The accumulator first, then B (see above).
+            if ((k0 == 0 && it >= 2 &&
+                 !mbar_wait(&sh->acc_empty[buf], (uint32_t)(((it >> 1) - 1) & 1), abort_flag)) ||
+                !mbar_wait(&sh->b_full[s], phase, abort_flag)) {
               quit = true;
               break;
             }
@@ -576,7 +591,7 @@ k_gemm_topk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
               // K steps of 16 inside this slice that reach column d (zeros past it).
               const int steps = min(4, ksteps - ka * 4);
               for (int kk = 0; kk < steps; ++kk)
-                mma_bf16(d_tmem, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2),
+                mma_bf16(tmem_base + (uint32_t)(buf * BN), da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2),
                          (ka > 0 || kk > 0) ? 1u : 0u);
             }
             mma_commit(&sh->b_empty[s]);
@@ -586,7 +601,7 @@ k_gemm_topk(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             }
           }
           if (quit) break;
-          mma_commit(&sh->acc_full[par]);
+          mma_commit(&sh->acc_full[buf]);
         }
         if (quit) break;
         mma_commit(&sh->a_empty);   // this issuer's MMAs of the unit done: its A panel may go
@@ -1204,7 +1219,7 @@ struct NormOrder {
 
 // BF16 copies of A (rows) and B^T (columns of B as rows) in norm order,
 // the 2-norms of the rounded rows of A and the column-group maxima of B.
-template <typename T>
+template <typename TA, typename TB>
 void launch_casts(const mad_matrix* A, const mad_matrix* B, int kp, const NormOrder& o,
                   __nv_bfloat16* Abf, __nv_bfloat16* Bbf, float* anorm, float* bgmax,
                   cudaStream_t st) {
@@ -1213,15 +1228,15 @@ void launch_casts(const mad_matrix* A, const mad_matrix* B, int kp, const NormOr
   const unsigned rgrid = (unsigned)(blocks < 152 * 16 ? blocks : 152 * 16);
   const unsigned cgrid = (unsigned)((n + 255) / 256);
   cudaMemsetAsync(o.hist, 0, 512 * sizeof(unsigned int), st);
-  k_row_buckets<T><<<rgrid, 256, 0, st>>>((const T*)A->values, m, A->cols, A->ld, o.bkt_a, o.hist);
-  k_col_buckets<T><<<cgrid, 256, 0, st>>>((const T*)B->values, B->rows, n, B->ld, o.bkt_b,
+  k_row_buckets<TA><<<rgrid, 256, 0, st>>>((const TA*)A->values, m, A->cols, A->ld, o.bkt_a, o.hist);
+  k_col_buckets<TB><<<cgrid, 256, 0, st>>>((const TB*)B->values, B->rows, n, B->ld, o.bkt_b,
                                           o.hist + 256);
   k_bucket_cursors<<<1, 256, 0, st>>>(o.hist, o.hist + 256, o.cur, o.cur + 256);
-  k_cast_rows_bf16<T><<<rgrid, 256, 0, st>>>((const T*)A->values, m, A->cols, A->ld, kp, o.bkt_a,
+  k_cast_rows_bf16<TA><<<rgrid, 256, 0, st>>>((const TA*)A->values, m, A->cols, A->ld, kp, o.bkt_a,
                                              o.cur, Abf, anorm, o.perm_a);
   k_claim_cols<<<cgrid, 256, 0, st>>>(o.bkt_b, n, o.cur + 256, o.pos_b, o.perm_b);
   dim3 grid((unsigned)((n + 31) / 32), (unsigned)((kp + 31) / 32));
-  k_cast_cols_bf16<T><<<grid, dim3(32, 8), 0, st>>>((const T*)B->values, B->rows, n, B->ld, kp,
+  k_cast_cols_bf16<TB><<<grid, dim3(32, 8), 0, st>>>((const TB*)B->values, B->rows, n, B->ld, kp,
                                                     o.pos_b, Bbf);
   // Every group of every column tile, the ones past n included (norm 0).
   const int64_t groups = (B->cols + BN - 1) / BN * (BN / kCols);
@@ -1312,8 +1327,11 @@ mad_status dense_comparator(mad_ctx* ctx, const mad_matrix* A, const mad_matrix*
   cudaMemsetAsync(g_theta, 0, 64, st);
   cudaMemsetAsync(pre_hist, 0, 4097 * 4, st);
 
-  if (A->dt == MAD_F64) launch_casts<double>(A, B, kp, ord, Abf, Bbf, anorm, bgmax, st);
-  else launch_casts<float>(A, B, kp, ord, Abf, Bbf, anorm, bgmax, st);
+  const bool a64 = A->dt == MAD_F64, b64 = B->dt == MAD_F64;
+  if (a64 && b64) launch_casts<double, double>(A, B, kp, ord, Abf, Bbf, anorm, bgmax, st);
+  else if (a64) launch_casts<double, float>(A, B, kp, ord, Abf, Bbf, anorm, bgmax, st);
+  else if (b64) launch_casts<float, double>(A, B, kp, ord, Abf, Bbf, anorm, bgmax, st);
+  else launch_casts<float, float>(A, B, kp, ord, Abf, Bbf, anorm, bgmax, st);
   count_launch(ctx, 7);
 
   CUtensorMap tmA, tmB;

@@ -47,6 +47,21 @@ def test_product_matches_bf16_reference(m, d, n, dtype):
     assert np.all(np.abs(C - ref) <= bound)
 
 
+@pytest.mark.parametrize("ta,tb", [(np.float64, np.float32), (np.float32, np.float64)])
+def test_product_of_mixed_types(ta, tb):
+    import paper_1506_03872_gb300 as mad
+    rng = _rng(77)
+    m, d, n = 200, 70, 530
+    A = rng.standard_normal((m, d)).astype(ta)
+    B = rng.standard_normal((d, n)).astype(tb)
+    tA, tB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    with mad.Context() as c:
+        C = mad.mad_debug_dense_product(c.ctx, mad.dense(tA), mad.dense(tB)).cpu().numpy()
+    Ab, Bb = _bf16(A).astype(np.float64), _bf16(B).astype(np.float64)
+    bound = d * 2.0 ** -23 * (np.abs(Ab) @ np.abs(Bb)) + 1e-30
+    assert np.all(np.abs(C - Ab @ Bb) <= bound)
+
+
 def _fp32_rescore(A, B, keys):
     """Lane-strided FP32 sums folded in halves, as the library computes them."""
     out = []
