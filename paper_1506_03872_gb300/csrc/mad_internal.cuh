@@ -102,7 +102,8 @@ struct SampleParams {
   int f_exp;                       // F
   // Hash.  Regioned (dense inputs): the key (a, b) starts probing in the
   // home region of row a, [hreg[a], hreg[a+1]), sized from row a's expected
-  // share of the diamonds; otherwise at mix(key) & hmask.  Probing is
+  // share of the diamonds (MAD_GRAM: of row a or b, see home_slot);
+  // otherwise at mix(key) & hmask.  Probing is
   // linear and wraps at hcap (for regioned hashes, the end of the regions,
   // read on the device and kept within the hcap_alloc allocated slots).
   unsigned long long* hkeys;
