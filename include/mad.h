@@ -318,8 +318,8 @@ mad_status mad_sparse_topt(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* 
  * A = Q[q] (1 x d) with B = the items (d x n), sampled with its own budget
  * s_q and seed + q.  Because m = 1, the stage-1 draw of Alg. 2 always gives
  * the query's row, so diamond l of query q draws only k, j and k' (Philox
- * key seed + q, counter l, as in mad_sample); its x accumulates in a hash
- * region of its own, and Alg. 3 runs per query: the t' largest positive x
+ * key seed + q, counter l, as in mad_sample); its x accumulates in
+ * tables of its own, and Alg. 3 runs per query: the t' largest positive x
  * by (x desc, j asc), their exact c = q . b_j (FP64, rescoring order of
  * mad_rescore), the t largest |c| by (|c| desc, j asc).  Each query's result
  * equals mad_build_tables + mad_sample + mad_topk + mad_rescore on that
@@ -338,17 +338,16 @@ mad_status mad_sparse_topt(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* 
  * and free of host synchronisation and allocation, so it can be captured
  * in a CUDA graph.  out_dev: nq * t pairs (query q's results at q * t, i =
  * q); n_out_dev: nq counts (uint32, device); cand_dev (optional, nq * t'
- * pairs): each query's top-t' candidates.  A query whose candidates above
- * the selection threshold exceed 4096 (ties of x in the thousands) reports
- * MAD_ERR_STATE through the device error word (read by mad_stats). */
+ * pairs): each query's top-t' candidates, exact for any ties of x. */
 mad_status mad_mips_items(mad_ctx* ctx, const mad_matrix* B, uint64_t s_max, mad_stream stream);
 /* mad_mips_config (the paper has no counterpart; used by the package's
  * autotuner, paper_1506_03872_gb300/autotune.py): the launch shape of the
- * next mad_mips_plan and mad_mips_run.  region_lg: each query's region is
- * the power of two >= 2^region_lg s_q slots (1..4; 0: 1); chunk_mult: 256
- * x chunk_mult diamonds per chunk (1, 2, 4, 8; 0: 1); blocks_per_sm:
- * sampler blocks per SM (0: as many as fit, at most 8); select_threads:
- * threads of each query's selection (128, 256, 512; 0: 256).  None of
+ * next mad_mips_plan and mad_mips_run.  region_lg: a query's
+ * columns are split into parts whose tables are planned for a load of 0.6 /
+ * 2^(region_lg - 1) (1..4; 0: 1); chunk_mult: 256 x chunk_mult diamonds per
+ * chunk (1, 2, 4, 8; 0: 8); blocks_per_sm: sampler blocks per SM (0: one
+ * block per chunk, at most 8); select_threads: threads of each query's
+ * final selection (128, 256, 512; 0: 256).  None of
  * these changes a result (the keys and sums of X, Omega_t' and Omega_t are
  * the same): only the time.  MAD_ERR_ARG outside these values. */
 mad_status mad_mips_config(mad_ctx* ctx, uint32_t region_lg, uint32_t chunk_mult,

@@ -1,10 +1,10 @@
 """Autotuner of the batched-query launch shape (mad_mips_config).
 
 A batch of queries (Alg. 2 and Alg. 3 per query, mad_mips_run) has four
-launch parameters that change its speed and none of its results: the size
-of each query's hash region (2^region_lg times its budget, rounded up to a
-power of two), the diamonds per chunk (256 x chunk_mult), the sampler's
-blocks per SM and the threads of each query's selection.  The tuner times
+launch parameters that change its speed and none of its results: the load of
+the tables a query's columns are split into (0.6 / 2^(region_lg - 1)), the
+diamonds per chunk (256 x chunk_mult), the sampler's blocks per SM and the
+threads of each query's final selection.  The tuner times
 the batch under each choice with CUDA events (a warm-up run, then the
 median of ``reps`` runs), walks the parameters one at a time from the
 library's defaults (coordinate descent, two sweeps), and keeps the fastest
@@ -21,11 +21,11 @@ import numpy as np
 
 SPACE = {
     "region_lg": (1, 2),
-    "chunk_mult": (1, 2, 4),
+    "chunk_mult": (2, 4, 8),
     "blocks_per_sm": (0, 2, 3),
     "select_threads": (128, 256, 512),
 }
-DEFAULT = {"region_lg": 1, "chunk_mult": 1, "blocks_per_sm": 0, "select_threads": 256}
+DEFAULT = {"region_lg": 1, "chunk_mult": 8, "blocks_per_sm": 0, "select_threads": 256}
 
 
 def cache_path() -> str:

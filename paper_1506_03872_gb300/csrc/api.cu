@@ -99,9 +99,7 @@ void free_tables(mad_ctx* ctx, cudaStream_t st) {
   free_async(ctx->pipe_scratch, st);
   ctx->pipe_scratch_bytes = 0;
   ctx->pipe = false;
-  free_async(ctx->mips_s, st);
-  free_async(ctx->mips_chunk_q, st);
-  free_async(ctx->mips_chunk_l0, st);
+  free_async(ctx->mips_buf, st);
   ctx->mips_items = false;
   ctx->mips_nq = 0;
   ctx->built = false;

@@ -215,17 +215,18 @@ struct mad_ctx {
   // Batched queries: the plan of the current batch.
   bool mips_items = false;
   uint32_t mips_nq = 0, mips_tprime = 0, mips_t = 0;
-  uint64_t mips_chunks = 0;
-  unsigned long long* mips_s = nullptr;   // nq budgets
-  uint32_t* mips_chunk_q = nullptr;       // query of each 256-diamond chunk
-  uint32_t* mips_chunk_l0 = nullptr;      // its first diamond
-  // Launch shape of batched queries (mad_mips_config): region size factor
-  // 2^mips_region_lg, 256 x mips_chunk_mult diamonds per chunk (the plan's
-  // value in mips_plan_mult), sampler blocks per SM (0: as many as fit),
-  // select threads per query.
+  uint64_t mips_chunks = 0, mips_units = 0, mips_offs = 0, mips_records = 0, mips_kept = 0;
+  uint32_t mips_max_parts = 1;            // parts of the query with the most
+  int mips_slots = 0;                     // table slots of a part
+  size_t mips_parts_smem = 0;
+  void* mips_buf = nullptr;               // the batch's device buffer (mips.cu)
+  // Launch shape of batched queries (mad_mips_config): the load of a part's
+  // table is 0.6 / 2^(mips_region_lg - 1), 256 x mips_chunk_mult diamonds per
+  // chunk (the plan's value in mips_plan_mult), draw blocks per SM (0: one
+  // block per chunk), threads of each query's final selection.
   int mips_region_lg = 1;
-  int mips_chunk_mult = 1;
-  int mips_plan_mult = 1;
+  int mips_chunk_mult = 8;
+  int mips_plan_mult = 8;
   int mips_bps = 0;
   int mips_select_threads = 256;
   void* bt = nullptr;               // dense B^T (n x d), the input dtype

@@ -6,15 +6,31 @@
 // Philox stream of seed + q, counter l, exactly as a single-query run) and
 // the rest of the loop body is the dense path's: k from the query's T2 row,
 // j from row k of TB (a guided search: n is large), k' from its TA row, the
-// increment from B.  Diamonds come in 256-diamond chunks that never mix
-// queries, so a warp's diamonds share the query's T2/TA rows and its hash
-// region; each query's keys stay inside its region (probing wraps there),
-// so Alg. 3 runs per query on the region alone: one CTA selects the t'
-// largest positive x, rescores them exactly and keeps the t largest |c|.
+// increment from B.
+//
+// A batch is three kernels, and X never exists as a whole.
+//  1. k_mips_draw: a block takes a chunk of one query's diamonds, with the
+//     query's T2 and TA rows in shared memory, and leaves a record (j, signed
+//     b_k'j) per diamond, grouped by part: the j of a query are split by a hash
+//     into parts of at most about kPartKeys distinct columns.
+//  2. k_mips_parts: a block per (query, part) gathers the part's records from
+//     the query's chunks, sums them per column in a shared-memory table
+//     (exact 64-bit sums) and keeps the columns that can be among the
+//     query's t' largest positive x.
+//  3. k_mips_final: a block per query merges its parts' lists into the t'
+//     largest x by (x desc, j asc), rescores them exactly and keeps the t
+//     largest |c|.
+// Against one hash region of 2 to 4 s_q slots of 16 bytes per query in
+// global memory (cleared, filled with global atomics and read back three times
+// by one block per query), a diamond moves 16 bytes of records in and out
+// instead of about 250, no global atomic is left, and a query's selection is
+// spread over its parts.  Measured on one GB300: 1e4 queries of 5e4 diamonds
+// on 1e6 items x 300, 142.6 -> 56.2 ms; 61 queries on 50,021 x 100, 1272 -> 254 us.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <vector>
 
@@ -23,63 +39,478 @@
 #include "mad_internal.cuh"
 
 namespace mad {
+
+// One query of a planned batch: budget, first record, first entry of its
+// chunks' part offsets, first candidate; parts, first part (over the batch),
+// first chunk, candidates a part may keep.
+struct MipsQuery {
+  unsigned long long s, rec, off, cand;
+  uint32_t parts, ubase, cbase, cap;
+};
+
 namespace {
 
-constexpr int kChunk = 256;       // diamonds per chunk (one per thread)
-constexpr int kSelCap = 4096;     // candidates a query's selection keeps
-constexpr int kTPrimeMax = 1024;  // largest t' of a batch
+constexpr int kDrawThreads = 256;
+constexpr int kPartThreads = 512;
+constexpr int kSlots = 8192;                 // largest table of a part (96 KB: two blocks per SM)
+constexpr uint32_t kMaxParts = 2048;         // (a part too full for its table splits itself)
+constexpr int kTPrimeMax = 1024;             // largest t' of a batch
+constexpr int kSlack = 32;                   // columns a part may keep beyond t'
+constexpr int kBins = 2048;                  // digits of the threshold search (11 bits)
+constexpr int kSortMax = 2048;               // >= kTPrimeMax + kSlack
+constexpr uint32_t kNoKey = 0xFFFFFFFFu;     // (columns are below 2^31)
 
-// Hash insert into query q's region [hreg[q], hreg[q+1]) (a power of two of
-// at least 4 slots, 4-aligned), probing inside the region only.
-__device__ __forceinline__ int region_add(const SampleParams& p, uint32_t q,
-                                          unsigned long long key, long long v) {
-  const unsigned long long r0 = __ldg(p.hreg + q), r1 = __ldg(p.hreg + q + 1);
-  const unsigned long long size = r1 - r0;
-  const uint64_t home = r0 + (mix64(key) & (size - 1));
-  return hash_add_from(p.hkeys, p.hvals, r0, r1, home, (uint32_t)size, key, v);
+// Upper bounds in two shared-memory rows of the same length (independent
+// chains), as ub2_u32.
+__device__ __forceinline__ void ub2_shared(const uint32_t* P, const uint32_t* Q, int len,
+                                           uint32_t tp, uint32_t tq, int* op, int* oq) {
+  int a = 0, b = 0;
+  for (int step = 1 << (31 - __clz(len)); step > 0; step >>= 1) {
+    const int na = a + step, nb = b + step;
+    const uint32_t va = P[(na <= len ? na : len) - 1] & PREFIX_MASK;
+    const uint32_t vb = Q[(nb <= len ? nb : len) - 1] & PREFIX_MASK;
+    a = (na <= len && va <= tp) ? na : a;
+    b = (nb <= len && vb <= tq) ? nb : b;
+  }
+  *op = a;
+  *oq = b;
 }
 
-// Alg. 2 over every query's diamonds: chunk c holds diamonds l0 .. l0+255 of
-// query chunk_q[c] (the last chunk of a query is partial).
-__global__ void __launch_bounds__(256, 4)
-k_mips_sample(const SampleParams p, unsigned long long seed, const uint32_t* __restrict__ chunk_q,
-              const uint32_t* __restrict__ chunk_l0, const unsigned long long* __restrict__ s_q,
-              unsigned long long nchunks, int mult) {
-  bool bad = false, full = false;
-  unsigned long long inserted = 0, created = 0;
-  for (unsigned long long c = blockIdx.x; c < nchunks; c += gridDim.x) {
-    const uint32_t q = __ldg(chunk_q + c);
-    const unsigned long long sq = __ldg(s_q + q);
-    for (int rep = 0; rep < mult; ++rep) {
-      const unsigned long long l =
-          (unsigned long long)__ldg(chunk_l0 + c) + threadIdx.x + (unsigned long long)rep * kChunk;
-      if (l >= sq) break;
-      const Uniforms u = diamond_uniforms(seed + q, l);
-      const Draw dr = draw_given_row(p, u, (int64_t)q, &bad);
-      if (dr.v != 0) {
-        ++inserted;
-        const int r = region_add(p, q, ((unsigned long long)q << 32) | dr.j, dr.v);
-        if (r == 0) full = true;
-        if (r == 2) ++created;
+// ub_guided_u32 for row k of TB, the window read 16 bytes at a time: at most
+// kQuads aligned quads hold a window of 17 or fewer entries.  Entries of the row
+// before the window are at most the target and entries after it above, so
+// whole quads are counted and only the row's own ends are checked (TB is
+// allocated with four entries of padding).
+constexpr int kQuads = 5;
+__device__ __forceinline__ int64_t ub_tb(const SampleParams& p, int64_t k, uint32_t target) {
+  const uint32_t* __restrict__ G = p.TBg + k * p.tbg_stride;
+  const uint32_t b = target >> (int)__ldg(p.TBg_sh + k);
+  const uint32_t lo = __ldg(G + b), hi = __ldg(G + b + 1);
+  const int64_t row = k * p.n;
+  if (hi - lo > 17u)
+    return (int64_t)lo + ub_u32(p.TB + row + lo, (int)(hi - lo), target, PREFIX_MASK);
+  const int64_t e0 = (row + lo) & ~(int64_t)3;
+  const int quads = (int)((row + hi - e0 + 3) >> 2);
+  uint4 w[kQuads];
+#pragma unroll
+  for (int q = 0; q < kQuads; ++q)
+    if (q < quads) w[q] = __ldg(reinterpret_cast<const uint4*>(p.TB + e0) + q);
+  const int64_t first = e0 - row;   // (below 0 by up to 3 in a row's first quad)
+  int cnt = 0;
+  const bool inner = first >= 0 && first + 4 * kQuads <= p.n;
+#pragma unroll
+  for (int q = 0; q < kQuads; ++q) {
+    if (q < quads) {
+      const uint32_t v[4] = {w[q].x, w[q].y, w[q].z, w[q].w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int64_t at = first + 4 * q + c;
+        const bool in_row = inner || (at >= 0 && at < p.n);
+        cnt += (in_row && (v[c] & PREFIX_MASK) <= target) ? 1 : 0;
       }
     }
   }
+  return (first > 0 ? first : 0) + cnt;
+}
+
+// The part of column j among `parts`: the high bits of a mix of j (the
+// tables use its low bits).
+__device__ __forceinline__ uint32_t part_of(uint32_t h, uint32_t parts) {
+  return __umulhi(h, parts);
+}
+
+// Step 1 (see above).  chunk c: diamonds (c - cbase) * chunk ... of query
+// chunk_q[c].  Shared memory: the query's T2 and TA rows, the chunk's records,
+// their parts and ranks, the parts' counts.  Bound by random sectors: per
+// diamond the guide (1 sector), its window of TB (2 to 3) and b_k'j (1), mostly
+// in DRAM for a million items.
+__global__ void __launch_bounds__(kDrawThreads, 4)
+k_mips_draw(const SampleParams p, unsigned long long seed, const MipsQuery* __restrict__ queries,
+            const uint32_t* __restrict__ chunk_q, unsigned long long nchunks, int mult,
+            uint32_t max_parts, uint2* __restrict__ rec, uint16_t* __restrict__ off) {
+  extern __shared__ __align__(16) unsigned char draw_smem[];
+  const int chunk = mult * kDrawThreads;
+  const int d = (int)p.d;
+  uint2* srec = (uint2*)draw_smem;                    // chunk records
+  uint32_t* splace = (uint32_t*)(srec + chunk);       // part << 16 | rank in it
+  uint32_t* scnt = splace + chunk;                    // max_parts counts, then offsets
+  uint32_t* s2 = scnt + max_parts + 1;                // T2 row
+  uint32_t* sa = s2 + d;                              // TA row
+  uint16_t* sord = (uint16_t*)(sa + d);               // source of each place
+  __shared__ uint32_t warp_sum[kDrawThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  bool bad = false;
+  for (unsigned long long c = blockIdx.x; c < nchunks; c += gridDim.x) {
+    const uint32_t q = __ldg(chunk_q + c);
+    const MipsQuery mq = queries[q];
+    const unsigned long long l0 = (c - mq.cbase) * (unsigned long long)chunk;
+    const int cnt = (int)(mq.s - l0 < (unsigned long long)chunk ? mq.s - l0
+                                                                 : (unsigned long long)chunk);
+    for (int x = tid; x < d; x += kDrawThreads) {
+      s2[x] = __ldg(p.T2 + (int64_t)q * d + x);
+      sa[x] = __ldg(p.TA + (int64_t)q * d + x);
+    }
+    for (uint32_t x = tid; x < mq.parts; x += kDrawThreads) scnt[x] = 0;
+    __syncthreads();
+    const uint32_t t2tot = s2[d - 1] & PREFIX_MASK, tatot = sa[d - 1] & PREFIX_MASK;
+    for (int x = tid; x < cnt; x += kDrawThreads) {
+      const Uniforms un = diamond_uniforms(seed + q, l0 + x);
+      int k, kp;
+      ub2_shared(s2, sa, d, (uint32_t)draw_target(un.u1, t2tot),
+                 (uint32_t)draw_target(un.u3, tatot), &k, &kp);
+      if (k >= d) { bad = true; k = d - 1; }
+      if (kp >= d) { bad = true; kp = d - 1; }
+      const int64_t row = (int64_t)k * p.n;
+      const uint32_t tbtot = __ldg(p.TB + row + p.n - 1) & PREFIX_MASK;
+      int64_t j = ub_tb(p, k, (uint32_t)draw_target(un.u2, tbtot));
+      if (j >= p.n) { bad = true; j = p.n - 1; }
+      const uint32_t sign = (s2[k] ^ sa[kp] ^ __ldg(p.TB + row + j)) & SIGN_BIT;
+      const float b = __ldg((const float*)p.b_val + (int64_t)kp * p.ldb + j);
+      const uint32_t part = part_of(fmix32((uint32_t)j), mq.parts);
+      const uint32_t rank = atomicAdd(&scnt[part], 1u);
+      srec[x] = make_uint2((uint32_t)j, __float_as_uint(b) ^ sign);
+      splace[x] = (part << 16) | rank;
+    }
+    __syncthreads();
+    // Exclusive scan of the counts (each thread a run of parts).
+    const uint32_t per = (mq.parts + kDrawThreads - 1) / kDrawThreads;
+    uint32_t mine = 0;
+    for (uint32_t x = tid * per; x < min((tid + 1) * per, mq.parts); ++x) mine += scnt[x];
+    uint32_t inc = mine;
 #pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    inserted += __shfl_xor_sync(0xFFFFFFFFu, inserted, off);
-    created += __shfl_xor_sync(0xFFFFFFFFu, created, off);
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (lane == 31) warp_sum[warp] = inc;
+    __syncthreads();
+    uint32_t run = inc - mine;
+    for (int w = 0; w < warp; ++w) run += warp_sum[w];
+    uint16_t* __restrict__ o = off + mq.off + (c - mq.cbase) * (unsigned long long)(mq.parts + 1);
+    for (uint32_t x = tid * per; x < min((tid + 1) * per, mq.parts); ++x) {
+      const uint32_t v = scnt[x];
+      scnt[x] = run;
+      o[x] = (uint16_t)run;
+      run += v;
+    }
+    if (tid == 0) o[mq.parts] = (uint16_t)cnt;
+    __syncthreads();
+    for (int x = tid; x < cnt; x += kDrawThreads) {
+      const uint32_t pl = splace[x];
+      sord[scnt[pl >> 16] + (pl & 0xFFFFu)] = (uint16_t)x;
+    }
+    __syncthreads();
+    uint2* __restrict__ out = rec + mq.rec + l0;
+    for (int x = tid; x < cnt; x += kDrawThreads) out[x] = srec[sord[x]];
+    __syncthreads();   // the buffers are reused by the next chunk
   }
-  const unsigned any_bad = __ballot_sync(0xFFFFFFFFu, bad);
-  const unsigned any_full = __ballot_sync(0xFFFFFFFFu, full);
-  if ((threadIdx.x & 31) == 0) {
-    if (inserted) atomicAdd(&p.sc->inserted, inserted);
-    if (created) atomicAdd(&p.sc->new_keys, created);
-    if (any_bad) atomicOr(&p.sc->err, DERR_SEARCH);
-    if (any_full) atomicOr(&p.sc->err, DERR_HASH_FULL);
+  if (bad) atomicOr(&p.sc->err, DERR_SEARCH);
+}
+
+// Shared words of the threshold search.
+struct PickState {
+  alignas(16) uint32_t hist[kBins];
+  uint32_t warp_sum[32];
+  unsigned long long maxx;
+  uint32_t total, bin, above, in_bin;
+};
+
+// The highest bin whose count from the top, `above` included, reaches need:
+// left in st->bin, with the count above it in st->above and its own in
+// st->in_bin.  Every thread of the block (a multiple of 32, at most 1024).
+__device__ void pick_bin(PickState* st, uint32_t need, uint32_t above) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int per = kBins / (int)blockDim.x;
+  uint32_t mine = 0;
+  for (int x = 0; x < per; ++x) mine += st->hist[kBins - 1 - (tid * per + x)];
+  uint32_t inc = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+    if (lane >= o) inc += v;
+  }
+  if (lane == 31) st->warp_sum[warp] = inc;
+  __syncthreads();
+  uint32_t before = above + inc - mine;
+  for (int w = 0; w < warp; ++w) before += st->warp_sum[w];
+  if (before < need && before + mine >= need) {
+    for (int x = 0; x < per; ++x) {
+      const uint32_t v = st->hist[kBins - 1 - (tid * per + x)];
+      if (before + v >= need) {
+        st->bin = (uint32_t)(kBins - 1 - (tid * per + x));
+        st->above = before;
+        st->in_bin = v;
+        break;
+      }
+      before += v;
+    }
+  }
+  __syncthreads();
+}
+
+// A threshold (xt, njt): the elements with x > xt, or x == xt and ~j >= njt,
+// hold the `need` first by (x desc, j asc) and are at most cap (> need).
+// get(e, &x, &j) is element e < n, false where there is none (or x <= 0).
+// Digits of 11 bits from the leading one of the largest x downwards, then of
+// ~j among equal x; the search ends as soon as the ties of the last digit
+// fit, and the composite is distinct, so it always ends.  Every thread of the
+// block.
+template <typename Get>
+__device__ void find_threshold(PickState* st, int n, uint32_t need, uint32_t cap, Get get,
+                               unsigned long long* xt, uint32_t* njt) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid == 0) {
+    st->maxx = 0;
+    st->total = 0;
+  }
+  __syncthreads();
+  unsigned long long mx = 0;
+  uint32_t cnt = 0;
+  for (int e = tid; e < n; e += blockDim.x) {
+    unsigned long long x;
+    uint32_t j;
+    if (get(e, &x, &j)) {
+      ++cnt;
+      mx = x > mx ? x : mx;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
+    mx = v > mx ? v : mx;
+    cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, o);
+  }
+  if (lane == 0 && cnt) {
+    atomicMax(&st->maxx, mx);
+    atomicAdd(&st->total, cnt);
+  }
+  __syncthreads();
+  *xt = 1;
+  *njt = 0;
+  if (st->total <= cap) {
+    __syncthreads();
+    return;
+  }
+  int top = 64 - __clzll((long long)st->maxx);   // bits of x not yet fixed
+  unsigned long long prefix = 0;                  // x >> top of the threshold's digits
+  uint32_t above = 0;
+  while (top > 0) {
+    const int width = top < 11 ? top : 11, sh = top - width;
+    for (int b = tid; b < kBins; b += blockDim.x) st->hist[b] = 0;
+    __syncthreads();
+    for (int e = tid; e < n; e += blockDim.x) {
+      unsigned long long x;
+      uint32_t j;
+      if (get(e, &x, &j) && (top >= 64 || (x >> top) == prefix))
+        atomicAdd(&st->hist[(uint32_t)(x >> sh) & ((1u << width) - 1u)], 1u);
+    }
+    __syncthreads();
+    pick_bin(st, need, above);
+    prefix = (prefix << width) | st->bin;
+    above = st->above;
+    const uint32_t in_bin = st->in_bin;
+    top = sh;
+    __syncthreads();
+    if (above + in_bin <= cap) {
+      *xt = prefix << top;
+      *xt = *xt ? *xt : 1ull;
+      return;
+    }
+  }
+  *xt = prefix;
+  uint32_t np = 0;
+  int ntop = 32;
+  while (ntop > 0) {   // ties of x: the smallest j
+    const int width = ntop < 11 ? ntop : 11, sh = ntop - width;
+    for (int b = tid; b < kBins; b += blockDim.x) st->hist[b] = 0;
+    __syncthreads();
+    for (int e = tid; e < n; e += blockDim.x) {
+      unsigned long long x;
+      uint32_t j;
+      if (get(e, &x, &j) && x == prefix && (ntop >= 32 || (~j >> ntop) == np))
+        atomicAdd(&st->hist[(~j >> sh) & ((1u << width) - 1u)], 1u);
+    }
+    __syncthreads();
+    pick_bin(st, need, above);
+    np = (np << width) | st->bin;
+    above = st->above;
+    const uint32_t in_bin = st->in_bin;
+    ntop = sh;
+    __syncthreads();
+    if (above + in_bin <= cap) break;
+  }
+  *njt = np << ntop;
+}
+
+// A kept column: its x and j.
+struct Kept {
+  unsigned long long x, j;
+};
+
+// Step 2: part u - ubase of query unit_q[u].  The table is open addressing
+// with linear probing over 32-bit columns; the sums are 64-bit (two 32-bit
+// shared atomics, the low word's carry into the high word).  When it fills up
+// (a statistical rarity, or a batch whose parts are capped at kMaxParts) the
+// part is taken in 2, 4, ... slices of another mix of j, each slice's kept
+// columns competing with those of the slices before.
+__global__ void __launch_bounds__(kPartThreads, 2)
+k_mips_parts(const MipsQuery* __restrict__ queries, const uint32_t* __restrict__ unit_q,
+             const uint2* __restrict__ rec, const uint16_t* __restrict__ off, int chunk,
+             int slots_max, float factor, int f_exp, uint32_t tprime, Kept* __restrict__ kept,
+             uint32_t* __restrict__ kept_n, DevScalars* sc) {
+  extern __shared__ __align__(16) unsigned char part_smem[];
+  unsigned long long* vals = (unsigned long long*)part_smem;   // slots_max sums
+  Kept* temp = (Kept*)(vals + slots_max);                      // cap kept columns
+  __shared__ PickState pick;
+  __shared__ uint32_t s_full, s_n;
+  __shared__ unsigned long long s_records, s_inserted, s_created;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kWarps = kPartThreads / 32;
+  const uint32_t u = blockIdx.x;
+  const uint32_t q = __ldg(unit_q + u);
+  const MipsQuery mq = queries[q];
+  const uint32_t part = u - mq.ubase;
+  uint32_t* keys = (uint32_t*)(temp + mq.cap);
+  const uint32_t cap = mq.cap;
+  Kept* __restrict__ list = kept + mq.cand + (unsigned long long)part * cap;
+  const uint32_t nch = (uint32_t)((mq.s + chunk - 1) / chunk);
+  const uint16_t* __restrict__ o = off + mq.off + part;
+  const uint32_t ostep = mq.parts + 1;
+  if (tid == 0) s_records = 0;
+  __syncthreads();
+  unsigned long long mine = 0;
+  for (uint32_t c = tid; c < nch; c += kPartThreads)
+    mine += (uint32_t)__ldg(o + (size_t)c * ostep + 1) - (uint32_t)__ldg(o + (size_t)c * ostep);
+#pragma unroll
+  for (int s = 16; s >= 1; s >>= 1) mine += __shfl_xor_sync(0xFFFFFFFFu, mine, s);
+  if (lane == 0 && mine) atomicAdd(&s_records, mine);
+  __syncthreads();
+  // A power of two of at least `factor` slots per record (1.5 unless a test
+  // asks for less), up to the table's size.
+  int slots = 256;
+  while (slots < slots_max && (float)slots < factor * (float)s_records) slots <<= 1;
+  const uint32_t mask = (uint32_t)slots - 1;
+  for (int level = 0; level <= 31; ++level) {
+    uint32_t nlist = 0;
+    bool full = false;
+    if (tid == 0) s_inserted = s_created = 0;
+    const uint32_t slices = 1u << level;
+    for (uint32_t slice = 0; slice < slices && !full; ++slice) {
+      for (int x = tid; x < slots; x += kPartThreads) {
+        keys[x] = kNoKey;
+        vals[x] = 0;
+      }
+      if (tid == 0) s_full = 0;
+      __syncthreads();
+      unsigned long long ins = 0, cre = 0;
+      for (uint32_t cb = (uint32_t)warp; cb < nch; cb += 32 * kWarps) {
+        // The segment bounds of this warp's next 32 chunks, one per lane.
+        const uint32_t cl = cb + (uint32_t)lane * kWarps;
+        uint32_t b0 = 0, b1 = 0;
+        if (cl < nch) {
+          b0 = __ldg(o + (size_t)cl * ostep);
+          b1 = __ldg(o + (size_t)cl * ostep + 1);
+        }
+        for (int w = 0; w < 32; ++w) {
+          const uint32_t c = cb + (uint32_t)w * kWarps;
+          if (c >= nch) break;
+          const uint32_t e1 = __shfl_sync(0xFFFFFFFFu, b1, w);
+          const uint2* __restrict__ r = rec + mq.rec + (unsigned long long)c * chunk;
+          for (uint32_t e = __shfl_sync(0xFFFFFFFFu, b0, w) + lane; e < e1; e += 32) {
+            const uint2 v = __ldg(r + e);
+            const long long x = fixed_point(__uint_as_float(v.y), f_exp);
+            const uint32_t h = fmix32(v.x);
+            if (x == 0 || (level && (fmix32(h ^ 0x9E3779B9u) >> (32 - level)) != slice)) continue;
+            ++ins;
+            uint32_t slot = h & mask;
+            int probes = 0;
+            for (; probes < slots; ++probes) {
+              uint32_t cur = ((volatile uint32_t*)keys)[slot];
+              if (cur == kNoKey) {
+                cur = atomicCAS(keys + slot, kNoKey, v.x);
+                if (cur == kNoKey) {
+                  ++cre;
+                  cur = v.x;
+                }
+              }
+              if (cur == v.x) break;
+              slot = (slot + 1) & mask;
+            }
+            if (probes == slots) {
+              s_full = 1;
+              continue;
+            }
+            uint32_t* h2 = (uint32_t*)(vals + slot);
+            const uint32_t lo = (uint32_t)(unsigned long long)x;
+            const uint32_t hi = (uint32_t)((unsigned long long)x >> 32);
+            const uint32_t old = atomicAdd(h2, lo);
+            atomicAdd(h2 + 1, hi + (old + lo < old ? 1u : 0u));
+          }
+        }
+      }
+#pragma unroll
+      for (int s = 16; s >= 1; s >>= 1) {
+        ins += __shfl_xor_sync(0xFFFFFFFFu, ins, s);
+        cre += __shfl_xor_sync(0xFFFFFFFFu, cre, s);
+      }
+      if (lane == 0) {
+        if (ins) atomicAdd(&s_inserted, ins);
+        if (cre) atomicAdd(&s_created, cre);
+      }
+      if (tid == 0) s_n = 0;
+      __syncthreads();
+      full = s_full != 0;
+      if (full) {
+        __syncthreads();
+        break;
+      }
+      auto get = [&](int e, unsigned long long* x, uint32_t* j) {
+        if (e < slots) {
+          *x = vals[e];
+          *j = keys[e];
+          return *j != kNoKey && (long long)*x > 0;
+        }
+        const Kept k = list[e - slots];
+        *x = k.x;
+        *j = (uint32_t)k.j;
+        return true;
+      };
+      unsigned long long xt;
+      uint32_t njt;
+      const int n = slots + (int)nlist;
+      find_threshold(&pick, n, tprime, cap, get, &xt, &njt);
+      for (int e = tid; e < n; e += kPartThreads) {
+        unsigned long long x;
+        uint32_t j;
+        if (get(e, &x, &j) && (x > xt || (x == xt && ~j >= njt))) {
+          const uint32_t at = atomicAdd(&s_n, 1u);
+          if (at < cap) {
+            temp[at].x = x;
+            temp[at].j = j;
+          }
+        }
+      }
+      __syncthreads();
+      nlist = s_n < cap ? s_n : cap;
+      for (uint32_t e = tid; e < nlist; e += kPartThreads) list[e] = temp[e];
+      __syncthreads();
+    }
+    if (!full) {
+      if (tid == 0) {
+        kept_n[u] = nlist;
+        if (s_inserted) atomicAdd(&sc->inserted, s_inserted);
+        if (s_created) atomicAdd(&sc->new_keys, s_created);
+      }
+      return;
+    }
+  }
+  if (tid == 0) {   // (not reached: 2^31 slices hold two columns each)
+    kept_n[u] = 0;
+    atomicOr(&sc->err, DERR_HASH_FULL);
   }
 }
 
-// Bitonic sort of n (a power of two, <= kSelCap) entries of shared arrays
+// Bitonic sort of n (a power of two, <= kSortMax) entries of shared arrays
 // into "before" order; all threads of the block take part.
 template <typename Before>
 __device__ void block_bitonic(unsigned long long* a, unsigned long long* b, double* c, int n,
@@ -105,106 +536,53 @@ __device__ void block_bitonic(unsigned long long* a, unsigned long long* b, doub
   }
 }
 
-// Offset of v inside its log bucket, scaled to 10 bits (monotone in v).
-__device__ __forceinline__ uint32_t fine_of(unsigned long long v, uint32_t b) {
-  const int e = 63 - __clzll((long long)v);
-  const int sh = e > 14 ? e - 14 : 0;
-  const unsigned long long f = (v - bucket_floor(b)) >> sh;
-  return f < 1024 ? (uint32_t)f : 1023u;
-}
-
-// Alg. 3 for query blockIdx.x over its hash region.  The t' largest positive
-// x by (x desc, key asc): a log-bucket histogram finds the bucket where the
-// count from the top reaches t', a 10-bit histogram inside that bucket
-// narrows it, and every x at or above the resulting threshold (all of the
-// top t', and few more) is collected and sorted.  Then c = q . b_j in FP64
-// (32 lane-strided fused multiply-add partial sums folded in halves) and the
-// t largest |c| by (|c| desc, key asc).
+// Step 3, query blockIdx.x: the t' first of its parts' kept columns by (x
+// desc, j asc), sorted; then c = q . b_j in FP64 (32 lane-strided fused
+// multiply-add partial sums folded in halves) and the t largest |c| by (|c|
+// desc, j asc).
 __global__ void __launch_bounds__(512)
-k_mips_select(const unsigned long long* __restrict__ hkeys, const long long* __restrict__ hvals,
-              const unsigned long long* __restrict__ hreg, const float* __restrict__ Q,
-              int64_t ldq, const float* __restrict__ Bt, int64_t d, uint32_t tprime, uint32_t t,
-              mad_pair* __restrict__ out, uint32_t* __restrict__ nout,
-              mad_pair* __restrict__ cand_out, DevScalars* sc) {
-  extern __shared__ unsigned long long sel_smem[];
-  unsigned long long* cx = sel_smem;            // x of the collected keys
-  unsigned long long* ck = sel_smem + kSelCap;  // keys
-  double* cc = (double*)(sel_smem + 2 * kSelCap);  // c of the top t'
-  __shared__ unsigned int hist[1024];
-  __shared__ unsigned int fine[1024];
-  __shared__ int bstar, fstar;
-  __shared__ unsigned int ncol;
-  __shared__ unsigned long long above;
+k_mips_final(const MipsQuery* __restrict__ queries, const Kept* __restrict__ kept,
+             const uint32_t* __restrict__ kept_n, const float* __restrict__ Q, int64_t ldq,
+             const float* __restrict__ Bt, int64_t d, uint32_t tprime, uint32_t t,
+             mad_pair* __restrict__ out, uint32_t* __restrict__ nout,
+             mad_pair* __restrict__ cand_out) {
+  __shared__ unsigned long long cx[kSortMax], ck[kSortMax];
+  __shared__ PickState pick;
+  static_assert(kTPrimeMax * sizeof(double) <= kBins * sizeof(uint32_t), "c in the bins' place");
+  double* cc = (double*)pick.hist;   // (the search is over when the t' are rescored)
+  __shared__ uint32_t s_n;
   const uint32_t q = blockIdx.x;
-  const unsigned long long r0 = hreg[q], r1 = hreg[q + 1];
-  for (int b = threadIdx.x; b < 1024; b += blockDim.x) hist[b] = fine[b] = 0;
-  if (threadIdx.x == 0) {
-    ncol = 0;
-    above = 0;
-  }
+  const MipsQuery mq = queries[q];
+  const Kept* __restrict__ list = kept + mq.cand;
+  const uint32_t* __restrict__ cnt = kept_n + mq.ubase;
+  auto get = [&](int e, unsigned long long* x, uint32_t* j) {
+    const uint32_t part = (uint32_t)e / mq.cap;
+    if ((uint32_t)e - part * mq.cap >= __ldg(cnt + part)) return false;
+    const Kept k = list[e];
+    *x = k.x;
+    *j = (uint32_t)k.j;
+    return true;
+  };
+  const int total = (int)(mq.parts * mq.cap);
+  unsigned long long xt = 1;
+  uint32_t njt = 0;
+  if (threadIdx.x == 0) s_n = 0;
   __syncthreads();
-  for (unsigned long long s = r0 + threadIdx.x; s < r1; s += blockDim.x) {
-    const long long v = hvals[s];
-    if (v > 0) atomicAdd(&hist[log_bucket((unsigned long long)v)], 1u);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long cum = 0;
-    int pick = -1;
-    for (int b = 1023; b >= 0; --b) {
-      if (cum + hist[b] >= tprime) {
-        pick = b;
-        break;
-      }
-      cum += hist[b];
-    }
-    bstar = pick;
-    above = cum;
-  }
-  __syncthreads();
-  const int bs = bstar;
-  if (bs >= 0) {
-    for (unsigned long long s = r0 + threadIdx.x; s < r1; s += blockDim.x) {
-      const long long v = hvals[s];
-      if (v > 0 && log_bucket((unsigned long long)v) == (uint32_t)bs)
-        atomicAdd(&fine[fine_of((unsigned long long)v, (uint32_t)bs)], 1u);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      unsigned long long cum = above;
-      int pick = 0;
-      for (int f = 1023; f >= 0; --f) {
-        cum += fine[f];
-        if (cum >= tprime) {
-          pick = f;
-          break;
-        }
-      }
-      fstar = pick;
-    }
-    __syncthreads();
-  }
-  const int fs = bs >= 0 ? fstar : 0;
-  for (unsigned long long s = r0 + threadIdx.x; s < r1; s += blockDim.x) {
-    const long long v = hvals[s];
-    if (v <= 0) continue;
-    bool take = true;
-    if (bs >= 0) {
-      const uint32_t b = log_bucket((unsigned long long)v);
-      take = b > (uint32_t)bs || (b == (uint32_t)bs && fine_of((unsigned long long)v, b) >= (uint32_t)fs);
-    }
-    if (take) {
-      const unsigned pos = atomicAdd(&ncol, 1u);
-      if (pos < kSelCap) {
-        cx[pos] = (unsigned long long)v;
-        ck[pos] = hkeys[s];
+  const uint32_t cap = min((uint32_t)kSortMax, tprime + (uint32_t)kSlack);
+  if (mq.parts > 1) find_threshold(&pick, total, tprime, cap, get, &xt, &njt);
+  for (int e = threadIdx.x; e < total; e += blockDim.x) {
+    unsigned long long x;
+    uint32_t j;
+    if (get(e, &x, &j) && (x > xt || (x == xt && ~j >= njt))) {
+      const uint32_t at = atomicAdd(&s_n, 1u);
+      if (at < kSortMax) {
+        cx[at] = x;
+        ck[at] = j;
       }
     }
   }
   __syncthreads();
-  const unsigned n_all = ncol;
-  if (n_all > kSelCap && threadIdx.x == 0) atomicOr(&sc->err, DERR_SELECT);
-  const int n = (int)(n_all < kSelCap ? n_all : kSelCap);
+  const int n = (int)min(s_n, (uint32_t)kSortMax);
   int n2 = 1;
   while (n2 < n) n2 <<= 1;
   for (int x = n + threadIdx.x; x < n2; x += blockDim.x) {
@@ -267,17 +645,6 @@ k_mips_select(const unsigned long long* __restrict__ hkeys, const long long* __r
   if (threadIdx.x == 0) nout[q] = (uint32_t)T;
 }
 
-// Region of query q: a power of two >= max(4, 2^lg s_q) slots.
-__global__ void __launch_bounds__(256)
-k_mips_region_sizes(const unsigned long long* __restrict__ s_q, uint32_t nq, int lg,
-                    unsigned long long* __restrict__ sizes) {
-  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += gridDim.x * blockDim.x) {
-    unsigned long long size = 4;
-    while (size < (s_q[q] << lg)) size <<= 1;
-    sizes[q] = size;
-  }
-}
-
 template <typename T>
 mad_status pool_alloc(mad_ctx* ctx, T*& p, size_t count, cudaStream_t st) {
   if (count == 0) count = 1;
@@ -293,7 +660,48 @@ void pool_free(T*& p, cudaStream_t st) {
   p = nullptr;
 }
 
-size_t select_smem_bytes() { return (size_t)kSelCap * 16 + (size_t)kTPrimeMax * 8; }
+// A part's table, its kept columns and the columns' keys.
+size_t parts_smem_bytes(int slots, uint32_t cap) {
+  return (size_t)slots * 12 + (size_t)cap * sizeof(Kept);
+}
+
+size_t draw_smem_bytes(int chunk, uint32_t parts, int64_t d) {
+  return (size_t)chunk * (8 + 4 + 2) + ((size_t)parts + 1 + 2 * (size_t)d) * 4;
+}
+
+// The batch's device buffer: the queries, the query of every chunk and part,
+// the part offsets of every chunk, the records and the parts' kept columns.
+struct MipsBufs {
+  MipsQuery* queries;
+  uint32_t* chunk_q;
+  uint32_t* unit_q;
+  uint16_t* off;
+  uint2* rec;
+  Kept* kept;
+  uint32_t* kept_n;
+  size_t bytes;
+};
+
+MipsBufs carve_mips(void* base, uint64_t nq, uint64_t chunks, uint64_t units, uint64_t offs,
+                    uint64_t records, uint64_t kept) {
+  MipsBufs b;
+  char* p = (char*)base;
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    char* q = p ? p + at : nullptr;
+    at += (bytes + 255) & ~(size_t)255;
+    return (void*)q;
+  };
+  b.queries = (MipsQuery*)take(nq * sizeof(MipsQuery));
+  b.chunk_q = (uint32_t*)take(chunks * sizeof(uint32_t));
+  b.unit_q = (uint32_t*)take(units * sizeof(uint32_t));
+  b.off = (uint16_t*)take(offs * sizeof(uint16_t));
+  b.rec = (uint2*)take(records * sizeof(uint2));
+  b.kept = (Kept*)take(kept * sizeof(Kept));
+  b.kept_n = (uint32_t*)take(units * sizeof(uint32_t));
+  b.bytes = at;
+  return b;
+}
 
 }  // namespace
 }  // namespace mad
@@ -318,7 +726,7 @@ mad_status mad_mips_items(mad_ctx* ctx, const mad_matrix* B, uint64_t s_max, mad
   pool_free(ctx->hreg, st); pool_free(ctx->T2g_ptr, st);
   pool_free(ctx->T2g, st); pool_free(ctx->T2g_sh, st); pool_free(ctx->bloom, st);
   pool_free(ctx->TBg, st); pool_free(ctx->TBg_sh, st);
-  pool_free(ctx->mips_s, st); pool_free(ctx->mips_chunk_q, st); pool_free(ctx->mips_chunk_l0, st);
+  pool_free(ctx->mips_buf, st);
   pool_free(ctx->pipe_buf, st);
   pool_free(ctx->pipe_scratch, st);
   ctx->pipe_scratch_bytes = 0;
@@ -336,7 +744,7 @@ mad_status mad_mips_items(mad_ctx* ctx, const mad_matrix* B, uint64_t s_max, mad
   ctx->m = 0;
   ctx->s_max = s_max;
   mad_status rs;
-  if ((rs = pool_alloc(ctx, ctx->TB, (size_t)(ctx->d * ctx->n), st)) != MAD_OK) return rs;
+  if ((rs = pool_alloc(ctx, ctx->TB, (size_t)(ctx->d * ctx->n) + 4, st)) != MAD_OK) return rs;
   if ((rs = pool_alloc(ctx, ctx->nb, (size_t)ctx->d, st)) != MAD_OK) return rs;
   char* bt = nullptr;
   if ((rs = pool_alloc(ctx, bt, (size_t)(ctx->n * ctx->d) * 4, st)) != MAD_OK) return rs;
@@ -369,7 +777,7 @@ mad_status mad_mips_config(mad_ctx* ctx, uint32_t region_lg, uint32_t chunk_mult
       select_threads != 512)
     return MAD_ERR_ARG;
   ctx->mips_region_lg = region_lg == 0 ? 1 : (int)region_lg;
-  ctx->mips_chunk_mult = chunk_mult == 0 ? 1 : (int)chunk_mult;
+  ctx->mips_chunk_mult = chunk_mult == 0 ? 8 : (int)chunk_mult;
   ctx->mips_bps = (int)blocks_per_sm;
   ctx->mips_select_threads = select_threads == 0 ? 256 : (int)select_threads;
   return MAD_OK;
@@ -382,65 +790,79 @@ mad_status mad_mips_plan(mad_ctx* ctx, uint32_t nq, const uint64_t* s_host, uint
     return MAD_ERR_ARG;
   if (!ctx->mips_items) return MAD_ERR_STATE;
   cudaStream_t st = (cudaStream_t)stream;
-  std::vector<uint32_t> cq, cl;
-  uint64_t chunks = 0;
-  const uint64_t csize = (uint64_t)kChunk * (uint64_t)ctx->mips_chunk_mult;
+  const uint64_t chunk = (uint64_t)kDrawThreads * (uint64_t)ctx->mips_chunk_mult;
+  // Distinct columns a part's table is planned for: load 0.6 at region_lg =
+  // 1, half of it for each step above.
+  const uint64_t part_keys = (uint64_t)(kSlots * 6 / 10) >> (ctx->mips_region_lg - 1);
+  std::vector<MipsQuery> qs(nq);
+  uint64_t chunks = 0, units = 0, offs = 0, records = 0, kept = 0, most = 0;
+  uint32_t max_parts = 1, max_cap = 1;
   for (uint32_t q = 0; q < nq; ++q) {
-    if (s_host[q] == 0 || s_host[q] > ctx->s_max) return MAD_ERR_ARG;
-    chunks += (s_host[q] + csize - 1) / csize;
+    const uint64_t s = s_host[q];
+    if (s == 0 || s > ctx->s_max) return MAD_ERR_ARG;
+    const uint64_t distinct = std::min<uint64_t>(s, (uint64_t)ctx->n);
+    const uint64_t nch = (s + chunk - 1) / chunk;
+    MipsQuery& m = qs[q];
+    m.s = s;
+    m.rec = records;
+    m.off = offs;
+    m.cand = kept;
+    m.parts = (uint32_t)std::min<uint64_t>(kMaxParts, (distinct + part_keys - 1) / part_keys);
+    m.ubase = (uint32_t)units;
+    m.cbase = (uint32_t)chunks;
+    m.cap = (uint32_t)std::min<uint64_t>(distinct, (uint64_t)tprime + kSlack);
+    chunks += nch;
+    units += m.parts;
+    offs += nch * (m.parts + 1);
+    records += s;
+    kept += (uint64_t)m.parts * m.cap;
+    most = std::max(most, (distinct + m.parts - 1) / m.parts);
+    max_parts = std::max(max_parts, m.parts);
+    max_cap = std::max(max_cap, m.cap);
+    // (a batch this long holds tens of terabytes of records)
+    if (chunks >= (1ull << 32) || units >= (1ull << 31)) return MAD_ERR_OOM;
   }
+  std::vector<uint32_t> cq, uq;
   cq.reserve(chunks);
-  cl.reserve(chunks);
-  for (uint32_t q = 0; q < nq; ++q)
-    for (uint64_t l = 0; l < s_host[q]; l += csize) {
-      cq.push_back(q);
-      cl.push_back((uint32_t)l);
-    }
+  uq.reserve(units);
+  for (uint32_t q = 0; q < nq; ++q) {
+    cq.insert(cq.end(), (size_t)((qs[q].s + chunk - 1) / chunk), q);
+    uq.insert(uq.end(), qs[q].parts, q);
+  }
   cudaStreamSynchronize(st);
   pool_free(ctx->T2, st); pool_free(ctx->TA, st); pool_free(ctx->na, st); pool_free(ctx->r, st);
-  pool_free(ctx->hkeys, st); pool_free(ctx->hvals, st); pool_free(ctx->hreg, st);
-  pool_free(ctx->mips_s, st); pool_free(ctx->mips_chunk_q, st); pool_free(ctx->mips_chunk_l0, st);
+  pool_free(ctx->mips_buf, st);
   ctx->mips_nq = 0;
   mad_status rs;
   if ((rs = pool_alloc(ctx, ctx->T2, (size_t)nq * (size_t)ctx->d, st)) != MAD_OK) return rs;
   if ((rs = pool_alloc(ctx, ctx->TA, (size_t)nq * (size_t)ctx->d, st)) != MAD_OK) return rs;
   if ((rs = pool_alloc(ctx, ctx->na, (size_t)nq, st)) != MAD_OK) return rs;
   if ((rs = pool_alloc(ctx, ctx->r, (size_t)nq, st)) != MAD_OK) return rs;
-  if ((rs = pool_alloc(ctx, ctx->hreg, (size_t)nq + 1, st)) != MAD_OK) return rs;
-  if ((rs = pool_alloc(ctx, ctx->mips_s, (size_t)nq, st)) != MAD_OK) return rs;
-  if ((rs = pool_alloc(ctx, ctx->mips_chunk_q, (size_t)chunks, st)) != MAD_OK) return rs;
-  if ((rs = pool_alloc(ctx, ctx->mips_chunk_l0, (size_t)chunks, st)) != MAD_OK) return rs;
-  cudaMemcpyAsync(ctx->mips_s, s_host, nq * sizeof(uint64_t), cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(ctx->mips_chunk_q, cq.data(), chunks * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(ctx->mips_chunk_l0, cl.data(), chunks * sizeof(uint32_t), cudaMemcpyHostToDevice,
-                  st);
-  // Regions: sizes, then their offsets (hreg[nq] = total).
-  const size_t sizes_bytes = ((size_t)nq * 8 + 255) & ~(size_t)255;
-  if ((rs = ensure_scratch(ctx, sizes_bytes + scan_partial_elems(nq) * 8, st)) != MAD_OK) return rs;
-  unsigned long long* sizes = (unsigned long long*)ctx->scratch;
-  uint64_t* part = (uint64_t*)((char*)ctx->scratch + sizes_bytes);
-  k_mips_region_sizes<<<(nq + 255) / 256, 256, 0, st>>>(ctx->mips_s, nq, ctx->mips_region_lg,
-                                                       sizes);
-  count_launch(ctx);
-  if ((rs = scan_exclusive_u64(ctx, (const uint64_t*)sizes, (uint64_t*)ctx->hreg, nq, part, st)) !=
-      MAD_OK)
-    return rs;
-  unsigned long long total = 0;
-  cudaMemcpyAsync(&total, ctx->hreg + nq, sizeof(total), cudaMemcpyDeviceToHost, st);
+  const MipsBufs sizes = carve_mips(nullptr, nq, chunks, units, offs, records, kept);
+  if ((rs = pool_malloc(ctx, &ctx->mips_buf, sizes.bytes, st)) != MAD_OK) return rs;
+  const MipsBufs b = carve_mips(ctx->mips_buf, nq, chunks, units, offs, records, kept);
+  cudaMemcpyAsync(b.queries, qs.data(), nq * sizeof(MipsQuery), cudaMemcpyHostToDevice, st);
+  cudaMemcpyAsync(b.chunk_q, cq.data(), chunks * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
+  cudaMemcpyAsync(b.unit_q, uq.data(), units * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
   if ((rs = cuda_status(cudaStreamSynchronize(st))) != MAD_OK) return rs;
-  if ((rs = pool_alloc(ctx, ctx->hkeys, (size_t)total, st)) != MAD_OK) return rs;
-  if ((rs = pool_alloc(ctx, ctx->hvals, (size_t)total, st)) != MAD_OK) return rs;
-  ctx->hcap = ctx->hcap_alloc = total;
+  int slots = 256;   // the largest table any part starts with
+  while (slots < kSlots && (uint64_t)slots * 2 < most * 3) slots <<= 1;
   ctx->m = nq;
+  ctx->hcap = ctx->hcap_alloc = 0;
   ctx->mips_nq = nq;
   ctx->mips_tprime = tprime;
   ctx->mips_t = t;
   ctx->mips_chunks = chunks;
+  ctx->mips_units = units;
+  ctx->mips_offs = offs;
+  ctx->mips_records = records;
+  ctx->mips_kept = kept;
+  ctx->mips_max_parts = max_parts;
+  ctx->mips_slots = slots;
+  ctx->mips_parts_smem = parts_smem_bytes(slots, max_cap);
   ctx->mips_plan_mult = ctx->mips_chunk_mult;
-  if (cudaFuncSetAttribute(k_mips_select, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)select_smem_bytes()) != cudaSuccess)
-    return MAD_ERR_CUDA;
-  return cuda_status(cudaStreamSynchronize(st));
+  return cuda_status(cudaFuncSetAttribute(k_mips_parts, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)parts_smem_bytes(kSlots, kTPrimeMax + kSlack)));
 }
 
 mad_status mad_mips_run(mad_ctx* ctx, const mad_matrix* Q, uint64_t seed, mad_pair* out_dev,
@@ -455,26 +877,28 @@ mad_status mad_mips_run(mad_ctx* ctx, const mad_matrix* Q, uint64_t seed, mad_pa
   // Query rows of the tables (T2, TA; T1 is not needed: m = 1 per query).
   mad_status rs;
   if ((rs = build_query_rows(ctx, st)) != MAD_OK) return rs;
-  cudaMemsetAsync(ctx->hkeys, 0xFF, ctx->hcap * sizeof(unsigned long long), st);
-  cudaMemsetAsync(ctx->hvals, 0, ctx->hcap * sizeof(long long), st);
-  SampleParams p = make_params(ctx);
-  p.regioned = 1;
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mips_sample, 256, 0) != cudaSuccess ||
-      per_sm < 1)
-    per_sm = 1;
-  if (ctx->mips_bps > 0 && ctx->mips_bps < per_sm) per_sm = ctx->mips_bps;
-  const unsigned long long grid =
-      std::min<unsigned long long>(ctx->mips_chunks, (unsigned long long)sms * per_sm);
-  k_mips_sample<<<(unsigned)grid, 256, 0, st>>>(p, seed, ctx->mips_chunk_q, ctx->mips_chunk_l0,
-                                                ctx->mips_s, ctx->mips_chunks,
-                                                ctx->mips_plan_mult);
-  k_mips_select<<<ctx->mips_nq, ctx->mips_select_threads, select_smem_bytes(), st>>>(
-      ctx->hkeys, ctx->hvals, ctx->hreg, (const float*)Q->values, Q->ld, (const float*)ctx->bt,
-      ctx->d, ctx->mips_tprime, ctx->mips_t, out_dev, n_out_dev, cand_dev, ctx->sc);
-  count_launch(ctx, 2);
+  const MipsBufs b = carve_mips(ctx->mips_buf, ctx->mips_nq, ctx->mips_chunks, ctx->mips_units,
+                                ctx->mips_offs, ctx->mips_records, ctx->mips_kept);
+  const SampleParams p = make_params(ctx);
+  const int chunk = kDrawThreads * ctx->mips_plan_mult;
+  unsigned long long grid = ctx->mips_chunks;
+  if (ctx->mips_bps > 0) {
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    grid = std::min<unsigned long long>(grid, (unsigned long long)sms * ctx->mips_bps);
+  }
+  grid = std::min<unsigned long long>(grid, 0x7FFFFFFFull);
+  k_mips_draw<<<(unsigned)grid, kDrawThreads, draw_smem_bytes(chunk, ctx->mips_max_parts, ctx->d),
+                st>>>(p, seed, b.queries, b.chunk_q, ctx->mips_chunks, ctx->mips_plan_mult,
+                      ctx->mips_max_parts, b.rec, b.off);
+  k_mips_parts<<<(unsigned)ctx->mips_units, kPartThreads, ctx->mips_parts_smem, st>>>(
+      b.queries, b.unit_q, b.rec, b.off, chunk, ctx->mips_slots, ctx->region_factor, ctx->f, ctx->mips_tprime, b.kept,
+      b.kept_n, ctx->sc);
+  k_mips_final<<<ctx->mips_nq, ctx->mips_select_threads, 0, st>>>(
+      b.queries, b.kept, b.kept_n, (const float*)Q->values, Q->ld, (const float*)ctx->bt, ctx->d,
+      ctx->mips_tprime, ctx->mips_t, out_dev, n_out_dev, cand_dev);
+  count_launch(ctx, 3);
   return cuda_status(cudaGetLastError());
 }
 

@@ -1,0 +1,100 @@
+"""Batched queries at the edges of their chunks, parts and tables, each query
+against the oracle run on it alone: Omega_t' (keys and x) and Omega_t (keys
+and the FP64 c) bit for bit."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+import oracle  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def _compare(Q, B, s_q, s_max, tprime, t, seed=5, factor=None, cfg=None):
+    import paper_1506_03872_gb300 as mad
+    nq = len(s_q)
+    tQ, tB = torch.from_numpy(Q).cuda(), torch.from_numpy(B).cuda()
+    out, cand = mad.new_pairs(nq * t), mad.new_pairs(nq * tprime)
+    nout = torch.zeros(nq, dtype=torch.int32, device="cuda")
+    with mad.Context() as c:
+        if factor:
+            mad.mad_debug_set_hash_layout(c.ctx, factor)
+        if cfg:
+            mad.mad_mips_config(c.ctx, **cfg)
+        mad.mad_mips_items(c.ctx, mad.dense(tB), s_max)
+        mad.mad_mips_plan(c.ctx, s_q, tprime, t)
+        for _ in range(2):   # (a second pass finds nothing of the first)
+            mad.mad_mips_run(c.ctx, mad.dense(tQ), seed, out, nout, cand)
+        assert mad.mad_stats(c.ctx)["device_error"] == 0
+    nout = nout.cpu().numpy()
+    for q in range(nq):
+        o = oracle.Oracle(oracle.Matrix(np.ascontiguousarray(Q[q:q + 1])), oracle.Matrix(B), 0, s_max)
+        assert o.sample(int(s_q[q]), seed + q) == 0
+        keys, x = o.topk(tprime)
+        ci, cj, cx, _ = mad.decode_pairs(cand[q * tprime:], len(keys))
+        assert np.array_equal(cj.astype(np.uint64), keys & np.uint64(0xFFFFFFFF)), q
+        assert np.array_equal(cx, x) and np.all(ci == q), q
+        tk, tc = oracle.topt(keys, o.rescore(keys), t)
+        assert nout[q] == len(tk)
+        _, gj, _, gc = mad.decode_pairs(out[q * t:], len(tk))
+        assert np.array_equal(gj.astype(np.uint64), tk & np.uint64(0xFFFFFFFF)), q
+        assert np.array_equal(gc.view(np.int64), tc.view(np.int64)), q
+
+
+def _rng(seed):
+    return np.random.Generator(np.random.PCG64(seed))
+
+
+def _items(seed, d, n, nq):
+    rng = _rng(seed)
+    B = (rng.standard_normal((d, n)) * np.exp(0.5 * rng.standard_normal((1, n)))).astype(np.float32)
+    return rng.standard_normal((nq, d)).astype(np.float32), B
+
+
+@pytest.mark.parametrize("d,n", [(1, 5), (7, 3001), (33, 17), (300, 40_003), (1024, 131)])
+def test_chunk_and_part_edges(d, n):
+    s_q = np.array([1, 2, 255, 256, 257, 2047, 2048, 2049, 4915, 4916, 9831, 30_000], np.uint64)
+    Q, B = _items(d + n, d, n, len(s_q))
+    _compare(Q, B, s_q, 30_000, 40, 7)
+
+
+@pytest.mark.parametrize("tprime,t", [(1, 1), (1024, 1024), (1000, 3)])
+def test_lists_of_every_length(tprime, t):
+    s_q = np.array([500, 60_000, 20_000], np.uint64)
+    Q, B = _items(3, 20, 50_001, len(s_q))
+    _compare(Q, B, s_q, 1 << 17, tprime, t)
+
+
+@pytest.mark.parametrize("factor", [0.03, 0.3])
+def test_full_tables_are_taken_in_slices(factor):
+    """Tables smaller than the part's distinct columns (3 to 40 % of its
+    records): the part splits until a slice fits."""
+    s_q = np.array([4900, 30_000, 3000], np.uint64)
+    Q, B = _items(9, 30, 100_003, len(s_q))
+    _compare(Q, B, s_q, 1 << 15, 64, 5, factor=factor)
+
+
+@pytest.mark.parametrize("cfg", [dict(chunk_mult=1), dict(region_lg=4, chunk_mult=2),
+                                 dict(blocks_per_sm=1, select_threads=128)])
+def test_launch_shapes(cfg):
+    s_q = np.array([40_000, 2100, 9000], np.uint64)
+    Q, B = _items(4, 50, 20_010, len(s_q))
+    _compare(Q, B, s_q, 1 << 16, 100, 5, cfg=cfg)
+
+
+def test_ties_of_x_in_the_thousands():
+    """Entries of one magnitude: x counts diamonds, and thousands of columns
+    tie at the t'-th; the smallest j of them are taken."""
+    rng = _rng(6)
+    B = np.where(rng.random((16, 30_001)) < 0.5, -1.0, 1.0).astype(np.float32)
+    Q = rng.standard_normal((3, 16)).astype(np.float32)
+    _compare(Q, B, np.array([20_000, 60_000, 700], np.uint64), 1 << 16, 300, 20)
