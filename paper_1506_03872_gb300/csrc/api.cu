@@ -574,7 +574,7 @@ mad_status mad_rescore(mad_ctx* ctx, const mad_pair* cand_dev, uint32_t ncand, u
   double* cvals = (double*)((char*)ctx->scratch + cv_off);
   if ((rs = rescore_items(ctx, cand_dev, ncand, ws.l0, cvals, st)) != MAD_OK) return rs;
   uint64_t nsel = 0;
-  if ((rs = select_list(ctx, ws, ncand, t, 8, &nsel, st)) != MAD_OK) return rs;
+  if ((rs = select_list(ctx, ws, ncand, t, 64, &nsel, st)) != MAD_OK) return rs;
   if ((rs = items_to_pairs(ctx, ws.out, nsel, cand_dev, cvals, out_dev, st)) != MAD_OK) return rs;
   DevScalars hs;
   if ((rs = read_scalars(ctx, &hs, st)) != MAD_OK) return rs;

@@ -1419,7 +1419,7 @@ mad_status dense_comparator(mad_ctx* ctx, const mad_matrix* A, const mad_matrix*
     count_launch(ctx);
   }
   uint64_t nsel = 0;
-  if ((rs = select_list(ctx, ws, ncand, kkeep, 4, &nsel, st)) != MAD_OK) return rs;
+  if ((rs = select_list(ctx, ws, ncand, kkeep, 32, &nsel, st)) != MAD_OK) return rs;
   const SelectWs ws2 = select_ws_carve(ws2b, kkeep, t ? t : 1);
   if (nsel) {
     const unsigned long long blocks = (nsel * 32 + 255) / 256;
@@ -1438,7 +1438,7 @@ mad_status dense_comparator(mad_ctx* ctx, const mad_matrix* A, const mad_matrix*
     count_launch(ctx);
   }
   uint64_t nt = 0;
-  if ((rs = select_list(ctx, ws2, nsel, t, 4, &nt, st)) != MAD_OK) return rs;
+  if ((rs = select_list(ctx, ws2, nsel, t, 32, &nt, st)) != MAD_OK) return rs;
   if (nt) {
     k_fp32_pairs<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(ws2.out, nt, cvals, out);
     count_launch(ctx);

@@ -353,10 +353,11 @@ struct SelectWs {
 };
 size_t select_ws_bytes(uint64_t n, uint64_t K);
 SelectWs select_ws_carve(void* base, uint64_t n, uint64_t K);
-// K largest of ws.l0[0..n) by (p desc, key asc), sorted into ws.out.  dp =
-// number of significant bytes of the largest p.  Asynchronous.
-mad_status select_list(mad_ctx* ctx, const SelectWs& ws, uint64_t n, uint64_t K, int dp,
-                       uint64_t* n_sel, cudaStream_t st);
+// K largest of ws.l0[0..n) by (p desc, key asc), sorted into ws.out.  pbits:
+// significant bits of the largest p; bi, bj: bits of the keys' i and j.
+// Asynchronous.
+mad_status select_list(mad_ctx* ctx, const SelectWs& ws, uint64_t n, uint64_t K, int pbits,
+                       uint64_t* n_sel, cudaStream_t st, int bi = 32, int bj = 32);
 // Omega_t': the K largest positive x of the hash, sorted into ws.out.
 // *n_pos receives the number of positive keys.  Synchronises once.
 mad_status select_from_hash(mad_ctx* ctx, const SelectWs& ws, uint64_t K, uint64_t* n_sel,
@@ -373,7 +374,7 @@ void tile_select_dev(mad_ctx* ctx, const Item* in, uint64_t cap, uint64_t K,
                      uint32_t* pos, Item* out, cudaStream_t st,
                      const unsigned int* gate = nullptr);
 // The same set, selected in one block when min(cap, *n_dev) <= 16384 (in no
-// particular order unless `sorted` and K <= 2048); longer lists fall back to
+// particular order unless `sorted`); longer lists fall back to
 // the tile kernels through the device word *gate (sorted output).
 void block_select_dev(mad_ctx* ctx, const Item* in, uint64_t cap, uint64_t K,
                       const unsigned long long* n_dev, bool sorted, Item* tile_sorted,
@@ -394,19 +395,18 @@ void select_hash_dev(mad_ctx* ctx, uint64_t K, const unsigned long long* hcap_de
 // inputs, whose small integer x tie in large numbers at the K-th value):
 // the x at or above the exact log-bucket threshold are compacted into list
 // (list_cap entries; more is reported as DERR_SELECT), the K first by
-// (x desc, key asc) are found by an MSB radix select on the device length
-// (ping-pong lists l1, l2 of list_cap entries) and collected into topk,
-// then sorted into out (K <= kDevSelectCap).  count[0..3] are device words.
+// (x desc, key asc) are found by a digit search on the device length and
+// collected into topk, then sorted into out (K <= kDevSelectCap).
+// count[0..3] are device words.
 void select_hash_dev_long(mad_ctx* ctx, uint64_t K, const unsigned long long* hcap_dev,
-                          void* state, unsigned long long* count, Item* list, Item* l1, Item* l2,
-                          uint64_t list_cap, Item* topk, Item* sorted, uint32_t* pos, Item* out,
-                          cudaStream_t st);
+                          void* state, unsigned long long* count, Item* list, uint64_t list_cap,
+                          Item* topk, Item* sorted, uint32_t* pos, Item* out, cudaStream_t st);
 // out[q] for q < min(cap, *n_dev) as in items_to_pairs; *n_out gets that
 // length.
 void items_to_pairs_dev(mad_ctx* ctx, const Item* items, uint64_t cap,
                         const unsigned long long* n_dev, const mad_pair* cand,
                         const double* cvals, mad_pair* out, uint32_t* n_out, cudaStream_t st);
-int significant_bytes(unsigned long long maxp);
+int significant_bits(unsigned long long maxp);
 mad_status export_x(mad_ctx* ctx, uint64_t* keys, int64_t* vals, uint64_t cap, uint64_t* n,
                     unsigned long long* counter, cudaStream_t st);
 // Sharded runs: X's occupied slots grouped by owner rank (offsets_host gets

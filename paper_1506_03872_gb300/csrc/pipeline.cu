@@ -32,8 +32,6 @@ struct PipeBufs {
   void* state;                  // selection state of Omega_t'
   unsigned long long* count;    // compacted candidates (device length)
   Item* list;                   // compacted items, list_cap
-  Item* l1;                     // ping-pong lists of the long selection (0/1
-  Item* l2;                     //   inputs), list_cap each
   Item* topk;                   // the K selected, unsorted (0/1 inputs), t'
   Item* sorted;                 // tile-sorted copy, kDevSelectCap
   uint32_t* pos;                // their input positions, kDevSelectCap
@@ -49,7 +47,7 @@ struct PipeBufs {
 
 size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// long_sel: the 0/1 pass's radix selection over list_cap candidates.
+// long_sel: the 0/1 pass's digit search over list_cap candidates.
 PipeBufs carve(void* base, uint64_t tprime, uint64_t t, uint64_t list_cap, bool long_sel) {
   PipeBufs b;
   char* p = (char*)base;
@@ -62,8 +60,6 @@ PipeBufs carve(void* base, uint64_t tprime, uint64_t t, uint64_t list_cap, bool 
   b.state = take(dev_select_state_bytes());
   b.count = (unsigned long long*)take(4 * sizeof(unsigned long long));
   b.list = (Item*)take(list_cap * sizeof(Item));
-  b.l1 = (Item*)take(long_sel ? list_cap * sizeof(Item) : 0);
-  b.l2 = (Item*)take(long_sel ? list_cap * sizeof(Item) : 0);
   b.topk = (Item*)take(long_sel ? tprime * sizeof(Item) : 0);
   b.sorted = (Item*)take(kDevSelectCap * sizeof(Item));
   b.pos = (uint32_t*)take(kDevSelectCap * sizeof(uint32_t));
@@ -121,8 +117,8 @@ mad_status enqueue_pass(mad_ctx* ctx, uint64_t seed, mad_pair* out_dev, uint32_t
   ctx->built = true;
   // Alg. 3: Omega_t' (its length min(t', compacted) on the device) ...
   if (long_sel)
-    select_hash_dev_long(ctx, ctx->pipe_tprime, hash_extent(ctx), b.state, b.count, b.list, b.l1,
-                         b.l2, ctx->pipe_list_cap, b.topk, b.sorted, b.pos, b.top, st);
+    select_hash_dev_long(ctx, ctx->pipe_tprime, hash_extent(ctx), b.state, b.count, b.list,
+                         ctx->pipe_list_cap, b.topk, b.sorted, b.pos, b.top, st);
   else
     select_hash_dev(ctx, ctx->pipe_tprime, hash_extent(ctx), b.state, b.count, b.list, b.sorted,
                   b.pos, b.top, st);

@@ -7,15 +7,14 @@
 //    positive x; the bucket where the count from the top reaches K gives a
 //    threshold that keeps all of the top K and few others; a second pass
 //    compacts the slots at or above it into items.
-// 2. MSB-first radix select on the composite, one byte per pass, starting
-//    at the highest nonzero byte of p: inside one 1024-thread block for
-//    short lists; otherwise across the grid, where each pass histograms the
-//    surviving tie set, the last block to finish picks the byte, and the
-//    next pass keeps only the survivors with that byte (passes whose work is
-//    already decided exit at once, so the host never waits between passes).
+// 2. MSB-first radix select on the composite: inside one 1024-thread block
+//    for short lists; otherwise across the grid, 11 bits a pass from the
+//    leading bit of the largest p downwards, then of the key among equal p;
+//    the last block of a pass picks the digit (passes whose work is already
+//    decided exit at once, so the host never waits between passes).
 // 3. Collection: every item whose composite is at least the threshold.
-// 4. Bitonic sort of the K items (shared-memory stages inside 2048-item
-//    chunks, global stages across chunks).
+// 4. Sorting of the K items: by counted ranks (up to 2048), by sorted tiles
+//    and pairwise merges (up to 2^17), else a bitonic network.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -30,6 +29,15 @@
 namespace mad {
 namespace {
 
+constexpr int kDigitBits = 11;
+constexpr int kDigitBins = 1 << kDigitBits;
+
+// How a key (i << 32) | j is packed for the digit search: i above the bj
+// bits of j, kb bits in all (32 and 64 where no shape is known).
+struct KeyPack {
+  int bj, kb;
+};
+
 struct SelState {
   unsigned int lhist[1024];   // log-bucket histogram of x (hash path)
   unsigned long long theta;   // collect threshold from the histogram
@@ -37,22 +45,19 @@ struct SelState {
   unsigned long long positive;
   unsigned int ticket3;
   unsigned int pad3;
-  unsigned long long n_cur;   // survivors in the current list
-  unsigned long long k_rem;   // survivors still to be taken
-  unsigned long long tp, tk;  // threshold composite (tk applies to ~key)
-  unsigned long long n_next;
-  unsigned int hist[256];
+  unsigned long long n_cur;   // items of the list
+  unsigned long long k_rem;   // ties of the digits fixed so far still to be taken
+  unsigned long long tp, tk;  // threshold composite (tk applies to ~packed key)
+  unsigned int hist[kDigitBins];
   unsigned int ticket;
-  unsigned int ticket2;
-  int cur;                    // 0: the compacted list, 1/2: ping-pong lists
+  int ptop, ktop;             // bits of p and of the packed key not fixed yet
   int done;
-  int picked;
-  int pad;
 };
 
-__device__ __forceinline__ uint32_t digit_of(const Item& it, int q, int dp) {
-  if (q < dp) return (uint32_t)(it.p >> (8 * (dp - 1 - q))) & 0xFFu;
-  return (uint32_t)((~it.key) >> (8 * (7 - (q - dp)))) & 0xFFu;
+// ~key, packed: larger for smaller keys.
+__device__ __forceinline__ unsigned long long packed_nk(unsigned long long key, KeyPack kp) {
+  const unsigned long long v = ((key >> 32) << kp.bj) | (key & 0xFFFFFFFFull);
+  return kp.kb < 64 ? ~v & ((1ull << kp.kb) - 1) : ~v;
 }
 
 // Warp-aggregated append of `it` when `want` (one counter atomic per warp
@@ -124,86 +129,129 @@ __device__ __forceinline__ void append_block1(Item* out, unsigned long long* cou
   append_block<1>(out, counter, w, v, cap);
 }
 
+// Start of the digit search: the K first of n items, p of at most ptop bits.
+__device__ __forceinline__ void sel_start(SelState* st, unsigned long long n,
+                                          unsigned long long K, int ptop, int kb) {
+  st->n_cur = n;
+  st->k_rem = K;
+  st->ptop = ptop;
+  st->ktop = kb;
+  st->done = n <= K ? 1 : 0;   // every item is taken: the threshold stays 0
+}
+
+__global__ void k_sel_start(SelState* st, unsigned long long n, unsigned long long K, int ptop,
+                            int kb) {
+  if (threadIdx.x == 0) sel_start(st, n, K, ptop, kb);
+}
+
+// One digit of the threshold composite: up to 11 bits of p below those fixed,
+// or of the packed ~key once p is fixed.  Every item whose fixed digits equal
+// the threshold's is counted in its bin; the last block to finish picks the
+// bin where the count from the top reaches k_rem.  No survivor lists: a
+// round reads the list once (16 of 24 bytes an item matter; L2 holds a million)
+// and writes nothing.  Bound by the shared-memory counters where few values
+// occur (0/1 counts: most items share one bin), so a warp's items in the bin
+// of its first lane go in with one addition.  Against byte digits with a
+// survivor list per round (16 rounds of two kernels, the first eight on the
+// zero bytes of a count: 35,000 items 8 x 50 us of same-bin additions, 550 us in
+// all): six passes of 3 to 8 us
+// (common neighbours of 20,011 nodes, fused pass 1003 -> 485 us; of 1e6 nodes,
+// 1e6 tied items, 209 -> 80 us).
 __global__ void __launch_bounds__(256)
-k_radix_hist(const Item* __restrict__ l0, const Item* __restrict__ l1,
-             const Item* __restrict__ l2, SelState* st, int q, int dp, int last_q) {
+k_sel_digit(const Item* __restrict__ list, SelState* st, KeyPack kp) {
   if (st->done) return;
-  __shared__ unsigned int h[256];
-  h[threadIdx.x] = 0;
+  __shared__ unsigned int h[kDigitBins];
+  for (int b = threadIdx.x; b < kDigitBins; b += blockDim.x) h[b] = 0;
   __syncthreads();
-  const Item* list = st->cur == 0 ? l0 : (st->cur == 1 ? l1 : l2);
-  const unsigned long long n = st->n_cur;
-  for (unsigned long long x = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; x < n;
-       x += (unsigned long long)gridDim.x * blockDim.x)
-    atomicAdd(&h[digit_of(list[x], q, dp)], 1u);
+  const unsigned long long n = st->n_cur, tp = st->tp, tk = st->tk;
+  const int ptop = st->ptop, ktop = st->ktop;
+  const bool on_p = ptop > 0;
+  const int top = on_p ? ptop : ktop;
+  const int width = top < kDigitBits ? top : kDigitBits, sh = top - width;
+  const unsigned int dmask = (1u << width) - 1u;
+  const int lane = threadIdx.x & 31;
+  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+  const unsigned long long rounds = (n + stride - 1) / stride;
+  for (unsigned long long r = 0; r < rounds; ++r) {
+    const unsigned long long x =
+        (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x + r * stride;
+    bool in = false;
+    unsigned int bin = 0;
+    if (x < n) {
+      const unsigned long long p = list[x].p;
+      if (on_p) {
+        in = top >= 64 || ((p ^ tp) >> top) == 0;
+        bin = (unsigned int)(p >> sh) & dmask;
+      } else if (p == tp) {
+        const unsigned long long nk = packed_nk(list[x].key, kp);
+        in = top >= 64 || ((nk ^ tk) >> top) == 0;
+        bin = (unsigned int)(nk >> sh) & dmask;
+      }
+    }
+    const unsigned int act = __ballot_sync(0xFFFFFFFFu, in);
+    if (!act) continue;
+    const int first = __ffs(act) - 1;
+    const unsigned int b0 = __shfl_sync(0xFFFFFFFFu, bin, first);
+    const unsigned int same = __ballot_sync(0xFFFFFFFFu, in && bin == b0);
+    if (lane == first) atomicAdd(&h[b0], (unsigned int)__popc(same));
+    else if (in && bin != b0) atomicAdd(&h[bin], 1u);
+  }
   __syncthreads();
-  if (h[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], h[threadIdx.x]);
+  for (int b = threadIdx.x; b < kDigitBins; b += blockDim.x)
+    if (h[b]) atomicAdd(&st->hist[b], h[b]);
   __threadfence();
   __shared__ unsigned int is_last;
   if (threadIdx.x == 0) is_last = (atomicAdd(&st->ticket, 1u) == gridDim.x - 1);
   __syncthreads();
   if (!is_last) return;
   __threadfence();
+  unsigned long long total = 0;
+  const int pick = block_pick_from_top<kDigitBins>(st->hist, st->k_rem, &total);
+  __shared__ unsigned long long s_above;
+  if (threadIdx.x == 0) s_above = 0;
+  __syncthreads();
+  unsigned long long above = 0;
+  for (int b = threadIdx.x; b < kDigitBins; b += blockDim.x)
+    if (b > pick) above += __ldcg(st->hist + b);
+  if (above) atomicAdd(&s_above, above);
+  __syncthreads();
   if (threadIdx.x == 0) {
-    volatile unsigned int* gh = st->hist;
-    unsigned long long above = 0;
-    int b = 255;
-    for (; b > 0; --b) {
-      const unsigned long long c = gh[b];
-      if (above + c >= st->k_rem) break;
-      above += c;
+    const unsigned long long ties = __ldcg(st->hist + pick);
+    st->k_rem -= s_above;
+    if (on_p) {
+      st->tp = tp | ((unsigned long long)pick << sh);
+      st->ptop = sh;
+    } else {
+      st->tk = tk | ((unsigned long long)pick << sh);
+      st->ktop = sh;
     }
-    const unsigned long long ties = gh[b];
-    st->k_rem -= above;
-    st->picked = b;
-    if (q < dp)
-      st->tp |= (unsigned long long)b << (8 * (dp - 1 - q));
-    else
-      st->tk |= (unsigned long long)b << (8 * (7 - (q - dp)));
-    // Every survivor with this byte is taken, or the threshold is complete.
-    if (ties == st->k_rem || q == last_q) st->done = 1;
+    // Every tie is taken, or the threshold is complete.
+    st->done = (ties == st->k_rem || (st->ptop == 0 && st->ktop == 0)) ? 1 : 0;
     st->ticket = 0;
-    st->n_next = 0;
   }
   __syncthreads();
-  st->hist[threadIdx.x] = 0;
+  for (int b = threadIdx.x; b < kDigitBins; b += blockDim.x) st->hist[b] = 0;
+}
+
+// Rounds that settle p of at most pbits bits and a packed key.
+int digit_rounds(int pbits, KeyPack kp) {
+  return (pbits + kDigitBits - 1) / kDigitBits + (kp.kb + kDigitBits - 1) / kDigitBits;
+}
+
+// The packing for the keys of a built context: rows below m, columns below n
+// (under MAD_SQUARE_SYM also pairs of inner indices, below d).
+KeyPack key_pack(const mad_ctx* ctx) {
+  const int64_t inner = (ctx->flags & MAD_SQUARE_SYM) ? ctx->d : 1;
+  const uint64_t rows = (uint64_t)(ctx->m > inner ? ctx->m : inner) - 1;
+  const uint64_t cols = (uint64_t)(ctx->n > inner ? ctx->n : inner) - 1;
+  int bi = 1, bj = 1;
+  while (bi < 32 && (rows >> bi)) ++bi;
+  while (bj < 32 && (cols >> bj)) ++bj;
+  return KeyPack{bj, bi + bj};
 }
 
 __global__ void __launch_bounds__(256)
-k_radix_filter(const Item* __restrict__ l0, Item* __restrict__ l1, Item* __restrict__ l2,
-               SelState* st, int q, int dp, uint64_t cap) {
-  if (st->done) return;
-  const int cur = st->cur;
-  const Item* list = cur == 0 ? l0 : (cur == 1 ? l1 : l2);
-  Item* out = cur == 1 ? l2 : l1;
-  const unsigned long long n = st->n_cur;
-  const uint32_t picked = (uint32_t)st->picked;
-  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-  const unsigned long long rounds = (n + stride - 1) / stride;
-  for (unsigned long long r = 0; r < rounds; ++r) {
-    const unsigned long long x = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x + r * stride;
-    bool want = false;
-    Item it;
-    if (x < n) {
-      it = list[x];
-      want = digit_of(it, q, dp) == picked;
-    }
-    append_block1(out, &st->n_next, want, it, cap);
-  }
-  __threadfence();
-  __shared__ unsigned int is_last;
-  if (threadIdx.x == 0) is_last = (atomicAdd(&st->ticket2, 1u) == gridDim.x - 1);
-  __syncthreads();
-  if (is_last && threadIdx.x == 0) {
-    __threadfence();
-    st->cur = cur == 1 ? 2 : 1;
-    st->n_cur = *((volatile unsigned long long*)&st->n_next);
-    st->ticket2 = 0;
-  }
-}
-
-__global__ void __launch_bounds__(256)
-k_collect(const Item* __restrict__ l0, unsigned long long n, const SelState* st,
+k_collect(const Item* __restrict__ l0, unsigned long long n, const SelState* st, KeyPack kp,
           Item* __restrict__ out, unsigned long long* counter, uint64_t cap) {
   const unsigned long long tp = st->tp, tk = st->tk;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
@@ -214,7 +262,7 @@ k_collect(const Item* __restrict__ l0, unsigned long long n, const SelState* st,
     Item it;
     if (x < n) {
       it = l0[x];
-      want = it.p > tp || (it.p == tp && (~it.key) >= tk);
+      want = it.p > tp || (it.p == tp && packed_nk(it.key, kp) >= tk);
     }
     append_block1(out, counter, want, it, cap);
   }
@@ -381,10 +429,8 @@ k_select_check(SelState* st, unsigned long long* counter, unsigned long long K,
 // writes the items ranked below K to their place.
 constexpr unsigned kTile = 2048;
 constexpr unsigned kTileSortMax = 1u << 17;
-// One-block selection (k_block_select, below): lists up to kBlockSel items,
-// sorted output up to kBlockSort items.
+// One-block selection (k_block_select, below): lists up to kBlockSel items.
 constexpr int kBlockSel = 16384;
-constexpr int kBlockSort = 2048;
 
 __device__ __forceinline__ bool item_before(unsigned long long ap, unsigned long long ak, uint32_t ai,
                                             unsigned long long bp, unsigned long long bk, uint32_t bi) {
@@ -433,12 +479,8 @@ k_tile_sort(const Item* __restrict__ in, unsigned n_max, unsigned K, Item* __res
     }
   }
   for (unsigned r = threadIdx.x; r < len; r += blockDim.x) {
-    if (pos_out) {
-      out[base + r] = in[si[r]];
-      pos_out[base + r] = si[r];
-    } else if (r < K) {
-      out[r] = in[si[r]];
-    }
+    out[base + r] = in[si[r]];
+    pos_out[base + r] = si[r];
   }
 }
 
@@ -472,6 +514,57 @@ k_merge_rank(const Item* __restrict__ tiles, const uint32_t* __restrict__ pos, u
     rank += lo;
   }
   if (rank < K) out[rank] = me;
+}
+
+// Lists of at most kTile items: every item's rank is counted directly.  A
+// block ranks 32 items, one per lane, its eight warps each against an eighth
+// of the list (held in shared memory, read as broadcasts), and writes those
+// ranked below K.  n * n compares, spread over n / 32 blocks, against the 66
+// barrier-separated steps of a 2048-item bitonic network in one block: 1000
+// items 35 -> 14 us, 100 items 32 -> 4.5 us.  With a gate, the kernel runs only when *gate is zero (the list was selected by
+// k_block_select).
+constexpr int kRankWarps = 8;
+__global__ void __launch_bounds__(32 * kRankWarps)
+k_rank_sort(const Item* __restrict__ in, unsigned n_max, unsigned K, Item* __restrict__ out,
+            const unsigned long long* n_dev, unsigned int* over_err, const unsigned int* gate) {
+  extern __shared__ ulonglong2 rank_pk[];   // (p, key)
+  __shared__ unsigned part[kRankWarps][32];
+  if (gate && *gate != 0u) return;
+  if (over_err && blockIdx.x == 0 && threadIdx.x == 0 && *n_dev > n_max)
+    atomicOr(over_err, DERR_SELECT);
+  const unsigned n = (unsigned)dev_len(n_max, n_dev);
+  const unsigned base = blockIdx.x * 32;
+  if (base >= n) return;
+  for (unsigned r = threadIdx.x; r < n; r += blockDim.x)
+    rank_pk[r] = make_ulonglong2(in[r].p, in[r].key);
+  __syncthreads();
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned e = base + lane < n ? base + lane : n - 1;
+  const unsigned long long p = rank_pk[e].x, key = rank_pk[e].y;
+  const unsigned per = (n + kRankWarps - 1) / kRankWarps;
+  const unsigned r1 = min(n, (warp + 1) * per);
+  unsigned rank = 0;
+#pragma unroll 4
+  for (unsigned r = warp * per; r < r1; ++r) {
+    const ulonglong2 o = rank_pk[r];
+    rank += item_before(o.x, o.y, r, p, key, e) ? 1u : 0u;
+  }
+  part[warp][lane] = rank;
+  __syncthreads();
+  if (warp == 0 && base + lane < n) {
+#pragma unroll
+    for (int w = 1; w < kRankWarps; ++w) rank += part[w][lane];
+    if (rank < K) out[rank] = in[e];
+  }
+}
+
+// out: the K first of in[0 .. min(n_max, *n_dev)), n_max <= kTile, sorted.
+void rank_sort(mad_ctx* ctx, const Item* in, uint64_t n_max, uint64_t K, Item* out,
+               const unsigned long long* n_dev, unsigned int* over_err, const unsigned int* gate,
+               cudaStream_t st) {
+  k_rank_sort<<<(unsigned)((n_max + 31) / 32), 32 * kRankWarps, n_max * sizeof(ulonglong2), st>>>(
+      in, (unsigned)n_max, (unsigned)K, out, n_dev, over_err, gate);
+  count_launch(ctx);
 }
 
 // Pairwise merge of sorted runs of length L (kTile times a power of two):
@@ -536,17 +629,20 @@ void sort_merge(mad_ctx* ctx, const SelectWs& ws, const Item* in, uint64_t n, cu
   if (cur != ws.out) cudaMemcpyAsync(ws.out, cur, n * sizeof(Item), cudaMemcpyDeviceToDevice, st);
 }
 
-// Sorted top K of `in[0..n)` by tiles (n <= kTileSortMax).  Uses l1 and l2
-// of the workspace as scratch; `in` may be ws.out.
+// Sorted top K of `in[0..n)` (n <= kTileSortMax): by rank up to kTile items,
+// else by tiles.  Uses l1 and l2 of the workspace as scratch; `in` may be
+// ws.out.
 void tile_select(mad_ctx* ctx, const SelectWs& ws, const Item* in, uint64_t n, uint64_t K,
                  cudaStream_t st) {
-  const unsigned tiles = (unsigned)((n + kTile - 1) / kTile);
-  if (tiles == 1 && in != ws.out) {
-    k_tile_sort<<<1, kTile / 2, 0, st>>>(in, (unsigned)n, (unsigned)K, ws.out, nullptr, nullptr,
-                                         nullptr);
-    count_launch(ctx);
+  if (n <= (uint64_t)kTile) {
+    if (in == ws.out) {
+      cudaMemcpyAsync(ws.l1, in, n * sizeof(Item), cudaMemcpyDeviceToDevice, st);
+      in = ws.l1;
+    }
+    rank_sort(ctx, in, n, K, ws.out, nullptr, nullptr, nullptr, st);
     return;
   }
+  const unsigned tiles = (unsigned)((n + kTile - 1) / kTile);
   uint32_t* pos = (uint32_t*)ws.l2;
   k_tile_sort<<<tiles, kTile / 2, 0, st>>>(in, (unsigned)n, (unsigned)K, ws.l1, pos, nullptr,
                                             nullptr);
@@ -673,9 +769,9 @@ void bitonic_sort(mad_ctx* ctx, Item* data, unsigned long long n, cudaStream_t s
 
 }  // namespace
 
-int significant_bytes(unsigned long long maxp) {
+int significant_bits(unsigned long long maxp) {
   int b = 1;
-  while (b < 8 && (maxp >> (8 * b)) != 0) ++b;
+  while (b < 64 && (maxp >> b) != 0) ++b;
   return b;
 }
 
@@ -704,8 +800,8 @@ SelectWs select_ws_carve(void* base, uint64_t n, uint64_t K) {
 
 void prefilter_select(mad_ctx* ctx, const SelectWs& ws, uint64_t n, uint64_t K, cudaStream_t st);
 
-mad_status select_list(mad_ctx* ctx, const SelectWs& ws, uint64_t n, uint64_t K, int dp,
-                       uint64_t* n_sel, cudaStream_t st) {
+mad_status select_list(mad_ctx* ctx, const SelectWs& ws, uint64_t n, uint64_t K, int pbits,
+                       uint64_t* n_sel, cudaStream_t st, int bi, int bj) {
   const uint64_t take = K < n ? K : n;
   *n_sel = take;
   if (take == 0) return MAD_OK;
@@ -714,7 +810,7 @@ mad_status select_list(mad_ctx* ctx, const SelectWs& ws, uint64_t n, uint64_t K,
   // pick the K largest, unordered, into ws.out (an MSB radix select), which
   // the tile sort then orders when K is short, else a bitonic network.
   if (n <= kTileSortMax) {
-    if (take <= (uint64_t)kBlockSort && take < n && n > (uint64_t)kTile)
+    if (take <= (uint64_t)kTile && take < n && n > (uint64_t)kTile)
       prefilter_select(ctx, ws, n, take, st);
     else if (take == n && n > (uint64_t)kTile)
       sort_merge(ctx, ws, ws.l0, n, st);
@@ -727,17 +823,15 @@ mad_status select_list(mad_ctx* ctx, const SelectWs& ws, uint64_t n, uint64_t K,
   } else {
     SelState* dst = (SelState*)ws.state;
     cudaMemsetAsync(dst, 0, sizeof(SelState), st);
-    const unsigned long long init[2] = {n, K};
-    cudaMemcpyAsync(&dst->n_cur, init, sizeof(init), cudaMemcpyHostToDevice, st);
-    const int digits = dp + 8;
+    const KeyPack kp{bj, bi + bj};
+    k_sel_start<<<1, 32, 0, st>>>(dst, n, K, pbits, kp.kb);
     const unsigned blocks = grid_for(n, 152 * 4);
-    for (int q = 0; q < digits; ++q) {
-      k_radix_hist<<<blocks, 256, 0, st>>>(ws.l0, ws.l1, ws.l2, dst, q, dp, digits - 1);
-      k_radix_filter<<<blocks, 256, 0, st>>>(ws.l0, ws.l1, ws.l2, dst, q, dp, ws.cap_n);
-      count_launch(ctx, 2);
-    }
+    const int rounds = digit_rounds(pbits, kp);
+    for (int q = 0; q < rounds; ++q) k_sel_digit<<<blocks, 256, 0, st>>>(ws.l0, dst, kp);
+    count_launch(ctx, 1 + rounds);
     cudaMemsetAsync(ws.counter, 0, sizeof(unsigned long long), st);
-    k_collect<<<grid_for(n, 152 * 8), 256, 0, st>>>(ws.l0, n, dst, ws.out, ws.counter, ws.cap_out);
+    k_collect<<<grid_for(n, 152 * 8), 256, 0, st>>>(ws.l0, n, dst, kp, ws.out, ws.counter,
+                                                    ws.cap_out);
     count_launch(ctx);
   }
   if (take <= kTileSortMax) {
@@ -770,7 +864,9 @@ mad_status select_from_hash(mad_ctx* ctx, const SelectWs& ws, uint64_t K, uint64
   if (e != cudaSuccess) return cuda_status(e);
   if (host[0] > ws.cap_n) return MAD_ERR_STATE;
   *n_pos = positive;
-  return select_list(ctx, ws, host[0], K, significant_bytes(host[1]), n_sel, st);
+  const KeyPack kp = key_pack(ctx);
+  return select_list(ctx, ws, host[0], K, significant_bits(host[1]), n_sel, st, kp.kb - kp.bj,
+                     kp.bj);
 }
 
 mad_status items_to_pairs(mad_ctx* ctx, const Item* items, uint64_t n, const mad_pair* cand,
@@ -784,6 +880,10 @@ mad_status items_to_pairs(mad_ctx* ctx, const Item* items, uint64_t n, const mad
 void tile_select_dev(mad_ctx* ctx, const Item* in, uint64_t cap, uint64_t K,
                      const unsigned long long* n_dev, unsigned int* over_err, Item* sorted,
                      uint32_t* pos, Item* out, cudaStream_t st, const unsigned int* gate) {
+  if (cap <= (uint64_t)kTile && !gate) {
+    rank_sort(ctx, in, cap, K, out, n_dev, over_err, nullptr, st);
+    return;
+  }
   const unsigned tiles = (unsigned)((cap + kTile - 1) / kTile);
   k_tile_sort<<<tiles, kTile / 2, 0, st>>>(in, (unsigned)cap, (unsigned)K, sorted, pos, n_dev,
                                             over_err, gate);
@@ -797,11 +897,10 @@ void tile_select_dev(mad_ctx* ctx, const Item* in, uint64_t cap, uint64_t K,
 // asc), for n <= kBlockSel, in one 1024-thread block: the p of every item
 // sit in shared memory and an MSB radix select (8-bit digits, from the
 // highest digit in which two items differ) finds the K-th largest p and how
-// many items equal to it are taken; among those
-// ties the smallest keys are found the same way.  The K items go to out in
-// no particular order, or sorted when `sorted` (K <= kBlockSort).  A longer
-// list sets *gate to 1 and writes nothing (the tile kernels, gated on that
-// word, select instead); otherwise *gate becomes 0.
+// many items equal to it are taken; among those ties the smallest keys are
+// found the same way.  The K items go to out in no particular order (k_rank_sort
+// orders them).  A longer list sets *gate to 1 and writes nothing (the tile
+// kernels, gated on that word, select instead); otherwise *gate becomes 0.
 
 // The digit of the K-th largest value among those counted in hist (256
 // bins, digit order): returns it and leaves in *rank the rank of that value
@@ -843,8 +942,8 @@ __device__ __forceinline__ void pick_digit(const unsigned int* hist, unsigned lo
 
 __global__ void __launch_bounds__(1024)
 k_block_select(const Item* __restrict__ in, unsigned long long cap, const unsigned long long* n_dev,
-               unsigned int K_max, Item* __restrict__ out, int sorted, unsigned int* gate) {
-  extern __shared__ unsigned long long bs_p[];   // kBlockSel values, then the sort buffers
+               unsigned int K_max, Item* __restrict__ out, unsigned int* gate) {
+  extern __shared__ unsigned long long bs_p[];   // kBlockSel values
   __shared__ unsigned int hist[256];
   __shared__ unsigned long long s_prefix, s_rank, s_kprefix, s_krank, s_diff;
   __shared__ int s_digit;
@@ -951,59 +1050,14 @@ k_block_select(const Item* __restrict__ in, unsigned long long cap, const unsign
   }
   const unsigned long long nk_min = s_kprefix;   // taken ties have ~key >= this
   // The selected items (their p values are still in shared memory).
-  const bool to_smem = sorted && K <= (unsigned long long)kBlockSort;
   __syncthreads();
-  unsigned long long* sp = bs_p + kBlockSel;   // sort buffers after the values
   for (unsigned long long x = threadIdx.x; x < n; x += blockDim.x) {
     const unsigned long long v = bs_p[x];
     bool take = K > 0 && v > pk;
     if (!take && K > 0 && v == pk) take = !key_select || ~in[x].key >= nk_min;
     if (take) {
       const unsigned int pos = atomicAdd(&s_out, 1u);
-      if (pos >= K) continue;   // (never: exactly K items qualify)
-      if (to_smem) {
-        sp[pos] = v;
-        sp[kBlockSort + pos] = in[x].key;
-        sp[2 * kBlockSort + pos] = in[x].aux;
-      } else {
-        out[pos] = in[x];
-      }
-    }
-  }
-  __syncthreads();
-  if (to_smem) {
-    const int m = (int)K;
-    int m2 = 1;
-    while (m2 < m) m2 <<= 1;
-    for (int x = m + threadIdx.x; x < m2; x += blockDim.x) {
-      sp[x] = 0;
-      sp[kBlockSort + x] = ~0ull;
-      sp[2 * kBlockSort + x] = 0;
-    }
-    __syncthreads();
-    unsigned long long* kk = sp + kBlockSort;
-    unsigned long long* aa = sp + 2 * kBlockSort;
-    for (int k = 2; k <= m2; k <<= 1) {
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int t = threadIdx.x; t < m2 / 2; t += blockDim.x) {
-          const int a = ((t & ~(j - 1)) << 1) | (t & (j - 1)), b = a + j;
-          const bool up = (a & k) == 0;
-          const bool b_first = sp[b] > sp[a] || (sp[b] == sp[a] && kk[b] < kk[a]);
-          if (b_first == up) {
-            const unsigned long long tp = sp[a], tk = kk[a], ta = aa[a];
-            sp[a] = sp[b]; kk[a] = kk[b]; aa[a] = aa[b];
-            sp[b] = tp; kk[b] = tk; aa[b] = ta;
-          }
-        }
-        __syncthreads();
-      }
-    }
-    for (int x = threadIdx.x; x < m; x += blockDim.x) {
-      Item it;
-      it.p = sp[x];
-      it.key = kk[x];
-      it.aux = aa[x];
-      out[x] = it;
+      if (pos < K) out[pos] = in[x];   // (exactly K items qualify)
     }
   }
   if (threadIdx.x == 0) *gate = 0u;
@@ -1116,24 +1170,27 @@ void block_select_dev(mad_ctx* ctx, const Item* in, uint64_t cap, uint64_t K,
                       uint32_t* pos, Item* out, unsigned int* gate, unsigned int* over_err,
                       cudaStream_t st) {
   static bool attr = false;
-  const size_t smem = (size_t)(kBlockSel + 3 * kBlockSort) * sizeof(unsigned long long);
+  const size_t smem = (size_t)kBlockSel * sizeof(unsigned long long);
   if (!attr) {
     cudaFuncSetAttribute(k_block_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     attr = true;
   }
-  if (sorted && K > (uint64_t)kBlockSort) {   // too many to sort in one block
+  if (sorted && (K > (uint64_t)kTile || cap <= (uint64_t)kTile)) {
+    // Too many for k_rank_sort, or a list short enough to be ranked at once.
     tile_select_dev(ctx, in, cap, K, n_dev, over_err, tile_sorted, pos, out, st);
     return;
   }
-  k_block_select<<<1, 1024, smem, st>>>(in, cap, n_dev, (unsigned int)K, out, sorted ? 1 : 0,
+  k_block_select<<<1, 1024, smem, st>>>(in, cap, n_dev, (unsigned int)K, sorted ? tile_sorted : out,
                                         gate);
   count_launch(ctx);
-  tile_select_dev(ctx, in, cap, K, n_dev, over_err, tile_sorted, pos, out, st, gate);
+  if (sorted) rank_sort(ctx, tile_sorted, K, K, out, n_dev, nullptr, gate, st);
+  if (cap > (uint64_t)kBlockSel)   // (a shorter list never leaves the block)
+    tile_select_dev(ctx, in, cap, K, n_dev, over_err, tile_sorted, pos, out, st, gate);
 }
 
 size_t dev_select_state_bytes() { return ((sizeof(SelState) + 255) / 256) * 256; }
 
-// The sorted top K (K <= kBlockSort < n <= kTileSortMax) of ws.l0[0..n) into
+// The sorted top K (K <= kTile < n <= kTileSortMax) of ws.l0[0..n) into
 // ws.out: the prefilter, then the one-block selection of the compacted
 // items; when more than kBlockSel of them tie into the threshold bin, the
 // tile kernels (gated on the block's word) select from the whole list.
@@ -1182,25 +1239,22 @@ void select_hash_dev(mad_ctx* ctx, uint64_t K, const unsigned long long* hcap_de
                    (unsigned int*)(count + 2), &ctx->sc->err, st);
 }
 
-// Device-length start of the radix selection: the list holds min(*count,
-// cap) items (more than cap: the compaction overflowed, reported); with no
-// more than K of them every one is taken (the threshold stays 0).
-__global__ void k_radix_init_dev(SelState* st, const unsigned long long* count, uint64_t cap,
-                                 unsigned long long K, unsigned int* err) {
+// Device-length start of the digit search: the list holds min(*count, cap)
+// items (more than cap: the compaction overflowed, reported), and the
+// largest x is known from the histogram pass.
+__global__ void k_sel_start_dev(SelState* st, const unsigned long long* count, uint64_t cap,
+                                unsigned long long K, int kb, unsigned int* err) {
   if (threadIdx.x != 0) return;
   const unsigned long long n = *count;
   if (n > cap) atomicOr(err, DERR_SELECT);
-  st->n_cur = n < cap ? n : cap;
-  st->k_rem = K;
-  st->cur = 0;
-  st->done = st->n_cur <= K ? 1 : 0;
+  sel_start(st, n < cap ? n : cap, K, 64 - __clzll((long long)st->maxp), kb);
 }
 
 // k_collect over a list of device length min(*count, cap).
 __global__ void __launch_bounds__(256)
 k_collect_dev(const Item* __restrict__ l0, const unsigned long long* count, uint64_t cap,
-              const SelState* st, Item* __restrict__ out, unsigned long long* counter,
-              uint64_t out_cap) {
+              const SelState* st, KeyPack kp, Item* __restrict__ out,
+              unsigned long long* counter, uint64_t out_cap) {
   const unsigned long long n0 = *count, n = n0 < cap ? n0 : cap;
   const unsigned long long tp = st->tp, tk = st->tk;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
@@ -1211,16 +1265,15 @@ k_collect_dev(const Item* __restrict__ l0, const unsigned long long* count, uint
     Item it;
     if (x < n) {
       it = l0[x];
-      want = it.p > tp || (it.p == tp && (~it.key) >= tk);
+      want = it.p > tp || (it.p == tp && packed_nk(it.key, kp) >= tk);
     }
     append_block1(out, counter, want, it, out_cap);
   }
 }
 
 void select_hash_dev_long(mad_ctx* ctx, uint64_t K, const unsigned long long* hcap_dev,
-                          void* state, unsigned long long* count, Item* list, Item* l1, Item* l2,
-                          uint64_t list_cap, Item* topk, Item* sorted, uint32_t* pos, Item* out,
-                          cudaStream_t st) {
+                          void* state, unsigned long long* count, Item* list, uint64_t list_cap,
+                          Item* topk, Item* sorted, uint32_t* pos, Item* out, cudaStream_t st) {
   SelState* dst = (SelState*)state;
   cudaMemsetAsync(dst, 0, sizeof(SelState), st);
   cudaMemsetAsync(count, 0, 4 * sizeof(unsigned long long), st);
@@ -1230,19 +1283,20 @@ void select_hash_dev_long(mad_ctx* ctx, uint64_t K, const unsigned long long* hc
   k_log_hist<<<blocks, 256, 0, st>>>(ctx->hvals, bound, K, dst, hcap_dev, 0);
   launch_compact_ge(ctx, blocks, st, ctx->hkeys, ctx->hvals, bound, dst, list, list_cap, count,
                     hcap_dev);
-  // The K first by (x desc, key asc): MSB radix select over the 8 bytes of
-  // x and the 8 of the key, on the device length.
-  k_radix_init_dev<<<1, 32, 0, st>>>(dst, count, list_cap, K, &ctx->sc->err);
+  // The K first by (x desc, key asc): the digit search on the device length.
+  // A count is at most the additions of s_max diamonds (two each under
+  // MAD_SQUARE_SYM).
+  const KeyPack kp = key_pack(ctx);
+  int pbits = 1;
+  while (pbits < 63 && ((2 * ctx->s_max) >> pbits)) ++pbits;
+  k_sel_start_dev<<<1, 32, 0, st>>>(dst, count, list_cap, K, kp.kb, &ctx->sc->err);
   const unsigned rb = grid_for(list_cap, 152 * 4);
-  constexpr int kDigits = 16;
-  for (int q = 0; q < kDigits; ++q) {
-    k_radix_hist<<<rb, 256, 0, st>>>(list, l1, l2, dst, q, 8, kDigits - 1);
-    k_radix_filter<<<rb, 256, 0, st>>>(list, l1, l2, dst, q, 8, list_cap);
-  }
-  k_collect_dev<<<grid_for(list_cap, 152 * 8), 256, 0, st>>>(list, count, list_cap, dst, topk,
+  const int rounds = digit_rounds(pbits, kp);
+  for (int q = 0; q < rounds; ++q) k_sel_digit<<<rb, 256, 0, st>>>(list, dst, kp);
+  k_collect_dev<<<grid_for(list_cap, 152 * 8), 256, 0, st>>>(list, count, list_cap, dst, kp, topk,
                                                              count + 1, K);
-  count_launch(ctx, 4 + 2 * kDigits);
-  // Sorted: the K items at count[1] through the tile sort.
+  count_launch(ctx, 4 + rounds);
+  // Sorted: the K items at count[1].
   tile_select_dev(ctx, topk, K, K, count + 1, &ctx->sc->err, sorted, pos, out, st);
 }
 
@@ -1387,7 +1441,7 @@ mad_status select_pairs(mad_ctx* ctx, const mad_pair* pairs, uint64_t n, uint64_
   cudaMemcpyAsync(&npos, counter, sizeof(npos), cudaMemcpyDeviceToHost, st);
   cudaError_t e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_status(e);
-  if ((rs = select_list(ctx, ws, npos, K, 8, n_sel, st)) != MAD_OK) return rs;
+  if ((rs = select_list(ctx, ws, npos, K, 64, n_sel, st)) != MAD_OK) return rs;
   if (*n_sel) {
     k_items_to_input_pairs<<<grid_for(*n_sel, 1u << 30), 256, 0, st>>>(ws.out, *n_sel, pairs, out);
     count_launch(ctx);

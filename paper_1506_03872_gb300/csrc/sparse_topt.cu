@@ -670,7 +670,7 @@ mad_status mad_sparse_topt(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* 
 
   // 3. The t largest candidates by (c desc, key asc).
   uint64_t nsel = 0;
-  if ((rs = select_list(ctx, w.sel_ws, count, t, 4, &nsel, st)) != MAD_OK) return rs;
+  if ((rs = select_list(ctx, w.sel_ws, count, t, 32, &nsel, st)) != MAD_OK) return rs;
   if (nsel) {
     k_sp_to_pairs<<<blocks_for(nsel, 1u << 30), 256, 0, st>>>(w.sel_ws.out, nsel, out_dev);
     count_launch(ctx);
