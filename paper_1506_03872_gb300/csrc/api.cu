@@ -364,6 +364,8 @@ mad_status mad_create(mad_ctx** out, uint32_t flags) {
   }
   if (e == cudaSuccess) e = cudaMalloc((void**)&ctx->sc, sizeof(DevScalars));
   if (e == cudaSuccess) e = cudaMemset(ctx->sc, 0, sizeof(DevScalars));
+  if (e == cudaSuccess) e = cudaMalloc(&ctx->bound_state, bound_state_bytes());
+  if (e == cudaSuccess) e = cudaMemset(ctx->bound_state, 0, bound_state_bytes());
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork2, cudaEventDisableTiming);
@@ -373,6 +375,7 @@ mad_status mad_create(mad_ctx** out, uint32_t flags) {
     if (ctx->ev_fork2) cudaEventDestroy(ctx->ev_fork2);
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->side) cudaStreamDestroy(ctx->side);
+    if (ctx->bound_state) cudaFree(ctx->bound_state);
     if (ctx->sc) cudaFree(ctx->sc);
     if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
     delete ctx;
@@ -395,6 +398,7 @@ void mad_destroy(mad_ctx* ctx) {
   free_tables(ctx, 0);
   if (ctx->scratch) cudaFreeAsync(ctx->scratch, 0);
   cudaStreamSynchronize(0);
+  cudaFree(ctx->bound_state);
   cudaFree(ctx->sc);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
   if (ctx->ev_fork2) cudaEventDestroy(ctx->ev_fork2);
@@ -572,9 +576,14 @@ mad_status mad_rescore(mad_ctx* ctx, const mad_pair* cand_dev, uint32_t ncand, u
   if ((rs = rescore_reserve(ctx, ncand, st)) != MAD_OK) return rs;
   const SelectWs ws = select_ws_carve(ctx->scratch, ncand, t);
   double* cvals = (double*)((char*)ctx->scratch + cv_off);
-  if ((rs = rescore_items(ctx, cand_dev, ncand, ws.l0, cvals, st)) != MAD_OK) return rs;
   uint64_t nsel = 0;
-  if ((rs = select_list(ctx, ws, ncand, t, 64, &nsel, st)) != MAD_OK) return rs;
+  if (rescore_bounded_applies(ctx, ncand, t)) {
+    const unsigned long long* kept = rescore_bounded(ctx, cand_dev, ncand, t, ws.l0, cvals, st);
+    if ((rs = select_list_dev(ctx, ws, ncand, kept, t, 64, &nsel, st)) != MAD_OK) return rs;
+  } else {
+    if ((rs = rescore_items(ctx, cand_dev, ncand, ws.l0, cvals, st)) != MAD_OK) return rs;
+    if ((rs = select_list(ctx, ws, ncand, t, 64, &nsel, st)) != MAD_OK) return rs;
+  }
   if ((rs = items_to_pairs(ctx, ws.out, nsel, cand_dev, cvals, out_dev, st)) != MAD_OK) return rs;
   DevScalars hs;
   if ((rs = read_scalars(ctx, &hs, st)) != MAD_OK) return rs;

@@ -244,6 +244,7 @@ struct mad_ctx {
   float region_factor = 1.5f;
   uint64_t hov_request = 0;
   mad::DevScalars* sc = nullptr;
+  void* bound_state = nullptr;      // rescore.cu's bounds (zeros between calls)
   // Scratch (select, scans); grown on demand.
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
@@ -358,6 +359,12 @@ SelectWs select_ws_carve(void* base, uint64_t n, uint64_t K);
 // Asynchronous.
 mad_status select_list(mad_ctx* ctx, const SelectWs& ws, uint64_t n, uint64_t K, int pbits,
                        uint64_t* n_sel, cudaStream_t st, int bi = 32, int bj = 32);
+// The same for a list of device length *n_dev <= n_max whose K largest are
+// known to be there (*n_sel = min(K, n_max)); waits for the length where the
+// list may be too long for a selection on the device.
+mad_status select_list_dev(mad_ctx* ctx, const SelectWs& ws, uint64_t n_max,
+                           const unsigned long long* n_dev, uint64_t K, int pbits,
+                           uint64_t* n_sel, cudaStream_t st);
 // Omega_t': the K largest positive x of the hash, sorted into ws.out.
 // *n_pos receives the number of positive keys.  Synchronises once.
 mad_status select_from_hash(mad_ctx* ctx, const SelectWs& ws, uint64_t K, uint64_t* n_sel,
@@ -461,6 +468,15 @@ int sort_bits(int64_t m);
 // Exact c for every candidate: items[q] = (bits |c|, key, q), cvals[q] = c.
 // With n_dev, the candidates are the first min(ncand, *n_dev).
 mad_status rescore_reserve(mad_ctx* ctx, uint64_t ncand, cudaStream_t st);
+// The t largest |c| of dense candidates, t small against their number: the
+// candidates that FP32 bounds cannot rule out go to items as above, in no
+// particular order (cvals only theirs), their count to the device word
+// returned (at least min(t, the number of candidates)).
+size_t bound_state_bytes();
+bool rescore_bounded_applies(const mad_ctx* ctx, uint64_t ncand, uint64_t t);
+const unsigned long long* rescore_bounded(mad_ctx* ctx, const mad_pair* cand, uint64_t ncand,
+                                          uint64_t t, Item* items, double* cvals, cudaStream_t st,
+                                          const unsigned long long* n_dev = nullptr);
 mad_status rescore_items(mad_ctx* ctx, const mad_pair* cand, uint64_t ncand, Item* items,
                          double* cvals, cudaStream_t st, const unsigned long long* n_dev = nullptr);
 

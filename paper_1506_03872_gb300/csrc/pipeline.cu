@@ -124,9 +124,14 @@ mad_status enqueue_pass(mad_ctx* ctx, uint64_t seed, mad_pair* out_dev, uint32_t
                   b.pos, b.top, st);
   items_to_pairs_dev(ctx, b.top, ctx->pipe_tprime, b.count, nullptr, nullptr, cand, counts_dev, st);
   // ... the exact c of each candidate, and Omega_t.
-  if ((rs = rescore_items(ctx, cand, ctx->pipe_tprime, b.rs_items, b.cvals, st, b.count)) != MAD_OK)
+  const unsigned long long* scored = b.count;
+  if (rescore_bounded_applies(ctx, ctx->pipe_tprime, ctx->pipe_t))
+    scored = rescore_bounded(ctx, cand, ctx->pipe_tprime, ctx->pipe_t, b.rs_items, b.cvals, st,
+                             b.count);
+  else if ((rs = rescore_items(ctx, cand, ctx->pipe_tprime, b.rs_items, b.cvals, st, b.count)) !=
+           MAD_OK)
     return rs;
-  block_select_dev(ctx, b.rs_items, ctx->pipe_tprime, ctx->pipe_t, b.count, true, b.rs_sorted,
+  block_select_dev(ctx, b.rs_items, ctx->pipe_tprime, ctx->pipe_t, scored, true, b.rs_sorted,
                    b.rs_pos, b.rs_out, (unsigned int*)(b.count + 3), nullptr, st);
   items_to_pairs_dev(ctx, b.rs_out, ctx->pipe_t, b.count, cand, b.cvals, out_dev, counts_dev + 1,
                      st);

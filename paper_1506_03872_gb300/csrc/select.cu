@@ -517,13 +517,14 @@ k_merge_rank(const Item* __restrict__ tiles, const uint32_t* __restrict__ pos, u
 }
 
 // Lists of at most kTile items: every item's rank is counted directly.  A
-// block ranks 32 items, one per lane, its eight warps each against an eighth
-// of the list (held in shared memory, read as broadcasts), and writes those
-// ranked below K.  n * n compares, spread over n / 32 blocks, against the 66
+// block ranks 32 items, one per lane, its warps each against a part of the list
+// (held in shared memory, read as broadcasts), and writes those ranked below
+// K.  n * n compares, spread over n / 32 blocks, against the 66
 // barrier-separated steps of a 2048-item bitonic network in one block: 1000
-// items 35 -> 14 us, 100 items 32 -> 4.5 us.  With a gate, the kernel runs only when *gate is zero (the list was selected by
-// k_block_select).
-constexpr int kRankWarps = 8;
+// items 35 -> 7 us (14 us with 8 warps a block instead of 32), 100 items 32 -> 4
+// us.  With a gate, the kernel runs only when *gate is zero (the list was
+// selected by k_block_select).
+constexpr int kRankWarps = 32;
 __global__ void __launch_bounds__(32 * kRankWarps)
 k_rank_sort(const Item* __restrict__ in, unsigned n_max, unsigned K, Item* __restrict__ out,
             const unsigned long long* n_dev, unsigned int* over_err, const unsigned int* gate) {
@@ -1186,6 +1187,23 @@ void block_select_dev(mad_ctx* ctx, const Item* in, uint64_t cap, uint64_t K,
   if (sorted) rank_sort(ctx, tile_sorted, K, K, out, n_dev, nullptr, gate, st);
   if (cap > (uint64_t)kBlockSel)   // (a shorter list never leaves the block)
     tile_select_dev(ctx, in, cap, K, n_dev, over_err, tile_sorted, pos, out, st, gate);
+}
+
+mad_status select_list_dev(mad_ctx* ctx, const SelectWs& ws, uint64_t n_max,
+                           const unsigned long long* n_dev, uint64_t K, int pbits,
+                           uint64_t* n_sel, cudaStream_t st) {
+  if (n_max <= kTileSortMax && K <= (uint64_t)kTile) {
+    *n_sel = K < n_max ? K : n_max;
+    unsigned int* gate = (unsigned int*)(ws.counter + 2);
+    block_select_dev(ctx, ws.l0, n_max, K, n_dev, true, ws.l1, (uint32_t*)ws.l2, ws.out, gate,
+                     nullptr, st);
+    return cuda_status(cudaGetLastError());
+  }
+  unsigned long long n = 0;
+  cudaMemcpyAsync(&n, n_dev, sizeof(n), cudaMemcpyDeviceToHost, st);
+  const cudaError_t e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return cuda_status(e);
+  return select_list(ctx, ws, n < n_max ? n : n_max, K, pbits, n_sel, st);
 }
 
 size_t dev_select_state_bytes() { return ((sizeof(SelState) + 255) / 256) * 256; }

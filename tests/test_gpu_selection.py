@@ -1,0 +1,81 @@
+"""Selection and re-ranking at the lengths where their kernels change: the K
+first pairs by (x desc, key asc) against numpy's sort, and the t largest |c|
+by FP32 bounds against the same call without them (t near the number of
+candidates takes the FP64 product of every candidate)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def _rng(seed):
+    return np.random.Generator(np.random.PCG64(seed))
+
+
+@pytest.mark.parametrize("kind", ["ties", "wide", "equal"])
+@pytest.mark.parametrize("n,K", [(1, 1), (31, 40), (33, 5), (2047, 2047), (2048, 100), (2049, 2049),
+                                 (40_000, 1000), (140_000, 3000), (300_000, 1), (300_000, 2048),
+                                 (300_000, 150_000)])
+def test_select_pairs(n, K, kind):
+    import paper_1506_03872_gb300 as mad
+    rng = _rng(n + K)
+    key = rng.choice(1 << 40, size=n, replace=False).astype(np.uint64)
+    i, j = key >> np.uint64(20), key & np.uint64((1 << 20) - 1)
+    if n > 100:   # indices that use all 32 bits
+        i[:50] += np.uint64((1 << 32) - (1 << 21))
+    x = {"ties": rng.integers(0, 4, n), "wide": rng.integers(-(1 << 61), 1 << 62, n),
+         "equal": np.full(n, 7)}[kind].astype(np.int64)
+    with mad.Context() as c:
+        out, cnt = mad.mad_select_pairs(c.ctx, mad.encode_pairs(i, j, x), n, K)
+    gi, gj, gx, _ = mad.decode_pairs(out, cnt)
+    keys = mad.keys_of(i, j)
+    pos = np.nonzero(x > 0)[0]
+    order = pos[np.lexsort((keys[pos], -x[pos]))][:K]
+    assert cnt == len(order)
+    assert np.array_equal(gx, x[order])
+    assert np.array_equal(mad.keys_of(gi, gj), keys[order])
+
+
+@pytest.mark.parametrize("kind", ["factors", "ties", "tiny", "mixed_scales"])
+@pytest.mark.parametrize("ta,tb,d", [(np.float32, np.float32, 100), (np.float64, np.float64, 33),
+                                     (np.float64, np.float32, 1), (np.float32, np.float64, 1024)])
+def test_bounded_rescore_equals_the_whole_one(kind, ta, tb, d):
+    import paper_1506_03872_gb300 as mad
+    rng = _rng(d)
+    m, n = 700, 900
+    A, B = rng.standard_normal((m, d)), rng.standard_normal((d, n))
+    if kind == "ties":
+        A, B = np.sign(A), np.sign(B)
+    if kind == "tiny":         # FP32 products below its range, FP64 entries below it
+        A[1:] *= 1e-30
+        B[:, 1:] *= 1e-18
+        if ta == np.float64:
+            A[5:] *= 1e-40
+    if kind == "mixed_scales":
+        A *= np.exp(6 * rng.standard_normal((m, 1)))
+        B *= np.exp(rng.standard_normal((1, n)))
+    tA = torch.from_numpy(A.astype(ta)).cuda()
+    tB = torch.from_numpy(B.astype(tb)).cuda()
+    flat = rng.permutation(m * n)
+    with mad.Context() as c:
+        c.build(mad.dense(tA), mad.dense(tB), 1024, keep=(tA, tB))
+        for ncand, t in ((4096, 1), (4097, 512), (20_000, 2049), (140_001, 700), (300_000, 5000)):
+            q = flat[:ncand]
+            if kind == "tiny":
+                q = q[(q // n > 0) & (q % n > 0)]
+            cand = mad.encode_pairs(q // n, q % n, np.arange(1, len(q) + 1))
+            whole, nw = mad.mad_rescore(c.ctx, cand, len(q), len(q))
+            for _ in range(2):
+                top, nt = mad.mad_rescore(c.ctx, cand, len(q), t)
+                assert nw == len(q) and nt == t
+                assert torch.equal(top, whole[:t])
