@@ -163,6 +163,10 @@ struct mad_ctx {
   int64_t m = 0, d = 0, n = 0;
   uint64_t nnz_a = 0, nnz_b = 0;
   uint64_t s_max = 0, sampled = 0;
+  // X is empty (cleared, nothing added since), and X was last written whole
+  // by the region builder (keys beyond a group's regions in the overflow
+  // table, where a later insert would not look for them).
+  bool x_empty = false, x_built = false;
   int e1 = 0, f = 0;
   unsigned long long t1_total = 0;
   // Owned device memory.
@@ -333,7 +337,8 @@ mad_status pilot_inserts(mad_ctx* ctx, uint64_t n, uint64_t* hits, cudaStream_t 
 // regions whole (dense, non-Gram, one sorted batch); X then needs no
 // clearing beforehand.
 bool x_builder_applies(const mad_ctx* ctx, uint64_t s);
-// fresh_x: X is empty and this call is its only filling (the fused pass):
+// fresh_x: X is empty and this call is its only filling (the fused pass, and
+// mad_sample of the whole budget):
 // where x_builder_applies, the home regions are built whole.
 mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first,
                        cudaStream_t st, bool fresh_x = false);

@@ -411,3 +411,36 @@ def test_csr_pass_matches_oracle_eager_and_from_a_graph(name):
         st = mad.mad_stats(c.ctx)
         sc = o.scalars()
         assert st["inserted"] == sc["inserted"] and st["diag_skipped"] == sc["diag_skipped"]
+
+
+@pytest.mark.parametrize("m,d,n,s", [(2051, 100, 3001, 200_000), (300, 25, 200, 5000),
+                                     (1, 40, 1000, 3000), (40_000, 20, 500, 300_000)])
+def test_steps_in_one_call_equal_steps_in_two(m, d, n, s):
+    """The whole budget into an empty X (built region by region) holds the X
+    of two calls (inserted key by key); pairs added afterwards, a reset and a
+    second filling find it as they would find a plain table."""
+    import paper_1506_03872_gb300 as mad
+    A, B = _inputs(91, m, d, n)
+    tA, tB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    (ok, ov), sc = _oracle_x(A, B, 0, s, 17)
+    with mad.Context() as c:
+        c.build(mad.dense(tA), mad.dense(tB), s, keep=(tA, tB))
+        for fill in range(2):
+            if fill == 0:
+                mad.mad_sample(c.ctx, s, 17)
+            else:
+                mad.mad_reset_hash(c.ctx)
+                mad.mad_sample(c.ctx, s // 3, 17)
+                mad.mad_sample(c.ctx, s - s // 3, 17, s // 3)
+            keys, vals, cnt = _export_sorted(mad, c.ctx, s + 1)
+            assert cnt == len(ok) and np.array_equal(keys, ok) and np.array_equal(vals, ov)
+            st = mad.mad_stats(c.ctx)
+            assert st["inserted"] == sc["inserted"] and st["distinct"] == len(ok)
+        mad.mad_reset_hash(c.ctx)
+        mad.mad_sample(c.ctx, s, 17)
+        k = torch.from_numpy(ok.view(np.int64).copy()).cuda()
+        v = torch.from_numpy(ov.copy()).cuda()
+        mad.mad_accumulate(c.ctx, k, v)
+        keys, vals, cnt = _export_sorted(mad, c.ctx, s + 1)
+        assert cnt == len(ok) and np.array_equal(keys, ok) and np.array_equal(vals, 2 * ov)
+        assert mad.mad_stats(c.ctx)["distinct"] == len(ok)
