@@ -78,6 +78,8 @@ void free_tables(mad_ctx* ctx, cudaStream_t st) {
   free_async(ctx->T2g_ptr, st);
   free_async(ctx->T2g, st);
   free_async(ctx->T2g_sh, st);
+  free_async(ctx->rdesc, st);
+  free_async(ctx->brow, st);
   free_async(ctx->bloom, st);
   free_async(ctx->T1g, st);
   free_async(ctx->TBg, st);
@@ -512,6 +514,11 @@ mad_status mad_build_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix*
   if ((rs = alloc(ctx, ctx->T2g, (size_t)gtotal, st)) != MAD_OK) return rs;
   ctx->t2g_total = gtotal;
   if (gtotal && (rs = t2_guide_fill(ctx, st)) != MAD_OK) return rs;
+  if (ctx->nnz_a < (1ull << 32) && ctx->nnz_b < (1ull << 32) && gtotal < (1ull << 32)) {
+    if ((rs = alloc(ctx, ctx->rdesc, (size_t)ctx->m, st)) != MAD_OK) return rs;
+    if ((rs = alloc(ctx, ctx->brow, (size_t)ctx->d, st)) != MAD_OK) return rs;
+    if ((rs = row_desc_fill(ctx, st)) != MAD_OK) return rs;
+  }
   // Closure filter: 16 bits per entry, a power of two of 64-bit words.
   const uint64_t nnz_c = (ctx->flags & MAD_GRAM) ? ctx->nnz_a : ctx->nnz_b;
   ctx->bloom_lg = 10;

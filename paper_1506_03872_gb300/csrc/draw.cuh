@@ -100,11 +100,10 @@ __device__ __forceinline__ Draw draw_given_row(const SampleParams& p, const Unif
   if (p.integer) {
     // b_k'j != 0: the entry (j, k') of A under MAD_GRAM, else (k', j) of B.
     // The filter settles most tests with one load; the rest search rows.
-    const unsigned long long ekey = (p.flags & MAD_GRAM)
-                                        ? (((unsigned long long)j << 32) | (unsigned long long)kp)
-                                        : (((unsigned long long)kp << 32) | (unsigned long long)j);
+    const bool gram = (p.flags & MAD_GRAM) != 0;
     bool hit = false;
-    if (p.bloom && !bloom_may_contain(p.bloom, p.bloom_shift, ekey)) {
+    if (p.bloom && !bloom_may_contain(p.bloom, p.bloom_shift, (uint32_t)(gram ? j : kp),
+                                      (uint32_t)(gram ? kp : j))) {
       hit = false;
     } else if (p.flags & MAD_GRAM) {
       const int64_t c0 = __ldg(p.b_ptr + kp), clen = __ldg(p.b_ptr + kp + 1) - c0;

@@ -86,8 +86,13 @@ struct SampleParams {
   const unsigned long long* T2g_ptr;
   const uint32_t* T2g;
   const uint8_t* T2g_sh;
+  // 0/1 rows in one load each (null when an index does not fit in 32 bits):
+  // of A, the row's start, length, T2 total and guide start; of B, its start
+  // and length.
+  const uint4* rdesc;
+  const uint2* brow;
   // Bloom filter over the entries the 0/1 closure test looks up (null when
-  // absent): word mix64(key) >> bloom_shift holds five bits of each key.
+  // absent; see bloom_probe).
   const unsigned long long* bloom;
   int bloom_shift;
   // Guide of T1 (null when absent): entry b counts the prefix entries
@@ -181,6 +186,8 @@ struct mad_ctx {
   unsigned long long* T2g_ptr = nullptr;  // guides of long 0/1 T2 rows
   uint32_t* T2g = nullptr;
   uint8_t* T2g_sh = nullptr;
+  uint4* rdesc = nullptr;                 // row descriptors of A (0/1 inputs)
+  uint2* brow = nullptr;                  // rows of B (0/1 inputs)
   unsigned long long* bloom = nullptr;    // closure-test filter (0/1 inputs)
   int bloom_lg = 0;
   uint32_t* T1g = nullptr;                // guide of T1
@@ -294,6 +301,9 @@ mad_status t2_guide_offsets(mad_ctx* ctx, cudaStream_t st);
 // MAD_GRAM, else B) into ctx->bloom (2^bloom_lg words, cleared here).
 mad_status build_bloom(mad_ctx* ctx, cudaStream_t st);
 mad_status t2_guide_fill(mad_ctx* ctx, cudaStream_t st);
+// Row descriptors into ctx->rdesc (m) and ctx->brow (d), after the guides'
+// offsets; nothing where they are not allocated.
+mad_status row_desc_fill(mad_ctx* ctx, cudaStream_t st);
 // Guides of the dense TB rows into ctx->TBg (d rows of ctx->tbg_stride =
 // 2^tb_guide_width(n) + 1 entries) and ctx->TBg_sh (d shifts).
 int tb_guide_width(int64_t n);

@@ -81,6 +81,7 @@ mad_status enqueue_csr_build(mad_ctx* ctx, cudaStream_t st) {
   if ((rs = build_tables_impl(ctx, st)) != MAD_OK) return rs;
   if ((rs = t2_guide_offsets(ctx, st)) != MAD_OK) return rs;
   if (ctx->t2g_total && (rs = t2_guide_fill(ctx, st)) != MAD_OK) return rs;
+  if ((rs = row_desc_fill(ctx, st)) != MAD_OK) return rs;
   if ((rs = build_bloom(ctx, st)) != MAD_OK) return rs;
   if ((rs = t1_guide_fill(ctx, st)) != MAD_OK) return rs;
   return clear_x(ctx, st);

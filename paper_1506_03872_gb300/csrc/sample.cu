@@ -130,7 +130,8 @@ __device__ __forceinline__ void flush_tally(const SampleParams& p, Tally& t) {
   }
 }
 
-// Diamonds in index order (0/1 CSR inputs; dense inputs with alias draws).
+// Diamonds in index order: dense inputs with alias draws, and 0/1 inputs whose
+// indices do not fit the row descriptors (k_sample_rows takes the others).
 template <bool kAlias>
 __global__ void __launch_bounds__(256)
 k_sample(const SampleParams p_, unsigned long long seed, unsigned long long first,
@@ -145,6 +146,83 @@ k_sample(const SampleParams p_, unsigned long long seed, unsigned long long firs
     Draw dr{};
     if (q < s) dr = draw_one_as<kAlias>(p, seed, first + q, &t.bad);
     accumulate(p, q < s, dr, t);
+  }
+  flush_tally(p, t);
+}
+
+// 0/1 inputs: the loop body of Alg. 2 with what it needs of a row in one load
+// (SampleParams::rdesc, brow); the draws are those of draw_given_row.  v is 1
+// where the diamond closes.  Every lane of the warp calls it.
+//
+// Bound by random sectors (about ten a diamond: T1's guide, the row, its guide
+// and window of T2, the two columns, the row of B, its column, the filter
+// word), at 53 % of DRAM's rate, 61 % of L2's and 64 % of L1's at once, so it
+// wants every warp the SM holds (32 registers).  Five arrays' worth of row data
+// in one 16-byte load, a cheaper filter mix and T2 guides of about four entries
+// a bucket took 1e8 diamonds on the graph of 1e6 nodes from 6.12 to 4.62 ms
+// (3e7 on 20,011 nodes, all in L2: 1.63 to 1.34).  Tried and dropped: the same
+// diamonds in the order of their rows (the sort costs what the locality
+// saves, 4.77 ms at best), windows read as 16-byte quads (registers spill,
+// 7.0 ms), and leaving the loop body early where the filter rules a diamond
+// out (the warp's lanes then run apart for good, 10.1 ms).
+__device__ __forceinline__ Draw draw_rows(const SampleParams& p, bool valid,
+                                          unsigned long long seed, unsigned long long ell,
+                                          bool* bad) {
+  const bool gram = (p.flags & MAD_GRAM) != 0;
+  Draw dr{};
+  bool maybe = false;
+  if (valid) {
+    const Uniforms u = diamond_uniforms(seed, ell);
+    int64_t i = ub_guided_u64(p.T1, p.m, p.T1g, p.t1g_sh, draw_target(u.u0, p.t1_total));
+    if (i >= p.m) { *bad = true; i = p.m - 1; }
+    const uint4 ra = __ldg(p.rdesc + i);
+    const uint32_t* __restrict__ row = p.T2 + ra.x;
+    const uint32_t target = (uint32_t)draw_target(u.u1, ra.z);
+    uint32_t pk =
+        ra.y >= (uint32_t)kGuideMin
+            ? (uint32_t)ub_guided_u32(row, p.T2g + ra.w, t2_guide_shift(ra.y, ra.z), target)
+            : (uint32_t)ub_u32(row, (int)ra.y, target, 0xFFFFFFFFu);
+    if (pk >= ra.y) { *bad = true; pk = ra.y - 1; }
+    const uint32_t pkp = (uint32_t)draw_target(u.u3, ra.y);
+    dr.i = (uint32_t)i;
+    dr.k = (uint32_t)__ldg(p.a_col + ra.x + pk);
+    dr.kp = (uint32_t)__ldg(p.a_col + ra.x + pkp);
+    const uint2 rb = __ldg(p.brow + dr.k);
+    dr.j = (uint32_t)__ldg(p.b_col + rb.x + (uint32_t)draw_target(u.u2, rb.y));
+    // b_k'j != 0: the entry (j, k') of A under MAD_GRAM, else (k', j) of B.
+    maybe = !p.bloom || bloom_may_contain(p.bloom, p.bloom_shift, gram ? dr.j : dr.kp,
+                                          gram ? dr.kp : dr.j);
+  }
+  // The few lanes whose diamond may close are searched while the others wait,
+  // and the warp goes on together.
+  if (__any_sync(0xFFFFFFFFu, maybe)) {
+    if (maybe) {
+      const uint2 rc = __ldg(p.brow + dr.kp);
+      const uint4 rj = gram ? __ldg(p.rdesc + dr.j) : make_uint4(0u, 0xFFFFFFFFu, 0u, 0u);
+      // (under MAD_GRAM b_k'j = a_jk': the shorter of the two sorted rows)
+      const bool hit = gram && rj.y < rc.y
+                           ? contains_sorted(p.a_col + rj.x, rj.y, (int32_t)dr.kp)
+                           : contains_sorted(p.b_col + rc.x, rc.y, (int32_t)dr.j);
+      dr.v = hit ? 1 : 0;
+    }
+    __syncwarp();
+  }
+  return dr;
+}
+
+__global__ void __launch_bounds__(256, 8)
+k_sample_rows(const SampleParams p_, unsigned long long seed, unsigned long long first,
+              unsigned long long s) {
+  const SampleParams p = resolve(p_);
+  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+  const unsigned long long rounds = (s + stride - 1) / stride;
+  Tally t;
+  unsigned long long x = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+  for (unsigned long long r = 0; r < rounds; ++r, x += stride) {
+    const bool valid = x < s;
+    const Draw dr = draw_rows(p, valid, seed, first + x, &t.bad);
+    accumulate(p, valid, dr, t);
+    __syncwarp();
   }
   flush_tally(p, t);
 }
@@ -706,15 +784,22 @@ unsigned grid_of(unsigned long long work, int full) {
 constexpr unsigned long long kSortBatch = 1ull << 26;
 
 // Pilot for hash sizing: counts the diamonds that would be inserted.
+template <bool kRows>
 __global__ void __launch_bounds__(256)
 k_pilot(const SampleParams p_, unsigned long long seed, unsigned long long n,
         unsigned long long* __restrict__ hits) {
   const SampleParams p = resolve(p_);
   bool bad = false;
   unsigned long long c = 0;
-  for (unsigned long long q = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
-       q += (unsigned long long)gridDim.x * blockDim.x) {
-    const Draw dr = draw_one_as<false>(p, seed, q, &bad);
+  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+  const unsigned long long rounds = (n + stride - 1) / stride;
+  unsigned long long q = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+  for (unsigned long long r = 0; r < rounds; ++r, q += stride) {
+    const bool valid = q < n;
+    Draw dr{};
+    if (kRows) dr = draw_rows(p, valid, seed, q, &bad);
+    else if (valid) dr = draw_one_as<false>(p, seed, q, &bad);
+    if (!valid) dr.v = 0;
     c += (dr.v != 0 && !((p.flags & MAD_EXCLUDE_DIAG) && dr.i == dr.j)) ? 1 : 0;
     if (p.flags & MAD_SQUARE_SYM)
       c += (dr.v != 0 && !((p.flags & MAD_EXCLUDE_DIAG) && dr.k == dr.kp)) ? 1 : 0;
@@ -755,8 +840,10 @@ SampleParams make_params(const mad_ctx* ctx) {
   p.T2g_ptr = ctx->T2g_ptr;
   p.T2g = ctx->T2g;
   p.T2g_sh = ctx->T2g_sh;
+  p.rdesc = ctx->rdesc;
+  p.brow = ctx->brow;
   p.bloom = ctx->bloom;
-  p.bloom_shift = 64 - ctx->bloom_lg;
+  p.bloom_shift = 40 - ctx->bloom_lg;
   p.TBg = ctx->TBg;
   p.tbg_stride = ctx->tbg_stride;
   p.TBg_sh = ctx->TBg_sh;
@@ -791,7 +878,12 @@ mad_status pilot_inserts(mad_ctx* ctx, uint64_t n, uint64_t* hits, cudaStream_t 
   unsigned long long* dev = (unsigned long long*)ctx->scratch;
   cudaMemsetAsync(dev, 0, sizeof(unsigned long long), st);
   const SampleParams p = make_params(ctx);
-  k_pilot<<<grid_of(n, full_grid<k_pilot>()), 256, 0, st>>>(p, 0x9E3779B97F4A7C15ull, n, dev);
+  if (p.rdesc)
+    k_pilot<true><<<grid_of(n, full_grid<k_pilot<true>>()), 256, 0, st>>>(
+        p, 0x9E3779B97F4A7C15ull, n, dev);
+  else
+    k_pilot<false><<<grid_of(n, full_grid<k_pilot<false>>()), 256, 0, st>>>(
+        p, 0x9E3779B97F4A7C15ull, n, dev);
   count_launch(ctx);
   unsigned long long h = 0;
   cudaMemcpyAsync(&h, dev, sizeof(h), cudaMemcpyDeviceToHost, st);
@@ -893,7 +985,9 @@ mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first, 
   if (!ctx->dense || p.alias) {
     phase_event(ctx, 0, st);
     phase_event(ctx, 1, st);
-    if (p.alias)
+    if (p.rdesc)
+      k_sample_rows<<<grid_of(s, full_grid<k_sample_rows>()), 256, 0, st>>>(p, seed, first, s);
+    else if (p.alias)
       k_sample<true><<<grid_of(s, full_grid<k_sample<true>>()), 256, 0, st>>>(p, seed, first, s);
     else
       k_sample<false><<<grid_of(s, full_grid<k_sample<false>>()), 256, 0, st>>>(p, seed, first, s);

@@ -639,12 +639,10 @@ k_a_rows_binary(const int64_t* __restrict__ a_ptr, const int32_t* __restrict__ a
 // ---------------------------------------------------------------------------
 // Guides of long 0/1 T2 rows.  Row i (L >= kGuideMin entries, total tot)
 // gets buckets of width 2^sh, sh the smallest shift leaving at most about
-// L/4 buckets, and nb + 1 guide entries: entry b is the number of the row's
+// L/2 buckets, and nb + 1 guide entries: entry b is the number of the row's
 // prefix entries below b << sh, so the first entry above a target t lies
 // between guide entries t >> sh and (t >> sh) + 1.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int bitlen_u32(uint32_t x) { return x ? 32 - __clz(x) : 0; }
-
 __global__ void __launch_bounds__(256)
 k_guide_sizes(const int64_t* __restrict__ a_ptr, const uint32_t* __restrict__ T2, int64_t m,
               unsigned long long* __restrict__ sizes, uint8_t* __restrict__ shift) {
@@ -656,9 +654,7 @@ k_guide_sizes(const int64_t* __restrict__ a_ptr, const uint32_t* __restrict__ T2
     if (len >= kGuideMin) {
       const uint32_t tot = T2[a0 + len - 1];
       if (tot > 0) {
-        const int want = bitlen_u32((uint32_t)(len / 8));
-        sh = bitlen_u32(tot - 1) - want;
-        if (sh < 0) sh = 0;
+        sh = t2_guide_shift((uint32_t)len, tot);
         size = (unsigned long long)((tot - 1) >> sh) + 2;   // nb + 1
       }
     }
@@ -951,6 +947,38 @@ mad_status t2_guide_offsets(mad_ctx* ctx, cudaStream_t st) {
   return scan_exclusive_u64(ctx, (const uint64_t*)sizes, (uint64_t*)ctx->T2g_ptr, m, part, st);
 }
 
+// Row descriptors of the 0/1 sampler: what a draw needs of row i of A (start,
+// length, T2 total, guide start) and of row k of B (start, length) in one load
+// each, instead of two row pointers, the row's last T2 entry, the guide's
+// pointer and its shift from five arrays.
+__global__ void __launch_bounds__(256)
+k_row_desc(const int64_t* __restrict__ a_ptr, const uint32_t* __restrict__ T2, int64_t m,
+           const unsigned long long* __restrict__ gptr, const int64_t* __restrict__ b_ptr, int64_t d,
+           uint4* __restrict__ rdesc, uint2* __restrict__ brow) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m || i < d; i += stride) {
+    if (i < m) {
+      const int64_t a0 = a_ptr[i], len = a_ptr[i + 1] - a0;
+      rdesc[i] = make_uint4((uint32_t)a0, (uint32_t)len, len ? T2[a0 + len - 1] : 0u,
+                            (uint32_t)gptr[i]);
+    }
+    if (i < d) {
+      const int64_t b0 = b_ptr[i];
+      brow[i] = make_uint2((uint32_t)b0, (uint32_t)(b_ptr[i + 1] - b0));
+    }
+  }
+}
+
+mad_status row_desc_fill(mad_ctx* ctx, cudaStream_t st) {
+  if (!ctx->rdesc) return MAD_OK;
+  const int64_t rows = ctx->m > ctx->d ? ctx->m : ctx->d;
+  const int64_t blocks64 = (rows + 255) / 256;
+  k_row_desc<<<(unsigned)(blocks64 < 152 * 8 ? blocks64 : 152 * 8), 256, 0, st>>>(
+      ctx->A.rowptr, ctx->T2, ctx->m, ctx->T2g_ptr, ctx->B.rowptr, ctx->d, ctx->rdesc, ctx->brow);
+  count_launch(ctx);
+  return cuda_status(cudaGetLastError());
+}
+
 // One warp per row of the closure matrix; every entry (row, col) sets its
 // five bits.
 __global__ void __launch_bounds__(256)
@@ -971,8 +999,8 @@ k_bloom_build(const int64_t* __restrict__ ptr, const int32_t* __restrict__ col, 
     const bool longrow = e1 - e0 > 32;
     if (r < rows && !longrow) {
       for (int64_t e = e0; e < e1; ++e) {
-        const unsigned long long h = mix64(((unsigned long long)r << 32) | (uint32_t)col[e]);
-        atomicOr(words + (h >> shift), bloom_bits(h));
+        const BloomProbe b = bloom_probe((uint32_t)r, (uint32_t)col[e], shift);
+        atomicOr(words + b.word, ((unsigned long long)b.hi << 32) | b.lo);
       }
     }
     unsigned lm = __ballot_sync(0xFFFFFFFFu, r < rows && longrow);
@@ -982,8 +1010,8 @@ k_bloom_build(const int64_t* __restrict__ ptr, const int32_t* __restrict__ col, 
       const unsigned long long rr = (unsigned long long)(base + (int64_t)src * warps + w);
       const int64_t f0 = __shfl_sync(0xFFFFFFFFu, e0, src), f1 = __shfl_sync(0xFFFFFFFFu, e1, src);
       for (int64_t e = f0 + lane; e < f1; e += 32) {
-        const unsigned long long h = mix64((rr << 32) | (uint32_t)col[e]);
-        atomicOr(words + (h >> shift), bloom_bits(h));
+        const BloomProbe b = bloom_probe((uint32_t)rr, (uint32_t)col[e], shift);
+        atomicOr(words + b.word, ((unsigned long long)b.hi << 32) | b.lo);
       }
     }
   }
@@ -997,7 +1025,7 @@ mad_status build_bloom(mad_ctx* ctx, cudaStream_t st) {
   cudaMemsetAsync(ctx->bloom, 0, (sizeof(unsigned long long) << ctx->bloom_lg), st);
   const int64_t blocks64 = (rows + 7) / 8;
   const unsigned blocks = (unsigned)(blocks64 < 152 * 16 ? blocks64 : 152 * 16);
-  k_bloom_build<<<blocks, 256, 0, st>>>(ptr, col, rows, 64 - ctx->bloom_lg, ctx->bloom);
+  k_bloom_build<<<blocks, 256, 0, st>>>(ptr, col, rows, 40 - ctx->bloom_lg, ctx->bloom);
   count_launch(ctx);
   return cuda_status(cudaGetLastError());
 }
