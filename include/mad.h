@@ -297,8 +297,8 @@ mad_status mad_dense_topt(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* B
  * 1}| among the stored entries of C (c_ij >= 1), sorted by (c desc, i asc,
  * j asc), with c as an exact integer in the double and x = 0: the same
  * pairs and counts as a full sparse product for any input.
- * Because c_ij <= min(nnz(a_i*), nnz(b_*j)), a pilot product of the ~2048
- * rows and columns of largest degree gives a lower bound theta on the t-th
+ * Because c_ij <= min(nnz(a_i*), nnz(b_*j)), a pilot product of the 256 to
+ * 2048 rows and columns of largest degree gives a lower bound theta on the t-th
  * largest count, and the main pass covers only rows and columns with at
  * least theta entries, keeping counts >= theta (MAD_SPARSE_NO_BOUND: every
  * row and column, the threshold filtering entries only).  Counts are

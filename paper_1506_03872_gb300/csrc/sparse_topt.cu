@@ -8,8 +8,8 @@
 // entry tau, no row with fewer than theta entries and no column of B with
 // fewer than theta entries can hold a pair of the top t, so:
 //
-//   1. pilot: the exact counts among the ~2048 rows of A and columns of B of
-//      largest degree; the t-th largest of them is such a theta (t entries
+//   1. pilot: the exact counts among the rows of A and columns of B of largest
+//      degree (16 sqrt(t) of each, 256 to 2048); the t-th largest of them is such a theta (t entries
 //      of C are at least that large);
 //   2. main pass over the rows with nnz >= theta against the columns with
 //      nnz >= theta only: B is filtered to those columns and relabelled by
@@ -29,15 +29,24 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 #include "mad_internal.cuh"
 
 namespace mad {
 namespace {
 
-constexpr int kSpBlock = 256;
+constexpr int kSpBlock = 512;
 constexpr int kSpWarps = kSpBlock / 32;
 constexpr uint32_t kSpWindowMax = 24576;       // labels per shared window (96 KB)
-constexpr uint32_t kPilot = 2048;              // rows and columns of the pilot
+// Rows and columns of the pilot: its pairs have to hold t large counts, so its
+// side grows with sqrt(t).  16 sqrt(t) measured best between 8 and 64 (2048 at
+// t = 1000, the size it always had) on graphs of 2e4 to 1e6 nodes: 1e6 nodes, t
+// = 1000: 1224, 1070, 1093, 1098 and 1193 us at 8, 16, 24, 32 and 64.
+uint32_t pilot_size(uint32_t t) {
+  const double want = 16.0 * std::sqrt((double)t);
+  return want < 256.0 ? 256u : want > 2048.0 ? 2048u : (uint32_t)want;
+}
 constexpr uint32_t kHistSmem = 4096;           // pilot histogram bins (clamped)
 constexpr uint32_t kHistGlobal = 65536;        // main-pass histogram bins (clamped)
 constexpr uint64_t kSpListCap = 1ull << 20;    // candidate list entries
@@ -129,72 +138,135 @@ __global__ void k_mark_deg(const uint32_t* __restrict__ cb, uint64_t n, uint32_t
     sel[j] = (cb[j] >= th && cb[j] > 0) ? 1u : 0u;
 }
 
+// colmap: the selected columns in order; bits: the selection as a bitmap.
 __global__ void k_colmap(const uint32_t* __restrict__ sel, const uint32_t* __restrict__ pre,
-                         uint64_t n, uint32_t* colmap) {
-  for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n;
-       j += (uint64_t)gridDim.x * blockDim.x)
-    if (sel[j]) colmap[pre[j]] = (uint32_t)j;
-}
-
-// Entries of each row of B whose column is selected (one warp per row).
-__global__ void k_bf_count(const int64_t* __restrict__ bptr, const int32_t* __restrict__ bcol,
-                           uint64_t d, const uint32_t* __restrict__ sel, uint32_t* len) {
-  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const unsigned lane = threadIdx.x & 31;
-  const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  for (uint64_t k = warp; k < d; k += nw) {
-    const int64_t e0 = bptr[k], e1 = bptr[k + 1];
-    unsigned c = 0;
-    for (int64_t e = e0 + lane; e < e1; e += 32) c += sel[bcol[e]];
-    for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(FULL, c, o);
-    if (lane == 0) len[k] = c;
+                         uint64_t n, uint32_t* colmap, uint32_t* bits) {
+  const uint64_t n_up = (n + 31) & ~31ull;
+  for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n_up;
+       j += (uint64_t)gridDim.x * blockDim.x) {
+    const bool on = j < n && sel[j];
+    const unsigned w = __ballot_sync(FULL, on);
+    if ((threadIdx.x & 31) == 0) bits[j >> 5] = w;
+    if (on) colmap[pre[j]] = (uint32_t)j;
   }
 }
 
-// The selected entries, relabelled by their column's rank, in order.
-__global__ void k_bf_fill(const int64_t* __restrict__ bptr, const int32_t* __restrict__ bcol,
-                          uint64_t d, const uint32_t* __restrict__ sel,
-                          const uint32_t* __restrict__ pre, const uint32_t* __restrict__ optr,
-                          uint32_t* ocol) {
-  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const unsigned lane = threadIdx.x & 31;
-  const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  for (uint64_t k = warp; k < d; k += nw) {
-    const int64_t e0 = bptr[k], e1 = bptr[k + 1];
-    uint32_t out = optr[k];
-    for (int64_t base = e0; base < e1; base += 32) {
-      const int64_t e = base + lane;
-      uint32_t j = 0, s = 0;
-      if (e < e1) {
-        j = (uint32_t)bcol[e];
-        s = sel[j];
-      }
-      const unsigned bal = __ballot_sync(FULL, s != 0);
-      if (s) ocol[out + __popc(bal & ((1u << lane) - 1))] = pre[j];
-      out += __popc(bal);
+// ---- B restricted to the selected columns -----------------------------------
+// The entries of B stay in order, so the filtered rows are a compaction of the
+// entry array: one bit per entry (k_bf_bits), the places from the bits' running
+// count (k_bf_emit), and a row's start is the count of selected entries before
+// it (k_bf_ptr).  Entries are read as one stream, 32 consecutive ones per warp
+// and load, whatever the rows' lengths, and looked up in a shared-memory bitmap
+// of the columns (a block per SM; columns past its 1.6 million bits are looked
+// up in L2).  A warp per row with a 4-byte L2 lookup per entry spent 148 us
+// counting and 178 us filling for 2e7 entries in rows of 20, twice per call;
+// the four kernels here take 78 us in all.
+constexpr int kBfThreads = 1024;
+constexpr int kBfPer = 8;                            // entries per thread and chunk
+constexpr uint32_t kBfChunk = kBfThreads * kBfPer;   // 256 words of bits
+constexpr size_t kBfBitmapMax = 200 * 1024;
+
+template <bool kShared>
+__global__ void __launch_bounds__(kBfThreads)
+k_bf_bits(const int32_t* __restrict__ bcol, uint64_t nnz, const uint32_t* __restrict__ bits,
+          uint64_t n, uint32_t* __restrict__ ebits, uint32_t* __restrict__ chunk_cnt) {
+  extern __shared__ uint32_t sbits[];
+  __shared__ uint32_t total[2];
+  const unsigned tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (kShared)
+    for (uint64_t w = tid; w < (n + 31) / 32; w += kBfThreads) sbits[w] = bits[w];
+  if (tid < 2) total[tid] = 0;
+  __syncthreads();
+  const uint64_t chunks = (nnz + kBfChunk - 1) / kBfChunk;
+  unsigned par = 0;
+  for (uint64_t c = blockIdx.x; c < chunks; c += gridDim.x, par ^= 1) {
+    int32_t j[kBfPer];
+#pragma unroll
+    for (int r = 0; r < kBfPer; ++r) {
+      const uint64_t e = c * kBfChunk + (uint64_t)r * kBfThreads + tid;
+      j[r] = e < nnz ? __ldcs(bcol + e) : -1;
     }
+    unsigned mine = 0;
+#pragma unroll
+    for (int r = 0; r < kBfPer; ++r) {
+      const uint32_t w = (uint32_t)j[r] >> 5;
+      const bool on = j[r] >= 0 && (((kShared ? sbits[w] : __ldg(bits + w)) >> (j[r] & 31)) & 1u);
+      const unsigned bal = __ballot_sync(FULL, on);
+      if (lane == 0) {
+        ebits[c * (kBfChunk / 32) + r * (kBfThreads / 32) + warp] = bal;
+        mine += __popc(bal);
+      }
+    }
+    if (lane == 0 && mine) atomicAdd(&total[par], mine);
+    __syncthreads();   // (the other chunk parity's counter is free again)
+    if (tid == 0) {
+      chunk_cnt[c] = total[par];
+      total[par ^ 1] = 0;
+    }
+    __syncthreads();
+  }
+}
+
+// Places of a chunk's entries: wpre[w] = selected entries before word w, and
+// the entries' labels.
+__global__ void __launch_bounds__(256)
+k_bf_emit(const int32_t* __restrict__ bcol, uint64_t nnz, const uint32_t* __restrict__ ebits,
+          const uint32_t* __restrict__ chunk_off, const uint32_t* __restrict__ pre,
+          uint32_t* __restrict__ wpre, uint32_t* __restrict__ ocol) {
+  constexpr unsigned kWords = kBfChunk / 32;   // one per thread
+  static_assert(kWords == 256, "a word per thread");
+  __shared__ uint32_t swpre[kWords], sword[kWords], wsum[8];
+  const unsigned tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint64_t chunks = (nnz + kBfChunk - 1) / kBfChunk;
+  for (uint64_t c = blockIdx.x; c < chunks; c += gridDim.x) {
+    const uint32_t word = ebits[c * kWords + tid];
+    uint32_t inc = __popc(word);
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(FULL, inc, o);
+      if ((int)lane >= o) inc += y;
+    }
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    uint32_t before = chunk_off[c] + inc - __popc(word);
+    for (unsigned w = 0; w < warp; ++w) before += wsum[w];
+    wpre[c * kWords + tid] = before;
+    swpre[tid] = before;
+    sword[tid] = word;
+    __syncthreads();
+#pragma unroll 4
+    for (unsigned w = warp; w < kWords; w += 8) {
+      const uint32_t bw = sword[w];
+      if (!bw) continue;
+      if ((bw >> lane) & 1u) {
+        const int32_t j = __ldcs(bcol + c * kBfChunk + 32 * w + lane);
+        ocol[swpre[w] + __popc(bw & ((1u << lane) - 1u))] = __ldg(pre + j);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Start of every filtered row.
+__global__ void k_bf_ptr(const int64_t* __restrict__ bptr, uint64_t d, uint64_t nnz,
+                         const uint32_t* __restrict__ ebits, const uint32_t* __restrict__ wpre,
+                         const uint32_t* __restrict__ total, uint32_t* __restrict__ optr) {
+  for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k <= d;
+       k += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t e = (uint64_t)bptr[k];
+    optr[k] = e < nnz ? wpre[e >> 5] + __popc(ebits[e >> 5] & ((1u << (e & 31)) - 1u)) : *total;
   }
 }
 
 // First position in [lo, hi) whose label is >= L (hi if none); labels
-// ascending.  All lanes of the warp call it with the same arguments.
-__device__ __forceinline__ uint32_t warp_lower_bound(const uint32_t* __restrict__ lab,
-                                                     uint32_t lo, uint32_t hi, uint32_t L,
-                                                     unsigned lane) {
-  while (hi - lo > 32) {
-    const uint32_t step = (hi - lo + 31) / 32;
-    const uint32_t pos = lo + lane * step;
-    const uint32_t v = pos < hi ? lab[pos] : 0xffffffffu;
-    const unsigned c = __popc(__ballot_sync(FULL, v < L));
-    if (c == 0) return lo;
-    const uint32_t nlo = lo + (c - 1) * step + 1;
-    const uint32_t nhi = lo + c * step < hi ? lo + c * step : hi;
-    lo = nlo;
-    hi = nhi;
+// ascending.
+__device__ __forceinline__ uint32_t lower_bound(const uint32_t* __restrict__ lab, uint32_t lo,
+                                                uint32_t hi, uint32_t L) {
+  while (lo < hi) {
+    const uint32_t mid = lo + ((hi - lo) >> 1);
+    if (__ldg(lab + mid) < L) lo = mid + 1;
+    else hi = mid;
   }
-  const uint32_t pos = lo + lane;
-  const uint32_t v = pos < hi ? lab[pos] : 0xffffffffu;
-  return lo + __popc(__ballot_sync(FULL, v < L));
+  return lo;
 }
 
 struct SpRowParams {
@@ -264,16 +336,44 @@ __global__ void __launch_bounds__(kSpBlock) k_spgemm_rowblock_topk(SpRowParams p
     for (uint32_t w0 = (lo / p.window) * p.window; w0 < p.nlab; w0 += p.window) {
       const uint32_t w1 = w0 + p.window < p.nlab ? w0 + p.window : p.nlab;
       const uint32_t L = lo > w0 ? lo : w0;
-      // Accumulate: warp per entry a_ik, lanes over row k of the filtered B.
-      for (int64_t q = a0 + warp; q < a1; q += kSpWarps) {
-        const uint32_t k = (uint32_t)p.acol[q];
-        const uint32_t b0 = p.bptr[k], b1 = p.bptr[k + 1];
-        if (b0 == b1) continue;
-        const uint32_t start = L == 0 ? b0 : warp_lower_bound(p.bcol, b0, b1, L, lane);
-        for (uint32_t e = start + lane; e < b1; e += 32) {
-          const uint32_t lab = p.bcol[e];
-          if (lab >= w1) break;
-          atomicAdd(&acc[lab - w0], 1u);
+      // Accumulate: each warp takes 32 of row i's entries at a time, every
+      // kSpWarps-th one (graphs are often numbered by weight, so that
+      // neighbouring entries are heavy together): lane l finds the part of its
+      // entry's filtered row inside the window (32 searches side by side), then
+      // the warp goes through the 32 parts in pieces of up to 32 labels, four
+      // pieces in flight.  A warp per entry in turn waited for four dependent
+      // loads on each (main pass on 1e6 nodes 865 us, now 576; with 512
+      // threads a row instead of 256, 480).
+      const uint32_t alen = (uint32_t)(a1 - a0);
+      for (uint32_t q0 = 0; q0 < alen; q0 += 32 * kSpWarps) {
+        uint32_t start = 0, len = 0;
+        const uint32_t q = q0 + lane * kSpWarps + warp;
+        if (q < alen) {
+          const uint32_t k = (uint32_t)__ldg(p.acol + a0 + q);
+          const uint32_t b0 = __ldg(p.bptr + k), b1 = __ldg(p.bptr + k + 1);
+          start = L == 0 ? b0 : lower_bound(p.bcol, b0, b1, L);
+          const uint32_t end = w1 == p.nlab ? b1 : lower_bound(p.bcol, start, b1, w1);
+          len = end - start;
+        }
+        unsigned todo = __ballot_sync(FULL, len != 0);
+        uint32_t s = 0, left = 0;   // the current part: its next label, labels left
+        while (todo || left) {
+          uint32_t v[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            if (left == 0 && todo) {
+              const int r = __ffs(todo) - 1;
+              todo &= todo - 1;
+              s = __shfl_sync(FULL, start, r);
+              left = __shfl_sync(FULL, len, r);
+            }
+            v[u] = lane < left ? __ldg(p.bcol + s + lane) : 0xffffffffu;
+            s += 32;
+            left = left > 32 ? left - 32 : 0;
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (v[u] != 0xffffffffu) atomicAdd(&acc[v[u] - w0], 1u);
         }
       }
       __syncthreads();
@@ -424,7 +524,8 @@ size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Scratch of one call.
 struct SpWs {
-  uint32_t *cb, *rorder, *corder, *sel, *pre, *colmap, *blen, *bp, *bcol, *part, *hist;
+  uint32_t *cb, *rorder, *corder, *sel, *pre, *colmap, *bits, *bp, *bcol, *part, *hist;
+  uint32_t *ebits, *wpre, *ccnt, *coff;
   unsigned long long *tiecnt, *tiepre, *part64;
   SpScalars* sc;
   SelectWs sel_ws;
@@ -438,7 +539,8 @@ size_t sp_ws_bytes(uint64_t m, uint64_t d, uint64_t n, uint64_t nnzb, uint64_t t
     off += align_up(bytes);
     return p;
   };
-  const uint64_t parts = scan_partial_elems((n > d ? n : d) + 1);
+  const uint64_t chunks = nnzb / kBfChunk + 1;
+  const uint64_t parts = scan_partial_elems((n > chunks ? n : chunks) + 1);
   SpWs w{};
   w.cb = (uint32_t*)take(4 * n);
   w.rorder = (uint32_t*)take(4 * m);
@@ -446,7 +548,11 @@ size_t sp_ws_bytes(uint64_t m, uint64_t d, uint64_t n, uint64_t nnzb, uint64_t t
   w.sel = (uint32_t*)take(4 * (n + 1));
   w.pre = (uint32_t*)take(4 * (n + 1));
   w.colmap = (uint32_t*)take(4 * n);
-  w.blen = (uint32_t*)take(4 * (d + 1));
+  w.bits = (uint32_t*)take(4 * (n / 32 + 1));
+  w.ebits = (uint32_t*)take(4 * chunks * (kBfChunk / 32));
+  w.wpre = (uint32_t*)take(4 * chunks * (kBfChunk / 32));
+  w.ccnt = (uint32_t*)take(4 * chunks);
+  w.coff = (uint32_t*)take(4 * (chunks + 1));
   w.bp = (uint32_t*)take(4 * (d + 1));
   w.bcol = (uint32_t*)take(4 * (nnzb ? nnzb : 1));
   w.part = (uint32_t*)take(4 * parts);
@@ -538,6 +644,8 @@ mad_status mad_sparse_topt(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* 
   const size_t smem_max = (size_t)kSpWindowMax * 4 + (size_t)kHistSmem * 4;
   cudaFuncSetAttribute(k_spgemm_rowblock_topk, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)smem_max);
+  cudaFuncSetAttribute(k_bf_bits<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)kBfBitmapMax);
 
   // Selected columns -> labels and the filtered, relabelled B.
   auto select_columns = [&](bool from_list, uint32_t h, uint32_t th) -> mad_status {
@@ -550,13 +658,21 @@ mad_status mad_sparse_topt(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* 
     count_launch(ctx);
     mad_status r = scan_exclusive_u32(ctx, w.sel, w.pre, n, w.part, st);
     if (r != MAD_OK) return r;
-    k_colmap<<<blocks_for(n, grid_stream), 256, 0, st>>>(w.sel, w.pre, n, w.colmap);
-    const unsigned wg = blocks_for(d * 32, (unsigned)sms * 16);
-    k_bf_count<<<wg, 256, 0, st>>>(B->rowptr, B->colidx, d, w.sel, w.blen);
+    k_colmap<<<blocks_for(n, grid_stream), 256, 0, st>>>(w.sel, w.pre, n, w.colmap, w.bits);
+    const uint64_t chunks = (nnzb + kBfChunk - 1) / kBfChunk;
+    const size_t bitmap = (size_t)((n + 31) / 32) * 4;
+    const unsigned bg = (unsigned)(chunks < (uint64_t)sms ? (chunks ? chunks : 1) : sms);
+    if (bitmap <= kBfBitmapMax)
+      k_bf_bits<true><<<bg, kBfThreads, bitmap, st>>>(B->colidx, nnzb, w.bits, n, w.ebits, w.ccnt);
+    else
+      k_bf_bits<false><<<bg, kBfThreads, 0, st>>>(B->colidx, nnzb, w.bits, n, w.ebits, w.ccnt);
     count_launch(ctx, 2);
-    if ((r = scan_exclusive_u32(ctx, w.blen, w.bp, d, w.part, st)) != MAD_OK) return r;
-    k_bf_fill<<<wg, 256, 0, st>>>(B->rowptr, B->colidx, d, w.sel, w.pre, w.bp, w.bcol);
-    count_launch(ctx);
+    if ((r = scan_exclusive_u32(ctx, w.ccnt, w.coff, chunks, w.part, st)) != MAD_OK) return r;
+    k_bf_emit<<<(unsigned)(chunks < grid_stream ? (chunks ? chunks : 1) : grid_stream), 256, 0, st>>>(
+        B->colidx, nnzb, w.ebits, w.coff, w.pre, w.wpre, w.bcol);
+    k_bf_ptr<<<blocks_for(d + 1, grid_stream), 256, 0, st>>>(B->rowptr, d, nnzb, w.ebits, w.wpre,
+                                                             w.coff + chunks, w.bp);
+    count_launch(ctx, 2);
     return cuda_status(cudaGetLastError());
   };
 
@@ -603,8 +719,9 @@ mad_status mad_sparse_topt(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* 
 
   // 1. Pilot: the heaviest rows against the heaviest columns, every stored
   //    entry counted into the histogram; its t-th largest is theta_0.
-  const uint32_t hr = (uint32_t)(rows_nz < kPilot ? rows_nz : kPilot);
-  const uint32_t hc = (uint32_t)(cols_nz < kPilot ? cols_nz : kPilot);
+  const uint32_t pilot = pilot_size(t);
+  const uint32_t hr = (uint32_t)(rows_nz < pilot ? rows_nz : pilot);
+  const uint32_t hc = (uint32_t)(cols_nz < pilot ? cols_nz : pilot);
   if ((rs = select_columns(true, hc, 0)) != MAD_OK) return rs;
   cudaMemsetAsync(w.hist, 0, 4 * kHistGlobal, st);
   // The pilot's rows are the first hr of the row order: count them through
