@@ -102,6 +102,8 @@ void free_tables(mad_ctx* ctx, cudaStream_t st) {
   ctx->pipe_scratch_bytes = 0;
   ctx->pipe = false;
   free_async(ctx->mips_buf, st);
+  free_async(ctx->mips_tb, st);
+  free_async(ctx->mips_blocks, st);
   ctx->mips_items = false;
   ctx->mips_nq = 0;
   ctx->built = false;

@@ -189,6 +189,12 @@ __device__ __forceinline__ int64_t ub_guided_u64(const uint64_t* __restrict__ P,
   return pos < len ? pos : len;
 }
 
+// FP32 sums of products against the exact c (d <= 1024, 32 lane partials
+// folded in halves): |c~ - c| <= kBoundEps sum |a_k b_k| + kBoundTiny (the
+// derivation stands with k_rescore_bound).
+constexpr float kBoundEps = 1.02f * 64.0f / 16777216.0f;
+constexpr float kBoundTiny = 1e-37f;
+
 // Bits of x (0 for 0).
 __device__ __forceinline__ int bitlen_u32(uint32_t x) { return x ? 32 - __clz(x) : 0; }
 

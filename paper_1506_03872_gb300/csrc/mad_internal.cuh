@@ -231,6 +231,8 @@ struct mad_ctx {
   int mips_slots = 0;                     // table slots of a part
   size_t mips_parts_smem = 0;
   void* mips_buf = nullptr;               // the batch's device buffer (mips.cu)
+  uint2* mips_tb = nullptr;               // total and bucket factor of every row of TB
+  uint4* mips_blocks = nullptr;           // TB's rows in 64-byte blocks (mips.cu)
   // Launch shape of batched queries (mad_mips_config): the load of a part's
   // table is 0.6 / 2^(mips_region_lg - 1), 256 x mips_chunk_mult diamonds per
   // chunk (the plan's value in mips_plan_mult), draw blocks per SM (0: one

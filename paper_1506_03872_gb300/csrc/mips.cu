@@ -25,7 +25,7 @@
 // by one block per query), a diamond moves 16 bytes of records in and out
 // instead of about 250, no global atomic is left, and a query's selection is
 // spread over its parts.  Measured on one GB300: 1e4 queries of 5e4 diamonds
-// on 1e6 items x 300, 142.6 -> 56.2 ms; 61 queries on 50,021 x 100, 1272 -> 254 us.
+// on 1e6 items x 300, 142 -> 43.9 ms; 61 queries on 50,021 x 100, 1300 -> 233 us.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -76,41 +76,92 @@ __device__ __forceinline__ void ub2_shared(const uint32_t* P, const uint32_t* Q,
   *oq = b;
 }
 
-// ub_guided_u32 for row k of TB, the window read 16 bytes at a time: at most
-// kQuads aligned quads hold a window of 17 or fewer entries.  Entries of the row
-// before the window are at most the target and entries after it above, so
-// whole quads are counted and only the row's own ends are checked (TB is
-// allocated with four entries of padding).
-constexpr int kQuads = 5;
-__device__ __forceinline__ int64_t ub_tb(const SampleParams& p, int64_t k, uint32_t target) {
-  const uint32_t* __restrict__ G = p.TBg + k * p.tbg_stride;
-  const uint32_t b = target >> (int)__ldg(p.TBg_sh + k);
-  const uint32_t lo = __ldg(G + b), hi = __ldg(G + b + 1);
-  const int64_t row = k * p.n;
-  if (hi - lo > 17u)
-    return (int64_t)lo + ub_u32(p.TB + row + lo, (int)(hi - lo), target, PREFIX_MASK);
-  const int64_t e0 = (row + lo) & ~(int64_t)3;
-  const int quads = (int)((row + hi - e0 + 3) >> 2);
-  uint4 w[kQuads];
-#pragma unroll
-  for (int q = 0; q < kQuads; ++q)
-    if (q < quads) w[q] = __ldg(reinterpret_cast<const uint4*>(p.TB + e0) + q);
-  const int64_t first = e0 - row;   // (below 0 by up to 3 in a row's first quad)
-  int cnt = 0;
-  const bool inner = first >= 0 && first + 4 * kQuads <= p.n;
-#pragma unroll
-  for (int q = 0; q < kQuads; ++q) {
-    if (q < quads) {
-      const uint32_t v[4] = {w[q].x, w[q].y, w[q].z, w[q].w};
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int64_t at = first + 4 * q + c;
-        const bool in_row = inner || (at >= 0 && at < p.n);
-        cnt += (in_row && (v[c] & PREFIX_MASK) <= target) ? 1 : 0;
+// ---- TB in 64-byte blocks ----------------------------------------------------
+// The draw of j is one aligned 64-byte read.  Row k's targets [0, total) are
+// cut into about n / kBlockKeys equal buckets, bucket of target t = t * mul /
+// 2^32; block b holds lo, the number of the row's entries at most bucket b's
+// first target, and entries lo, lo + 1, ... up to 15 of them (sign bits
+// included), padded with entries above every target.  The first entry above
+// a target of the bucket is among entries lo .. lo', lo' the next block's lo, so
+// it is in the block when lo' - lo < 15 (all but 0.1 % of the buckets where
+// six entries a bucket are expected); otherwise TB is searched between the two.
+// Against the row guides of tb_guide_build (two entries of the guide, then a
+// window of up to 17 entries of TB at any alignment: three or four 64-byte
+// fetches from DRAM for a million items, 383 bytes a diamond with b_k'j) this
+// is one, for 10.7 bytes an entry of TB instead of at most 4: 1e4 queries of 5e4
+// diamonds, draws 38.3 -> 29.1 ms.
+constexpr int kBlockKeys = 6;
+constexpr int kBlockEnts = 15;
+
+__host__ __device__ inline int64_t tb_blocks(int64_t n) { return (n + kBlockKeys - 1) / kBlockKeys; }
+
+// First target of bucket b: the smallest t with t * mul >= b * 2^32.
+__device__ __forceinline__ unsigned long long bucket_first(unsigned long long b,
+                                                           unsigned long long mul) {
+  return ((b << 32) + mul - 1) / mul;
+}
+
+// Row k's total, mul and blocks [k (nb + 1), (k + 1) (nb + 1)); the last block
+// only ends the one before it.
+__global__ void __launch_bounds__(256)
+k_mips_blocks(const uint32_t* __restrict__ TB, int64_t d, int64_t n, uint2* __restrict__ tb_row,
+              uint4* __restrict__ blocks) {
+  const int64_t nb = tb_blocks(n);
+  for (int64_t k = blockIdx.y; k < d; k += gridDim.y) {
+    const uint32_t* __restrict__ row = TB + k * n;
+    const uint32_t tot = __ldg(row + n - 1) & PREFIX_MASK;
+    // (t mul < 2^32 nb for t < tot, so every bucket is below nb)
+    const unsigned long long mul = tot ? ((unsigned long long)nb << 32) / tot : 0ull;
+    const uint32_t m32 = mul < 0xFFFFFFFFull ? (uint32_t)mul : 0xFFFFFFFFu;
+    if (blockIdx.x == 0 && threadIdx.x == 0) tb_row[k] = make_uint2(tot, m32);
+    uint4* __restrict__ out = blocks + k * (nb + 1) * 4;
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b <= nb;
+         b += (int64_t)gridDim.x * blockDim.x) {
+      uint32_t lo = (uint32_t)n;
+      if (m32) {
+        const unsigned long long first = bucket_first((unsigned long long)b, m32);
+        if (b == 0) lo = (uint32_t)ub_u32(row, (int)n, 0u, PREFIX_MASK);
+        else if (first < tot) lo = (uint32_t)ub_u32(row, (int)n, (uint32_t)first, PREFIX_MASK);
       }
+      uint32_t v[16];
+      v[0] = lo;
+#pragma unroll
+      for (int c = 0; c < kBlockEnts; ++c) {
+        const int64_t e = (int64_t)lo + c;
+        v[1 + c] = e < n ? __ldg(row + e) : PREFIX_MASK;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        out[4 * b + q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     }
   }
-  return (first > 0 ? first : 0) + cnt;
+}
+
+// First entry of row k of TB above target and its sign bit.
+__device__ __forceinline__ int64_t ub_block(const SampleParams& p, const uint4* __restrict__ blocks,
+                                            int64_t nb, int64_t k, uint32_t mul, uint32_t target,
+                                            uint32_t* sign) {
+  const uint4* __restrict__ blk = blocks + (k * (nb + 1) + __umulhi(target, mul)) * 4;
+  const uint4 a = __ldg(blk), b = __ldg(blk + 1), c = __ldg(blk + 2), e = __ldg(blk + 3);
+  const uint32_t v[kBlockEnts] = {a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x,
+                                  c.y, c.z, c.w, e.x, e.y, e.z, e.w};
+  int cnt = 0;
+  uint32_t s = 0;
+#pragma unroll
+  for (int u = kBlockEnts - 1; u >= 0; --u) {
+    const bool le = (v[u] & PREFIX_MASK) <= target;
+    cnt += le ? 1 : 0;
+    s = le ? s : v[u];
+  }
+  *sign = s & SIGN_BIT;
+  if (cnt < kBlockEnts) return (int64_t)a.x + cnt;
+  // Every entry held is at most the target: search on to the next block's lo.
+  const uint32_t* __restrict__ row = p.TB + k * p.n;
+  const uint32_t lo = a.x + kBlockEnts, hi = __ldg((const uint32_t*)(blk + 4));
+  const int64_t j =
+      (int64_t)lo + (hi > lo ? ub_u32(row + lo, (int)(hi - lo), target, PREFIX_MASK) : 0);
+  if (j < p.n) *sign = __ldg(row + j) & SIGN_BIT;
+  return j;
 }
 
 // The part of column j among `parts`: the high bits of a mix of j (the
@@ -121,25 +172,31 @@ __device__ __forceinline__ uint32_t part_of(uint32_t h, uint32_t parts) {
 
 // Step 1 (see above).  chunk c: diamonds (c - cbase) * chunk ... of query
 // chunk_q[c].  Shared memory: the query's T2 and TA rows, the chunk's records,
-// their parts and ranks, the parts' counts.  Bound by random sectors: per
-// diamond the guide (1 sector), its window of TB (2 to 3) and b_k'j (1), mostly
-// in DRAM for a million items.
+// their parts and ranks, the parts' counts.  Bound by DRAM's random reads: per
+// diamond a block of TB (64 bytes) and b_k'j (a sector, fetched as 64 bytes) for
+// a million items, 3.4e10 of them a second; 2 to 5 resident blocks per SM measure
+// the same, 6 leave too little L1 (8.46 instead of 6.59 ms for 1500 queries).
 __global__ void __launch_bounds__(kDrawThreads, 4)
 k_mips_draw(const SampleParams p, unsigned long long seed, const MipsQuery* __restrict__ queries,
             const uint32_t* __restrict__ chunk_q, unsigned long long nchunks, int mult,
-            uint32_t max_parts, uint2* __restrict__ rec, uint16_t* __restrict__ off) {
+            uint32_t max_parts, const uint2* __restrict__ tb_row,
+            const uint4* __restrict__ blocks, uint2* __restrict__ rec,
+            uint16_t* __restrict__ off) {
   extern __shared__ __align__(16) unsigned char draw_smem[];
   const int chunk = mult * kDrawThreads;
   const int d = (int)p.d;
   uint2* srec = (uint2*)draw_smem;                    // chunk records
-  uint32_t* splace = (uint32_t*)(srec + chunk);       // part << 16 | rank in it
+  uint2* stb = srec + chunk;                          // total and mul of TB's rows
+  uint32_t* splace = (uint32_t*)(stb + d);            // part << 16 | rank in it
   uint32_t* scnt = splace + chunk;                    // max_parts counts, then offsets
   uint32_t* s2 = scnt + max_parts + 1;                // T2 row
   uint32_t* sa = s2 + d;                              // TA row
   uint16_t* sord = (uint16_t*)(sa + d);               // source of each place
   __shared__ uint32_t warp_sum[kDrawThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t nb = tb_blocks(p.n);
   bool bad = false;
+  for (int x = tid; x < d; x += kDrawThreads) stb[x] = __ldg(tb_row + x);
   for (unsigned long long c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const uint32_t q = __ldg(chunk_q + c);
     const MipsQuery mq = queries[q];
@@ -160,11 +217,11 @@ k_mips_draw(const SampleParams p, unsigned long long seed, const MipsQuery* __re
                  (uint32_t)draw_target(un.u3, tatot), &k, &kp);
       if (k >= d) { bad = true; k = d - 1; }
       if (kp >= d) { bad = true; kp = d - 1; }
-      const int64_t row = (int64_t)k * p.n;
-      const uint32_t tbtot = __ldg(p.TB + row + p.n - 1) & PREFIX_MASK;
-      int64_t j = ub_tb(p, k, (uint32_t)draw_target(un.u2, tbtot));
+      const uint2 tb = stb[k];
+      uint32_t sj;
+      int64_t j = ub_block(p, blocks, nb, k, tb.y, (uint32_t)draw_target(un.u2, tb.x), &sj);
       if (j >= p.n) { bad = true; j = p.n - 1; }
-      const uint32_t sign = (s2[k] ^ sa[kp] ^ __ldg(p.TB + row + j)) & SIGN_BIT;
+      const uint32_t sign = sj ^ ((s2[k] ^ sa[kp]) & SIGN_BIT);
       const float b = __ldg((const float*)p.b_val + (int64_t)kp * p.ldb + j);
       const uint32_t part = part_of(fmix32((uint32_t)j), mq.parts);
       const uint32_t rank = atomicAdd(&scnt[part], 1u);
@@ -211,7 +268,6 @@ k_mips_draw(const SampleParams p, unsigned long long seed, const MipsQuery* __re
 struct PickState {
   alignas(16) uint32_t hist[kBins];
   uint32_t warp_sum[32];
-  unsigned long long maxx;
   uint32_t total, bin, above, in_bin;
 };
 
@@ -251,39 +307,30 @@ __device__ void pick_bin(PickState* st, uint32_t need, uint32_t above) {
 // A threshold (xt, njt): the elements with x > xt, or x == xt and ~j >= njt,
 // hold the `need` first by (x desc, j asc) and are at most cap (> need).
 // get(e, &x, &j) is element e < n, false where there is none (or x <= 0).
-// Digits of 11 bits from the leading one of the largest x downwards, then of
-// ~j among equal x; the search ends as soon as the ties of the last digit
+// First the logarithmic bucket of x (16 to an octave: for a few hundred of
+// several thousand that is mostly enough), then digits of 11 bits below it, then
+// of ~j among equal x; the search ends as soon as the ties of the last step
 // fit, and the composite is distinct, so it always ends.  Every thread of the
 // block.
 template <typename Get>
 __device__ void find_threshold(PickState* st, int n, uint32_t need, uint32_t cap, Get get,
                                unsigned long long* xt, uint32_t* njt) {
   const int tid = threadIdx.x, lane = tid & 31;
-  if (tid == 0) {
-    st->maxx = 0;
-    st->total = 0;
-  }
+  if (tid == 0) st->total = 0;
+  for (int b = tid; b < kBins; b += blockDim.x) st->hist[b] = 0;
   __syncthreads();
-  unsigned long long mx = 0;
   uint32_t cnt = 0;
   for (int e = tid; e < n; e += blockDim.x) {
     unsigned long long x;
     uint32_t j;
     if (get(e, &x, &j)) {
       ++cnt;
-      mx = x > mx ? x : mx;
+      atomicAdd(&st->hist[log_bucket(x)], 1u);
     }
   }
 #pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) {
-    const unsigned long long v = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
-    mx = v > mx ? v : mx;
-    cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, o);
-  }
-  if (lane == 0 && cnt) {
-    atomicMax(&st->maxx, mx);
-    atomicAdd(&st->total, cnt);
-  }
+  for (int o = 16; o >= 1; o >>= 1) cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, o);
+  if (lane == 0 && cnt) atomicAdd(&st->total, cnt);
   __syncthreads();
   *xt = 1;
   *njt = 0;
@@ -291,9 +338,19 @@ __device__ void find_threshold(PickState* st, int n, uint32_t need, uint32_t cap
     __syncthreads();
     return;
   }
-  int top = 64 - __clzll((long long)st->maxx);   // bits of x not yet fixed
-  unsigned long long prefix = 0;                  // x >> top of the threshold's digits
-  uint32_t above = 0;
+  pick_bin(st, need, 0);
+  const uint32_t b0 = st->bin;
+  uint32_t above = st->above;
+  const uint32_t in_b0 = st->in_bin;
+  __syncthreads();
+  if (above + in_b0 <= cap) {
+    *xt = bucket_floor(b0);
+    return;
+  }
+  // The bucket's values share their leading bits: the exponent's and four more.
+  const int ex = (int)(b0 >> 4);
+  int top = ex >= 4 ? ex - 4 : 0;                      // bits of x not yet fixed
+  unsigned long long prefix = bucket_floor(b0) >> top;  // x >> top of the threshold
   while (top > 0) {
     const int width = top < 11 ? top : 11, sh = top - width;
     for (int b = tid; b < kBins; b += blockDim.x) st->hist[b] = 0;
@@ -604,10 +661,49 @@ k_mips_final(const MipsQuery* __restrict__ queries, const Kept* __restrict__ kep
       cand_out[(size_t)q * tprime + x] = pr;
     }
   }
-  // Exact rescoring, one warp per candidate.
+  // Exact rescoring, one warp per candidate; when t is a small part of K, only
+  // of the candidates that FP32 bounds leave (as k_rescore_bound: FP64 runs at
+  // a sixty-fourth of FP32, and t' = 100 products of d = 300 cost a query 12 us
+  // of it): a candidate whose U lies below t others' L is not among the t largest.
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const float* __restrict__ a = Q + (int64_t)q * ldq;
+  static_assert(kSortMax >= 2 * kTPrimeMax, "bounds in the upper half of cx");
+  float2* lu = (float2*)(cx + kTPrimeMax);
+  const bool bounded = 4 * (int)t <= K;
+  if (bounded) {
+    for (int x = warp; x < K; x += warps) {
+      const float* __restrict__ b = Bt + (int64_t)(uint32_t)ck[x] * d;
+      float c = 0.0f, s = 0.0f;
+      for (int64_t k = lane; k < d; k += 32) {
+        c = fmaf(a[k], b[k], c);
+        s = fmaf(fabsf(a[k]), fabsf(b[k]), s);
+      }
+#pragma unroll
+      for (int off = 16; off >= 1; off >>= 1) {
+        c += __shfl_xor_sync(0xFFFFFFFFu, c, off);
+        s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+      }
+      if (lane == 0) {
+        const float inf = __int_as_float(0x7F800000);
+        const bool known = s < inf && fabsf(c) < inf;
+        const float e = fmaf(s, kBoundEps, kBoundTiny);
+        lu[x] = known ? make_float2(fabsf(c) - e, fabsf(c) + e) : make_float2(0.0f, inf);
+      }
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < K; x += blockDim.x) {
+      const float up = lu[x].y;
+      int over = 0;
+      for (int y = 0; y < K; ++y) over += lu[y].x > up ? 1 : 0;
+      if (over >= (int)t) ck[x] = ~0ull;   // sorts last, as a padding entry
+    }
+    __syncthreads();
+  }
   for (int x = warp; x < K; x += warps) {
+    if (ck[x] == ~0ull) {
+      if (lane == 0) cc[x] = -1.0;
+      continue;
+    }
     const float* __restrict__ b = Bt + (int64_t)(uint32_t)ck[x] * d;
     double acc = 0.0;
     for (int64_t k = lane; k < d; k += 32) acc = __fma_rn((double)a[k], (double)b[k], acc);
@@ -666,7 +762,7 @@ size_t parts_smem_bytes(int slots, uint32_t cap) {
 }
 
 size_t draw_smem_bytes(int chunk, uint32_t parts, int64_t d) {
-  return (size_t)chunk * (8 + 4 + 2) + ((size_t)parts + 1 + 2 * (size_t)d) * 4;
+  return (size_t)chunk * (8 + 4 + 2) + ((size_t)parts + 1 + 4 * (size_t)d) * 4;
 }
 
 // The batch's device buffer: the queries, the query of every chunk and part,
@@ -726,7 +822,8 @@ mad_status mad_mips_items(mad_ctx* ctx, const mad_matrix* B, uint64_t s_max, mad
   pool_free(ctx->hreg, st); pool_free(ctx->T2g_ptr, st);
   pool_free(ctx->T2g, st); pool_free(ctx->T2g_sh, st); pool_free(ctx->bloom, st);
   pool_free(ctx->TBg, st); pool_free(ctx->TBg_sh, st);
-  pool_free(ctx->mips_buf, st);
+  pool_free(ctx->mips_buf, st); pool_free(ctx->mips_tb, st);
+  pool_free(ctx->mips_blocks, st);
   pool_free(ctx->pipe_buf, st);
   pool_free(ctx->pipe_scratch, st);
   ctx->pipe_scratch_bytes = 0;
@@ -744,17 +841,22 @@ mad_status mad_mips_items(mad_ctx* ctx, const mad_matrix* B, uint64_t s_max, mad
   ctx->m = 0;
   ctx->s_max = s_max;
   mad_status rs;
-  if ((rs = pool_alloc(ctx, ctx->TB, (size_t)(ctx->d * ctx->n) + 4, st)) != MAD_OK) return rs;
+  if ((rs = pool_alloc(ctx, ctx->TB, (size_t)(ctx->d * ctx->n), st)) != MAD_OK) return rs;
   if ((rs = pool_alloc(ctx, ctx->nb, (size_t)ctx->d, st)) != MAD_OK) return rs;
   char* bt = nullptr;
   if ((rs = pool_alloc(ctx, bt, (size_t)(ctx->n * ctx->d) * 4, st)) != MAD_OK) return rs;
   ctx->bt = bt;
-  ctx->tbg_stride = ((int64_t)1 << tb_guide_width(ctx->n)) + 1;
-  if ((rs = pool_alloc(ctx, ctx->TBg_sh, (size_t)ctx->d, st)) != MAD_OK) return rs;
-  if ((rs = pool_alloc(ctx, ctx->TBg, (size_t)(ctx->d * ctx->tbg_stride), st)) != MAD_OK) return rs;
+  if ((rs = pool_alloc(ctx, ctx->mips_tb, (size_t)ctx->d, st)) != MAD_OK) return rs;
+  if ((rs = pool_alloc(ctx, ctx->mips_blocks,
+                       (size_t)ctx->d * (size_t)(tb_blocks(ctx->n) + 1) * 4, st)) != MAD_OK)
+    return rs;
   cudaMemsetAsync(ctx->sc, 0, sizeof(DevScalars), st);
   if ((rs = build_item_tables(ctx, st)) != MAD_OK) return rs;
-  if ((rs = tb_guide_build(ctx, st)) != MAD_OK) return rs;
+  const int64_t nb = tb_blocks(ctx->n);
+  const int64_t bx = (nb + 256) / 256;
+  k_mips_blocks<<<dim3((unsigned)(bx < 1024 ? bx : 1024), (unsigned)ctx->d), 256, 0, st>>>(
+      ctx->TB, ctx->d, ctx->n, ctx->mips_tb, ctx->mips_blocks);
+  count_launch(ctx);
   DevScalars hs;
   cudaMemcpyAsync(&hs, ctx->sc, sizeof(hs), cudaMemcpyDeviceToHost, st);
   if ((rs = cuda_status(cudaStreamSynchronize(st))) != MAD_OK) return rs;
@@ -891,7 +993,7 @@ mad_status mad_mips_run(mad_ctx* ctx, const mad_matrix* Q, uint64_t seed, mad_pa
   grid = std::min<unsigned long long>(grid, 0x7FFFFFFFull);
   k_mips_draw<<<(unsigned)grid, kDrawThreads, draw_smem_bytes(chunk, ctx->mips_max_parts, ctx->d),
                 st>>>(p, seed, b.queries, b.chunk_q, ctx->mips_chunks, ctx->mips_plan_mult,
-                      ctx->mips_max_parts, b.rec, b.off);
+                      ctx->mips_max_parts, ctx->mips_tb, ctx->mips_blocks, b.rec, b.off);
   k_mips_parts<<<(unsigned)ctx->mips_units, kPartThreads, ctx->mips_parts_smem, st>>>(
       b.queries, b.unit_q, b.rec, b.off, chunk, ctx->mips_slots, ctx->region_factor, ctx->f, ctx->mips_tprime, b.kept,
       b.kept_n, ctx->sc);

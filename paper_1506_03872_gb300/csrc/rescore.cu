@@ -87,8 +87,7 @@ k_rescore_dense(const mad_pair* __restrict__ cand, unsigned long long ncand_max,
 // of that sum and of L and U, and 1e-37 for products that underflow.  A
 // candidate whose sums are not finite, or with an FP64 entry that is nonzero but
 // below FP32's normal range, always stays (U = inf).
-constexpr float kBoundEps = 1.02f * 64.0f / 16777216.0f;
-constexpr float kBoundTiny = 1e-37f;
+// (kBoundEps, kBoundTiny)
 constexpr int kBoundBins = 4096;
 
 struct BoundState {
