@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -233,23 +234,32 @@ k_sample_rows(const SampleParams p_, unsigned long long seed, unsigned long long
 // order is row order; the T1 search itself is left to the draw kernel,
 // where neighbouring diamonds search the same few lines of T1.  At most
 // 2^kSortBitsMax buckets (a few rows each; measured on the dense factor
-// workload, 2^14 buckets made sampling 3.7 % slower than 2^15).  One block
-// per SM takes a contiguous chunk of the diamonds and counts them per
-// bucket in shared memory (step 1), the counts become per-(bucket, block)
-// offsets (steps 2 and 3), and each block places its diamonds by
-// shared-memory counts (step 4): no global atomics and no per-diamond
-// record between the steps.
+// workload, 2^14 buckets made sampling 3.7 % slower than 2^15).
+//
+// Two levels: the top kCoarseBits of the bucket across the grid, then the rest
+// inside each coarse bucket.
+//  1. k_sort_hist: a block counts its contiguous chunk of the diamonds per coarse
+//     bucket; the counts, bucket by bucket and block by block, are scanned.
+//  2. k_sort_scatter: the same chunk again, a tile of 8192 diamonds at a time: a
+//     tile is ordered by coarse bucket in shared memory, so that its records
+//     (diamond index and the bucket's low bits, one word) leave in runs of about
+//     eight, whole sectors.
+//  3. k_sort_fine: a block per coarse bucket (equal slices of a uniform target:
+//     equal counts) orders its records by the low bits in shared memory and
+//     writes indices and bucket offsets in order.
+// Bound by Philox in the first two (35 us a pass over 1e7 diamonds).  One level
+// over all 2^16 buckets kept a count per (bucket, block), as many as there were
+// diamonds, through four passes (40 MB: 67 us of sums and offsets), and wrote
+// each index to a sector of its own (94 us): 206 us with the histogram, now 123
+// (cold caches, one by one; the fused pass 965 -> 930 us).
 constexpr int kSortBitsMax = 16;
-// Above 2^15 buckets the shared-memory counters are 16 bits, two to a word:
-// the buckets are equal slices of the uniform target range, each at most
-// 2^-15 of it, so a block's chunk (at most 2^26 / #SMs diamonds) puts about
-// 14 diamonds into a bucket, far below 2^16.
-constexpr uint32_t kWideSort = 1u << 15;
-// Row stride of the per-(block, bucket) counts: a power-of-two number of
-// buckets plus 64 words, so that the rows of successive blocks do not all
-// start on the same memory channel (the column passes read one entry of
-// every row).
-__host__ __device__ __forceinline__ size_t sort_row(uint32_t nbk) { return (size_t)nbk + 64; }
+constexpr int kCoarseBits = 10;
+constexpr int kSortThreads = 1024;
+constexpr int kTilePer = 8;                             // diamonds per thread and tile
+constexpr int kSortTile = kSortThreads * kTilePer;
+constexpr int kIdxBits = 26;                            // diamond index in a record
+constexpr uint32_t kIdxMask = (1u << kIdxBits) - 1u;
+constexpr uint32_t kFineStage = 24576;                  // records k_sort_fine holds in shared memory
 
 __device__ __forceinline__ uint32_t sort_bucket(unsigned long long ell, uint2 key,
                                                 unsigned long long t1_total, int shift) {
@@ -258,106 +268,176 @@ __device__ __forceinline__ uint32_t sort_bucket(unsigned long long ell, uint2 ke
   return (uint32_t)(draw_target(u0, t1_total) >> shift);
 }
 
-// Step 1: H[g * sort_row(nbk) + b] = diamonds of block g's chunk in bucket b.
-template <bool Packed>
-__global__ void __launch_bounds__(1024)
+// Step 1: H[c * gridDim.x + g] = diamonds of block g's chunk in coarse bucket c.
+__global__ void __launch_bounds__(kSortThreads, 2)
 k_sort_hist(const DevScalars* __restrict__ sc, unsigned long long seed, unsigned long long first,
-            unsigned long long s, unsigned long long chunk, uint32_t nbk,
+            unsigned long long s, unsigned long long chunk, int coarse, int fine,
             unsigned int* __restrict__ H) {
-  extern __shared__ unsigned int sort_cnt[];
-  const uint32_t words = Packed ? nbk / 2 : nbk;
-  for (uint32_t b = threadIdx.x; b < words; b += blockDim.x) sort_cnt[b] = 0;
+  __shared__ unsigned int cnt[1 << kCoarseBits];
+  const int nc = 1 << coarse;
+  for (int b = threadIdx.x; b < nc; b += kSortThreads) cnt[b] = 0;
   __syncthreads();
   const unsigned long long t1_total = sc->t1_total;
-  const int shift = sc->sort_shift;
+  const int shift = sc->sort_shift + fine;
   const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
   const unsigned long long q0 = (unsigned long long)blockIdx.x * chunk;
   const unsigned long long q1 = q0 + chunk < s ? q0 + chunk : s;
-  for (unsigned long long q = q0 + threadIdx.x; q < q1; q += blockDim.x) {
-    const uint32_t b = sort_bucket(first + q, key, t1_total, shift);
-    if (Packed) atomicAdd(&sort_cnt[b >> 1], 1u << ((b & 1u) << 4));
-    else atomicAdd(&sort_cnt[b], 1u);
+  for (unsigned long long q = q0 + threadIdx.x; q < q1; q += kSortThreads)
+    atomicAdd(&cnt[sort_bucket(first + q, key, t1_total, shift)], 1u);
+  __syncthreads();
+  for (int b = threadIdx.x; b < nc; b += kSortThreads)
+    H[(size_t)b * gridDim.x + blockIdx.x] = cnt[b];
+}
+
+// Exclusive scan of one value per thread over a 1024-thread block.
+__device__ __forceinline__ uint32_t block_exclusive_1024(uint32_t v, uint32_t* warp_sum) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) warp_sum[warp] = inc;
+  __syncthreads();
+  if (warp == 0) {
+    const uint32_t w = warp_sum[lane];
+    uint32_t wi = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, wi, o);
+      if (lane >= o) wi += y;
+    }
+    warp_sum[lane] = wi - w;
   }
   __syncthreads();
-  unsigned int* __restrict__ row = H + (size_t)blockIdx.x * sort_row(nbk);
-  for (uint32_t b = threadIdx.x; b < nbk; b += blockDim.x)
-    row[b] = Packed ? (sort_cnt[b >> 1] >> ((b & 1u) << 4)) & 0xFFFFu : sort_cnt[b];
+  return warp_sum[warp] + inc - v;
 }
 
-// Step 2: tot[b] = sum over the blocks of H[g][b].
-__global__ void __launch_bounds__(256)
-k_sort_colsum(const unsigned int* __restrict__ H, uint32_t nbk, int blocks,
-              unsigned int* __restrict__ tot) {
-  const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nbk) return;
-  unsigned int acc = 0;
-#pragma unroll 16
-  for (int g = 0; g < blocks; ++g) acc += H[(size_t)g * sort_row(nbk) + b];
-  tot[b] = acc;
-}
+struct SortTile {
+  uint32_t cur[1 << kCoarseBits];    // next place of each coarse bucket
+  uint32_t cnt[1 << kCoarseBits];    // this tile's counts
+  uint32_t off[1 << kCoarseBits];    // their exclusive scan
+  uint32_t rec[kSortTile];
+  uint16_t bkt[kSortTile];
+  uint32_t warp_sum[32];
+};
 
-// Step 3 (after the exclusive scan of tot into base): H[g][b] becomes the
-// first position of block g's diamonds of bucket b.  Thirty-two loads are
-// in flight before their stores (one thread walks all the blocks of its
-// bucket; splitting the walk over more threads measured slower).
-__global__ void __launch_bounds__(256)
-k_sort_coloff(unsigned int* __restrict__ H, uint32_t nbk, int blocks,
-              const unsigned int* __restrict__ base) {
-  constexpr int kBatch = 32;
-  const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nbk) return;
-  const size_t row = sort_row(nbk);
-  unsigned int acc = base[b];
-  int g = 0;
-  for (; g + kBatch <= blocks; g += kBatch) {
-    unsigned int c[kBatch];
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) c[u] = H[(size_t)(g + u) * row + b];
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      H[(size_t)(g + u) * row + b] = acc;
-      acc += c[u];
-    }
-  }
-  for (; g < blocks; ++g) {
-    const unsigned int c = H[(size_t)g * row + b];
-    H[(size_t)g * row + b] = acc;
-    acc += c;
-  }
-}
-
-// Step 4: order[position] = q for every diamond q of the block's chunk.
-// Unpacked: the block's offsets are staged as shared-memory cursors.
-// Packed: a 16-bit shared-memory count gives the rank, added to the offset
-// read from H.
-template <bool Packed>
-__global__ void __launch_bounds__(1024)
+// Step 2: rec[place] = low bucket bits << kIdxBits | q for every diamond q of
+// the block's chunk, in coarse bucket order (off: the scanned counts).
+__global__ void __launch_bounds__(kSortThreads, 2)
 k_sort_scatter(const DevScalars* __restrict__ sc, unsigned long long seed,
                unsigned long long first, unsigned long long s, unsigned long long chunk,
-               uint32_t nbk, const unsigned int* __restrict__ H, uint32_t* __restrict__ order) {
-  extern __shared__ unsigned int sort_cnt[];
-  const unsigned int* __restrict__ row = H + (size_t)blockIdx.x * sort_row(nbk);
-  if (Packed) {
-    for (uint32_t w = threadIdx.x; w < nbk / 2; w += blockDim.x) sort_cnt[w] = 0;
-  } else {
-    for (uint32_t b = threadIdx.x; b < nbk; b += blockDim.x) sort_cnt[b] = row[b];
-  }
-  __syncthreads();
+               int coarse, int fine, const unsigned int* __restrict__ off,
+               uint32_t* __restrict__ rec) {
+  extern __shared__ __align__(16) unsigned char sort_smem[];
+  SortTile& sh = *reinterpret_cast<SortTile*>(sort_smem);
+  const int tid = threadIdx.x, nc = 1 << coarse;
+  static_assert((1 << kCoarseBits) == kSortThreads, "a coarse bucket per thread");
+  sh.cur[tid] = tid < nc ? off[(size_t)tid * gridDim.x + blockIdx.x] : 0u;
   const unsigned long long t1_total = sc->t1_total;
   const int shift = sc->sort_shift;
+  const uint32_t fmask = (1u << fine) - 1u;
   const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
   const unsigned long long q0 = (unsigned long long)blockIdx.x * chunk;
   const unsigned long long q1 = q0 + chunk < s ? q0 + chunk : s;
-  for (unsigned long long q = q0 + threadIdx.x; q < q1; q += blockDim.x) {
-    const uint32_t b = sort_bucket(first + q, key, t1_total, shift);
-    unsigned int pos;
-    if (Packed) {
-      const uint32_t sh = (b & 1u) << 4;
-      pos = __ldg(row + b) + ((atomicAdd(&sort_cnt[b >> 1], 1u << sh) >> sh) & 0xFFFFu);
-    } else {
-      pos = atomicAdd(&sort_cnt[b], 1u);
+  for (unsigned long long base = q0; base < q1; base += kSortTile) {
+    const uint32_t n = (uint32_t)(q1 - base < (unsigned long long)kSortTile ? q1 - base : kSortTile);
+    sh.cnt[tid] = 0;
+    __syncthreads();
+    uint32_t b[kTilePer], rank[kTilePer];
+#pragma unroll
+    for (int u = 0; u < kTilePer; ++u) {
+      const uint32_t x = tid + u * kSortThreads;
+      b[u] = 0;
+      rank[u] = 0;
+      if (x < n) {
+        b[u] = sort_bucket(first + base + x, key, t1_total, shift);
+        rank[u] = atomicAdd(&sh.cnt[b[u] >> fine], 1u);
+      }
     }
-    order[pos] = (uint32_t)q;
+    __syncthreads();
+    const uint32_t mine = sh.cnt[tid];
+    sh.off[tid] = block_exclusive_1024(mine, sh.warp_sum);
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kTilePer; ++u) {
+      const uint32_t x = tid + u * kSortThreads;
+      if (x < n) {
+        const uint32_t c = b[u] >> fine, at = sh.off[c] + rank[u];
+        sh.rec[at] = ((b[u] & fmask) << kIdxBits) | (uint32_t)(base + x);
+        sh.bkt[at] = (uint16_t)c;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kTilePer; ++u) {
+      const uint32_t x = tid + u * kSortThreads;
+      if (x < n) {
+        const uint32_t c = sh.bkt[x];
+        rec[sh.cur[c] + x - sh.off[c]] = sh.rec[x];
+      }
+    }
+    __syncthreads();
+    sh.cur[tid] += mine;
+  }
+}
+
+// Step 3, coarse bucket blockIdx.x: its records by their low bits into order
+// (indices alone) and the first place of each of its buckets into base
+// (base[nbk] = s).  Longer than kFineStage, it is written in place order
+// straight to memory.  With no low bits the records are the order already.
+__global__ void __launch_bounds__(kSortThreads, 2)
+k_sort_fine(const uint32_t* __restrict__ rec, const unsigned int* __restrict__ off, int blocks,
+            int fine, unsigned int s, uint32_t* __restrict__ order,
+            unsigned int* __restrict__ base) {
+  extern __shared__ uint32_t stage[];
+  __shared__ uint32_t cur[1 << (kSortBitsMax - kCoarseBits)];
+  const uint32_t c = blockIdx.x, nf = 1u << fine;
+  const uint32_t p0 = off[(size_t)c * blocks], p1 = off[(size_t)(c + 1) * blocks];
+  const uint32_t tid = threadIdx.x;
+  if (c + 1 == gridDim.x && tid == 0) base[(size_t)gridDim.x << fine] = s;
+  if (fine == 0) {
+    if (tid == 0) base[c] = p0;
+    return;
+  }
+  const uint32_t n = p1 - p0;
+  if (tid < nf) cur[tid] = 0;
+  __syncthreads();
+  for (uint32_t x = tid; x < n; x += kSortThreads) atomicAdd(&cur[rec[p0 + x] >> kIdxBits], 1u);
+  __syncthreads();
+  if (tid < 32) {   // nf <= 64 counts: two per lane
+    const uint32_t a = 2 * tid < nf ? cur[2 * tid] : 0u;
+    const uint32_t d = 2 * tid + 1 < nf ? cur[2 * tid + 1] : 0u;
+    uint32_t inc = a + d;
+#pragma unroll
+    for (uint32_t o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (tid >= o) inc += y;
+    }
+    const uint32_t ex = inc - a - d;
+    if (2 * tid < nf) {
+      cur[2 * tid] = ex;
+      base[c * nf + 2 * tid] = p0 + ex;
+    }
+    if (2 * tid + 1 < nf) {
+      cur[2 * tid + 1] = ex + a;
+      base[c * nf + 2 * tid + 1] = p0 + ex + a;
+    }
+  }
+  __syncthreads();
+  if (n <= kFineStage) {
+    for (uint32_t x = tid; x < n; x += kSortThreads) {
+      const uint32_t r = rec[p0 + x];
+      stage[atomicAdd(&cur[r >> kIdxBits], 1u)] = r & kIdxMask;
+    }
+    __syncthreads();
+    for (uint32_t x = tid; x < n; x += kSortThreads) order[p0 + x] = stage[x];
+  } else {
+    for (uint32_t x = tid; x < n; x += kSortThreads) {
+      const uint32_t r = rec[p0 + x];
+      order[p0 + atomicAdd(&cur[r >> kIdxBits], 1u)] = r & kIdxMask;
+    }
   }
 }
 
@@ -901,26 +981,28 @@ int sort_bits(int64_t m) {
 
 uint64_t sort_buckets(int64_t m) { return 1ull << sort_bits(m); }
 
-// Blocks of the sort (one per SM).
+// Blocks of the sort (two per SM).
 int sort_blocks() {
   static int blocks = 0;
   if (!blocks) {
-    int dev = 0;
+    int dev = 0, sms = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&blocks, cudaDevAttrMultiProcessorCount, dev);
-    if (blocks < 1) blocks = 1;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    blocks = 2 * (sms < 1 ? 1 : sms);
   }
   return blocks;
 }
 
-// Scratch of the sort and the draws for one batch: the per-(block, bucket)
-// counts, bucket totals and offsets, the scan's partials, the diamond
-// indices in bucket order, and each diamond's key and increment.
+// Scratch of the sort and the draws for one batch: the per-(coarse bucket,
+// block) counts and offsets, the bucket offsets, the scan's partials, the
+// records in coarse order, the diamond indices in bucket order, and each
+// diamond's key and increment.
 struct SortScratch {
   unsigned int* H;
-  unsigned int* tot;
+  unsigned int* off;
   unsigned int* base;
   unsigned int* part;
+  uint32_t* rec;
   uint32_t* order;
   unsigned long long* keys;
   long long* vals;
@@ -940,10 +1022,13 @@ SortScratch carve_sort(void* p, uint64_t nbk, int blocks, uint64_t batch, int re
     off += (bytes + 255) & ~(size_t)255;
     return (void*)q;
   };
-  c.H = (unsigned int*)take(sort_row((uint32_t)nbk) * blocks * sizeof(unsigned int));
-  c.tot = (unsigned int*)take(nbk * sizeof(unsigned int));
+  const uint64_t counts = std::min<uint64_t>(nbk, 1ull << kCoarseBits) * (uint64_t)blocks;
+  c.H = (unsigned int*)take(counts * sizeof(unsigned int));
+  c.off = (unsigned int*)take((counts + 1) * sizeof(unsigned int));
   c.base = (unsigned int*)take((nbk + 1) * sizeof(unsigned int));
-  c.part = (unsigned int*)take(scan_partial_elems(nbk) * sizeof(unsigned int));
+  c.part = (unsigned int*)take(scan_partial_elems(counts) * sizeof(unsigned int));
+  // (records are the order itself when there is no second level)
+  c.rec = (uint32_t*)take(nbk > (1ull << kCoarseBits) ? batch * sizeof(uint32_t) : 0);
   c.order = (uint32_t*)take(batch * sizeof(uint32_t));
   c.keys = (unsigned long long*)take(batch * recs * sizeof(unsigned long long));
   c.vals = (long long*)take(batch * recs * sizeof(long long));
@@ -1000,19 +1085,15 @@ mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first, 
   const int full_insert = full_grid<k_insert>();
   const uint64_t nbk = sort_buckets(ctx->m);
   const int blocks = sort_blocks();
-  const bool packed = nbk > kWideSort;
-  const size_t sort_smem = (packed ? nbk / 2 : nbk) * sizeof(unsigned int);
-  static size_t smem_set = 0;
-  if (sort_smem > 48 * 1024 && smem_set < sort_smem) {
-    cudaFuncSetAttribute(k_sort_hist<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sort_smem);
-    cudaFuncSetAttribute(k_sort_hist<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sort_smem);
-    cudaFuncSetAttribute(k_sort_scatter<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sort_smem);
-    cudaFuncSetAttribute(k_sort_scatter<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sort_smem);
-    smem_set = sort_smem;
+  const int bits = sort_bits(ctx->m);
+  const int coarse = bits < kCoarseBits ? bits : kCoarseBits, fine = bits - coarse;
+  static bool sort_attr = false;
+  if (!sort_attr) {
+    cudaFuncSetAttribute(k_sort_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(SortTile));
+    cudaFuncSetAttribute(k_sort_fine, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(kFineStage * sizeof(uint32_t)));
+    sort_attr = true;
   }
   const uint64_t batch = s < kSortBatch ? s : kSortBatch;
   // An empty X filled by one batch, keys owned by their drawn row: the
@@ -1037,23 +1118,16 @@ mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first, 
     const uint64_t n = (s - done) < batch ? (s - done) : batch;
     phase_event(ctx, 0, st);
     const unsigned long long chunk = (n + blocks - 1) / blocks;
-    const unsigned cols = (unsigned)((nbk + 255) / 256);
-    if (packed)
-      k_sort_hist<true><<<blocks, 1024, sort_smem, st>>>(ctx->sc, seed, first + done, n, chunk,
-                                                         (uint32_t)nbk, w.H);
-    else
-      k_sort_hist<false><<<blocks, 1024, sort_smem, st>>>(ctx->sc, seed, first + done, n, chunk,
-                                                          (uint32_t)nbk, w.H);
-    k_sort_colsum<<<cols, 256, 0, st>>>(w.H, (uint32_t)nbk, blocks, w.tot);
-    if ((rs = scan_exclusive_u32(ctx, w.tot, w.base, nbk, w.part, st)) != MAD_OK) return rs;
-    k_sort_coloff<<<cols, 256, 0, st>>>(w.H, (uint32_t)nbk, blocks, w.base);
-    if (packed)
-      k_sort_scatter<true><<<blocks, 1024, sort_smem, st>>>(ctx->sc, seed, first + done, n, chunk,
-                                                            (uint32_t)nbk, w.H, w.order);
-    else
-      k_sort_scatter<false><<<blocks, 1024, sort_smem, st>>>(ctx->sc, seed, first + done, n,
-                                                             chunk, (uint32_t)nbk, w.H, w.order);
-    count_launch(ctx, 4);
+    uint32_t* rec = fine ? w.rec : w.order;
+    const uint64_t counts = (uint64_t)blocks << coarse;
+    k_sort_hist<<<blocks, kSortThreads, 0, st>>>(ctx->sc, seed, first + done, n, chunk, coarse,
+                                                 fine, w.H);
+    if ((rs = scan_exclusive_u32(ctx, w.H, w.off, counts, w.part, st)) != MAD_OK) return rs;
+    k_sort_scatter<<<blocks, kSortThreads, sizeof(SortTile), st>>>(
+        ctx->sc, seed, first + done, n, chunk, coarse, fine, w.off, rec);
+    k_sort_fine<<<1u << coarse, kSortThreads, fine ? kFineStage * sizeof(uint32_t) : 0, st>>>(
+        w.rec, w.off, blocks, fine, (unsigned)n, w.order, w.base);
+    count_launch(ctx, 3);
     phase_event(ctx, 1, st);
     k_sample_sorted<<<grid_of(n, full_sorted), 256, 0, st>>>(p, seed, first + done, n, w.order,
                                                              w.keys, w.vals);
