@@ -108,6 +108,7 @@ void free_tables(mad_ctx* ctx, cudaStream_t st) {
   ctx->mips_nq = 0;
   ctx->built = false;
   ctx->regioned = false;
+  ctx->shape.valid = false;
 }
 
 template <typename T>
@@ -122,9 +123,10 @@ mad_status alloc(mad_ctx* ctx, T*& p, size_t count, cudaStream_t st) {
 
 // Read the device scalars (synchronises the stream).
 mad_status read_scalars(mad_ctx* ctx, DevScalars* hs, cudaStream_t st) {
-  cudaMemcpyAsync(hs, ctx->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, st);
+  cudaMemcpyAsync(ctx->pinned, ctx->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, st);
   const cudaError_t e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_status(e);
+  std::memcpy(hs, ctx->pinned, sizeof(DevScalars));
   ctx->device_error = hs->err;
   return MAD_OK;
 }
@@ -232,6 +234,28 @@ mad_status check_inputs(const mad_ctx* ctx, const mad_matrix* A, const mad_matri
 // for s_max, or an explicit capacity).
 mad_status alloc_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* B, uint64_t s_max,
                         bool dense, cudaStream_t st) {
+  // A rebuild of the shape whose tables are there keeps them: every table, the
+  // hash's regions and X are written again from the new contents.  (Freeing
+  // and allocating some twenty buffers took about 30 us of a plain search.)
+  const mad_ctx::TableShape want = {true,       A->rows, A->cols,           B->cols,
+                                    B->dt,      s_max,   ctx->hcap_request, ctx->hov_request};
+  const mad_ctx::TableShape& have = ctx->shape;
+  if (dense && have.valid && have.m == want.m && have.d == want.d && have.n == want.n &&
+      have.b_dt == want.b_dt && have.s_max == want.s_max &&
+      have.hcap_request == want.hcap_request && have.hov_request == want.hov_request) {
+    free_async(ctx->pipe_buf, st);
+    free_async(ctx->pipe_scratch, st);
+    ctx->pipe_scratch_bytes = 0;
+    ctx->pipe = false;
+    ctx->built = false;
+    ctx->A = *A;
+    ctx->B = *B;
+    ctx->sampled = 0;
+    ctx->x_empty = ctx->x_built = false;
+    if (ctx->regioned)
+      ctx->hcap = ctx->hcap_alloc = hash_region_bound((uint64_t)ctx->m, s_max) + ctx->hov;
+    return MAD_OK;
+  }
   free_tables(ctx, st);
   ctx->A = *A;
   ctx->B = *B;
@@ -299,6 +323,7 @@ mad_status alloc_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* B, 
     if ((rs = alloc(ctx, ctx->hkeys, cap, st)) != MAD_OK) return rs;
     if ((rs = alloc(ctx, ctx->hvals, cap, st)) != MAD_OK) return rs;
   }
+  if (dense && !(ctx->flags & (MAD_WEDGE | MAD_ALIAS))) ctx->shape = want;
   return MAD_OK;
 }
 
@@ -320,11 +345,12 @@ mad_status enqueue_dense_build(mad_ctx* ctx, cudaStream_t st, bool clear_x) {
 // Host mirrors of the device scalars after a dense build (synchronises).
 mad_status finish_dense_build(mad_ctx* ctx, cudaStream_t st) {
   DevScalars hs;
-  unsigned long long used = 0;
+  unsigned long long* used_host = (unsigned long long*)((char*)ctx->pinned + 2048);
   if (ctx->regioned)
-    cudaMemcpyAsync(&used, ctx->hreg + ctx->m, sizeof(used), cudaMemcpyDeviceToHost, st);
+    cudaMemcpyAsync(used_host, ctx->hreg + ctx->m, sizeof(*used_host), cudaMemcpyDeviceToHost, st);
   mad_status rs = read_scalars(ctx, &hs, st);
   if (rs != MAD_OK) return rs;
+  const unsigned long long used = ctx->regioned ? *used_host : 0;
   if (hs.err & DERR_OVERFLOW) return MAD_ERR_OVERFLOW;
   if ((hs.err & DERR_EMPTY) || hs.maxr_bits == 0u || hs.maxb_bits == 0u) return MAD_ERR_EMPTY;
   if (ctx->regioned) {
@@ -396,6 +422,7 @@ mad_status mad_create(mad_ctx** out, uint32_t flags) {
   if (e == cudaSuccess) e = cudaMemset(ctx->sc, 0, sizeof(DevScalars));
   if (e == cudaSuccess) e = cudaMalloc(&ctx->bound_state, bound_state_bytes());
   if (e == cudaSuccess) e = cudaMemset(ctx->bound_state, 0, bound_state_bytes());
+  if (e == cudaSuccess) e = cudaMallocHost(&ctx->pinned, 4096);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork2, cudaEventDisableTiming);
@@ -405,6 +432,7 @@ mad_status mad_create(mad_ctx** out, uint32_t flags) {
     if (ctx->ev_fork2) cudaEventDestroy(ctx->ev_fork2);
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->side) cudaStreamDestroy(ctx->side);
+    if (ctx->pinned) cudaFreeHost(ctx->pinned);
     if (ctx->bound_state) cudaFree(ctx->bound_state);
     if (ctx->sc) cudaFree(ctx->sc);
     if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
@@ -428,6 +456,7 @@ void mad_destroy(mad_ctx* ctx) {
   free_tables(ctx, 0);
   if (ctx->scratch) cudaFreeAsync(ctx->scratch, 0);
   cudaStreamSynchronize(0);
+  cudaFreeHost(ctx->pinned);
   cudaFree(ctx->bound_state);
   cudaFree(ctx->sc);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
@@ -595,6 +624,12 @@ mad_status mad_topk(mad_ctx* ctx, uint32_t tprime, mad_pair* out_dev, uint32_t* 
   if (!ctx->built) return MAD_ERR_STATE;
   cudaStream_t st = (cudaStream_t)stream;
   DevScalars hs;
+  if (ctx->regioned && tprime > 0) {
+    uint64_t nsel = 0;
+    const mad_status rd = topk_dense(ctx, tprime, out_dev, &nsel, &hs, st);
+    if (rd == MAD_OK) *n_out_host = (uint32_t)nsel;
+    return rd;
+  }
   mad_status rs = read_scalars(ctx, &hs, st);
   if (rs != MAD_OK) return rs;
   if ((rs = device_error_status(hs.err)) != MAD_OK) return rs;

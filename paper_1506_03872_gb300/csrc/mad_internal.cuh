@@ -258,6 +258,15 @@ struct mad_ctx {
   uint64_t hov_request = 0;
   mad::DevScalars* sc = nullptr;
   void* bound_state = nullptr;      // rescore.cu's bounds (zeros between calls)
+  void* pinned = nullptr;           // 4 KB of pinned host memory for read-backs
+  // The shape whose tables are allocated (dense tables without the optional
+  // ones): a rebuild of the same shape keeps them.
+  struct TableShape {
+    bool valid = false;
+    int64_t m = 0, d = 0, n = 0;
+    int32_t b_dt = 0;
+    uint64_t s_max = 0, hcap_request = 0, hov_request = 0;
+  } shape;
   // Scratch (select, scans); grown on demand.
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
@@ -386,6 +395,10 @@ mad_status select_list_dev(mad_ctx* ctx, const SelectWs& ws, uint64_t n_max,
 // *n_pos receives the number of positive keys.  Synchronises once.
 mad_status select_from_hash(mad_ctx* ctx, const SelectWs& ws, uint64_t K, uint64_t* n_sel,
                             uint64_t* n_pos, cudaStream_t st);
+// Omega_t' of a regioned (dense) hash into out, sorted, with the scalars read
+// on the way; synchronises.
+mad_status topk_dense(mad_ctx* ctx, uint64_t K, mad_pair* out, uint64_t* n_sel, DevScalars* hs,
+                      cudaStream_t st);
 mad_status items_to_pairs(mad_ctx* ctx, const Item* items, uint64_t n, const mad_pair* cand,
                           const double* cvals, mad_pair* out, cudaStream_t st);
 // Device-driven selection: every length comes from device memory, so the

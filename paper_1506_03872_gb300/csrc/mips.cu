@@ -830,6 +830,7 @@ mad_status mad_mips_items(mad_ctx* ctx, const mad_matrix* B, uint64_t s_max, mad
   ctx->pipe = false;
   ctx->built = false;
   ctx->mips_items = false;
+  ctx->shape.valid = false;
   ctx->mips_nq = 0;
   ctx->B = *B;
   ctx->dense = true;
