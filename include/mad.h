@@ -503,8 +503,10 @@ mad_status mad_debug_draws(mad_ctx* ctx, uint64_t seed, uint64_t first, uint64_t
  * overflow table in the fused pass (mad_pipeline_run); a full overflow
  * table is reported as MAD_ERR_HASH_FULL by mad_pipeline_status.  The
  * step-wise mad_sample probes the regions as one table and reports
- * MAD_ERR_HASH_FULL past its probe limit.  MAD_ERR_ARG outside these
- * ranges. */
+ * MAD_ERR_HASH_FULL past its probe limit.  For batched queries region_factor
+ * scales the tables of a query's parts (1.5 slots per record), and a nonzero
+ * overflow_slots makes mad_mips_items build the guides of long item tables.
+ * MAD_ERR_ARG outside these ranges. */
 mad_status mad_debug_set_hash_layout(mad_ctx* ctx, float region_factor, uint64_t overflow_slots);
 
 /* As mad_debug_draws for an arbitrary device list of diamond indices. */

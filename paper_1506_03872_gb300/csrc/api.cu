@@ -84,6 +84,8 @@ void free_tables(mad_ctx* ctx, cudaStream_t st) {
   free_async(ctx->T1g, st);
   free_async(ctx->TBg, st);
   free_async(ctx->TBg_sh, st);
+  free_async(ctx->tb_row, st);
+  free_async(ctx->tb_blocks, st);
   free_async(ctx->TK, st);
   free_async(ctx->TAc, st);
   free_async(ctx->nac, st);
@@ -102,8 +104,6 @@ void free_tables(mad_ctx* ctx, cudaStream_t st) {
   ctx->pipe_scratch_bytes = 0;
   ctx->pipe = false;
   free_async(ctx->mips_buf, st);
-  free_async(ctx->mips_tb, st);
-  free_async(ctx->mips_blocks, st);
   ctx->mips_items = false;
   ctx->mips_nq = 0;
   ctx->built = false;

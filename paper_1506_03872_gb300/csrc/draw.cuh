@@ -46,7 +46,7 @@ __device__ __forceinline__ Draw draw_given_row(const SampleParams& p, const Unif
   uint32_t e_k, e_kp = 0;
   if (p.integer) {
     const uint32_t t2tot = __ldg(p.T2 + a0 + alen - 1);
-    const uint32_t target = (uint32_t)draw_target(u.u1, t2tot);
+    const uint32_t target = draw_target32(u.u1, t2tot);
     if (p.T2g && alen >= kGuideMin) {
       pk = ub_guided_u32(p.T2 + a0, p.T2g + __ldg(p.T2g_ptr + i), (int)__ldg(p.T2g_sh + i), target);
     } else {
@@ -57,8 +57,8 @@ __device__ __forceinline__ Draw draw_given_row(const SampleParams& p, const Unif
     const uint32_t t2tot = __ldg(p.T2 + a0 + alen - 1) & mask;
     const uint32_t tatot = __ldg(p.TA + a0 + alen - 1) & mask;
     int a, b;
-    ub2_u32(p.T2 + a0, p.TA + a0, (int)alen, (uint32_t)draw_target(u.u1, t2tot),
-            (uint32_t)draw_target(u.u3, tatot), mask, &a, &b);
+    ub2_u32(p.T2 + a0, p.TA + a0, (int)alen, draw_target32(u.u1, t2tot),
+            draw_target32(u.u3, tatot), mask, &a, &b);
     pk = a;
     pkp = b;
   }
@@ -82,7 +82,7 @@ __device__ __forceinline__ Draw draw_given_row(const SampleParams& p, const Unif
     pj = (int64_t)draw_target(u.u2, (unsigned long long)blen);
   } else {
     const uint32_t tbtot = __ldg(p.TB + b0 + blen - 1) & mask;
-    const uint32_t target = (uint32_t)draw_target(u.u2, tbtot);
+    const uint32_t target = draw_target32(u.u2, tbtot);
     if (p.TBg) {
       pj = ub_guided_u32(p.TB + b0, p.TBg + k * p.tbg_stride, (int)__ldg(p.TBg_sh + k), target,
                          mask);

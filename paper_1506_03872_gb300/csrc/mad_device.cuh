@@ -68,6 +68,12 @@ __device__ __forceinline__ unsigned long long draw_target(unsigned long long u,
   return __umul64hi(u, total);
 }
 
+// The same for a 32-bit total: two multiplies instead of the 64 x 64-bit one's.
+__device__ __forceinline__ uint32_t draw_target32(unsigned long long u, uint32_t total) {
+  const unsigned long long hi = (u >> 32) * total + __umulhi((uint32_t)u, total);
+  return (uint32_t)(hi >> 32);
+}
+
 // First position p in [0, len) with prefix[p] > target (masking the sign
 // bit of row tables).  Clamped to len-1 when the table is inconsistent.
 __device__ __forceinline__ int64_t search_u64(const uint64_t* __restrict__ prefix, int64_t len,
@@ -220,6 +226,53 @@ __device__ __forceinline__ void ub2_u32(const uint32_t* __restrict__ P, const ui
   }
   *op = a;
   *oq = b;
+}
+
+// ---- TB in 64-byte blocks ----------------------------------------------------
+// The draw of j is one aligned 64-byte read.  Row k's targets [0, total) are
+// cut into about n / kBlockKeys equal buckets, bucket of target t = t * mul /
+// 2^32; block b holds lo, the number of the row's entries at most bucket b's
+// first target, and entries lo, lo + 1, ... up to 15 of them (sign bits
+// included), padded with entries above every target.  The first entry above
+// a target of the bucket is among entries lo .. lo', lo' the next block's lo, so
+// it is in the block when lo' - lo < 15 (all but 0.1 % of the buckets where
+// six entries a bucket are expected); otherwise TB is searched between the two.
+// Against the row guides of tb_guide_build (two entries of the guide, then a
+// window of up to 17 entries of TB at any alignment: three or four 64-byte
+// fetches from DRAM for a million items, 383 bytes a diamond with b_k'j) this
+// is one, for 10.7 bytes an entry of TB instead of at most 4: 1e4 queries of 5e4
+// diamonds, draws 38.3 -> 29.1 ms.
+
+// First target of bucket b: the smallest t with t * mul >= b * 2^32.
+__device__ __forceinline__ unsigned long long bucket_first(unsigned long long b,
+                                                           unsigned long long mul) {
+  return ((b << 32) + mul - 1) / mul;
+}
+
+// First entry of row k of TB above target and its sign bit.
+__device__ __forceinline__ int64_t ub_block(const SampleParams& p, int64_t nb, int64_t k,
+                                            uint32_t mul, uint32_t target, uint32_t* sign) {
+  const uint4* __restrict__ blk = p.tb_blocks + (k * (nb + 1) + __umulhi(target, mul)) * 4;
+  const uint4 a = __ldg(blk), b = __ldg(blk + 1), c = __ldg(blk + 2), e = __ldg(blk + 3);
+  const uint32_t v[kBlockEnts] = {a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x,
+                                  c.y, c.z, c.w, e.x, e.y, e.z, e.w};
+  int cnt = 0;
+  uint32_t s = 0;
+#pragma unroll
+  for (int u = kBlockEnts - 1; u >= 0; --u) {
+    const bool le = (v[u] & PREFIX_MASK) <= target;
+    cnt += le ? 1 : 0;
+    s = le ? s : v[u];
+  }
+  *sign = s & SIGN_BIT;
+  if (cnt < kBlockEnts) return (int64_t)a.x + cnt;
+  // Every entry held is at most the target: search on to the next block's lo.
+  const uint32_t* __restrict__ row = p.TB + k * p.n;
+  const uint32_t lo = a.x + kBlockEnts, hi = __ldg((const uint32_t*)(blk + 4));
+  const int64_t j =
+      (int64_t)lo + (hi > lo ? ub_u32(row + lo, (int)(hi - lo), target, PREFIX_MASK) : 0);
+  if (j < p.n) *sign = __ldg(row + j) & SIGN_BIT;
+  return j;
 }
 
 // A length known only on the device: min(cap, *n_dev), or cap itself when

@@ -104,6 +104,10 @@ struct SampleParams {
   const uint32_t* TBg;
   int64_t tbg_stride;
   const uint8_t* TBg_sh;
+  // TB's rows in 64-byte blocks (null when absent, see ub_block), and each row's
+  // total and bucket factor.
+  const uint4* tb_blocks;
+  const uint2* tb_row;
   int f_exp;                       // F
   // Hash.  Regioned (dense inputs): the key (a, b) starts probing in the
   // home region of row a, [hreg[a], hreg[a+1]), sized from row a's expected
@@ -196,6 +200,8 @@ struct mad_ctx {
   uint32_t* TBg = nullptr;                // guides of the TB rows (fixed row stride)
   int64_t tbg_stride = 0;
   uint8_t* TBg_sh = nullptr;
+  uint2* tb_row = nullptr;                // total and bucket factor of every row of TB
+  uint4* tb_blocks = nullptr;             // TB's rows in 64-byte blocks (in place of TBg)
   // Wedge sampling (MAD_WEDGE): the centre table TK over k (its inclusive
   // prefix starts at TK + TK_shift), its total and scale exponent, the
   // column norms of A and, for dense non-Gram inputs, the column tables.
@@ -231,8 +237,6 @@ struct mad_ctx {
   int mips_slots = 0;                     // table slots of a part
   size_t mips_parts_smem = 0;
   void* mips_buf = nullptr;               // the batch's device buffer (mips.cu)
-  uint2* mips_tb = nullptr;               // total and bucket factor of every row of TB
-  uint4* mips_blocks = nullptr;           // TB's rows in 64-byte blocks (mips.cu)
   // Launch shape of batched queries (mad_mips_config): the load of a part's
   // table is 0.6 / 2^(mips_region_lg - 1), 256 x mips_chunk_mult diamonds per
   // chunk (the plan's value in mips_plan_mult), draw blocks per SM (0: one
@@ -315,7 +319,18 @@ mad_status t2_guide_fill(mad_ctx* ctx, cudaStream_t st);
 // Row descriptors into ctx->rdesc (m) and ctx->brow (d), after the guides'
 // offsets; nothing where they are not allocated.
 mad_status row_desc_fill(mad_ctx* ctx, cudaStream_t st);
-// Guides of the dense TB rows into ctx->TBg (d rows of ctx->tbg_stride =
+// Batched queries: TB in 64-byte blocks of kBlockEnts entries, about kBlockKeys of them new in
+// each (see ub_block): 10.7 bytes an entry of TB, built up to 2^31 entries (23
+// GB); longer tables get the guides, at most 4 bytes an entry.
+constexpr int kBlockKeys = 6;
+constexpr int kBlockEnts = 15;
+__host__ __device__ inline int64_t tb_blocks(int64_t n) { return (n + kBlockKeys - 1) / kBlockKeys; }
+inline bool tb_blocks_apply(int64_t d, int64_t n) { return d * n <= (1ll << 31); }
+inline size_t tb_blocks_quads(int64_t d, int64_t n) {
+  return (size_t)d * (size_t)(tb_blocks(n) + 1) * 4;
+}
+// The blocks where ctx->tb_blocks is allocated, else the
+// guides of the dense TB rows into ctx->TBg (d rows of ctx->tbg_stride =
 // 2^tb_guide_width(n) + 1 entries) and ctx->TBg_sh (d shifts).
 int tb_guide_width(int64_t n);
 mad_status tb_guide_build(mad_ctx* ctx, cudaStream_t st);

@@ -76,92 +76,42 @@ __device__ __forceinline__ void ub2_shared(const uint32_t* P, const uint32_t* Q,
   *oq = b;
 }
 
-// ---- TB in 64-byte blocks ----------------------------------------------------
-// The draw of j is one aligned 64-byte read.  Row k's targets [0, total) are
-// cut into about n / kBlockKeys equal buckets, bucket of target t = t * mul /
-// 2^32; block b holds lo, the number of the row's entries at most bucket b's
-// first target, and entries lo, lo + 1, ... up to 15 of them (sign bits
-// included), padded with entries above every target.  The first entry above
-// a target of the bucket is among entries lo .. lo', lo' the next block's lo, so
-// it is in the block when lo' - lo < 15 (all but 0.1 % of the buckets where
-// six entries a bucket are expected); otherwise TB is searched between the two.
-// Against the row guides of tb_guide_build (two entries of the guide, then a
-// window of up to 17 entries of TB at any alignment: three or four 64-byte
-// fetches from DRAM for a million items, 383 bytes a diamond with b_k'j) this
-// is one, for 10.7 bytes an entry of TB instead of at most 4: 1e4 queries of 5e4
-// diamonds, draws 38.3 -> 29.1 ms.
-constexpr int kBlockKeys = 6;
-constexpr int kBlockEnts = 15;
-
-__host__ __device__ inline int64_t tb_blocks(int64_t n) { return (n + kBlockKeys - 1) / kBlockKeys; }
-
-// First target of bucket b: the smallest t with t * mul >= b * 2^32.
-__device__ __forceinline__ unsigned long long bucket_first(unsigned long long b,
-                                                           unsigned long long mul) {
-  return ((b << 32) + mul - 1) / mul;
-}
-
-// Row k's total, mul and blocks [k (nb + 1), (k + 1) (nb + 1)); the last block
-// only ends the one before it.
-__global__ void __launch_bounds__(256)
-k_mips_blocks(const uint32_t* __restrict__ TB, int64_t d, int64_t n, uint2* __restrict__ tb_row,
-              uint4* __restrict__ blocks) {
-  const int64_t nb = tb_blocks(n);
-  for (int64_t k = blockIdx.y; k < d; k += gridDim.y) {
-    const uint32_t* __restrict__ row = TB + k * n;
-    const uint32_t tot = __ldg(row + n - 1) & PREFIX_MASK;
-    // (t mul < 2^32 nb for t < tot, so every bucket is below nb)
-    const unsigned long long mul = tot ? ((unsigned long long)nb << 32) / tot : 0ull;
-    const uint32_t m32 = mul < 0xFFFFFFFFull ? (uint32_t)mul : 0xFFFFFFFFu;
-    if (blockIdx.x == 0 && threadIdx.x == 0) tb_row[k] = make_uint2(tot, m32);
-    uint4* __restrict__ out = blocks + k * (nb + 1) * 4;
-    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b <= nb;
-         b += (int64_t)gridDim.x * blockDim.x) {
-      uint32_t lo = (uint32_t)n;
-      if (m32) {
-        const unsigned long long first = bucket_first((unsigned long long)b, m32);
-        if (b == 0) lo = (uint32_t)ub_u32(row, (int)n, 0u, PREFIX_MASK);
-        else if (first < tot) lo = (uint32_t)ub_u32(row, (int)n, (uint32_t)first, PREFIX_MASK);
-      }
-      uint32_t v[16];
-      v[0] = lo;
+// The j search where the blocks are not built (tb_blocks_apply): row k's guide,
+// and its window of TB 16 bytes at a time: at most kQuads aligned quads hold a
+// window of 17 or fewer entries.  Entries of the row before the window are at
+// most the target and entries after it above, so whole quads are counted and
+// only the row's own ends are checked (TB is allocated with four entries of
+// padding).
+constexpr int kQuads = 5;
+__device__ __forceinline__ int64_t ub_tb(const SampleParams& p, int64_t k, uint32_t target) {
+  const uint32_t* __restrict__ G = p.TBg + k * p.tbg_stride;
+  const uint32_t b = target >> (int)__ldg(p.TBg_sh + k);
+  const uint32_t lo = __ldg(G + b), hi = __ldg(G + b + 1);
+  const int64_t row = k * p.n;
+  if (hi - lo > 17u)
+    return (int64_t)lo + ub_u32(p.TB + row + lo, (int)(hi - lo), target, PREFIX_MASK);
+  const int64_t e0 = (row + lo) & ~(int64_t)3;
+  const int quads = (int)((row + hi - e0 + 3) >> 2);
+  uint4 w[kQuads];
 #pragma unroll
-      for (int c = 0; c < kBlockEnts; ++c) {
-        const int64_t e = (int64_t)lo + c;
-        v[1 + c] = e < n ? __ldg(row + e) : PREFIX_MASK;
-      }
+  for (int q = 0; q < kQuads; ++q)
+    if (q < quads) w[q] = __ldg(reinterpret_cast<const uint4*>(p.TB + e0) + q);
+  const int64_t first = e0 - row;   // (below 0 by up to 3 in a row's first quad)
+  int cnt = 0;
+  const bool inner = first >= 0 && first + 4 * kQuads <= p.n;
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        out[4 * b + q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+  for (int q = 0; q < kQuads; ++q) {
+    if (q < quads) {
+      const uint32_t v[4] = {w[q].x, w[q].y, w[q].z, w[q].w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int64_t at = first + 4 * q + c;
+        const bool in_row = inner || (at >= 0 && at < p.n);
+        cnt += (in_row && (v[c] & PREFIX_MASK) <= target) ? 1 : 0;
+      }
     }
   }
-}
-
-// First entry of row k of TB above target and its sign bit.
-__device__ __forceinline__ int64_t ub_block(const SampleParams& p, const uint4* __restrict__ blocks,
-                                            int64_t nb, int64_t k, uint32_t mul, uint32_t target,
-                                            uint32_t* sign) {
-  const uint4* __restrict__ blk = blocks + (k * (nb + 1) + __umulhi(target, mul)) * 4;
-  const uint4 a = __ldg(blk), b = __ldg(blk + 1), c = __ldg(blk + 2), e = __ldg(blk + 3);
-  const uint32_t v[kBlockEnts] = {a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x,
-                                  c.y, c.z, c.w, e.x, e.y, e.z, e.w};
-  int cnt = 0;
-  uint32_t s = 0;
-#pragma unroll
-  for (int u = kBlockEnts - 1; u >= 0; --u) {
-    const bool le = (v[u] & PREFIX_MASK) <= target;
-    cnt += le ? 1 : 0;
-    s = le ? s : v[u];
-  }
-  *sign = s & SIGN_BIT;
-  if (cnt < kBlockEnts) return (int64_t)a.x + cnt;
-  // Every entry held is at most the target: search on to the next block's lo.
-  const uint32_t* __restrict__ row = p.TB + k * p.n;
-  const uint32_t lo = a.x + kBlockEnts, hi = __ldg((const uint32_t*)(blk + 4));
-  const int64_t j =
-      (int64_t)lo + (hi > lo ? ub_u32(row + lo, (int)(hi - lo), target, PREFIX_MASK) : 0);
-  if (j < p.n) *sign = __ldg(row + j) & SIGN_BIT;
-  return j;
+  return (first > 0 ? first : 0) + cnt;
 }
 
 // The part of column j among `parts`: the high bits of a mix of j (the
@@ -176,12 +126,11 @@ __device__ __forceinline__ uint32_t part_of(uint32_t h, uint32_t parts) {
 // diamond a block of TB (64 bytes) and b_k'j (a sector, fetched as 64 bytes) for
 // a million items, 3.4e10 of them a second; 2 to 5 resident blocks per SM measure
 // the same, 6 leave too little L1 (8.46 instead of 6.59 ms for 1500 queries).
+template <bool kBlocks>
 __global__ void __launch_bounds__(kDrawThreads, 4)
 k_mips_draw(const SampleParams p, unsigned long long seed, const MipsQuery* __restrict__ queries,
             const uint32_t* __restrict__ chunk_q, unsigned long long nchunks, int mult,
-            uint32_t max_parts, const uint2* __restrict__ tb_row,
-            const uint4* __restrict__ blocks, uint2* __restrict__ rec,
-            uint16_t* __restrict__ off) {
+            uint32_t max_parts, uint2* __restrict__ rec, uint16_t* __restrict__ off) {
   extern __shared__ __align__(16) unsigned char draw_smem[];
   const int chunk = mult * kDrawThreads;
   const int d = (int)p.d;
@@ -196,7 +145,8 @@ k_mips_draw(const SampleParams p, unsigned long long seed, const MipsQuery* __re
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t nb = tb_blocks(p.n);
   bool bad = false;
-  for (int x = tid; x < d; x += kDrawThreads) stb[x] = __ldg(tb_row + x);
+  if (kBlocks)
+    for (int x = tid; x < d; x += kDrawThreads) stb[x] = __ldg(p.tb_row + x);
   for (unsigned long long c = blockIdx.x; c < nchunks; c += gridDim.x) {
     const uint32_t q = __ldg(chunk_q + c);
     const MipsQuery mq = queries[q];
@@ -213,14 +163,23 @@ k_mips_draw(const SampleParams p, unsigned long long seed, const MipsQuery* __re
     for (int x = tid; x < cnt; x += kDrawThreads) {
       const Uniforms un = diamond_uniforms(seed + q, l0 + x);
       int k, kp;
-      ub2_shared(s2, sa, d, (uint32_t)draw_target(un.u1, t2tot),
-                 (uint32_t)draw_target(un.u3, tatot), &k, &kp);
+      ub2_shared(s2, sa, d, draw_target32(un.u1, t2tot),
+                 draw_target32(un.u3, tatot), &k, &kp);
       if (k >= d) { bad = true; k = d - 1; }
       if (kp >= d) { bad = true; kp = d - 1; }
-      const uint2 tb = stb[k];
       uint32_t sj;
-      int64_t j = ub_block(p, blocks, nb, k, tb.y, (uint32_t)draw_target(un.u2, tb.x), &sj);
-      if (j >= p.n) { bad = true; j = p.n - 1; }
+      int64_t j;
+      if (kBlocks) {
+        const uint2 tb = stb[k];
+        j = ub_block(p, nb, k, tb.y, draw_target32(un.u2, tb.x), &sj);
+        if (j >= p.n) { bad = true; j = p.n - 1; }
+      } else {
+        const int64_t row = (int64_t)k * p.n;
+        const uint32_t tot = __ldg(p.TB + row + p.n - 1) & PREFIX_MASK;
+        j = ub_tb(p, k, draw_target32(un.u2, tot));
+        if (j >= p.n) { bad = true; j = p.n - 1; }
+        sj = __ldg(p.TB + row + j) & SIGN_BIT;
+      }
       const uint32_t sign = sj ^ ((s2[k] ^ sa[kp]) & SIGN_BIT);
       const float b = __ldg((const float*)p.b_val + (int64_t)kp * p.ldb + j);
       const uint32_t part = part_of(fmix32((uint32_t)j), mq.parts);
@@ -822,8 +781,8 @@ mad_status mad_mips_items(mad_ctx* ctx, const mad_matrix* B, uint64_t s_max, mad
   pool_free(ctx->hreg, st); pool_free(ctx->T2g_ptr, st);
   pool_free(ctx->T2g, st); pool_free(ctx->T2g_sh, st); pool_free(ctx->bloom, st);
   pool_free(ctx->TBg, st); pool_free(ctx->TBg_sh, st);
-  pool_free(ctx->mips_buf, st); pool_free(ctx->mips_tb, st);
-  pool_free(ctx->mips_blocks, st);
+  pool_free(ctx->mips_buf, st); pool_free(ctx->tb_row, st);
+  pool_free(ctx->tb_blocks, st);
   pool_free(ctx->pipe_buf, st);
   pool_free(ctx->pipe_scratch, st);
   ctx->pipe_scratch_bytes = 0;
@@ -842,22 +801,25 @@ mad_status mad_mips_items(mad_ctx* ctx, const mad_matrix* B, uint64_t s_max, mad
   ctx->m = 0;
   ctx->s_max = s_max;
   mad_status rs;
-  if ((rs = pool_alloc(ctx, ctx->TB, (size_t)(ctx->d * ctx->n), st)) != MAD_OK) return rs;
+  if ((rs = pool_alloc(ctx, ctx->TB, (size_t)(ctx->d * ctx->n) + 4, st)) != MAD_OK) return rs;
   if ((rs = pool_alloc(ctx, ctx->nb, (size_t)ctx->d, st)) != MAD_OK) return rs;
   char* bt = nullptr;
   if ((rs = pool_alloc(ctx, bt, (size_t)(ctx->n * ctx->d) * 4, st)) != MAD_OK) return rs;
   ctx->bt = bt;
-  if ((rs = pool_alloc(ctx, ctx->mips_tb, (size_t)ctx->d, st)) != MAD_OK) return rs;
-  if ((rs = pool_alloc(ctx, ctx->mips_blocks,
-                       (size_t)ctx->d * (size_t)(tb_blocks(ctx->n) + 1) * 4, st)) != MAD_OK)
-    return rs;
+  // (a test asks for the guides by an overflow table of the debug layout)
+  if (ctx->hov_request == 0 && tb_blocks_apply(ctx->d, ctx->n)) {
+    if ((rs = pool_alloc(ctx, ctx->tb_row, (size_t)ctx->d, st)) != MAD_OK) return rs;
+    if ((rs = pool_alloc(ctx, ctx->tb_blocks, tb_blocks_quads(ctx->d, ctx->n), st)) != MAD_OK)
+      return rs;
+  } else {
+    ctx->tbg_stride = ((int64_t)1 << tb_guide_width(ctx->n)) + 1;
+    if ((rs = pool_alloc(ctx, ctx->TBg_sh, (size_t)ctx->d, st)) != MAD_OK) return rs;
+    if ((rs = pool_alloc(ctx, ctx->TBg, (size_t)(ctx->d * ctx->tbg_stride), st)) != MAD_OK)
+      return rs;
+  }
   cudaMemsetAsync(ctx->sc, 0, sizeof(DevScalars), st);
   if ((rs = build_item_tables(ctx, st)) != MAD_OK) return rs;
-  const int64_t nb = tb_blocks(ctx->n);
-  const int64_t bx = (nb + 256) / 256;
-  k_mips_blocks<<<dim3((unsigned)(bx < 1024 ? bx : 1024), (unsigned)ctx->d), 256, 0, st>>>(
-      ctx->TB, ctx->d, ctx->n, ctx->mips_tb, ctx->mips_blocks);
-  count_launch(ctx);
+  if ((rs = tb_guide_build(ctx, st)) != MAD_OK) return rs;
   DevScalars hs;
   cudaMemcpyAsync(&hs, ctx->sc, sizeof(hs), cudaMemcpyDeviceToHost, st);
   if ((rs = cuda_status(cudaStreamSynchronize(st))) != MAD_OK) return rs;
@@ -992,9 +954,15 @@ mad_status mad_mips_run(mad_ctx* ctx, const mad_matrix* Q, uint64_t seed, mad_pa
     grid = std::min<unsigned long long>(grid, (unsigned long long)sms * ctx->mips_bps);
   }
   grid = std::min<unsigned long long>(grid, 0x7FFFFFFFull);
-  k_mips_draw<<<(unsigned)grid, kDrawThreads, draw_smem_bytes(chunk, ctx->mips_max_parts, ctx->d),
-                st>>>(p, seed, b.queries, b.chunk_q, ctx->mips_chunks, ctx->mips_plan_mult,
-                      ctx->mips_max_parts, ctx->mips_tb, ctx->mips_blocks, b.rec, b.off);
+  const size_t draw_smem = draw_smem_bytes(chunk, ctx->mips_max_parts, ctx->d);
+  if (p.tb_blocks)
+    k_mips_draw<true><<<(unsigned)grid, kDrawThreads, draw_smem, st>>>(
+        p, seed, b.queries, b.chunk_q, ctx->mips_chunks, ctx->mips_plan_mult, ctx->mips_max_parts,
+        b.rec, b.off);
+  else
+    k_mips_draw<false><<<(unsigned)grid, kDrawThreads, draw_smem, st>>>(
+        p, seed, b.queries, b.chunk_q, ctx->mips_chunks, ctx->mips_plan_mult, ctx->mips_max_parts,
+        b.rec, b.off);
   k_mips_parts<<<(unsigned)ctx->mips_units, kPartThreads, ctx->mips_parts_smem, st>>>(
       b.queries, b.unit_q, b.rec, b.off, chunk, ctx->mips_slots, ctx->region_factor, ctx->f, ctx->mips_tprime, b.kept,
       b.kept_n, ctx->sc);

@@ -178,18 +178,18 @@ __device__ __forceinline__ Draw draw_rows(const SampleParams& p, bool valid,
     if (i >= p.m) { *bad = true; i = p.m - 1; }
     const uint4 ra = __ldg(p.rdesc + i);
     const uint32_t* __restrict__ row = p.T2 + ra.x;
-    const uint32_t target = (uint32_t)draw_target(u.u1, ra.z);
+    const uint32_t target = draw_target32(u.u1, ra.z);
     uint32_t pk =
         ra.y >= (uint32_t)kGuideMin
             ? (uint32_t)ub_guided_u32(row, p.T2g + ra.w, t2_guide_shift(ra.y, ra.z), target)
             : (uint32_t)ub_u32(row, (int)ra.y, target, 0xFFFFFFFFu);
     if (pk >= ra.y) { *bad = true; pk = ra.y - 1; }
-    const uint32_t pkp = (uint32_t)draw_target(u.u3, ra.y);
+    const uint32_t pkp = draw_target32(u.u3, ra.y);
     dr.i = (uint32_t)i;
     dr.k = (uint32_t)__ldg(p.a_col + ra.x + pk);
     dr.kp = (uint32_t)__ldg(p.a_col + ra.x + pkp);
     const uint2 rb = __ldg(p.brow + dr.k);
-    dr.j = (uint32_t)__ldg(p.b_col + rb.x + (uint32_t)draw_target(u.u2, rb.y));
+    dr.j = (uint32_t)__ldg(p.b_col + rb.x + draw_target32(u.u2, rb.y));
     // b_k'j != 0: the entry (j, k') of A under MAD_GRAM, else (k', j) of B.
     maybe = !p.bloom || bloom_may_contain(p.bloom, p.bloom_shift, gram ? dr.j : dr.kp,
                                           gram ? dr.kp : dr.j);
@@ -446,6 +446,15 @@ k_sort_fine(const uint32_t* __restrict__ rec, const unsigned int* __restrict__ o
 // v = 0 or an excluded diagonal) and its increment to vals[q].  Under
 // MAD_SQUARE_SYM the same increment for the pair (k, k') goes to keys[s +
 // q] and vals[s + q] (Sec. 3.2.3).  k_insert adds them to X.
+//
+// The draws are draw_given_row's, written out for dense inputs of one type.
+// Issue slots and L1 bind it together (54 % and 62 % of their rates, 680
+// instructions a diamond before, DRAM 23 %): without the branches on input
+// kinds and with 32-bit totals multiplied as such the fused pass went from 930
+// to 907 us.  TB in 64-byte blocks, as the batched queries draw, is slower here
+// (972 us: TB and its guides are in L2, and a block reads twice their bytes),
+// and so are 7 or 8 blocks per SM (935 us).
+template <typename TBV>
 __global__ void __launch_bounds__(256, 6)
 k_sample_sorted(const SampleParams p_, unsigned long long seed, unsigned long long first,
                 unsigned long long s, const uint32_t* __restrict__ order,
@@ -453,13 +462,37 @@ k_sample_sorted(const SampleParams p_, unsigned long long seed, unsigned long lo
   const bool sqsym = (p_.flags & MAD_SQUARE_SYM) != 0;
   const SampleParams p = resolve(p_);
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+  const int d = (int)p.d;
   bool bad = false;
   unsigned long long diag = 0;
   for (unsigned long long q = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; q < s;
        q += stride) {
     const Uniforms u = diamond_uniforms(seed, first + __ldcs(order + q));
-    const int64_t i = draw_row_i(p, u.u0, &bad);
-    const Draw dr = draw_given_row(p, u, i, &bad);
+    Draw dr;
+    {
+      const int64_t i = draw_row_i(p, u.u0, &bad);
+      const uint32_t* __restrict__ r2 = p.T2 + i * p.d;
+      const uint32_t* __restrict__ ra = p.TA + i * p.d;
+      int k, kp;
+      ub2_u32(r2, ra, d, draw_target32(u.u1, __ldg(r2 + d - 1) & PREFIX_MASK),
+              draw_target32(u.u3, __ldg(ra + d - 1) & PREFIX_MASK), PREFIX_MASK, &k, &kp);
+      if (k >= d) { bad = true; k = d - 1; }
+      if (kp >= d) { bad = true; kp = d - 1; }
+      uint32_t sign = __ldg(r2 + k) ^ __ldg(ra + kp);
+      const uint32_t* __restrict__ row = p.TB + (int64_t)k * p.n;
+      int64_t j = ub_guided_u32(row, p.TBg + k * p.tbg_stride, (int)__ldg(p.TBg_sh + k),
+                                draw_target32(u.u2, __ldg(row + p.n - 1) & PREFIX_MASK),
+                                PREFIX_MASK);
+      if (j >= p.n) { bad = true; j = p.n - 1; }
+      sign ^= __ldg(row + j);
+      const TBV b = __ldg((const TBV*)p.b_val + (int64_t)kp * p.ldb + j);
+      dr.i = (uint32_t)i;
+      dr.k = (uint32_t)k;
+      dr.j = (uint32_t)j;
+      dr.kp = (uint32_t)kp;
+      dr.v = fixed_point((float)b, p.f_exp);
+      if (!(p.flags & MAD_NONNEG) && (sign & SIGN_BIT)) dr.v = -dr.v;
+    }
     unsigned long long key = EMPTY_KEY;
     if ((p.flags & MAD_EXCLUDE_DIAG) && dr.i == dr.j) {
       ++diag;
@@ -927,6 +960,8 @@ SampleParams make_params(const mad_ctx* ctx) {
   p.TBg = ctx->TBg;
   p.tbg_stride = ctx->tbg_stride;
   p.TBg_sh = ctx->TBg_sh;
+  p.tb_blocks = ctx->tb_blocks;
+  p.tb_row = ctx->tb_row;
   p.f_exp = ctx->f;
   p.hkeys = ctx->hkeys;
   p.hvals = ctx->hvals;
@@ -1081,7 +1116,6 @@ mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first, 
     phase_event(ctx, 3, st);
     return cuda_status(cudaGetLastError());
   }
-  const int full_sorted = full_grid<k_sample_sorted>();
   const int full_insert = full_grid<k_insert>();
   const uint64_t nbk = sort_buckets(ctx->m);
   const int blocks = sort_blocks();
@@ -1129,8 +1163,12 @@ mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first, 
         w.rec, w.off, blocks, fine, (unsigned)n, w.order, w.base);
     count_launch(ctx, 3);
     phase_event(ctx, 1, st);
-    k_sample_sorted<<<grid_of(n, full_sorted), 256, 0, st>>>(p, seed, first + done, n, w.order,
-                                                             w.keys, w.vals);
+    if (ctx->B.dt == MAD_F64)
+      k_sample_sorted<double><<<grid_of(n, full_grid<k_sample_sorted<double>>()), 256, 0, st>>>(
+          p, seed, first + done, n, w.order, w.keys, w.vals);
+    else
+      k_sample_sorted<float><<<grid_of(n, full_grid<k_sample_sorted<float>>()), 256, 0, st>>>(
+          p, seed, first + done, n, w.order, w.keys, w.vals);
     count_launch(ctx);
     phase_event(ctx, 2, st);
     if (build_x) {

@@ -1173,7 +1173,51 @@ int tb_guide_width(int64_t n) {
   return full < cap ? full : cap;
 }
 
+// Row k's total, mul and blocks [k (nb + 1), (k + 1) (nb + 1)); the last block
+// only ends the one before it.
+__global__ void __launch_bounds__(256)
+k_tb_blocks(const uint32_t* __restrict__ TB, int64_t d, int64_t n, uint2* __restrict__ tb_row,
+              uint4* __restrict__ blocks) {
+  const int64_t nb = tb_blocks(n);
+  for (int64_t k = blockIdx.y; k < d; k += gridDim.y) {
+    const uint32_t* __restrict__ row = TB + k * n;
+    const uint32_t tot = __ldg(row + n - 1) & PREFIX_MASK;
+    // (t mul < 2^32 nb for t < tot, so every bucket is below nb)
+    const unsigned long long mul = tot ? ((unsigned long long)nb << 32) / tot : 0ull;
+    const uint32_t m32 = mul < 0xFFFFFFFFull ? (uint32_t)mul : 0xFFFFFFFFu;
+    if (blockIdx.x == 0 && threadIdx.x == 0) tb_row[k] = make_uint2(tot, m32);
+    uint4* __restrict__ out = blocks + k * (nb + 1) * 4;
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b <= nb;
+         b += (int64_t)gridDim.x * blockDim.x) {
+      uint32_t lo = (uint32_t)n;
+      if (m32) {
+        const unsigned long long first = bucket_first((unsigned long long)b, m32);
+        if (b == 0) lo = (uint32_t)ub_u32(row, (int)n, 0u, PREFIX_MASK);
+        else if (first < tot) lo = (uint32_t)ub_u32(row, (int)n, (uint32_t)first, PREFIX_MASK);
+      }
+      uint32_t v[16];
+      v[0] = lo;
+#pragma unroll
+      for (int c = 0; c < kBlockEnts; ++c) {
+        const int64_t e = (int64_t)lo + c;
+        v[1 + c] = e < n ? __ldg(row + e) : PREFIX_MASK;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        out[4 * b + q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    }
+  }
+}
+
 mad_status tb_guide_build(mad_ctx* ctx, cudaStream_t st) {
+  if (ctx->tb_blocks) {
+    const int64_t bx = (tb_blocks(ctx->n) + 256) / 256;
+    k_tb_blocks<<<dim3((unsigned)(bx < 1024 ? bx : 1024),
+                       (unsigned)(ctx->d < 65535 ? ctx->d : 65535)),
+                  256, 0, st>>>(ctx->TB, ctx->d, ctx->n, ctx->tb_row, ctx->tb_blocks);
+    count_launch(ctx);
+    return cuda_status(cudaGetLastError());
+  }
   const int W = tb_guide_width(ctx->n);
   const int64_t xblocks = (ctx->n + 1023) / 1024;   // four entries per thread
   const dim3 grid((unsigned)(xblocks < 64 ? xblocks : 64),

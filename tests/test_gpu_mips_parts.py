@@ -19,7 +19,7 @@ def _built():
         pytest.skip("no CUDA device")
 
 
-def _compare(Q, B, s_q, s_max, tprime, t, seed=5, factor=None, cfg=None):
+def _compare(Q, B, s_q, s_max, tprime, t, seed=5, factor=None, cfg=None, guides=False):
     import paper_1506_03872_gb300 as mad
     nq = len(s_q)
     tQ, tB = torch.from_numpy(Q).cuda(), torch.from_numpy(B).cuda()
@@ -28,6 +28,8 @@ def _compare(Q, B, s_q, s_max, tprime, t, seed=5, factor=None, cfg=None):
     with mad.Context() as c:
         if factor:
             mad.mad_debug_set_hash_layout(c.ctx, factor)
+        if guides:
+            mad.mad_debug_set_hash_layout(c.ctx, 1.5, 1 << 14)
         if cfg:
             mad.mad_mips_config(c.ctx, **cfg)
         mad.mad_mips_items(c.ctx, mad.dense(tB), s_max)
@@ -98,3 +100,14 @@ def test_ties_of_x_in_the_thousands():
     B = np.where(rng.random((16, 30_001)) < 0.5, -1.0, 1.0).astype(np.float32)
     Q = rng.standard_normal((3, 16)).astype(np.float32)
     _compare(Q, B, np.array([20_000, 60_000, 700], np.uint64), 1 << 16, 300, 20)
+
+
+@pytest.mark.parametrize("d,n", [(7, 3001), (33, 17), (300, 40_003), (2, 1)])
+def test_row_guides_draw_what_the_blocks_draw(d, n):
+    """Item tables too long for 64-byte blocks are drawn from through their
+    row guides (asked for here by the debug layout's overflow table)."""
+    s_q = np.array([1, 300, 5000, 30_000], np.uint64)
+    Q, B = _items(d * n, d, n, len(s_q))
+    B[0, ::3] = 0.0
+    _compare(Q, B, s_q, 30_000, 40, 7)
+    _compare(Q, B, s_q, 30_000, 40, 7, guides=True)
