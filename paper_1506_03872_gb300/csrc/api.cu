@@ -530,6 +530,9 @@ mad_status mad_build_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix*
   }
   const bool pilot = ctx->hcap_request == 0 && !wedge;
   cudaMemsetAsync(ctx->sc, 0, sizeof(DevScalars), st);
+  if (ctx->nnz_a < (1ull << 32) && ctx->nnz_b < (1ull << 32) &&
+      (rs = alloc(ctx, ctx->brow, (size_t)ctx->d, st)) != MAD_OK)
+    return rs;
   if ((rs = build_tables_impl(ctx, st)) != MAD_OK) return rs;
   DevScalars hs;
   if ((rs = read_scalars(ctx, &hs, st)) != MAD_OK) return rs;
@@ -545,9 +548,8 @@ mad_status mad_build_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix*
   if ((rs = alloc(ctx, ctx->T2g, (size_t)gtotal, st)) != MAD_OK) return rs;
   ctx->t2g_total = gtotal;
   if (gtotal && (rs = t2_guide_fill(ctx, st)) != MAD_OK) return rs;
-  if (ctx->nnz_a < (1ull << 32) && ctx->nnz_b < (1ull << 32) && gtotal < (1ull << 32)) {
+  if (ctx->brow && gtotal < (1ull << 32)) {
     if ((rs = alloc(ctx, ctx->rdesc, (size_t)ctx->m, st)) != MAD_OK) return rs;
-    if ((rs = alloc(ctx, ctx->brow, (size_t)ctx->d, st)) != MAD_OK) return rs;
     if ((rs = row_desc_fill(ctx, st)) != MAD_OK) return rs;
   }
   // Closure filter: 16 bits per entry, a power of two of 64-bit words.
@@ -564,16 +566,17 @@ mad_status mad_build_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix*
   if (pilot) {
     // Fraction of diamonds that add to X, from kPilot diamonds of a fixed
     // seed; the table holds s_max times that fraction plus six standard
-    // deviations at load 1/16 (and never more than s_max / 0.6 slots).
-    // Measured on GB300: scattered inserts into a table at load 0.46 took
-    // 3.3x longer than at load 0.06 with the same number of probes.
+    // deviations at load 1/4 or less (and never more than s_max / 0.6
+    // slots).  The sampler takes the same time at loads of 1/16 to 0.4 (4.67 ms for
+    // 1e8 diamonds on 1e6 nodes); clearing X and the two passes over it do not
+    // (the search 6438 us at 1/16, 6257 at 1/4, 6202 at 0.4).
     const uint64_t kPilot = 1ull << 20;
     uint64_t hits = 0;
     if ((rs = pilot_inserts(ctx, kPilot, &hits, st)) != MAD_OK) return rs;
     const double f = (double)hits / (double)kPilot;
     const double f_hi = f + 6.0 * std::sqrt(f * (1.0 - f) / (double)kPilot) + 8.0 / (double)kPilot;
     const double per = (ctx->flags & MAD_SQUARE_SYM) ? 2.0 : 1.0;  // inserts per diamond
-    const double want = std::min(((double)s_max * std::min(f_hi, per) + 4096.0) * 16.0,
+    const double want = std::min(((double)s_max * std::min(f_hi, per) + 4096.0) * 4.0,
                                  per * (double)s_max / 0.6);
     uint64_t cap = 1024;
     while ((double)cap < want && cap < (1ull << 40)) cap <<= 1;

@@ -316,8 +316,8 @@ mad_status t2_guide_offsets(mad_ctx* ctx, cudaStream_t st);
 // MAD_GRAM, else B) into ctx->bloom (2^bloom_lg words, cleared here).
 mad_status build_bloom(mad_ctx* ctx, cudaStream_t st);
 mad_status t2_guide_fill(mad_ctx* ctx, cudaStream_t st);
-// Row descriptors into ctx->rdesc (m) and ctx->brow (d), after the guides'
-// offsets; nothing where they are not allocated.
+// Row descriptors into ctx->rdesc (m), after the guides' offsets; nothing where
+// they are not allocated (ctx->brow is filled with the tables).
 mad_status row_desc_fill(mad_ctx* ctx, cudaStream_t st);
 // Batched queries: TB in 64-byte blocks of kBlockEnts entries, about kBlockKeys of them new in
 // each (see ub_block): 10.7 bytes an entry of TB, built up to 2^31 entries (23

@@ -105,8 +105,12 @@ __device__ __forceinline__ float to_f32(double v, bool* unsafe) {
 }
 
 // U of every candidate (into the first half of its cvals slot) and tau.
-// A warp per candidate, two in flight: bound by the latency of the rows.
-template <typename TA, typename TB>
+// A warp per candidate, four in flight; kVec: FP32 rows on 16-byte boundaries (d
+// and the leading dimension multiples of four), read 16 bytes a lane.  Bound by
+// the latency of the rows (1e5 candidates of d = 100: 48 us with two in flight
+// and 4-byte loads, 27 us so; 80 MB are 12 us of reading).
+constexpr int kBoundAhead = 4;
+template <typename TA, typename TB, bool kVec>
 __global__ void __launch_bounds__(256)
 k_rescore_bound(const mad_pair* __restrict__ cand, unsigned long long ncand_max,
                 const TA* __restrict__ A, int64_t lda, const TB* __restrict__ Bt, int64_t d,
@@ -119,37 +123,62 @@ k_rescore_bound(const mad_pair* __restrict__ cand, unsigned long long ncand_max,
   const int lane = threadIdx.x & 31;
   const unsigned long long warp = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const unsigned long long warps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-  for (unsigned long long q0 = warp; q0 < ncand; q0 += 2 * warps) {
-    float c[2], s[2];
-    bool valid[2], unsafe[2];
+  // A warp's candidates are consecutive, kBoundAhead at a time.
+  for (unsigned long long q0 = warp * kBoundAhead; q0 < ncand; q0 += kBoundAhead * warps) {
+    float c[kBoundAhead], s[kBoundAhead];
+    bool valid[kBoundAhead], unsafe[kBoundAhead];
+    const TA* a[kBoundAhead];
+    const TB* b[kBoundAhead];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const unsigned long long q = q0 + (unsigned long long)u * warps;
+    for (int u = 0; u < kBoundAhead; ++u) {
+      const unsigned long long q = q0 + u;
       c[u] = s[u] = 0.0f;
-      valid[u] = unsafe[u] = false;
-      if (q >= ncand) continue;
-      const uint32_t i = cand[q].i, j = cand[q].j;
+      unsafe[u] = false;
+      const uint32_t i = q < ncand ? cand[q].i : 0xFFFFFFFFu, j = q < ncand ? cand[q].j : 0u;
       valid[u] = i < m && j < n;
-      if (!valid[u]) continue;
-      const TA* __restrict__ a = A + (int64_t)i * lda;
-      const TB* __restrict__ b = Bt + (int64_t)j * d;
-#pragma unroll 4
+      a[u] = A + (valid[u] ? (int64_t)i * lda : 0);
+      b[u] = Bt + (valid[u] ? (int64_t)j * d : 0);
+    }
+    if (kVec) {
+      // 16 bytes a lane: a row of 128 FP32 entries in one load.
+      for (int64_t k = 4 * lane; k < d; k += 128) {
+        float4 x[kBoundAhead], y[kBoundAhead];
+#pragma unroll
+        for (int u = 0; u < kBoundAhead; ++u) {
+          x[u] = __ldg(reinterpret_cast<const float4*>(a[u] + k));
+          y[u] = __ldg(reinterpret_cast<const float4*>(b[u] + k));
+        }
+#pragma unroll
+        for (int u = 0; u < kBoundAhead; ++u) {
+          const float xs[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+          const float ys[4] = {y[u].x, y[u].y, y[u].z, y[u].w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            c[u] = fmaf(xs[e], ys[e], c[u]);
+            s[u] = fmaf(fabsf(xs[e]), fabsf(ys[e]), s[u]);
+          }
+        }
+      }
+    } else {
       for (int64_t k = lane; k < d; k += 32) {
-        const float x = to_f32(a[k], &unsafe[u]), y = to_f32(b[k], &unsafe[u]);
-        c[u] = fmaf(x, y, c[u]);
-        s[u] = fmaf(fabsf(x), fabsf(y), s[u]);
+#pragma unroll
+        for (int u = 0; u < kBoundAhead; ++u) {
+          const float x = to_f32(a[u][k], &unsafe[u]), y = to_f32(b[u][k], &unsafe[u]);
+          c[u] = fmaf(x, y, c[u]);
+          s[u] = fmaf(fabsf(x), fabsf(y), s[u]);
+        }
       }
     }
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1)
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < kBoundAhead; ++u) {
         c[u] += __shfl_xor_sync(0xFFFFFFFFu, c[u], off);
         s[u] += __shfl_xor_sync(0xFFFFFFFFu, s[u], off);
       }
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const unsigned long long q = q0 + (unsigned long long)u * warps;
+    for (int u = 0; u < kBoundAhead; ++u) {
+      const unsigned long long q = q0 + u;
       const bool any_unsafe = __any_sync(0xFFFFFFFFu, unsafe[u]);
       if (q >= ncand || lane != 0) continue;
       if (!valid[u]) atomicOr(&sc->err, DERR_SEARCH);   // outside the matrices
@@ -368,7 +397,7 @@ struct __align__(16) GramRec {
   long long lo_start, hub_start;
 };
 
-constexpr int kRgUnit = 64;        // candidates a block takes at a time
+constexpr int kRgUnit = 64;        // most candidates a block takes at a time
 constexpr int kRgThreads = 1024;
 constexpr int kRgKeep = 8;         // hub columns a thread keeps between set and clear
 
@@ -460,7 +489,7 @@ __device__ __forceinline__ uint32_t count_row_in_bits(const uint32_t* bits, int6
 __global__ void __launch_bounds__(kRgThreads, 1)
 k_rescore_bitmap(const GramRec* __restrict__ rec, unsigned long long ncand_max,
                  const unsigned long long* n_dev, const int32_t* __restrict__ a_col, int64_t m,
-                 int64_t d, double* __restrict__ cvals, Item* __restrict__ items,
+                 int64_t d, int unit, double* __restrict__ cvals, Item* __restrict__ items,
                  DevScalars* sc, unsigned long long* next_unit) {
   extern __shared__ uint32_t bits[];
   __shared__ GramRec s_rec[kRgUnit];
@@ -471,7 +500,7 @@ k_rescore_bitmap(const GramRec* __restrict__ rec, unsigned long long ncand_max,
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t words = (uint32_t)((d + 31) >> 5);
   for (uint32_t w = tid; w < words; w += kRgThreads) bits[w] = 0u;
-  const unsigned long long units = (ncand + kRgUnit - 1) / kRgUnit;
+  const unsigned long long units = (ncand + unit - 1) / unit;
   // Units from a counter: their cost varies with the number of hubs in
   // them (one bitmap per hub), so a fixed assignment left some blocks
   // twice the mean work.
@@ -481,8 +510,8 @@ k_rescore_bitmap(const GramRec* __restrict__ rec, unsigned long long ncand_max,
     __syncthreads();
     const unsigned long long u = s_unit;
     if (u >= units) break;
-    const unsigned long long p0 = u * kRgUnit;
-    const int n = (int)(ncand - p0 < (unsigned long long)kRgUnit ? ncand - p0 : kRgUnit);
+    const unsigned long long p0 = u * unit;
+    const int n = (int)(ncand - p0 < (unsigned long long)unit ? ncand - p0 : unit);
     if (tid < n) {
       const uint4* src = reinterpret_cast<const uint4*>(rec + p0 + tid);
       uint4* dst = reinterpret_cast<uint4*>(s_rec + tid);
@@ -625,10 +654,14 @@ mad_status rescore_gram_grouped(mad_ctx* ctx, const mad_pair* cand, uint64_t nca
   k_rg_scatter<<<grid, 256, 0, st>>>(cand, ncand, n_dev, ctx->A.rowptr, ctx->m, off, rec);
   count_launch(ctx);
   const size_t smem = gram_bitmap_bytes(ctx->d);
-  const unsigned long long units = (ncand + kRgUnit - 1) / kRgUnit;
   const int full = rescore_bitmap_grid(smem);
+  // Two units a block where there are few candidates (1000 of a graph of 20,011
+  // nodes in units of 64 kept 16 blocks busy: 66 us; in units of 4, 19 us).
+  const unsigned long long share = ncand / (2ull * (unsigned)full);
+  const int unit = (int)(share < 4 ? 4 : share < (unsigned)kRgUnit ? share : kRgUnit);
+  const unsigned long long units = (ncand + unit - 1) / unit;
   k_rescore_bitmap<<<(unsigned)(units < (unsigned long long)full ? units : full), kRgThreads, smem,
-                     st>>>(rec, ncand, n_dev, ctx->A.colidx, ctx->m, ctx->d, cvals, items,
+                     st>>>(rec, ncand, n_dev, ctx->A.colidx, ctx->m, ctx->d, unit, cvals, items,
                            ctx->sc, next_unit);
   count_launch(ctx);
   return cuda_status(cudaGetLastError());
@@ -648,11 +681,22 @@ template <typename TA, typename TB>
 void launch_bounded(mad_ctx* ctx, const mad_pair* cand, uint64_t ncand, uint64_t t, Item* items,
                     double* cvals, const unsigned long long* n_dev, cudaStream_t st) {
   BoundState* bs = (BoundState*)ctx->bound_state;
-  const unsigned long long warps2 = (ncand * 16 + 255) / 256;   // two candidates a warp
+  const unsigned long long bound_blocks = (ncand * 32 / kBoundAhead + 255) / 256;
   const unsigned long long blocks = (ncand + 255) / 256;
-  k_rescore_bound<TA, TB><<<(unsigned)(warps2 < 152 * 8 ? warps2 : 152 * 8), 256, 0, st>>>(
-      cand, ncand, (const TA*)ctx->A.values, ctx->A.ld, (const TB*)ctx->bt, ctx->d, ctx->m, ctx->n,
-      (unsigned)t, cvals, bs, ctx->sc, n_dev);
+  const unsigned bgrid = (unsigned)(bound_blocks < 152 * 8 ? bound_blocks : 152 * 8);
+  bool vec = false;
+  if constexpr (sizeof(TA) == 4 && sizeof(TB) == 4)
+    vec = ctx->d % 4 == 0 && ctx->A.ld % 4 == 0 && ((uintptr_t)ctx->A.values & 15) == 0;
+  if (vec) {
+    if constexpr (sizeof(TA) == 4 && sizeof(TB) == 4)
+      k_rescore_bound<TA, TB, true><<<bgrid, 256, 0, st>>>(
+          cand, ncand, (const TA*)ctx->A.values, ctx->A.ld, (const TB*)ctx->bt, ctx->d, ctx->m,
+          ctx->n, (unsigned)t, cvals, bs, ctx->sc, n_dev);
+  } else {
+    k_rescore_bound<TA, TB, false><<<bgrid, 256, 0, st>>>(
+        cand, ncand, (const TA*)ctx->A.values, ctx->A.ld, (const TB*)ctx->bt, ctx->d, ctx->m,
+        ctx->n, (unsigned)t, cvals, bs, ctx->sc, n_dev);
+  }
   k_rescore_kept<TA, TB><<<(unsigned)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, st>>>(
       cand, ncand, (const TA*)ctx->A.values, ctx->A.ld, (const TB*)ctx->bt, ctx->d, cvals, items,
       bs, n_dev);

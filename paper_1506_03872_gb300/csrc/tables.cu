@@ -569,12 +569,29 @@ k_a_rows_short(const T* __restrict__ A, int64_t m, int d, int64_t lda,
 // indices (generators often number nodes by weight) go to different warps.
 // A warp per row, as for the long rows, spent a chain of dependent loads on
 // every short row in turn.
+// (brow: start and length of every row of B, filled by k_b_row_desc first.)
+__global__ void __launch_bounds__(256)
+k_b_row_desc(const int64_t* __restrict__ b_ptr, int64_t d, uint2* __restrict__ brow) {
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < d;
+       k += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b0 = b_ptr[k];
+    brow[k] = make_uint2((uint32_t)b0, (uint32_t)(b_ptr[k + 1] - b0));
+  }
+}
+
 constexpr int64_t kShortRow = 32;
+constexpr int kRowAhead = 8;   // 32-entry pieces of a long row in flight
 
 __global__ void __launch_bounds__(256)
 k_a_rows_binary(const int64_t* __restrict__ a_ptr, const int32_t* __restrict__ a_col,
-                const int64_t* __restrict__ b_ptr, int64_t m, uint32_t* __restrict__ T2,
-                unsigned long long* __restrict__ r64, DevScalars* sc) {
+                const int64_t* __restrict__ b_ptr, const uint2* __restrict__ brow, int64_t m,
+                uint32_t* __restrict__ T2, unsigned long long* __restrict__ r64, DevScalars* sc) {
+  // Bound by the lookups of the entries' weights, one load each where the row
+  // descriptors of B are there (two row pointers: 177 us for 2e7 entries, 146 so).
+  auto weight = [&](int32_t k) -> unsigned long long {
+    return brow ? (unsigned long long)__ldg(&brow[k].y)
+                : (unsigned long long)(b_ptr[k + 1] - b_ptr[k]);
+  };
   const int lane = threadIdx.x & 31;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   bool over = false;
@@ -595,8 +612,7 @@ k_a_rows_binary(const int64_t* __restrict__ a_ptr, const int32_t* __restrict__ a
         for (int u = 0; u < 8; ++u) {
           q[u] = 0;
           if (e0 + u < a1) {
-            const int32_t k = a_col[e0 + u];
-            q[u] = (unsigned long long)(b_ptr[k + 1] - b_ptr[k]);
+            q[u] = weight(a_col[e0 + u]);
           }
         }
 #pragma unroll
@@ -615,20 +631,30 @@ k_a_rows_binary(const int64_t* __restrict__ a_ptr, const int32_t* __restrict__ a
       const int src = __ffs(lm) - 1;
       lm &= lm - 1;
       const int64_t r0 = __shfl_sync(0xFFFFFFFFu, a0, src), r1 = __shfl_sync(0xFFFFFFFFu, a1, src);
+      // kRowAhead x 32 entries' weights in flight: the longest row alone sets
+      // the kernel's time (4266 entries: 134 rounds of two dependent loads).
       unsigned long long carry = 0;
-      for (int64_t b = r0; b < r1; b += 32) {
-        const int64_t e = b + lane;
-        unsigned long long q = 0;
-        if (e < r1) {
-          const int32_t k = a_col[e];
-          q = (unsigned long long)(b_ptr[k + 1] - b_ptr[k]);
+      for (int64_t b = r0; b < r1; b += 32 * kRowAhead) {
+        int32_t k[kRowAhead];
+        unsigned long long q[kRowAhead];
+#pragma unroll
+        for (int u = 0; u < kRowAhead; ++u) {
+          const int64_t e = b + 32 * u + lane;
+          k[u] = e < r1 ? a_col[e] : -1;
         }
-        const unsigned long long inc = warp_inclusive_u64(q, lane) + carry;
-        if (e < r1) {
-          if (inc > 0xFFFFFFFFull) over = true;
-          T2[e] = (uint32_t)inc;
+#pragma unroll
+        for (int u = 0; u < kRowAhead; ++u)
+          q[u] = k[u] >= 0 ? weight(k[u]) : 0ull;
+#pragma unroll
+        for (int u = 0; u < kRowAhead; ++u) {
+          const int64_t e = b + 32 * u + lane;
+          const unsigned long long inc = warp_inclusive_u64(q[u], lane) + carry;
+          if (e < r1) {
+            if (inc > 0xFFFFFFFFull) over = true;
+            T2[e] = (uint32_t)inc;
+          }
+          carry = __shfl_sync(0xFFFFFFFFu, inc, 31);
         }
-        carry = __shfl_sync(0xFFFFFFFFu, inc, 31);
       }
       if (lane == 0) r64[base + (int64_t)src * warps + w] = (unsigned long long)(r1 - r0) * carry;
     }
@@ -688,13 +714,30 @@ k_guide_fill(const int64_t* __restrict__ a_ptr, const uint32_t* __restrict__ T2,
       const unsigned long long n = __shfl_sync(0xFFFFFFFFu, nr, src);
       const int64_t a0 = a_ptr[i], len = a_ptr[i + 1] - a0;
       const int sh = shift[i];
-      for (unsigned long long b = lane; b < n; b += 32) {
-        const unsigned long long thr = b << sh;   // count the entries below thr
-        uint32_t cnt;
-        if (thr == 0) cnt = 0;
-        else if (thr > 0xFFFFFFFFull) cnt = (uint32_t)len;
-        else cnt = (uint32_t)ub_u32(T2 + a0, (int)len, (uint32_t)(thr - 1), 0xFFFFFFFFu);
-        G[g0 + b] = cnt;
+      // Entry e writes the guide entries of the bucket starts in (T2[e-1],
+      // T2[e]] (guide entry b counts the entries below b << sh); the last one
+      // also those past it.
+      for (int64_t base_e = 0; base_e < len; base_e += 32 * kRowAhead) {
+        uint32_t v[kRowAhead], pv[kRowAhead];
+#pragma unroll
+        for (int u = 0; u < kRowAhead; ++u) {
+          const int64_t e = base_e + 32 * u + lane;
+          v[u] = e < len ? T2[a0 + e] : 0u;
+          pv[u] = e < len && e > 0 ? T2[a0 + e - 1] : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < kRowAhead; ++u) {
+          const int64_t e = base_e + 32 * u + lane;
+          if (e < len) {
+            const unsigned long long b_lo = e ? (unsigned long long)(pv[u] >> sh) + 1 : 0;
+            unsigned long long b_end = (unsigned long long)(v[u] >> sh) + 1;
+            b_end = b_end < n ? b_end : n;
+            for (unsigned long long b = b_lo; b < b_end; ++b) G[g0 + b] = (uint32_t)e;
+            if (e == len - 1)
+              for (unsigned long long b = b_end > b_lo ? b_end : b_lo; b < n; ++b)
+                G[g0 + b] = (uint32_t)len;
+          }
+        }
       }
     }
   }
@@ -948,33 +991,25 @@ mad_status t2_guide_offsets(mad_ctx* ctx, cudaStream_t st) {
 }
 
 // Row descriptors of the 0/1 sampler: what a draw needs of row i of A (start,
-// length, T2 total, guide start) and of row k of B (start, length) in one load
-// each, instead of two row pointers, the row's last T2 entry, the guide's
-// pointer and its shift from five arrays.
+// length, T2 total, guide start) in one load (and of row k of B, k_b_row_desc),
+// instead of two row pointers, the row's last T2 entry, the guide's pointer and
+// its shift from five arrays.
 __global__ void __launch_bounds__(256)
 k_row_desc(const int64_t* __restrict__ a_ptr, const uint32_t* __restrict__ T2, int64_t m,
-           const unsigned long long* __restrict__ gptr, const int64_t* __restrict__ b_ptr, int64_t d,
-           uint4* __restrict__ rdesc, uint2* __restrict__ brow) {
+           const unsigned long long* __restrict__ gptr, uint4* __restrict__ rdesc) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m || i < d; i += stride) {
-    if (i < m) {
-      const int64_t a0 = a_ptr[i], len = a_ptr[i + 1] - a0;
-      rdesc[i] = make_uint4((uint32_t)a0, (uint32_t)len, len ? T2[a0 + len - 1] : 0u,
-                            (uint32_t)gptr[i]);
-    }
-    if (i < d) {
-      const int64_t b0 = b_ptr[i];
-      brow[i] = make_uint2((uint32_t)b0, (uint32_t)(b_ptr[i + 1] - b0));
-    }
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
+    const int64_t a0 = a_ptr[i], len = a_ptr[i + 1] - a0;
+    rdesc[i] = make_uint4((uint32_t)a0, (uint32_t)len, len ? T2[a0 + len - 1] : 0u,
+                          (uint32_t)gptr[i]);
   }
 }
 
 mad_status row_desc_fill(mad_ctx* ctx, cudaStream_t st) {
   if (!ctx->rdesc) return MAD_OK;
-  const int64_t rows = ctx->m > ctx->d ? ctx->m : ctx->d;
-  const int64_t blocks64 = (rows + 255) / 256;
+  const int64_t blocks64 = (ctx->m + 255) / 256;
   k_row_desc<<<(unsigned)(blocks64 < 152 * 8 ? blocks64 : 152 * 8), 256, 0, st>>>(
-      ctx->A.rowptr, ctx->T2, ctx->m, ctx->T2g_ptr, ctx->B.rowptr, ctx->d, ctx->rdesc, ctx->brow);
+      ctx->A.rowptr, ctx->T2, ctx->m, ctx->T2g_ptr, ctx->rdesc);
   count_launch(ctx);
   return cuda_status(cudaGetLastError());
 }
@@ -998,9 +1033,16 @@ k_bloom_build(const int64_t* __restrict__ ptr, const int32_t* __restrict__ col, 
     }
     const bool longrow = e1 - e0 > 32;
     if (r < rows && !longrow) {
-      for (int64_t e = e0; e < e1; ++e) {
-        const BloomProbe b = bloom_probe((uint32_t)r, (uint32_t)col[e], shift);
-        atomicOr(words + b.word, ((unsigned long long)b.hi << 32) | b.lo);
+      for (int64_t f = e0; f < e1; f += kRowAhead) {
+        int32_t c[kRowAhead];
+#pragma unroll
+        for (int u = 0; u < kRowAhead; ++u) c[u] = f + u < e1 ? col[f + u] : -1;
+#pragma unroll
+        for (int u = 0; u < kRowAhead; ++u) {
+          if (c[u] < 0) continue;
+          const BloomProbe b = bloom_probe((uint32_t)r, (uint32_t)c[u], shift);
+          atomicOr(words + b.word, ((unsigned long long)b.hi << 32) | b.lo);
+        }
       }
     }
     unsigned lm = __ballot_sync(0xFFFFFFFFu, r < rows && longrow);
@@ -1009,9 +1051,19 @@ k_bloom_build(const int64_t* __restrict__ ptr, const int32_t* __restrict__ col, 
       lm &= lm - 1;
       const unsigned long long rr = (unsigned long long)(base + (int64_t)src * warps + w);
       const int64_t f0 = __shfl_sync(0xFFFFFFFFu, e0, src), f1 = __shfl_sync(0xFFFFFFFFu, e1, src);
-      for (int64_t e = f0 + lane; e < f1; e += 32) {
-        const BloomProbe b = bloom_probe((uint32_t)rr, (uint32_t)col[e], shift);
-        atomicOr(words + b.word, ((unsigned long long)b.hi << 32) | b.lo);
+      for (int64_t f = f0; f < f1; f += 32 * kRowAhead) {
+        int32_t c[kRowAhead];
+#pragma unroll
+        for (int u = 0; u < kRowAhead; ++u) {
+          const int64_t e = f + 32 * u + lane;
+          c[u] = e < f1 ? col[e] : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < kRowAhead; ++u) {
+          if (c[u] < 0) continue;
+          const BloomProbe b = bloom_probe((uint32_t)rr, (uint32_t)c[u], shift);
+          atomicOr(words + b.word, ((unsigned long long)b.hi << 32) | b.lo);
+        }
       }
     }
   }
@@ -1283,8 +1335,14 @@ mad_status build_tables_impl(mad_ctx* ctx, cudaStream_t st, bool side_branch) {
   if (ctx->integer) {
     const int64_t blocks64 = (ctx->m + 7) / 8;
     const unsigned blocks = (unsigned)(blocks64 < 152 * 16 ? blocks64 : 152 * 16);
-    k_a_rows_binary<<<blocks, 256, 0, st>>>(ctx->A.rowptr, ctx->A.colidx, ctx->B.rowptr, ctx->m,
-                                            ctx->T2, ctx->r64, ctx->sc);
+    if (ctx->brow) {
+      const int64_t rb = (ctx->d + 255) / 256;
+      k_b_row_desc<<<(unsigned)(rb < 152 * 8 ? rb : 152 * 8), 256, 0, st>>>(ctx->B.rowptr, ctx->d,
+                                                                          ctx->brow);
+      count_launch(ctx);
+    }
+    k_a_rows_binary<<<blocks, 256, 0, st>>>(ctx->A.rowptr, ctx->A.colidx, ctx->B.rowptr, ctx->brow,
+                                            ctx->m, ctx->T2, ctx->r64, ctx->sc);
     count_launch(ctx);
   } else {
     if (side_branch) {
