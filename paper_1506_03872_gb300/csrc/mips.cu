@@ -25,7 +25,7 @@
 // by one block per query), a diamond moves 16 bytes of records in and out
 // instead of about 250, no global atomic is left, and a query's selection is
 // spread over its parts.  Measured on one GB300: 1e4 queries of 5e4 diamonds
-// on 1e6 items x 300, 142 -> 43.9 ms; 61 queries on 50,021 x 100, 1300 -> 233 us.
+// on 1e6 items x 300, 142 -> 32.3 ms; 61 queries on 50,021 x 100, 1300 -> 200 us.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -52,6 +52,8 @@ namespace {
 
 constexpr int kDrawThreads = 256;
 constexpr int kPartThreads = 512;
+constexpr int kGroup = kPartThreads;         // chunks of a part scanned together
+constexpr int kAhead = 4;                    // records of a thread in flight
 constexpr int kSlots = 8192;                 // largest table of a part (96 KB: two blocks per SM)
 constexpr uint32_t kMaxParts = 2048;         // (a part too full for its table splits itself)
 constexpr int kTPrimeMax = 1024;             // largest t' of a batch
@@ -59,6 +61,7 @@ constexpr int kSlack = 32;                   // columns a part may keep beyond t
 constexpr int kBins = 2048;                  // digits of the threshold search (11 bits)
 constexpr int kSortMax = 2048;               // >= kTPrimeMax + kSlack
 constexpr uint32_t kNoKey = 0xFFFFFFFFu;     // (columns are below 2^31)
+static_assert(4 * kPartThreads <= kBins, "the warps' queues (64 records each) share the histogram's words");
 
 // Upper bounds in two shared-memory rows of the same length (independent
 // chains), as ub2_u32.
@@ -124,7 +127,8 @@ __device__ __forceinline__ uint32_t part_of(uint32_t h, uint32_t parts) {
 // chunk_q[c].  Shared memory: the query's T2 and TA rows, the chunk's records,
 // their parts and ranks, the parts' counts.  Bound by DRAM's random reads: per
 // diamond a block of TB (64 bytes) and b_k'j (a sector, fetched as 64 bytes) for
-// a million items, 3.4e10 of them a second; 2 to 5 resident blocks per SM measure
+// a million items, 4.5e10 of them a second (random reads reach 3.9e10 over 4.4 GB
+// and more where items repeat); 2 to 5 resident blocks per SM measure
 // the same, 6 leave too little L1 (8.46 instead of 6.59 ms for 1500 queries).
 template <bool kBlocks>
 __global__ void __launch_bounds__(kDrawThreads, 4)
@@ -160,8 +164,10 @@ k_mips_draw(const SampleParams p, unsigned long long seed, const MipsQuery* __re
     for (uint32_t x = tid; x < mq.parts; x += kDrawThreads) scnt[x] = 0;
     __syncthreads();
     const uint32_t t2tot = s2[d - 1] & PREFIX_MASK, tatot = sa[d - 1] & PREFIX_MASK;
-    for (int x = tid; x < cnt; x += kDrawThreads) {
-      const Uniforms un = diamond_uniforms(seed + q, l0 + x);
+    // (Whole warps: the blocks of TB are read by a warp's lanes together.)
+    for (int x0 = warp * 32; x0 < cnt; x0 += kDrawThreads) {
+      const int x = x0 + lane;
+      const Uniforms un = diamond_uniforms(seed + q, l0 + (x < cnt ? x : cnt - 1));
       int k, kp;
       ub2_shared(s2, sa, d, draw_target32(un.u1, t2tot),
                  draw_target32(un.u3, tatot), &k, &kp);
@@ -182,6 +188,7 @@ k_mips_draw(const SampleParams p, unsigned long long seed, const MipsQuery* __re
       }
       const uint32_t sign = sj ^ ((s2[k] ^ sa[kp]) & SIGN_BIT);
       const float b = __ldg((const float*)p.b_val + (int64_t)kp * p.ldb + j);
+      if (x >= cnt) continue;
       const uint32_t part = part_of(fmix32((uint32_t)j), mq.parts);
       const uint32_t rank = atomicAdd(&scnt[part], 1u);
       srec[x] = make_uint2((uint32_t)j, __float_as_uint(b) ^ sign);
@@ -369,6 +376,15 @@ struct Kept {
 // (a statistical rarity, or a batch whose parts are capped at kMaxParts) the
 // part is taken in 2, 4, ... slices of another mix of j, each slice's kept
 // columns competing with those of the slices before.
+//
+// The part's records lie in one run per chunk of the query: the runs' offsets are
+// scanned (kGroup chunks at a time) and the records dealt out evenly, four of a
+// lane read at a time.  Bound by the instructions of the inserts (55 % of the issue
+// slots with the loads' latency hidden): a warp that probes until the last of its
+// records is placed takes eight to ten steps for two on average, so a record whose
+// first slot is taken (a third of them) waits in the warp's queue until 32
+// such can probe on together: 14.5 ms for 5e8 diamonds, 9.6 so (four slots per
+// load 14.6, four records probing side by side 13.7).
 __global__ void __launch_bounds__(kPartThreads, 2)
 k_mips_parts(const MipsQuery* __restrict__ queries, const uint32_t* __restrict__ unit_q,
              const uint2* __restrict__ rec, const uint16_t* __restrict__ off, int chunk,
@@ -379,7 +395,7 @@ k_mips_parts(const MipsQuery* __restrict__ queries, const uint32_t* __restrict__
   Kept* temp = (Kept*)(vals + slots_max);                      // cap kept columns
   __shared__ PickState pick;
   __shared__ uint32_t s_full, s_n;
-  __shared__ unsigned long long s_records, s_inserted, s_created;
+  __shared__ unsigned long long s_inserted, s_created;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kWarps = kPartThreads / 32;
   const uint32_t u = blockIdx.x;
@@ -392,19 +408,45 @@ k_mips_parts(const MipsQuery* __restrict__ queries, const uint32_t* __restrict__
   const uint32_t nch = (uint32_t)((mq.s + chunk - 1) / chunk);
   const uint16_t* __restrict__ o = off + mq.off + part;
   const uint32_t ostep = mq.parts + 1;
-  if (tid == 0) s_records = 0;
-  __syncthreads();
-  unsigned long long mine = 0;
-  for (uint32_t c = tid; c < nch; c += kPartThreads)
-    mine += (uint32_t)__ldg(o + (size_t)c * ostep + 1) - (uint32_t)__ldg(o + (size_t)c * ostep);
+  // Chunks g0 .. of the part: soff[c] the records of those before chunk g0 + c,
+  // srun[c] + e the place of record e of them after chunk g0's first record;
+  // returns how many they are.
+  __shared__ uint32_t soff[kGroup], srun[kGroup];
+  uint2* queue = (uint2*)pick.hist + 64 * warp;
+  auto scan_group = [&](uint32_t g0) -> uint32_t {
+    const uint32_t c = g0 + tid;
+    uint32_t b0 = 0, len = 0;
+    if (c < nch) {
+      b0 = __ldg(o + (size_t)c * ostep);
+      len = (uint32_t)__ldg(o + (size_t)c * ostep + 1) - b0;
+    }
+    uint32_t inc = len;
 #pragma unroll
-  for (int s = 16; s >= 1; s >>= 1) mine += __shfl_xor_sync(0xFFFFFFFFu, mine, s);
-  if (lane == 0 && mine) atomicAdd(&s_records, mine);
-  __syncthreads();
+    for (int s = 1; s < 32; s <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, inc, s);
+      if (lane >= s) inc += v;
+    }
+    __syncthreads();   // (the words may still be read)
+    if (lane == 31) pick.warp_sum[warp] = inc;
+    __syncthreads();
+    uint32_t before = inc - len, total = 0;
+    for (int w = 0; w < kWarps; ++w) {
+      const uint32_t v = pick.warp_sum[w];
+      before += w < warp ? v : 0u;
+      total += v;
+    }
+    soff[tid] = before;
+    srun[tid] = (uint32_t)tid * (uint32_t)chunk + b0 - before;
+    __syncthreads();
+    return total;
+  };
+  unsigned long long records = 0;
+  uint32_t in_group = 0;
+  for (uint32_t g0 = 0; g0 < nch; g0 += kGroup) records += in_group = scan_group(g0);
   // A power of two of at least `factor` slots per record (1.5 unless a test
   // asks for less), up to the table's size.
   int slots = 256;
-  while (slots < slots_max && (float)slots < factor * (float)s_records) slots <<= 1;
+  while (slots < slots_max && (float)slots < factor * (float)records) slots <<= 1;
   const uint32_t mask = (uint32_t)slots - 1;
   for (int level = 0; level <= 31; ++level) {
     uint32_t nlist = 0;
@@ -412,58 +454,91 @@ k_mips_parts(const MipsQuery* __restrict__ queries, const uint32_t* __restrict__
     if (tid == 0) s_inserted = s_created = 0;
     const uint32_t slices = 1u << level;
     for (uint32_t slice = 0; slice < slices && !full; ++slice) {
-      for (int x = tid; x < slots; x += kPartThreads) {
-        keys[x] = kNoKey;
-        vals[x] = 0;
-      }
+      for (int x = tid; x < slots / 4; x += kPartThreads)
+        ((uint4*)keys)[x] = make_uint4(kNoKey, kNoKey, kNoKey, kNoKey);
+      for (int x = tid; x < slots / 2; x += kPartThreads)
+        ((uint4*)vals)[x] = make_uint4(0u, 0u, 0u, 0u);
       if (tid == 0) s_full = 0;
       __syncthreads();
       unsigned long long ins = 0, cre = 0;
-      for (uint32_t cb = (uint32_t)warp; cb < nch; cb += 32 * kWarps) {
-        // The segment bounds of this warp's next 32 chunks, one per lane.
-        const uint32_t cl = cb + (uint32_t)lane * kWarps;
-        uint32_t b0 = 0, b1 = 0;
-        if (cl < nch) {
-          b0 = __ldg(o + (size_t)cl * ostep);
-          b1 = __ldg(o + (size_t)cl * ostep + 1);
+      auto add = [&](uint32_t slot, long long x) {
+        uint32_t* h2 = (uint32_t*)(vals + slot);
+        const uint32_t lo = (uint32_t)(unsigned long long)x;
+        const uint32_t hi = (uint32_t)((unsigned long long)x >> 32);
+        const uint32_t old = atomicAdd(h2, lo);
+        atomicAdd(h2 + 1, hi + (old + lo < old ? 1u : 0u));
+      };
+      // The slots after its first, of a record that found that taken.
+      auto probe_on = [&](uint2 v) {
+        uint32_t slot = fmix32(v.x) & mask;
+        int probes = 1;
+        for (; probes < slots; ++probes) {
+          slot = (slot + 1) & mask;
+          const uint32_t cur = atomicCAS(keys + slot, kNoKey, v.x);
+          if (cur == kNoKey || cur == v.x) {
+            cre += cur == kNoKey ? 1 : 0;
+            add(slot, fixed_point(__uint_as_float(v.y), f_exp));
+            break;
+          }
         }
-        for (int w = 0; w < 32; ++w) {
-          const uint32_t c = cb + (uint32_t)w * kWarps;
-          if (c >= nch) break;
-          const uint32_t e1 = __shfl_sync(0xFFFFFFFFu, b1, w);
-          const uint2* __restrict__ r = rec + mq.rec + (unsigned long long)c * chunk;
-          for (uint32_t e = __shfl_sync(0xFFFFFFFFu, b0, w) + lane; e < e1; e += 32) {
-            const uint2 v = __ldg(r + e);
-            const long long x = fixed_point(__uint_as_float(v.y), f_exp);
-            const uint32_t h = fmix32(v.x);
-            if (x == 0 || (level && (fmix32(h ^ 0x9E3779B9u) >> (32 - level)) != slice)) continue;
-            ++ins;
-            uint32_t slot = h & mask;
-            int probes = 0;
-            for (; probes < slots; ++probes) {
-              uint32_t cur = ((volatile uint32_t*)keys)[slot];
-              if (cur == kNoKey) {
-                cur = atomicCAS(keys + slot, kNoKey, v.x);
-                if (cur == kNoKey) {
-                  ++cre;
-                  cur = v.x;
-                }
+        if (probes == slots) s_full = 1;
+      };
+      int waiting = 0;   // of the warp
+      for (uint32_t g0 = 0; g0 < nch; g0 += kGroup) {
+        if (nch > (uint32_t)kGroup) in_group = scan_group(g0);
+        const int runs = (int)(nch - g0 < (uint32_t)kGroup ? nch - g0 : (uint32_t)kGroup);
+        const uint2* __restrict__ r = rec + mq.rec + (unsigned long long)g0 * chunk;
+        // A warp's records: an even share of them, in a row.
+        const uint32_t share = ((in_group + kPartThreads - 1) / kPartThreads) * 32;
+        const uint32_t end = min(in_group, (warp + 1) * share);
+        int run = 0;   // the last run that starts at or before the lane's record
+        for (uint32_t base = warp * share; base < end; base += 32 * kAhead) {
+          uint2 v[kAhead];
+#pragma unroll
+          for (int a = 0; a < kAhead; ++a) {
+            const uint32_t e = base + 32 * a + lane;
+            v[a] = make_uint2(0u, 0u);
+            if (e < end) {
+              if (run + 1 < runs && soff[run + 1] <= e) {
+                ++run;
+                if (run + 1 < runs && soff[run + 1] <= e)
+                  for (int step = 1 << (31 - __clz(runs)); step > 0; step >>= 1)
+                    if (run + step < runs && soff[run + step] <= e) run += step;
               }
-              if (cur == v.x) break;
-              slot = (slot + 1) & mask;
+              v[a] = __ldg(r + (uint32_t)(srun[run] + e));
             }
-            if (probes == slots) {
-              s_full = 1;
-              continue;
+          }
+#pragma unroll
+          for (int a = 0; a < kAhead; ++a) {
+            const long long x = fixed_point(__uint_as_float(v[a].y), f_exp);   // (0: no record)
+            const uint32_t h = fmix32(v[a].x), slot = h & mask;
+            const bool in = x != 0 && !(level && (fmix32(h ^ 0x9E3779B9u) >> (32 - level)) != slice);
+            bool wait = false;
+            if (in) {
+              ++ins;
+              const uint32_t cur = atomicCAS(keys + slot, kNoKey, v[a].x);
+              if (cur == kNoKey || cur == v[a].x) {
+                cre += cur == kNoKey ? 1 : 0;
+                add(slot, x);
+              } else {
+                wait = true;
+              }
             }
-            uint32_t* h2 = (uint32_t*)(vals + slot);
-            const uint32_t lo = (uint32_t)(unsigned long long)x;
-            const uint32_t hi = (uint32_t)((unsigned long long)x >> 32);
-            const uint32_t old = atomicAdd(h2, lo);
-            atomicAdd(h2 + 1, hi + (old + lo < old ? 1u : 0u));
+            const uint32_t left = __ballot_sync(0xFFFFFFFFu, wait);
+            if (left) {
+              if (wait) queue[waiting + __popc(left & ((1u << lane) - 1u))] = v[a];
+              waiting += __popc(left);
+              __syncwarp();
+              if (waiting >= 32) {
+                waiting -= 32;
+                probe_on(queue[waiting + lane]);
+                __syncwarp();
+              }
+            }
           }
         }
       }
+      if (lane < waiting) probe_on(queue[lane]);
 #pragma unroll
       for (int s = 16; s >= 1; s >>= 1) {
         ins += __shfl_xor_sync(0xFFFFFFFFu, ins, s);
@@ -483,8 +558,9 @@ k_mips_parts(const MipsQuery* __restrict__ queries, const uint32_t* __restrict__
       auto get = [&](int e, unsigned long long* x, uint32_t* j) {
         if (e < slots) {
           *x = vals[e];
+          if ((long long)*x <= 0) return false;   // (0 in a free slot)
           *j = keys[e];
-          return *j != kNoKey && (long long)*x > 0;
+          return true;
         }
         const Kept k = list[e - slots];
         *x = k.x;
