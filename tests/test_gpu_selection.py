@@ -24,6 +24,7 @@ def _rng(seed):
 
 @pytest.mark.parametrize("kind", ["ties", "wide", "equal"])
 @pytest.mark.parametrize("n,K", [(1, 1), (31, 40), (33, 5), (2047, 2047), (2048, 100), (2049, 2049),
+                                 (8193, 8193), (32_768, 32_768), (32_769, 30_000),
                                  (40_000, 1000), (140_000, 3000), (300_000, 1), (300_000, 2048),
                                  (300_000, 150_000)])
 def test_select_pairs(n, K, kind):
