@@ -480,10 +480,22 @@ __device__ __forceinline__ BloomProbe bloom_probe(uint32_t a, uint32_t b, int sh
   return p;
 }
 
+// kFar: the word is the first that L2 drops again.
+template <bool kFar = false>
 __device__ __forceinline__ bool bloom_may_contain(const unsigned long long* __restrict__ words,
                                                   int shift, uint32_t a, uint32_t b) {
   const BloomProbe p = bloom_probe(a, b, shift);
-  const uint2 w = __ldg(reinterpret_cast<const uint2*>(words) + p.word);
+  const uint2* __restrict__ at = reinterpret_cast<const uint2*>(words) + p.word;
+  uint2 w;
+  if (kFar) {
+    unsigned long long policy;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    asm("ld.global.nc.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
+        : "=r"(w.x), "=r"(w.y)
+        : "l"(at), "l"(policy));
+  } else {
+    w = __ldg(at);
+  }
   return (w.x & p.lo) == p.lo && (w.y & p.hi) == p.hi;
 }
 

@@ -166,6 +166,7 @@ k_sample(const SampleParams p_, unsigned long long seed, unsigned long long firs
 // saves, 4.77 ms at best), windows read as 16-byte quads (registers spill,
 // 7.0 ms), and leaving the loop body early where the filter rules a diamond
 // out (the warp's lanes then run apart for good, 10.1 ms).
+template <bool kFar>
 __device__ __forceinline__ Draw draw_rows(const SampleParams& p, bool valid,
                                           unsigned long long seed, unsigned long long ell,
                                           bool* bad) {
@@ -191,8 +192,8 @@ __device__ __forceinline__ Draw draw_rows(const SampleParams& p, bool valid,
     const uint2 rb = __ldg(p.brow + dr.k);
     dr.j = (uint32_t)__ldg(p.b_col + rb.x + draw_target32(u.u2, rb.y));
     // b_k'j != 0: the entry (j, k') of A under MAD_GRAM, else (k', j) of B.
-    maybe = !p.bloom || bloom_may_contain(p.bloom, p.bloom_shift, gram ? dr.j : dr.kp,
-                                          gram ? dr.kp : dr.j);
+    maybe = !p.bloom || bloom_may_contain<kFar>(p.bloom, p.bloom_shift, gram ? dr.j : dr.kp,
+                                                gram ? dr.kp : dr.j);
   }
   // The few lanes whose diamond may close are searched while the others wait,
   // and the warp goes on together.
@@ -211,6 +212,7 @@ __device__ __forceinline__ Draw draw_rows(const SampleParams& p, bool valid,
   return dr;
 }
 
+template <bool kFar>
 __global__ void __launch_bounds__(256, 8)
 k_sample_rows(const SampleParams p_, unsigned long long seed, unsigned long long first,
               unsigned long long s) {
@@ -221,7 +223,7 @@ k_sample_rows(const SampleParams p_, unsigned long long seed, unsigned long long
   unsigned long long x = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
   for (unsigned long long r = 0; r < rounds; ++r, x += stride) {
     const bool valid = x < s;
-    const Draw dr = draw_rows(p, valid, seed, first + x, &t.bad);
+    const Draw dr = draw_rows<kFar>(p, valid, seed, first + x, &t.bad);
     accumulate(p, valid, dr, t);
     __syncwarp();
   }
@@ -910,7 +912,7 @@ k_pilot(const SampleParams p_, unsigned long long seed, unsigned long long n,
   for (unsigned long long r = 0; r < rounds; ++r, q += stride) {
     const bool valid = q < n;
     Draw dr{};
-    if (kRows) dr = draw_rows(p, valid, seed, q, &bad);
+    if (kRows) dr = draw_rows<false>(p, valid, seed, q, &bad);
     else if (valid) dr = draw_one_as<false>(p, seed, q, &bad);
     if (!valid) dr.v = 0;
     c += (dr.v != 0 && !((p.flags & MAD_EXCLUDE_DIAG) && dr.i == dr.j)) ? 1 : 0;
@@ -1105,9 +1107,23 @@ mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first, 
   if (!ctx->dense || p.alias) {
     phase_event(ctx, 0, st);
     phase_event(ctx, 1, st);
-    if (p.rdesc)
-      k_sample_rows<<<grid_of(s, full_grid<k_sample_rows>()), 256, 0, st>>>(p, seed, first, s);
-    else if (p.alias)
+    if (p.rdesc) {
+      // The filter's words are read evenly, the rows' tables by the rows' weights:
+      // where they do not fit into L2 together, the words do not stay there (1e8
+      // diamonds, 160 + 64 MB of tables and words: 4.68 -> 4.44 ms; 2e7 on 32 + 16
+      // MB, which fit: 0.838 -> 0.849 with the same hint).
+      int dev = 0, l2 = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+      const uint64_t bytes =
+          4 * (uint64_t)(ctx->nnz_a + ctx->nnz_b) + (p.bloom ? 8ull << ctx->bloom_lg : 0ull);
+      if (p.bloom && bytes > (uint64_t)l2)
+        k_sample_rows<true><<<grid_of(s, full_grid<k_sample_rows<true>>()), 256, 0, st>>>(
+            p, seed, first, s);
+      else
+        k_sample_rows<false><<<grid_of(s, full_grid<k_sample_rows<false>>()), 256, 0, st>>>(
+            p, seed, first, s);
+    } else if (p.alias)
       k_sample<true><<<grid_of(s, full_grid<k_sample<true>>()), 256, 0, st>>>(p, seed, first, s);
     else
       k_sample<false><<<grid_of(s, full_grid<k_sample<false>>()), 256, 0, st>>>(p, seed, first, s);
