@@ -156,24 +156,30 @@ mad_status clear_hash(mad_ctx* ctx, cudaStream_t st) {
   return cuda_status(cudaGetLastError());
 }
 
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
 // X of the region builder's layout re-inserted as a plain table, so that
-// further pairs can be added to it (synchronises).
+// further pairs can be added to it (asynchronous: the count of its keys, at most
+// one per diamond unless replays of a captured call added some, stays on the
+// device; a plain table stays one).
 mad_status x_to_table(mad_ctx* ctx, cudaStream_t st) {
-  DevScalars hs;
-  mad_status rs = read_scalars(ctx, &hs, st);
-  if (rs != MAD_OK) return rs;
-  const uint64_t cap = hs.new_keys ? hs.new_keys : 1;
+  const uint64_t slots = hash_slot_bound(ctx);
+  const uint64_t cap = ctx->x_captured || ctx->sampled > slots ? slots : ctx->sampled;
   void* tmp = nullptr;
-  if ((rs = pool_malloc(ctx, &tmp, 2 * cap * sizeof(uint64_t), st)) != MAD_OK) return rs;
-  uint64_t* keys = (uint64_t*)tmp;
+  mad_status rs = pool_malloc(ctx, &tmp, 256 + 2 * cap * sizeof(uint64_t), st);
+  if (rs != MAD_OK) return rs;
+  unsigned long long* count = (unsigned long long*)tmp;
+  uint64_t* keys = (uint64_t*)((char*)tmp + 256);
   int64_t* vals = (int64_t*)(keys + cap);
-  uint64_t n = 0;
-  if ((rs = ensure_scratch(ctx, 256, st)) == MAD_OK &&
-      (rs = export_x(ctx, keys, vals, cap, &n, (unsigned long long*)ctx->scratch, st)) == MAD_OK &&
+  if ((rs = export_x_enqueue(ctx, keys, vals, cap, count, st)) == MAD_OK &&
       (rs = clear_x_slots(ctx, st)) == MAD_OK) {
     cudaMemsetAsync(&ctx->sc->new_keys, 0, sizeof(unsigned long long), st);
-    rs = accumulate_pairs(ctx, keys, vals, n < cap ? n : cap, st);
-    ctx->x_built = false;
+    rs = accumulate_pairs(ctx, keys, vals, cap, st, count);
   }
   cudaFreeAsync(tmp, st);
   return rs;
@@ -598,13 +604,14 @@ mad_status mad_sample(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first_di
   // The whole budget into an empty X leaves no diamond to add later: the home
   // regions are built whole, as in the fused pass (1e7 diamonds on 200000 x 100
   // factors: insert phase 359 -> 212 us, the search 1471 -> 1328 us).  Not while a stream is captured
-  // (a replay would change X's layout unseen), nor with a test's layout.
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+  // (a replay would change X's layout unseen) or once one was (its replays add
+  // to a plain table), nor with a test's layout.
+  const bool captured = capturing((cudaStream_t)stream);
+  ctx->x_captured |= captured;
   const bool fresh = s == ctx->s_max && ctx->sampled == 0 && ctx->x_empty &&
                      ctx->region_factor == 1.5f && ctx->hov_request == 0 &&
                      !(ctx->flags & (MAD_WEDGE | MAD_ALIAS)) && x_builder_applies(ctx, s) &&
-                     cudaStreamIsCapturing((cudaStream_t)stream, &cap) == cudaSuccess &&
-                     cap == cudaStreamCaptureStatusNone;
+                     !ctx->x_captured;
   const mad_status rs = sample_impl(ctx, s, seed, first_diamond, (cudaStream_t)stream, fresh);
   if (s > 0) ctx->x_empty = false;
   if (rs == MAD_OK) {
@@ -778,9 +785,12 @@ mad_status mad_accumulate(mad_ctx* ctx, const uint64_t* keys_dev, const int64_t*
   if (!ctx || (n && (!keys_dev || !vals_dev))) return MAD_ERR_ARG;
   if (!ctx->built) return MAD_ERR_STATE;
   if (n == 0) return MAD_OK;
+  const bool captured = capturing((cudaStream_t)stream);
+  ctx->x_captured |= captured;
   if (ctx->x_built) {
     const mad_status rs = x_to_table(ctx, (cudaStream_t)stream);
     if (rs != MAD_OK) return rs;
+    if (!captured) ctx->x_built = false;   // (captured: the layout changes with the replay)
   }
   ctx->x_empty = false;
   return accumulate_pairs(ctx, keys_dev, vals_dev, n, (cudaStream_t)stream);

@@ -565,8 +565,10 @@ k_insert(const SampleParams p_, const unsigned long long* __restrict__ keys,
 // Counts the keys it creates, not diamonds.
 __global__ void __launch_bounds__(256)
 k_accumulate(const SampleParams p_, const unsigned long long* __restrict__ keys,
-             const long long* __restrict__ vals, unsigned long long n) {
+             const long long* __restrict__ vals, unsigned long long n_max,
+             const unsigned long long* n_dev) {
   const SampleParams p = resolve(p_);
+  const unsigned long long n = dev_len(n_max, n_dev);
   Tally t;
   for (unsigned long long q = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (unsigned long long)gridDim.x * blockDim.x) {
@@ -1213,11 +1215,11 @@ mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first, 
 }
 
 mad_status accumulate_pairs(mad_ctx* ctx, const uint64_t* keys, const int64_t* vals, uint64_t n,
-                            cudaStream_t st) {
+                            cudaStream_t st, const unsigned long long* n_dev) {
   if (n == 0) return MAD_OK;
   const SampleParams p = make_params(ctx);
   k_accumulate<<<grid_of(n, full_grid<k_accumulate>()), 256, 0, st>>>(
-      p, (const unsigned long long*)keys, (const long long*)vals, n);
+      p, (const unsigned long long*)keys, (const long long*)vals, n, n_dev);
   count_launch(ctx);
   return cuda_status(cudaGetLastError());
 }

@@ -444,3 +444,41 @@ def test_steps_in_one_call_equal_steps_in_two(m, d, n, s):
         keys, vals, cnt = _export_sorted(mad, c.ctx, s + 1)
         assert cnt == len(ok) and np.array_equal(keys, ok) and np.array_equal(vals, 2 * ov)
         assert mad.mad_stats(c.ctx)["distinct"] == len(ok)
+
+
+def test_captured_accumulate_onto_a_whole_budget():
+    """Pairs added by a captured call to an X filled by one mad_sample: each
+    replay adds them once, also after later eager calls and a refilled X."""
+    import paper_1506_03872_gb300 as mad
+    m, d, n, s = 2051, 60, 3001, 100_000
+    A, B = _inputs(92, m, d, n)
+    tA, tB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    (ok, ov), _ = _oracle_x(A, B, 0, s, 17)
+    k = torch.from_numpy(ok.view(np.int64).copy()).cuda()
+    v = torch.from_numpy(ov.copy()).cuda()
+    with mad.Context() as c:
+        c.build(mad.dense(tA), mad.dense(tB), s, keep=(tA, tB))
+
+        def check(times):
+            keys, vals, cnt = _export_sorted(mad, c.ctx, 2 * s)
+            assert cnt == len(ok)
+            assert np.array_equal(keys, ok) and np.array_equal(vals, times * ov)
+
+        mad.mad_sample(c.ctx, s, 17)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            mad.mad_accumulate(c.ctx, k, v)
+        check(1)
+        for r in range(2):
+            g.replay()
+            check(r + 2)
+        mad.mad_accumulate(c.ctx, k, v)
+        check(4)
+        mad.mad_reset_hash(c.ctx)
+        mad.mad_sample(c.ctx, s, 17)
+        check(1)
+        g.replay()
+        check(2)
+        mad.mad_accumulate(c.ctx, k, v)
+        check(3)
