@@ -325,7 +325,7 @@ mad_status mad_sparse_topt(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* 
  * equals mad_build_tables + mad_sample + mad_topk + mad_rescore on that
  * query alone with the same s_max.
  *
- * mad_mips_items: item-side tables (TB with per-row guides, row norms, the
+ * mad_mips_items: item-side tables (TB and its 64-byte blocks or row guides, row norms, the
  * items transposed for rescoring) for dense B (d x n, F32, n < 2^31).  B
  * must stay alive and unchanged while the context uses it.  s_max bounds
  * every query budget (it fixes the fixed-point scale F).  Synchronises.
