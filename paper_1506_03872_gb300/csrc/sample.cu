@@ -240,20 +240,22 @@ k_sample_rows(const SampleParams p_, unsigned long long seed, unsigned long long
 //
 // Two levels: the top kCoarseBits of the bucket across the grid, then the rest
 // inside each coarse bucket.
-//  1. k_sort_hist: a block counts its contiguous chunk of the diamonds per coarse
-//     bucket; the counts, bucket by bucket and block by block, are scanned.
-//  2. k_sort_scatter: the same chunk again, a tile of 8192 diamonds at a time: a
-//     tile is ordered by coarse bucket in shared memory, so that its records
+//  1. k_sort_scatter: a block takes a contiguous chunk of the diamonds, a tile of
+//     8192 at a time: a tile is ordered by coarse bucket in shared memory, takes
+//     its places in the buckets' slots with one atomic per bucket, and its records
 //     (diamond index and the bucket's low bits, one word) leave in runs of about
-//     eight, whole sectors.
-//  3. k_sort_fine: a block per coarse bucket (equal slices of a uniform target:
-//     equal counts) orders its records by the low bits in shared memory and
-//     writes indices and bucket offsets in order.
-// Bound by Philox in the first two (35 us a pass over 1e7 diamonds).  One level
+//     eight, whole sectors.  The target is uniform, so a coarse bucket gets
+//     s * width / total diamonds give or take: it has slots for that and three
+//     standard deviations, and what is more goes to a list of its own (some ten of
+//     1e7 diamonds).  No pass counts the diamonds first.
+//  2. k_sort_fine: a block per coarse bucket orders its records by the low bits in
+//     shared memory and writes indices and bucket offsets in order.
+// Bound by Philox and the scatter's shared-memory steps.  One level
 // over all 2^16 buckets kept a count per (bucket, block), as many as there were
 // diamonds, through four passes (40 MB: 67 us of sums and offsets), and wrote
-// each index to a sector of its own (94 us): 206 us with the histogram, now 123
-// (cold caches, one by one; the fused pass 965 -> 930 us).
+// each index to a sector of its own (94 us): 206 us with the histogram; two levels
+// with a counting pass (34 us) and a scan of its counts 123; without them 89 (cold
+// caches, one by one; the fused pass 965 -> 930 -> 904 with other changes -> 874 us).
 constexpr int kSortBitsMax = 16;
 constexpr int kCoarseBits = 10;
 constexpr int kSortThreads = 1024;
@@ -270,25 +272,14 @@ __device__ __forceinline__ uint32_t sort_bucket(unsigned long long ell, uint2 ke
   return (uint32_t)(draw_target(u0, t1_total) >> shift);
 }
 
-// Step 1: H[c * gridDim.x + g] = diamonds of block g's chunk in coarse bucket c.
-__global__ void __launch_bounds__(kSortThreads, 2)
-k_sort_hist(const DevScalars* __restrict__ sc, unsigned long long seed, unsigned long long first,
-            unsigned long long s, unsigned long long chunk, int coarse, int fine,
-            unsigned int* __restrict__ H) {
-  __shared__ unsigned int cnt[1 << kCoarseBits];
-  const int nc = 1 << coarse;
-  for (int b = threadIdx.x; b < nc; b += kSortThreads) cnt[b] = 0;
-  __syncthreads();
-  const unsigned long long t1_total = sc->t1_total;
-  const int shift = sc->sort_shift + fine;
-  const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
-  const unsigned long long q0 = (unsigned long long)blockIdx.x * chunk;
-  const unsigned long long q1 = q0 + chunk < s ? q0 + chunk : s;
-  for (unsigned long long q = q0 + threadIdx.x; q < q1; q += kSortThreads)
-    atomicAdd(&cnt[sort_bucket(first + q, key, t1_total, shift)], 1u);
-  __syncthreads();
-  for (int b = threadIdx.x; b < nc; b += kSortThreads)
-    H[(size_t)b * gridDim.x + blockIdx.x] = cnt[b];
+// Slots of a coarse bucket (see above): the same in every block of both kernels.
+// shift: of a coarse bucket; slots_max bounds them all together.
+__device__ __forceinline__ uint32_t coarse_slots(unsigned long long s, unsigned long long total,
+                                                 int shift, unsigned long long slots_max) {
+  const double mean = (double)s * ldexp(1.0, shift) / (double)total;
+  const unsigned long long used = ((total - 1) >> shift) + 1, most = slots_max / used;
+  const unsigned long long want = (unsigned long long)(fmin(mean, 4e9) + 3.0 * sqrt(mean)) + 1;
+  return (uint32_t)(want < most ? want : most);
 }
 
 // Exclusive scan of one value per thread over a 1024-thread block.
@@ -317,29 +308,39 @@ __device__ __forceinline__ uint32_t block_exclusive_1024(uint32_t v, uint32_t* w
 }
 
 struct SortTile {
-  uint32_t cur[1 << kCoarseBits];    // next place of each coarse bucket
+  uint32_t cur[1 << kCoarseBits];    // the tile's first place in each coarse bucket
   uint32_t cnt[1 << kCoarseBits];    // this tile's counts
   uint32_t off[1 << kCoarseBits];    // their exclusive scan
   uint32_t rec[kSortTile];
   uint16_t bkt[kSortTile];
   uint32_t warp_sum[32];
+  uint32_t slots;
 };
 
-// Step 2: rec[place] = low bucket bits << kIdxBits | q for every diamond q of
-// the block's chunk, in coarse bucket order (off: the scanned counts).
+// Places given out in each coarse bucket, and the length of the list of those
+// beyond its slots.
+struct SortTaken {
+  unsigned int n[1 << kCoarseBits], over;
+};
+
+// Step 1: rec[c * slots + place] = low bucket bits << kIdxBits | q for every
+// diamond q of the block's chunk, c its coarse bucket; places from slots on go to
+// over instead, with c.  taken: the places given out, zero at first.
 __global__ void __launch_bounds__(kSortThreads, 2)
 k_sort_scatter(const DevScalars* __restrict__ sc, unsigned long long seed,
                unsigned long long first, unsigned long long s, unsigned long long chunk,
-               int coarse, int fine, const unsigned int* __restrict__ off,
-               uint32_t* __restrict__ rec) {
+               int coarse, int fine, unsigned long long slots_max, SortTaken* taken,
+               uint32_t* __restrict__ rec, uint2* __restrict__ over) {
   extern __shared__ __align__(16) unsigned char sort_smem[];
   SortTile& sh = *reinterpret_cast<SortTile*>(sort_smem);
   const int tid = threadIdx.x, nc = 1 << coarse;
   static_assert((1 << kCoarseBits) == kSortThreads, "a coarse bucket per thread");
-  sh.cur[tid] = tid < nc ? off[(size_t)tid * gridDim.x + blockIdx.x] : 0u;
+  if (tid == 0) sh.slots = coarse_slots(s, sc->t1_total, sc->sort_shift + fine, slots_max);
   const unsigned long long t1_total = sc->t1_total;
   const int shift = sc->sort_shift;
   const uint32_t fmask = (1u << fine) - 1u;
+  __syncthreads();
+  const uint32_t slots = sh.slots;
   const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
   const unsigned long long q0 = (unsigned long long)blockIdx.x * chunk;
   const unsigned long long q1 = q0 + chunk < s ? q0 + chunk : s;
@@ -360,6 +361,7 @@ k_sort_scatter(const DevScalars* __restrict__ sc, unsigned long long seed,
     }
     __syncthreads();
     const uint32_t mine = sh.cnt[tid];
+    sh.cur[tid] = tid < nc && mine ? atomicAdd(&taken->n[tid], mine) : 0u;
     sh.off[tid] = block_exclusive_1024(mine, sh.warp_sum);
     __syncthreads();
 #pragma unroll
@@ -376,38 +378,54 @@ k_sort_scatter(const DevScalars* __restrict__ sc, unsigned long long seed,
     for (int u = 0; u < kTilePer; ++u) {
       const uint32_t x = tid + u * kSortThreads;
       if (x < n) {
-        const uint32_t c = sh.bkt[x];
-        rec[sh.cur[c] + x - sh.off[c]] = sh.rec[x];
+        const uint32_t c = sh.bkt[x], at = sh.cur[c] + x - sh.off[c];
+        if (at < slots) rec[(size_t)c * slots + at] = sh.rec[x];
+        else over[atomicAdd(&taken->over, 1u)] = make_uint2(c, sh.rec[x]);
       }
     }
     __syncthreads();
-    sh.cur[tid] += mine;
   }
 }
 
-// Step 3, coarse bucket blockIdx.x: its records by their low bits into order
+// Step 2, coarse bucket blockIdx.x: its records by their low bits into order
 // (indices alone) and the first place of each of its buckets into base
 // (base[nbk] = s).  Longer than kFineStage, it is written in place order
-// straight to memory.  With no low bits the records are the order already.
+// straight to memory.
 __global__ void __launch_bounds__(kSortThreads, 2)
-k_sort_fine(const uint32_t* __restrict__ rec, const unsigned int* __restrict__ off, int blocks,
-            int fine, unsigned int s, uint32_t* __restrict__ order,
+k_sort_fine(const DevScalars* __restrict__ sc, const uint32_t* __restrict__ rec,
+            const uint2* __restrict__ over, const SortTaken* __restrict__ taken, int fine,
+            unsigned long long s, unsigned long long slots_max, uint32_t* __restrict__ order,
             unsigned int* __restrict__ base) {
   extern __shared__ uint32_t stage[];
   __shared__ uint32_t cur[1 << (kSortBitsMax - kCoarseBits)];
+  __shared__ uint32_t warp_sum[32], s_slots, s_p0;
   const uint32_t c = blockIdx.x, nf = 1u << fine;
-  const uint32_t p0 = off[(size_t)c * blocks], p1 = off[(size_t)(c + 1) * blocks];
-  const uint32_t tid = threadIdx.x;
-  if (c + 1 == gridDim.x && tid == 0) base[(size_t)gridDim.x << fine] = s;
-  if (fine == 0) {
-    if (tid == 0) base[c] = p0;
-    return;
-  }
-  const uint32_t n = p1 - p0;
+  const uint32_t tid = threadIdx.x, lane = tid & 31;
+  if (c + 1 == gridDim.x && tid == 0) base[(size_t)gridDim.x << fine] = (unsigned int)s;
+  // The places before it: those of the coarse buckets before it.
+  uint32_t before = tid < c ? taken->n[tid] : 0u;
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
+  if (lane == 0) warp_sum[tid >> 5] = before;
   if (tid < nf) cur[tid] = 0;
+  if (tid == 0) s_slots = coarse_slots(s, sc->t1_total, sc->sort_shift + fine, slots_max);
   __syncthreads();
-  for (uint32_t x = tid; x < n; x += kSortThreads) atomicAdd(&cur[rec[p0 + x] >> kIdxBits], 1u);
+  if (tid < 32) {
+    uint32_t v = warp_sum[tid];
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    if (tid == 0) s_p0 = v;
+  }
+  const uint32_t n = taken->n[c], held = min(n, s_slots);
+  const uint32_t listed = n > held ? taken->over : 0u;
+  const uint32_t* __restrict__ mine = rec + (size_t)c * s_slots;
+  for (uint32_t x = tid; x < held; x += kSortThreads) atomicAdd(&cur[mine[x] >> kIdxBits], 1u);
+  for (uint32_t x = tid; x < listed; x += kSortThreads) {
+    const uint2 e = over[x];
+    if (e.x == c) atomicAdd(&cur[e.y >> kIdxBits], 1u);
+  }
   __syncthreads();
+  const uint32_t p0 = s_p0;
   if (tid < 32) {   // nf <= 64 counts: two per lane
     const uint32_t a = 2 * tid < nf ? cur[2 * tid] : 0u;
     const uint32_t d = 2 * tid + 1 < nf ? cur[2 * tid + 1] : 0u;
@@ -428,19 +446,18 @@ k_sort_fine(const uint32_t* __restrict__ rec, const unsigned int* __restrict__ o
     }
   }
   __syncthreads();
-  if (n <= kFineStage) {
-    for (uint32_t x = tid; x < n; x += kSortThreads) {
-      const uint32_t r = rec[p0 + x];
-      stage[atomicAdd(&cur[r >> kIdxBits], 1u)] = r & kIdxMask;
-    }
-    __syncthreads();
-    for (uint32_t x = tid; x < n; x += kSortThreads) order[p0 + x] = stage[x];
-  } else {
-    for (uint32_t x = tid; x < n; x += kSortThreads) {
-      const uint32_t r = rec[p0 + x];
-      order[p0 + atomicAdd(&cur[r >> kIdxBits], 1u)] = r & kIdxMask;
-    }
+  uint32_t* __restrict__ out = n <= kFineStage ? stage : order + p0;
+  for (uint32_t x = tid; x < held; x += kSortThreads) {
+    const uint32_t r = mine[x];
+    out[atomicAdd(&cur[r >> kIdxBits], 1u)] = r & kIdxMask;
   }
+  for (uint32_t x = tid; x < listed; x += kSortThreads) {
+    const uint2 e = over[x];
+    if (e.x == c) out[atomicAdd(&cur[e.y >> kIdxBits], 1u)] = e.y & kIdxMask;
+  }
+  if (n > kFineStage) return;
+  __syncthreads();
+  for (uint32_t x = tid; x < n; x += kSortThreads) order[p0 + x] = stage[x];
 }
 
 // Diamonds in row order (dense inputs): order[q] = l - first.  Draws only:
@@ -1032,15 +1049,21 @@ int sort_blocks() {
   return blocks;
 }
 
-// Scratch of the sort and the draws for one batch: the per-(coarse bucket,
-// block) counts and offsets, the bucket offsets, the scan's partials, the
-// records in coarse order, the diamond indices in bucket order, and each
-// diamond's key and increment.
+// Slots of the coarse buckets together (coarse_slots): the diamonds, one more
+// bucket of at most 2 s / nc, and three deviations for each.
+uint64_t sort_slots(uint64_t nbk, uint64_t batch) {
+  const uint64_t nc = std::min<uint64_t>(nbk, 1ull << kCoarseBits);
+  const double most = 2.0 * (double)batch / (double)nc;
+  return batch + (uint64_t)most + nc * ((uint64_t)(3.0 * std::sqrt(most)) + 2);
+}
+
+// Scratch of the sort and the draws for one batch: the coarse buckets' counts,
+// the bucket offsets, the records in coarse order, the diamond indices in bucket
+// order, and each diamond's key and increment (the sort's list of records beyond
+// their slots uses the keys' memory before them).
 struct SortScratch {
-  unsigned int* H;
-  unsigned int* off;
+  SortTaken* taken;
   unsigned int* base;
-  unsigned int* part;
   uint32_t* rec;
   uint32_t* order;
   unsigned long long* keys;
@@ -1052,7 +1075,7 @@ struct SortScratch {
 };
 
 // recs: records per diamond (2 under MAD_SQUARE_SYM).
-SortScratch carve_sort(void* p, uint64_t nbk, int blocks, uint64_t batch, int recs) {
+SortScratch carve_sort(void* p, uint64_t nbk, uint64_t batch, int recs) {
   SortScratch c;
   char* b = (char*)p;
   size_t off = 0;
@@ -1061,13 +1084,9 @@ SortScratch carve_sort(void* p, uint64_t nbk, int blocks, uint64_t batch, int re
     off += (bytes + 255) & ~(size_t)255;
     return (void*)q;
   };
-  const uint64_t counts = std::min<uint64_t>(nbk, 1ull << kCoarseBits) * (uint64_t)blocks;
-  c.H = (unsigned int*)take(counts * sizeof(unsigned int));
-  c.off = (unsigned int*)take((counts + 1) * sizeof(unsigned int));
+  c.taken = (SortTaken*)take(sizeof(SortTaken));
   c.base = (unsigned int*)take((nbk + 1) * sizeof(unsigned int));
-  c.part = (unsigned int*)take(scan_partial_elems(counts) * sizeof(unsigned int));
-  // (records are the order itself when there is no second level)
-  c.rec = (uint32_t*)take(nbk > (1ull << kCoarseBits) ? batch * sizeof(uint32_t) : 0);
+  c.rec = (uint32_t*)take(sort_slots(nbk, batch) * sizeof(uint32_t));
   c.order = (uint32_t*)take(batch * sizeof(uint32_t));
   c.keys = (unsigned long long*)take(batch * recs * sizeof(unsigned long long));
   c.vals = (long long*)take(batch * recs * sizeof(long long));
@@ -1083,7 +1102,7 @@ int sort_records(const mad_ctx* ctx) { return (ctx->flags & MAD_SQUARE_SYM) ? 2 
 size_t sample_scratch_bytes(const mad_ctx* ctx, uint64_t s) {
   if (!ctx->dense || s == 0) return 0;
   const uint64_t batch = s < kSortBatch ? s : kSortBatch;
-  return carve_sort(nullptr, sort_buckets(ctx->m), sort_blocks(), batch, sort_records(ctx)).bytes;
+  return carve_sort(nullptr, sort_buckets(ctx->m), batch, sort_records(ctx)).bytes;
 }
 
 // Buckets per group of the X builder: about 640 diamonds of s_max per group
@@ -1165,21 +1184,19 @@ mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first, 
   }
   mad_status rs = ensure_scratch(ctx, sample_scratch_bytes(ctx, s), st);
   if (rs != MAD_OK) return rs;
-  const SortScratch w = carve_sort(ctx->scratch, nbk, blocks, batch, sort_records(ctx));
+  const SortScratch w = carve_sort(ctx->scratch, nbk, batch, sort_records(ctx));
   for (uint64_t done = 0; done < s; done += batch) {
     const uint64_t n = (s - done) < batch ? (s - done) : batch;
     phase_event(ctx, 0, st);
     const unsigned long long chunk = (n + blocks - 1) / blocks;
-    uint32_t* rec = fine ? w.rec : w.order;
-    const uint64_t counts = (uint64_t)blocks << coarse;
-    k_sort_hist<<<blocks, kSortThreads, 0, st>>>(ctx->sc, seed, first + done, n, chunk, coarse,
-                                                 fine, w.H);
-    if ((rs = scan_exclusive_u32(ctx, w.H, w.off, counts, w.part, st)) != MAD_OK) return rs;
+    const uint64_t slots = sort_slots(nbk, batch);
+    cudaMemsetAsync(w.taken, 0, sizeof(SortTaken), st);
     k_sort_scatter<<<blocks, kSortThreads, sizeof(SortTile), st>>>(
-        ctx->sc, seed, first + done, n, chunk, coarse, fine, w.off, rec);
-    k_sort_fine<<<1u << coarse, kSortThreads, fine ? kFineStage * sizeof(uint32_t) : 0, st>>>(
-        w.rec, w.off, blocks, fine, (unsigned)n, w.order, w.base);
-    count_launch(ctx, 3);
+        ctx->sc, seed, first + done, n, chunk, coarse, fine, slots, w.taken, w.rec,
+        (uint2*)w.keys);
+    k_sort_fine<<<1u << coarse, kSortThreads, kFineStage * sizeof(uint32_t), st>>>(
+        ctx->sc, w.rec, (const uint2*)w.keys, w.taken, fine, n, slots, w.order, w.base);
+    count_launch(ctx, 2);
     phase_event(ctx, 1, st);
     if (ctx->B.dt == MAD_F64)
       k_sample_sorted<double><<<grid_of(n, full_grid<k_sample_sorted<double>>()), 256, 0, st>>>(
