@@ -37,6 +37,7 @@
 #include "draw.cuh"
 #include "mad_device.cuh"
 #include "mad_internal.cuh"
+#include "mips_shape.h"
 
 namespace mad {
 
@@ -50,12 +51,10 @@ struct MipsQuery {
 
 namespace {
 
-constexpr int kDrawThreads = 256;
 constexpr int kPartThreads = 512;
 constexpr int kGroup = kPartThreads;         // chunks of a part scanned together
 constexpr int kAhead = 4;                    // records of a thread in flight
 constexpr int kSlots = 8192;                 // largest table of a part (96 KB: two blocks per SM)
-constexpr uint32_t kMaxParts = 2048;         // (a part too full for its table splits itself)
 constexpr int kTPrimeMax = 1024;             // largest t' of a batch
 constexpr int kSlack = 32;                   // columns a part may keep beyond t'
 constexpr int kBins = 2048;                  // digits of the threshold search (11 bits)
@@ -796,10 +795,6 @@ size_t parts_smem_bytes(int slots, uint32_t cap) {
   return (size_t)slots * 12 + (size_t)cap * sizeof(Kept);
 }
 
-size_t draw_smem_bytes(int chunk, uint32_t parts, int64_t d) {
-  return (size_t)chunk * (8 + 4 + 2) + ((size_t)parts + 1 + 4 * (size_t)d) * 4;
-}
-
 // The batch's device buffer: the queries, the query of every chunk and part,
 // the part offsets of every chunk, the records and the parts' kept columns.
 struct MipsBufs {
@@ -846,7 +841,7 @@ mad_status mad_mips_items(mad_ctx* ctx, const mad_matrix* B, uint64_t s_max, mad
   if (B->fmt != MAD_DENSE_ROWMAJOR || B->dt != MAD_F32 || !B->values || B->rows <= 0 ||
       B->cols <= 0 || B->ld < B->cols)
     return MAD_ERR_ARG;
-  if (B->cols >= (1ll << 31) || B->rows > 1024) return MAD_ERR_UNSUPPORTED;
+  if (B->cols >= (1ll << 31) || B->rows > kItemDimMax) return MAD_ERR_UNSUPPORTED;
   if (ctx->flags) return MAD_ERR_UNSUPPORTED;   // plain |q . b_j|, no Gram or sign flags
   cudaStream_t st = (cudaStream_t)stream;
   cudaStreamSynchronize(st);
@@ -1002,8 +997,16 @@ mad_status mad_mips_plan(mad_ctx* ctx, uint32_t nq, const uint64_t* s_host, uint
   ctx->mips_slots = slots;
   ctx->mips_parts_smem = parts_smem_bytes(slots, max_cap);
   ctx->mips_plan_mult = ctx->mips_chunk_mult;
-  return cuda_status(cudaFuncSetAttribute(k_mips_parts, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)parts_smem_bytes(kSlots, kTPrimeMax + kSlack)));
+  cudaError_t e = cudaFuncSetAttribute(k_mips_draw<true>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDrawSmemMax);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_mips_draw<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kDrawSmemMax);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_mips_parts, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)parts_smem_bytes(kSlots, kTPrimeMax + kSlack));
+  if (e != cudaSuccess) ctx->mips_nq = 0;   // no plan: a run is refused
+  return cuda_status(e);
 }
 
 mad_status mad_mips_run(mad_ctx* ctx, const mad_matrix* Q, uint64_t seed, mad_pair* out_dev,
@@ -1039,9 +1042,12 @@ mad_status mad_mips_run(mad_ctx* ctx, const mad_matrix* Q, uint64_t seed, mad_pa
     k_mips_draw<false><<<(unsigned)grid, kDrawThreads, draw_smem, st>>>(
         p, seed, b.queries, b.chunk_q, ctx->mips_chunks, ctx->mips_plan_mult, ctx->mips_max_parts,
         b.rec, b.off);
+  // The next two kernels read addresses out of what this one writes.
+  if ((rs = cuda_status(cudaGetLastError())) != MAD_OK) return rs;
   k_mips_parts<<<(unsigned)ctx->mips_units, kPartThreads, ctx->mips_parts_smem, st>>>(
       b.queries, b.unit_q, b.rec, b.off, chunk, ctx->mips_slots, ctx->region_factor, ctx->f, ctx->mips_tprime, b.kept,
       b.kept_n, ctx->sc);
+  if ((rs = cuda_status(cudaGetLastError())) != MAD_OK) return rs;
   k_mips_final<<<ctx->mips_nq, ctx->mips_select_threads, 0, st>>>(
       b.queries, b.kept, b.kept_n, (const float*)Q->values, Q->ld, (const float*)ctx->bt, ctx->d,
       ctx->mips_tprime, ctx->mips_t, out_dev, n_out_dev, cand_dev);

@@ -111,3 +111,28 @@ def test_row_guides_draw_what_the_blocks_draw(d, n):
     B[0, ::3] = 0.0
     _compare(Q, B, s_q, 30_000, 40, 7)
     _compare(Q, B, s_q, 30_000, 40, 7, guides=True)
+
+
+def test_many_parts_of_long_items():
+    """More than 1,015 parts at d = 1024: a draw block asks for more than the
+    48 KB a kernel gets unasked.  The launch shape changes no result, so the
+    same batch in 127 parts a query is the reference."""
+    import paper_1506_03872_gb300 as mad
+    d, n, nq, tprime, t = 1024, 630_000, 2, 50, 5
+    g = torch.Generator(device="cuda").manual_seed(3)
+    B = torch.randn((d, n), generator=g, device="cuda")
+    Q = torch.randn((nq, d), generator=g, device="cuda")
+    got = []
+    with mad.Context() as c:
+        mad.mad_mips_items(c.ctx, mad.dense(B), 700_000)
+        for cfg in (dict(), dict(region_lg=4)):
+            out, cand = mad.new_pairs(nq * t), mad.new_pairs(nq * tprime)
+            nout = torch.zeros(nq, dtype=torch.int32, device="cuda")
+            mad.mad_mips_config(c.ctx, **cfg)
+            mad.mad_mips_plan(c.ctx, np.array([650_000, 300], np.uint64), tprime, t)
+            mad.mad_mips_run(c.ctx, mad.dense(Q), 5, out, nout, cand)
+            assert mad.mad_stats(c.ctx)["device_error"] == 0
+            got.append((nout, out, cand))
+    assert got[0][0].tolist() == [t, t]
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
