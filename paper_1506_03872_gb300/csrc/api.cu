@@ -673,13 +673,16 @@ mad_status mad_rescore(mad_ctx* ctx, const mad_pair* cand_dev, uint32_t ncand, u
   double* cvals = (double*)((char*)ctx->scratch + cv_off);
   uint64_t nsel = 0;
   if (rescore_bounded_applies(ctx, ncand, t)) {
+    // Candidates outside the matrices are reported and left out of the list, so
+    // fewer than t of it may be written: its device length bounds the reads.
     const unsigned long long* kept = rescore_bounded(ctx, cand_dev, ncand, t, ws.l0, cvals, st);
     if ((rs = select_list_dev(ctx, ws, ncand, kept, t, 64, &nsel, st)) != MAD_OK) return rs;
+    items_to_pairs_dev(ctx, ws.out, nsel, kept, cand_dev, cvals, out_dev, nullptr, st);
   } else {
     if ((rs = rescore_items(ctx, cand_dev, ncand, ws.l0, cvals, st)) != MAD_OK) return rs;
     if ((rs = select_list(ctx, ws, ncand, t, 64, &nsel, st)) != MAD_OK) return rs;
+    if ((rs = items_to_pairs(ctx, ws.out, nsel, cand_dev, cvals, out_dev, st)) != MAD_OK) return rs;
   }
-  if ((rs = items_to_pairs(ctx, ws.out, nsel, cand_dev, cvals, out_dev, st)) != MAD_OK) return rs;
   DevScalars hs;
   if ((rs = read_scalars(ctx, &hs, st)) != MAD_OK) return rs;
   if ((rs = device_error_status(hs.err)) != MAD_OK) return rs;

@@ -401,9 +401,9 @@ SelectWs select_ws_carve(void* base, uint64_t n, uint64_t K);
 // Asynchronous.
 mad_status select_list(mad_ctx* ctx, const SelectWs& ws, uint64_t n, uint64_t K, int pbits,
                        uint64_t* n_sel, cudaStream_t st, int bi = 32, int bj = 32);
-// The same for a list of device length *n_dev <= n_max whose K largest are
-// known to be there (*n_sel = min(K, n_max)); waits for the length where the
-// list may be too long for a selection on the device.
+// The same for a list of device length *n_dev <= n_max: ws.out holds min(K,
+// *n_dev) items, of which *n_sel is an upper bound (readers go by *n_dev); waits
+// for the length where the list may be too long for a selection on the device.
 mad_status select_list_dev(mad_ctx* ctx, const SelectWs& ws, uint64_t n_max,
                            const unsigned long long* n_dev, uint64_t K, int pbits,
                            uint64_t* n_sel, cudaStream_t st);
@@ -454,8 +454,8 @@ void select_hash_dev(mad_ctx* ctx, uint64_t K, const unsigned long long* hcap_de
 void select_hash_dev_long(mad_ctx* ctx, uint64_t K, const unsigned long long* hcap_dev,
                           void* state, unsigned long long* count, Item* list, uint64_t list_cap,
                           Item* topk, Item* sorted, uint32_t* pos, Item* out, cudaStream_t st);
-// out[q] for q < min(cap, *n_dev) as in items_to_pairs; *n_out gets that
-// length.
+// out[q] for q < min(cap, *n_dev) as in items_to_pairs; *n_out (when given) gets
+// that length.
 void items_to_pairs_dev(mad_ctx* ctx, const Item* items, uint64_t cap,
                         const unsigned long long* n_dev, const mad_pair* cand,
                         const double* cvals, mad_pair* out, uint32_t* n_out, cudaStream_t st);

@@ -136,8 +136,7 @@ mad_status enqueue_pass(mad_ctx* ctx, uint64_t seed, mad_pair* out_dev, uint32_t
     return rs;
   block_select_dev(ctx, b.rs_items, ctx->pipe_tprime, ctx->pipe_t, scored, true, b.rs_sorted,
                    b.rs_pos, b.rs_out, (unsigned int*)(b.count + 3), nullptr, st);
-  items_to_pairs_dev(ctx, b.rs_out, ctx->pipe_t, b.count, cand, b.cvals, out_dev, counts_dev + 1,
-                     st);
+  items_to_pairs_dev(ctx, b.rs_out, ctx->pipe_t, scored, cand, b.cvals, out_dev, counts_dev + 1, st);
   return cuda_status(cudaGetLastError());
 }
 

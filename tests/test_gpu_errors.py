@@ -150,3 +150,28 @@ def test_injected_allocation_failure_returns_oom(monkeypatch, nth):
         mad.mad_sample(c.ctx, 50_000, 3)
         _, n = mad.mad_topk(c.ctx, 100)
         assert n == 100
+
+
+@pytest.mark.parametrize("inside", [0, 3, 99])
+@pytest.mark.parametrize("ncand,t", [(4096, 100), (20_000, 2048), (140_000, 2048), (140_000, 5000)])
+def test_candidates_outside_the_matrices_are_reported(ncand, t, inside):
+    """Fewer than t candidates inside the matrices (rows and columns swapped,
+    say): an error status, nothing read past what was selected, and a correct
+    call once the tables are built again."""
+    import paper_1506_03872_gb300 as mad
+    m, n = 500, 900
+    A, B = _dense_inputs(m, 10, n)
+    i = np.full(ncand, m) + np.arange(ncand) % 7
+    j = np.arange(ncand) % n
+    i[ncand // 2:ncand // 2 + inside] = 1
+    flat = np.arange(ncand) * 3 % (m * n)
+    good = mad.encode_pairs(flat // n, flat % n, np.arange(1, ncand + 1))
+    with mad.Context() as c:
+        c.build(mad.dense(A), mad.dense(B), 1024, keep=(A, B))
+        want, nw = mad.mad_rescore(c.ctx, good, ncand, t)
+        with pytest.raises(mad.MadError) as e:
+            mad.mad_rescore(c.ctx, mad.encode_pairs(i, j, np.arange(1, ncand + 1)), ncand, t)
+        assert e.value.status == mad.MAD_ERR_STATE
+        c.build(mad.dense(A), mad.dense(B), 1024, keep=(A, B))
+        got, ng = mad.mad_rescore(c.ctx, good, ncand, t)
+        assert ng == nw == t and torch.equal(got, want)
