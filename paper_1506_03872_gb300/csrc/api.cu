@@ -675,7 +675,8 @@ mad_status mad_rescore(mad_ctx* ctx, const mad_pair* cand_dev, uint32_t ncand, u
   if (rescore_bounded_applies(ctx, ncand, t)) {
     // Candidates outside the matrices are reported and left out of the list, so
     // fewer than t of it may be written: its device length bounds the reads.
-    const unsigned long long* kept = rescore_bounded(ctx, cand_dev, ncand, t, ws.l0, cvals, st);
+    const unsigned long long* kept =
+        rescore_bounded(ctx, ctx->bound_state, cand_dev, ncand, t, ws.l0, cvals, st);
     if ((rs = select_list_dev(ctx, ws, ncand, kept, t, 64, &nsel, st)) != MAD_OK) return rs;
     items_to_pairs_dev(ctx, ws.out, nsel, kept, cand_dev, cvals, out_dev, nullptr, st);
   } else {

@@ -262,7 +262,7 @@ struct mad_ctx {
   float region_factor = 1.5f;
   uint64_t hov_request = 0;
   mad::DevScalars* sc = nullptr;
-  void* bound_state = nullptr;      // rescore.cu's bounds (zeros between calls)
+  void* bound_state = nullptr;      // bounds of mad_rescore (rescore_bounded)
   void* pinned = nullptr;           // 4 KB of pinned host memory for read-backs
   // The shape whose tables are allocated (dense tables without the optional
   // ones): a rebuild of the same shape keeps them.
@@ -523,8 +523,11 @@ mad_status rescore_reserve(mad_ctx* ctx, uint64_t ncand, cudaStream_t st);
 // returned (at least min(t, the number of candidates)).
 size_t bound_state_bytes();
 bool rescore_bounded_applies(const mad_ctx* ctx, uint64_t ncand, uint64_t t);
-const unsigned long long* rescore_bounded(mad_ctx* ctx, const mad_pair* cand, uint64_t ncand,
-                                          uint64_t t, Item* items, double* cvals, cudaStream_t st,
+// state: bound_state_bytes() of device memory, zeros between calls (one for each
+// of the calls that may run at the same time: the context's, the pass's own).
+const unsigned long long* rescore_bounded(mad_ctx* ctx, void* state, const mad_pair* cand,
+                                          uint64_t ncand, uint64_t t, Item* items, double* cvals,
+                                          cudaStream_t st,
                                           const unsigned long long* n_dev = nullptr);
 mad_status rescore_items(mad_ctx* ctx, const mad_pair* cand, uint64_t ncand, Item* items,
                          double* cvals, cudaStream_t st, const unsigned long long* n_dev = nullptr);

@@ -31,6 +31,7 @@ namespace {
 struct PipeBufs {
   void* state;                  // selection state of Omega_t'
   unsigned long long* count;    // compacted candidates (device length)
+  void* bound;                  // bounds of the rescore (dense inputs; zeros between runs)
   Item* list;                   // compacted items, list_cap
   Item* topk;                   // the K selected, unsorted (0/1 inputs), t'
   Item* sorted;                 // tile-sorted copy, kDevSelectCap
@@ -59,6 +60,7 @@ PipeBufs carve(void* base, uint64_t tprime, uint64_t t, uint64_t list_cap, bool 
   };
   b.state = take(dev_select_state_bytes());
   b.count = (unsigned long long*)take(4 * sizeof(unsigned long long));
+  b.bound = take(long_sel ? 0 : bound_state_bytes());
   b.list = (Item*)take(list_cap * sizeof(Item));
   b.topk = (Item*)take(long_sel ? tprime * sizeof(Item) : 0);
   b.sorted = (Item*)take(kDevSelectCap * sizeof(Item));
@@ -129,8 +131,8 @@ mad_status enqueue_pass(mad_ctx* ctx, uint64_t seed, mad_pair* out_dev, uint32_t
   // ... the exact c of each candidate, and Omega_t.
   const unsigned long long* scored = b.count;
   if (rescore_bounded_applies(ctx, ctx->pipe_tprime, ctx->pipe_t))
-    scored = rescore_bounded(ctx, cand, ctx->pipe_tprime, ctx->pipe_t, b.rs_items, b.cvals, st,
-                             b.count);
+    scored = rescore_bounded(ctx, b.bound, cand, ctx->pipe_tprime, ctx->pipe_t, b.rs_items, b.cvals,
+                             st, b.count);
   else if ((rs = rescore_items(ctx, cand, ctx->pipe_tprime, b.rs_items, b.cvals, st, b.count)) !=
            MAD_OK)
     return rs;
@@ -163,6 +165,9 @@ mad_status mad_pipeline_plan(mad_ctx* ctx, const mad_matrix* A, const mad_matrix
   ctx->pipe_list_cap = csr ? std::max<uint64_t>(kDevSelectCap, ctx->hcap_alloc) : kDevSelectCap;
   const PipeBufs sizes = carve(nullptr, tprime, t, ctx->pipe_list_cap, csr);
   if ((rs = pool_malloc(ctx, &ctx->pipe_buf, sizes.bytes, st)) != MAD_OK) return rs;
+  if (!csr)
+    cudaMemsetAsync(carve(ctx->pipe_buf, tprime, t, ctx->pipe_list_cap, csr).bound, 0,
+                    bound_state_bytes(), st);
   // The scratch every launch of a run needs, owned by the pass.
   size_t scratch = csr ? csr_build_scratch_bytes(ctx) : dense_build_scratch_bytes(ctx);
   if (sample_scratch_bytes(ctx, s) > scratch) scratch = sample_scratch_bytes(ctx, s);

@@ -678,9 +678,8 @@ void launch_dense(mad_ctx* ctx, const mad_pair* cand, uint64_t ncand, Item* item
 }
 
 template <typename TA, typename TB>
-void launch_bounded(mad_ctx* ctx, const mad_pair* cand, uint64_t ncand, uint64_t t, Item* items,
-                    double* cvals, const unsigned long long* n_dev, cudaStream_t st) {
-  BoundState* bs = (BoundState*)ctx->bound_state;
+void launch_bounded(mad_ctx* ctx, BoundState* bs, const mad_pair* cand, uint64_t ncand, uint64_t t,
+                    Item* items, double* cvals, const unsigned long long* n_dev, cudaStream_t st) {
   const unsigned long long bound_blocks = (ncand * 32 / kBoundAhead + 255) / 256;
   const unsigned long long blocks = (ncand + 255) / 256;
   const unsigned bgrid = (unsigned)(bound_blocks < 152 * 8 ? bound_blocks : 152 * 8);
@@ -725,18 +724,19 @@ size_t bound_state_bytes() { return sizeof(BoundState); }
 // cost more than the FP64 sums they save (two launches of about 5 us against
 // 1.6 ns a candidate at d = 100).
 bool rescore_bounded_applies(const mad_ctx* ctx, uint64_t ncand, uint64_t t) {
-  return ctx->dense && ctx->bound_state && ncand >= 4096 && t <= ncand / 8;
+  return ctx->dense && ncand >= 4096 && t <= ncand / 8;
 }
 
-const unsigned long long* rescore_bounded(mad_ctx* ctx, const mad_pair* cand, uint64_t ncand,
-                                          uint64_t t, Item* items, double* cvals, cudaStream_t st,
-                                          const unsigned long long* n_dev) {
+const unsigned long long* rescore_bounded(mad_ctx* ctx, void* state, const mad_pair* cand,
+                                          uint64_t ncand, uint64_t t, Item* items, double* cvals,
+                                          cudaStream_t st, const unsigned long long* n_dev) {
+  BoundState* bs = (BoundState*)state;
   const bool a64 = ctx->A.dt == MAD_F64, b64 = ctx->B.dt == MAD_F64;
-  if (a64 && b64) launch_bounded<double, double>(ctx, cand, ncand, t, items, cvals, n_dev, st);
-  else if (a64) launch_bounded<double, float>(ctx, cand, ncand, t, items, cvals, n_dev, st);
-  else if (b64) launch_bounded<float, double>(ctx, cand, ncand, t, items, cvals, n_dev, st);
-  else launch_bounded<float, float>(ctx, cand, ncand, t, items, cvals, n_dev, st);
-  return &((BoundState*)ctx->bound_state)->kept;
+  if (a64 && b64) launch_bounded<double, double>(ctx, bs, cand, ncand, t, items, cvals, n_dev, st);
+  else if (a64) launch_bounded<double, float>(ctx, bs, cand, ncand, t, items, cvals, n_dev, st);
+  else if (b64) launch_bounded<float, double>(ctx, bs, cand, ncand, t, items, cvals, n_dev, st);
+  else launch_bounded<float, float>(ctx, bs, cand, ncand, t, items, cvals, n_dev, st);
+  return &bs->kept;
 }
 
 mad_status rescore_items(mad_ctx* ctx, const mad_pair* cand, uint64_t ncand, Item* items,

@@ -502,3 +502,37 @@ def test_row_order_with_coarse_buckets_beyond_their_slots(m, s):
             keys, vals, cnt = _export_sorted(mad, c.ctx, s + 1)
             assert cnt == len(ok) and np.array_equal(keys, ok) and np.array_equal(vals, ov)
             assert mad.mad_stats(c.ctx)["inserted"] == sc["inserted"]
+
+
+def test_replays_beside_eager_rescoring():
+    """A captured pass replayed on one stream while mad_rescore runs on
+    another: both rule candidates out by bounds, each by its own."""
+    import paper_1506_03872_gb300 as mad
+    m, d, n, s, tprime, t, ncand = 2051, 100, 3001, 200_000, 6000, 30, 60_000
+    A, B = _inputs(94, m, d, n)
+    tA, tB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    flat = _rng(95).permutation(m * n)[:ncand]
+    pairs = mad.encode_pairs(flat // n, flat % n, np.arange(1, ncand + 1))
+    side = torch.cuda.Stream()
+    with mad.Context() as c:
+        mad.mad_pipeline_plan(c.ctx, mad.dense(tA), mad.dense(tB), s, tprime, t)
+        out, cand = mad.new_pairs(t), mad.new_pairs(tprime)
+        counts = torch.zeros(2, dtype=torch.int32, device="cuda")
+        mad.mad_pipeline_run(c.ctx, 51, out, counts, cand)
+        torch.cuda.synchronize()
+        mad.mad_pipeline_status(c.ctx)
+        _check(mad, out, counts, cand, _oracle_pass(A, B, 0, s, 51, tprime, t))
+        want, wc = out.clone(), counts.clone()
+        top, nt = mad.mad_rescore(c.ctx, pairs, ncand, t)
+        top = top.clone()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            mad.mad_pipeline_run(c.ctx, 51, out, counts, cand)
+        for _ in range(100):
+            with torch.cuda.stream(side):
+                g.replay()
+            for _ in range(2):
+                got, ng = mad.mad_rescore(c.ctx, pairs, ncand, t)
+                assert ng == nt and torch.equal(got[:ng], top[:nt])
+            side.synchronize()
+            assert torch.equal(counts, wc) and torch.equal(out, want)
