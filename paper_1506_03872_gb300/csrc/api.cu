@@ -151,38 +151,11 @@ mad_status clear_hash(mad_ctx* ctx, cudaStream_t st) {
   if (rs != MAD_OK) return rs;
   cudaMemsetAsync(&ctx->sc->inserted, 0, 5 * sizeof(unsigned long long), st);
   ctx->sampled = 0;
-  ctx->x_empty = true;
-  ctx->x_built = false;
-  return cuda_status(cudaGetLastError());
-}
-
-bool capturing(cudaStream_t st) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
-  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
-  cudaGetLastError();
-  return true;
-}
-
-// X of the region builder's layout re-inserted as a plain table, so that
-// further pairs can be added to it (asynchronous: the count of its keys, at most
-// one per diamond unless replays of a captured call added some, stays on the
-// device; a plain table stays one).
-mad_status x_to_table(mad_ctx* ctx, cudaStream_t st) {
-  const uint64_t slots = hash_slot_bound(ctx);
-  const uint64_t cap = ctx->x_captured || ctx->sampled > slots ? slots : ctx->sampled;
-  void* tmp = nullptr;
-  mad_status rs = pool_malloc(ctx, &tmp, 256 + 2 * cap * sizeof(uint64_t), st);
-  if (rs != MAD_OK) return rs;
-  unsigned long long* count = (unsigned long long*)tmp;
-  uint64_t* keys = (uint64_t*)((char*)tmp + 256);
-  int64_t* vals = (int64_t*)(keys + cap);
-  if ((rs = export_x_enqueue(ctx, keys, vals, cap, count, st)) == MAD_OK &&
-      (rs = clear_x_slots(ctx, st)) == MAD_OK) {
-    cudaMemsetAsync(&ctx->sc->new_keys, 0, sizeof(unsigned long long), st);
-    rs = accumulate_pairs(ctx, keys, vals, cap, st, count);
+  if (!stream_capturing(st)) {   // (a captured one clears X when it is replayed)
+    ctx->x_empty = true;
+    ctx->x_overflow = ctx->x_pass_captured;
   }
-  cudaFreeAsync(tmp, st);
-  return rs;
+  return cuda_status(cudaGetLastError());
 }
 
 }  // namespace
@@ -191,6 +164,13 @@ namespace mad {
 
 mad_status read_device_scalars(mad_ctx* ctx, DevScalars* hs, cudaStream_t st) {
   return read_scalars(ctx, hs, st);
+}
+
+bool stream_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
 }
 
 mad_status clear_x(mad_ctx* ctx, cudaStream_t st) { return clear_x_slots(ctx, st); }
@@ -257,7 +237,7 @@ mad_status alloc_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* B, 
     ctx->A = *A;
     ctx->B = *B;
     ctx->sampled = 0;
-    ctx->x_empty = ctx->x_built = false;
+    ctx->x_empty = ctx->x_overflow = ctx->x_pass_captured = false;
     if (ctx->regioned)
       ctx->hcap = ctx->hcap_alloc = hash_region_bound((uint64_t)ctx->m, s_max) + ctx->hov;
     return MAD_OK;
@@ -272,7 +252,7 @@ mad_status alloc_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* B, 
   ctx->n = B->cols;
   ctx->s_max = s_max;
   ctx->sampled = 0;
-  ctx->x_empty = ctx->x_built = false;
+  ctx->x_empty = ctx->x_overflow = ctx->x_pass_captured = false;
   mad_status rs = MAD_OK;
   if (!dense) {
     int64_t na = 0, nb = 0;
@@ -606,18 +586,22 @@ mad_status mad_sample(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first_di
   // factors: insert phase 359 -> 212 us, the search 1471 -> 1328 us).  Not while a stream is captured
   // (a replay would change X's layout unseen) or once one was (its replays add
   // to a plain table), nor with a test's layout.
-  const bool captured = capturing((cudaStream_t)stream);
+  cudaStream_t st = (cudaStream_t)stream;
+  const bool captured = stream_capturing(st);
   ctx->x_captured |= captured;
   const bool fresh = s == ctx->s_max && ctx->sampled == 0 && ctx->x_empty &&
                      ctx->region_factor == 1.5f && ctx->hov_request == 0 &&
                      !(ctx->flags & (MAD_WEDGE | MAD_ALIAS)) && x_builder_applies(ctx, s) &&
                      !ctx->x_captured;
-  const mad_status rs = sample_impl(ctx, s, seed, first_diamond, (cudaStream_t)stream, fresh);
-  if (s > 0) ctx->x_empty = false;
-  if (rs == MAD_OK) {
-    ctx->sampled += s;
-    if (fresh) ctx->x_built = true;
+  mad_status rs;
+  if (s > 0 && !fresh && ctx->x_overflow) {
+    if ((rs = fold_overflow(ctx, st)) != MAD_OK) return rs;
+    if (!captured) ctx->x_overflow = ctx->x_pass_captured;
   }
+  rs = sample_impl(ctx, s, seed, first_diamond, st, fresh);
+  if (s > 0) ctx->x_empty = false;
+  ctx->x_overflow |= fresh;
+  if (rs == MAD_OK) ctx->sampled += s;
   return rs;
 }
 
@@ -789,15 +773,16 @@ mad_status mad_accumulate(mad_ctx* ctx, const uint64_t* keys_dev, const int64_t*
   if (!ctx || (n && (!keys_dev || !vals_dev))) return MAD_ERR_ARG;
   if (!ctx->built) return MAD_ERR_STATE;
   if (n == 0) return MAD_OK;
-  const bool captured = capturing((cudaStream_t)stream);
+  cudaStream_t st = (cudaStream_t)stream;
+  const bool captured = stream_capturing(st);
   ctx->x_captured |= captured;
-  if (ctx->x_built) {
-    const mad_status rs = x_to_table(ctx, (cudaStream_t)stream);
+  if (ctx->x_overflow || captured) {   // (X may have been built whole again before a replay)
+    const mad_status rs = fold_overflow(ctx, st);
     if (rs != MAD_OK) return rs;
-    if (!captured) ctx->x_built = false;   // (captured: the layout changes with the replay)
+    if (!captured) ctx->x_overflow = ctx->x_pass_captured;
   }
   ctx->x_empty = false;
-  return accumulate_pairs(ctx, keys_dev, vals_dev, n, (cudaStream_t)stream);
+  return accumulate_pairs(ctx, keys_dev, vals_dev, n, st);
 }
 
 mad_status mad_select_pairs(mad_ctx* ctx, const mad_pair* pairs_dev, uint64_t n, uint32_t K,

@@ -432,6 +432,7 @@ __device__ __forceinline__ int hash_add_from(unsigned long long* __restrict__ ke
       const unsigned long long prev = atomicCAS(keys + g + pick, EMPTY_KEY, key);
       if (prev != EMPTY_KEY && prev != key) {
         slot = g + pick;  // taken by another key: look again from here
+        --probes;         // (counted again there)
         continue;
       }
       created = prev == EMPTY_KEY ? 2 : 0;
@@ -499,6 +500,13 @@ __device__ __forceinline__ bool bloom_may_contain(const unsigned long long* __re
   return (w.x & p.lo) == p.lo && (w.y & p.hi) == p.hi;
 }
 
+// Place of column b in a home region of `size` slots (a power of two).  A region
+// built whole (k_build_x) and one filled by k_insert place their keys alike, so
+// that either finds what the other left.
+__device__ __forceinline__ unsigned long long region_offset(uint32_t b, unsigned long long size) {
+  return (size <= (1ull << 32) ? (unsigned long long)fmix32(b) : mix64(b)) & (size - 1);
+}
+
 // First slot probed for key = (a << 32) | b.
 //
 // The home regions are sized for the diamonds whose row i is theirs.  Under
@@ -513,20 +521,20 @@ __device__ __forceinline__ bool bloom_may_contain(const unsigned long long* __re
 // at most 1.21, whatever the order of the rows.
 __device__ __forceinline__ uint64_t home_slot(const SampleParams& p, unsigned long long key) {
   if (p.regioned) {
-    const unsigned long long h = mix64(key);
-    const uint32_t a = (uint32_t)(key >> 32);
+    const uint32_t a = (uint32_t)(key >> 32), b = (uint32_t)key;
     unsigned long long r0 = p.hreg[a];
     unsigned long long size = p.hreg[a + 1] - r0;  // a power of two
     if (p.flags & MAD_GRAM) {
-      const uint32_t b = (uint32_t)key;
+      const unsigned long long h = mix64(key);
       const unsigned long long rb = p.hreg[b];
       const unsigned long long sb = p.hreg[b + 1] - rb;
       if (__umul64hi(h, size + sb) >= size) {
         r0 = rb;
         size = sb;
       }
+      return r0 + (h & (size - 1));
     }
-    return r0 + (h & (size - 1));
+    return r0 + region_offset(b, size);
   }
   return mix64(key) & p.hmask;
 }

@@ -172,11 +172,15 @@ struct mad_ctx {
   int64_t m = 0, d = 0, n = 0;
   uint64_t nnz_a = 0, nnz_b = 0;
   uint64_t s_max = 0, sampled = 0;
-  // X is empty (cleared, nothing added since), and X was last written whole
-  // by the region builder (keys beyond a group's regions in the overflow
-  // table, where a later insert would not look for them).
-  bool x_empty = false, x_built = false;
-  bool x_captured = false;   // a captured call adds to X as a plain table
+  // What is known of X when a call is enqueued; replays of captured calls may
+  // change X unseen, so each is stated on its safe side.
+  //   x_empty: cleared by a call that ran, nothing added since.
+  //   x_overflow: X may have been written whole by the region builder, with keys
+  //     in the overflow table, where adding calls do not look (fold_overflow).
+  //   x_captured: a captured call adds to X when it is replayed.
+  //   x_pass_captured: a captured pass writes X whole when it is replayed.
+  bool x_empty = false, x_overflow = false;
+  bool x_captured = false, x_pass_captured = false;
   int e1 = 0, f = 0;
   unsigned long long t1_total = 0;
   // Owned device memory.
@@ -460,9 +464,6 @@ void items_to_pairs_dev(mad_ctx* ctx, const Item* items, uint64_t cap,
                         const unsigned long long* n_dev, const mad_pair* cand,
                         const double* cvals, mad_pair* out, uint32_t* n_out, cudaStream_t st);
 int significant_bits(unsigned long long maxp);
-// (export_x_enqueue leaves the count in *counter and does not wait for it.)
-mad_status export_x_enqueue(mad_ctx* ctx, uint64_t* keys, int64_t* vals, uint64_t cap,
-                            unsigned long long* counter, cudaStream_t st);
 mad_status export_x(mad_ctx* ctx, uint64_t* keys, int64_t* vals, uint64_t cap, uint64_t* n,
                     unsigned long long* counter, cudaStream_t st);
 // Sharded runs: X's occupied slots grouped by owner rank (offsets_host gets
@@ -486,9 +487,14 @@ mad_status wedge_sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t f
 mad_status wedge_draws_impl(mad_ctx* ctx, uint64_t seed, uint64_t first, const uint64_t* ells,
                             uint64_t count, uint32_t* oi, uint32_t* ok, uint32_t* oj,
                             uint32_t* okp, int64_t* ov, cudaStream_t st);
-// sample.cu: (key, value) pairs added to X (min(n, *n_dev) with a device count).
+// sample.cu: (key, value) pairs added to X.
 mad_status accumulate_pairs(mad_ctx* ctx, const uint64_t* keys, const int64_t* vals, uint64_t n,
-                            cudaStream_t st, const unsigned long long* n_dev = nullptr);
+                            cudaStream_t st);
+// sample.cu: an X that may have been built whole made a plain table, to which
+// pairs can be added (nothing where X is never built whole).
+mad_status fold_overflow(mad_ctx* ctx, cudaStream_t st);
+// Whether calls on the stream are being captured into a graph.
+bool stream_capturing(cudaStream_t st);
 // dense_topt.cu: the comparator; dense_out != NULL writes the full product.
 mad_status dense_comparator(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* B, uint32_t t,
                             uint32_t rescore, mad_pair* out, uint32_t* n_out, float* dense_out,

@@ -118,7 +118,8 @@ mad_status enqueue_pass(mad_ctx* ctx, uint64_t seed, mad_pair* out_dev, uint32_t
   if ((rs = sample_impl(ctx, ctx->pipe_s, seed, 0, st, true)) != MAD_OK) return rs;
   ctx->sampled = ctx->pipe_s;
   ctx->x_empty = false;
-  ctx->x_built = fresh;
+  ctx->x_overflow |= fresh;
+  ctx->x_pass_captured |= fresh && stream_capturing(st);
   ctx->built = true;
   // Alg. 3: Omega_t' (its length min(t', compacted) on the device) ...
   if (long_sel)

@@ -582,10 +582,8 @@ k_insert(const SampleParams p_, const unsigned long long* __restrict__ keys,
 // Counts the keys it creates, not diamonds.
 __global__ void __launch_bounds__(256)
 k_accumulate(const SampleParams p_, const unsigned long long* __restrict__ keys,
-             const long long* __restrict__ vals, unsigned long long n_max,
-             const unsigned long long* n_dev) {
+             const long long* __restrict__ vals, unsigned long long n) {
   const SampleParams p = resolve(p_);
-  const unsigned long long n = dev_len(n_max, n_dev);
   Tally t;
   for (unsigned long long q = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (unsigned long long)gridDim.x * blockDim.x) {
@@ -609,16 +607,20 @@ k_accumulate(const SampleParams p_, const unsigned long long* __restrict__ keys,
 // contiguous.  A block builds them in shared memory from the diamonds of its
 // buckets (those of its last row that fall into later buckets included) and
 // stores them with plain coalesced writes, so X is written once and never read
-// back from DRAM.  Every key probes linearly from its home slot through its
-// group's regions, taken as one circular table; a key that finds them all
-// full goes to the overflow table after the regions, [hreg[m], hreg[m] + O),
-// a plain linear-probing hash.  Groups whose regions exceed the
+// back from DRAM.  Every key probes linearly from its home slot (home_slot) to
+// the end of its group's regions; a key that finds no place before it goes to
+// the overflow table after the regions, [hreg[m], hreg[m] + O), a plain
+// linear-probing hash (a key in two groups or so, at the loads of 1/3 to 2/3
+// that the regions are sized for).  So the regions are what k_insert would
+// leave, but for those keys, and k_fold_overflow makes X a plain table again
+// before anything else is added to it.  Groups whose regions exceed the
 // shared-memory image are "heavy": a first kernel clears their regions and
 // the diamonds of their rows are added with global atomics (the same
-// circular probing) by whichever block holds them in its own buckets.
+// probing) by whichever block holds them in its own buckets.
 // Each diamond is added exactly once, so X is the same set of
 // (key, sum) as the one k_insert builds (the sums are exact integers).
 constexpr int kImageSlots = 3072;   // 48 KB: keys, then values
+constexpr int kSpill = 32;          // slots after a group's regions in the image
 constexpr int kRowCache = 256;      // owned rows whose hreg a block keeps in shared memory
 
 // R[h] for a group boundary h (see above): 1 + #{r : T1[r] < h << gs}, read
@@ -692,15 +694,14 @@ k_group_prep(const SampleParams p_, const unsigned int* __restrict__ base, uint3
   }
 }
 
-// Global insert of key into the circular table [lo, hi) from slot, then,
-// when it is full, into the overflow table.  1 existing key, 2 new key, 0
-// both full.
-__device__ __forceinline__ int add_span_or_overflow(const SampleParams& p, unsigned long long lo,
-                                                    unsigned long long hi, unsigned long long slot,
+// Global insert of key into [slot, hi) from slot on, then, when that is full,
+// into the overflow table.  1 existing key, 2 new key, 0 both full.
+__device__ __forceinline__ int add_span_or_overflow(const SampleParams& p, unsigned long long hi,
+                                                    unsigned long long slot,
                                                     unsigned long long ov0, uint64_t ov_slots,
                                                     unsigned long long key, long long v) {
-  if (lo < hi) {
-    const int r = hash_add_from(p.hkeys, p.hvals, lo, hi, slot, (uint32_t)(hi - lo), key, v);
+  if (slot < hi) {   // (hi - slot probes end before the wrap)
+    const int r = hash_add_from(p.hkeys, p.hvals, slot, hi, slot, (uint32_t)(hi - slot), key, v);
     if (r) return r;
   }
   return hash_add_from(p.hkeys, p.hvals, ov0, ov0 + ov_slots, ov0 + (mix64(key) & (ov_slots - 1)),
@@ -723,7 +724,7 @@ k_build_x(const SampleParams p_, const unsigned long long* __restrict__ keys,
           uint32_t nbk, int lg_group, uint32_t ngroups, uint64_t ov_slots,
           const uint32_t* __restrict__ R, const unsigned char* __restrict__ heavy,
           const uint32_t* __restrict__ qend_g) {
-  // kImageSlots keys (4 or 8 bytes), then kImageSlots 8-byte values.
+  // kImageSlots + kSpill keys (4 or 8 bytes), then as many 8-byte values.
   extern __shared__ __align__(16) unsigned long long img[];
   using IKey = typename std::conditional<kNarrow, uint32_t, unsigned long long>::type;
   constexpr IKey kEmptyI = (IKey)~(IKey)0;
@@ -747,13 +748,15 @@ k_build_x(const SampleParams p_, const unsigned long long* __restrict__ keys,
   if (!hv && cached)
     for (uint32_t x = threadIdx.x; x <= r1 - r0; x += blockDim.x)
       s_off[x] = (uint32_t)(p.hreg[r0 + x] - lo);
-  const uint32_t span32 = (uint32_t)span;
+  // Keys that reach the end of the regions go on into the spill slots, which
+  // leave for the overflow table at the end, beside the image's stores.
+  const uint32_t span32 = (uint32_t)span, end32 = hv ? 0u : span32 + kSpill;
   unsigned long long q = q0 + threadIdx.x;
   unsigned long long key = q < qend ? keys[q] : EMPTY_KEY;
   long long v = q < qend ? vals[q] : 0;
   IKey* ik = (IKey*)img;
-  unsigned long long* iv = (unsigned long long*)((char*)img + kImageSlots * sizeof(IKey));
-  for (uint32_t x = 4 * threadIdx.x; x < span32; x += 4 * blockDim.x) {
+  unsigned long long* iv = (unsigned long long*)((char*)img + (kImageSlots + kSpill) * sizeof(IKey));
+  for (uint32_t x = 4 * threadIdx.x; x < end32; x += 4 * blockDim.x) {
     if (kNarrow) {
       *(uint4*)(ik + x) = make_uint4(~0u, ~0u, ~0u, ~0u);
     } else {
@@ -779,9 +782,11 @@ k_build_x(const SampleParams p_, const unsigned long long* __restrict__ keys,
     const bool own = !hv && i >= r0 && i < r1;
     int res;
     if (own) {
-      // Linear probe of the image from the home slot, wrapping at its end
-      // (the group's regions form one circular table), four slots per
-      // step (two 16-byte shared loads; regions start on 4-slot groups).
+      // Linear probe of the image from the home slot to its end, four slots
+      // per step (two 16-byte shared loads; regions start on 4-slot groups).
+      // The probes left end the loop at the image's end, so the wraps below are
+      // never taken; the loop compiled without them costs the pass 3 us, and
+      // ended by the position instead of the count 15 us (849 -> 852, 865).
       // A stale EMPTY is caught by the CAS; a key once set never changes.
       // Image positions are 32-bit (the image holds kImageSlots slots).
       uint32_t roff, rsz;
@@ -793,10 +798,10 @@ k_build_x(const SampleParams p_, const unsigned long long* __restrict__ keys,
         roff = (uint32_t)(a - lo);
         rsz = (uint32_t)(__ldg(p.hreg + i + 1) - a);
       }
-      uint32_t x = roff + (fmix32((uint32_t)k) & (rsz - 1));
+      uint32_t x = roff + (uint32_t)region_offset((uint32_t)k, rsz);
       const IKey kk = kNarrow ? (IKey)(((i - r0) << 24) | (uint32_t)k) : (IKey)k;
       res = 0;
-      for (uint32_t probes = 0; probes < span32;) {
+      for (uint32_t probes = 0, left = end32 - x; probes < left;) {
         const uint32_t gx = x & ~3u;
         IKey k4[4];
         if (kNarrow) {
@@ -814,7 +819,7 @@ k_build_x(const SampleParams p_, const unsigned long long* __restrict__ keys,
           pick = ((uint32_t)u >= start && (k4[u] == kk || k4[u] == kEmptyI)) ? (uint32_t)u : pick;
         if (pick == 4) {
           probes += 4 - start;
-          x = gx + 4 < span32 ? gx + 4 : 0;
+          x = gx + 4 < end32 ? gx + 4 : 0;
           continue;
         }
         probes += pick - start + 1;
@@ -834,9 +839,9 @@ k_build_x(const SampleParams p_, const unsigned long long* __restrict__ keys,
           res = prev == kEmptyI ? 2 : 1;
           break;
         }
-        x = slot + 1 < span32 ? slot + 1 : 0;   // taken by another key: go on after it
+        x = slot + 1 < end32 ? slot + 1 : 0;   // taken by another key: go on after it
       }
-      if (res == 0) res = add_span_or_overflow(p, 0, 0, 0, ov0, ov_slots, k, w);
+      if (res == 0) res = add_span_or_overflow(p, 0, 0, ov0, ov_slots, k, w);
     } else {
       if (q >= q1) continue;   // the owner's extension: not this block's
       const unsigned long long ex = i ? __ldg(p.T1 + i - 1) : 0ull;
@@ -844,32 +849,65 @@ k_build_x(const SampleParams p_, const unsigned long long* __restrict__ keys,
       og = og < ngroups - 1 ? og : ngroups - 1;
       if (!heavy[og]) continue;   // its owner builds it
       const unsigned long long rlo = __ldg(p.hreg + i), rhi = __ldg(p.hreg + i + 1);
-      const unsigned long long home = rlo + (fmix32((uint32_t)k) & (rhi - rlo - 1));
-      res = add_span_or_overflow(p, p.hreg[R[og]], p.hreg[R[og + 1]], home, ov0, ov_slots, k, w);
+      const unsigned long long home = rlo + region_offset((uint32_t)k, rhi - rlo);
+      res = add_span_or_overflow(p, p.hreg[R[og + 1]], home, ov0, ov_slots, k, w);
     }
     ++t.inserted;
     if (res == 0) t.full = true;
     if (res == 2) ++t.created;
   }
   __syncthreads();
-  // The image, 16 bytes per store (regions start on 4-slot groups), keys
-  // widened back to (i << 32) | j.
+  // Image keys widened back to (i << 32) | j.
+  auto wide = [&](uint32_t x) -> unsigned long long {
+    const IKey a = ik[x];
+    if (a == kEmptyI) return EMPTY_KEY;
+    return kNarrow ? ((unsigned long long)(r0 + ((uint32_t)a >> 24)) << 32) | ((uint32_t)a & 0xFFFFFFu)
+                   : (unsigned long long)a;
+  };
+  // A spilled key is in no other block's hands: a claimed slot of the overflow
+  // table is its own, and the claim's round trip passes beside the stores below.
+  unsigned long long spilled = EMPTY_KEY, at = 0, prev = EMPTY_KEY;
+  if (threadIdx.x < kSpill && !hv) spilled = wide(span32 + threadIdx.x);
+  if (spilled != EMPTY_KEY) {
+    at = mix64(spilled) & (ov_slots - 1);
+    prev = atomicCAS(p.hkeys + ov0 + at, EMPTY_KEY, spilled);
+  }
+  // The image, 16 bytes per store (regions start on 4-slot groups).
   for (uint32_t x = 2 * threadIdx.x; x < span32; x += 2 * blockDim.x) {
-    unsigned long long k0, k1;
-    if (kNarrow) {
-      const uint32_t a = ik[x], b = ik[x + 1];
-      k0 = a == ~0u ? EMPTY_KEY
-                    : ((unsigned long long)(r0 + (a >> 24)) << 32) | (a & 0xFFFFFFu);
-      k1 = b == ~0u ? EMPTY_KEY
-                    : ((unsigned long long)(r0 + (b >> 24)) << 32) | (b & 0xFFFFFFu);
-    } else {
-      k0 = (unsigned long long)ik[x];
-      k1 = (unsigned long long)ik[x + 1];
-    }
-    *(ulonglong2*)(p.hkeys + lo + x) = make_ulonglong2(k0, k1);
+    *(ulonglong2*)(p.hkeys + lo + x) = make_ulonglong2(wide(x), wide(x + 1));
     *(longlong2*)(p.hvals + lo + x) = make_longlong2((long long)iv[x], (long long)iv[x + 1]);
   }
+  if (spilled != EMPTY_KEY) {
+    for (uint64_t probes = 1; prev != EMPTY_KEY && probes < ov_slots; ++probes) {
+      at = (at + 1) & (ov_slots - 1);
+      prev = atomicCAS(p.hkeys + ov0 + at, EMPTY_KEY, spilled);
+    }
+    if (prev == EMPTY_KEY) p.hvals[ov0 + at] = (long long)iv[span32 + threadIdx.x];
+    else t.full = true;
+  }
   flush_tally_block(p, t);
+}
+
+// The overflow table's keys moved into the regions, where k_insert and
+// k_accumulate look for them: X is a plain table afterwards.  (Each key is in
+// one place, so none is counted as new; one that finds no place stays and is
+// reported.)
+__global__ void __launch_bounds__(256)
+k_fold_overflow(const SampleParams p_, uint64_t ov_slots) {
+  const SampleParams p = resolve(p_);
+  const unsigned long long ov0 = p.hreg[p.m];
+  if (ov0 + ov_slots > p.hcap_alloc) return;   // reported by k_group_prep
+  for (unsigned long long x = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+       x < ov_slots; x += (unsigned long long)gridDim.x * blockDim.x) {
+    const unsigned long long key = p.hkeys[ov0 + x];
+    if (key == EMPTY_KEY) continue;
+    if (hash_add(p, key, p.hvals[ov0 + x]) == 0) {
+      atomicOr(&p.sc->err, DERR_HASH_FULL);
+      continue;
+    }
+    p.hkeys[ov0 + x] = EMPTY_KEY;
+    p.hvals[ov0 + x] = 0;
+  }
 }
 
 // Diagnostic twin of k_sample: writes each diamond's draws instead of
@@ -1173,11 +1211,11 @@ mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first, 
   // Narrow image keys when every column index fits in 24 bits.
   const bool narrow = ctx->n <= (1ll << 24);
   const size_t image_smem =
-      (size_t)kImageSlots * ((narrow ? sizeof(uint32_t) : sizeof(unsigned long long)) +
+      (size_t)(kImageSlots + kSpill) * ((narrow ? sizeof(uint32_t) : sizeof(unsigned long long)) +
                              sizeof(unsigned long long));
   static bool image_attr = false;
   if (build_x && !image_attr) {
-    const int wide_smem = (int)(2 * (size_t)kImageSlots * sizeof(unsigned long long));
+    const int wide_smem = (int)(2 * (size_t)(kImageSlots + kSpill) * sizeof(unsigned long long));
     cudaFuncSetAttribute(k_build_x<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide_smem);
     cudaFuncSetAttribute(k_build_x<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide_smem);
     image_attr = true;
@@ -1231,12 +1269,20 @@ mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first, 
   return cuda_status(cudaGetLastError());
 }
 
+mad_status fold_overflow(mad_ctx* ctx, cudaStream_t st) {
+  if (!x_builder_applies(ctx, ctx->s_max)) return MAD_OK;   // X is never built whole
+  k_fold_overflow<<<grid_of(ctx->hov, full_grid<k_fold_overflow>()), 256, 0, st>>>(
+      make_params(ctx), ctx->hov);
+  count_launch(ctx);
+  return cuda_status(cudaGetLastError());
+}
+
 mad_status accumulate_pairs(mad_ctx* ctx, const uint64_t* keys, const int64_t* vals, uint64_t n,
-                            cudaStream_t st, const unsigned long long* n_dev) {
+                            cudaStream_t st) {
   if (n == 0) return MAD_OK;
   const SampleParams p = make_params(ctx);
   k_accumulate<<<grid_of(n, full_grid<k_accumulate>()), 256, 0, st>>>(
-      p, (const unsigned long long*)keys, (const long long*)vals, n, n_dev);
+      p, (const unsigned long long*)keys, (const long long*)vals, n);
   count_launch(ctx);
   return cuda_status(cudaGetLastError());
 }

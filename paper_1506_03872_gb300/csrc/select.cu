@@ -1620,8 +1620,8 @@ mad_status select_pairs(mad_ctx* ctx, const mad_pair* pairs, uint64_t n, uint64_
   return cuda_status(cudaStreamSynchronize(st));
 }
 
-mad_status export_x_enqueue(mad_ctx* ctx, uint64_t* keys, int64_t* vals, uint64_t cap,
-                            unsigned long long* counter, cudaStream_t st) {
+mad_status export_x(mad_ctx* ctx, uint64_t* keys, int64_t* vals, uint64_t cap, uint64_t* n,
+                    unsigned long long* counter, cudaStream_t st) {
   cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st);
   k_export<<<grid_for(hash_slot_bound(ctx), 152 * 8), 256, 0, st>>>(ctx->hkeys, ctx->hvals,
                                                                     hash_slot_bound(ctx),
@@ -1629,13 +1629,6 @@ mad_status export_x_enqueue(mad_ctx* ctx, uint64_t* keys, int64_t* vals, uint64_
                                                          (long long*)vals, cap, counter,
                                                          hash_extent(ctx));
   count_launch(ctx);
-  return cuda_status(cudaGetLastError());
-}
-
-mad_status export_x(mad_ctx* ctx, uint64_t* keys, int64_t* vals, uint64_t cap, uint64_t* n,
-                    unsigned long long* counter, cudaStream_t st) {
-  const mad_status rs = export_x_enqueue(ctx, keys, vals, cap, counter, st);
-  if (rs != MAD_OK) return rs;
   unsigned long long cnt = 0;
   cudaMemcpyAsync(&cnt, counter, sizeof(cnt), cudaMemcpyDeviceToHost, st);
   const cudaError_t e = cudaStreamSynchronize(st);

@@ -536,3 +536,93 @@ def test_replays_beside_eager_rescoring():
                 assert ng == nt and torch.equal(got[:ng], top[:nt])
             side.synchronize()
             assert torch.equal(counts, wc) and torch.equal(out, want)
+
+
+def test_captured_clear_and_pass_around_eager_additions():
+    """A captured mad_reset_hash clears X, and a captured pass fills it, when
+    they are replayed, not when they are captured: pairs added before, between
+    and after replays are each added once."""
+    import paper_1506_03872_gb300 as mad
+    m, d, n, s = 2051, 60, 3001, 100_000
+    A, B = _inputs(96, m, d, n)
+    tA, tB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    (ok, ov), _ = _oracle_x(A, B, 0, s, 17)
+    k = torch.from_numpy(ok.view(np.int64).copy()).cuda()
+    v = torch.from_numpy(ov.copy()).cuda()
+    with mad.Context() as c:
+        def check(times):
+            keys, vals, cnt = _export_sorted(mad, c.ctx, 2 * s)
+            assert cnt == (len(ok) if times else 0) == mad.mad_stats(c.ctx)["distinct"]
+            if times:
+                assert np.array_equal(keys, ok) and np.array_equal(vals, times * ov)
+
+        def capture(call):
+            torch.cuda.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                call()
+            return g
+
+        c.build(mad.dense(tA), mad.dense(tB), s, keep=(tA, tB))
+        mad.mad_sample(c.ctx, s, 17)
+        clear = capture(lambda: mad.mad_reset_hash(c.ctx))
+        mad.mad_accumulate(c.ctx, k, v)
+        check(2)
+        clear.replay()
+        check(0)
+        mad.mad_sample(c.ctx, s, 17)
+        check(1)
+        mad.mad_reset_hash(c.ctx)
+        mad.mad_sample(c.ctx, s, 17)      # (region by region again)
+        capture(lambda: mad.mad_reset_hash(c.ctx))
+        mad.mad_sample(c.ctx, s // 2, 17)
+        mad.mad_sample(c.ctx, s - s // 2, 17, s // 2)
+        check(2)
+
+        mad.mad_pipeline_plan(c.ctx, mad.dense(tA), mad.dense(tB), s, 100, 10)
+        out, counts = mad.new_pairs(10), torch.zeros(2, dtype=torch.int32, device="cuda")
+        mad.mad_pipeline_run(c.ctx, 17, out, counts)
+        mad.mad_pipeline_status(c.ctx)
+        run = capture(lambda: mad.mad_pipeline_run(c.ctx, 17, out, counts))
+        add = capture(lambda: mad.mad_accumulate(c.ctx, k, v))
+        mad.mad_accumulate(c.ctx, k, v)
+        check(2)
+        mad.mad_reset_hash(c.ctx)
+        check(0)
+        run.replay()
+        mad.mad_accumulate(c.ctx, k, v)
+        mad.mad_accumulate(c.ctx, k, v)
+        check(3)
+        run.replay()
+        check(1)
+        add.replay()
+        check(2)
+
+
+@pytest.mark.parametrize("m,s,scale,factor", [(300, 50_000, 1.0, 0.75), (2051, 200_000, 3.0, 0.75),
+                                              (2051, 200_000, 3.0, 1.5), (7, 60_000, 1.0, 1.5)])
+def test_keys_past_their_group_are_folded_back(m, s, scale, factor):
+    """Keys of a pass that found no place before their group's end lie in the
+    overflow table; pairs added to that X find them.  (Regions of 0.75 of the
+    expected diamonds hold X as one table where the rows' sizes are even;
+    one row of many thousand keys past its own region is beyond the probe
+    limit of any adding call.)"""
+    import paper_1506_03872_gb300 as mad
+    A, B = _inputs(97, m, 40, 90_001 if m == 7 else 3001)
+    A *= np.exp(scale * _rng(98).standard_normal((m, 1))).astype(np.float32)
+    tA, tB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    (ok, ov), _ = _oracle_x(A, B, 0, s, 3)
+    k = torch.from_numpy(ok.view(np.int64).copy()).cuda()
+    v = torch.from_numpy(ov.copy()).cuda()
+    with mad.Context() as c:
+        mad.mad_debug_set_hash_layout(c.ctx, factor, 1 << 18)
+        mad.mad_pipeline_plan(c.ctx, mad.dense(tA), mad.dense(tB), s, 100, 10)
+        out, counts = mad.new_pairs(10), torch.zeros(2, dtype=torch.int32, device="cuda")
+        mad.mad_pipeline_run(c.ctx, 3, out, counts)
+        mad.mad_pipeline_status(c.ctx)
+        mad.mad_accumulate(c.ctx, k[::2].contiguous(), v[::2].contiguous())
+        mad.mad_accumulate(c.ctx, k[1::2].contiguous(), v[1::2].contiguous())
+        keys, vals, cnt = _export_sorted(mad, c.ctx, 2 * s)
+        st = mad.mad_stats(c.ctx)
+        assert st["device_error"] == 0 and st["distinct"] == len(ok) == cnt
+        assert np.array_equal(keys, ok) and np.array_equal(vals, 2 * ov)
