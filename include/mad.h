@@ -40,7 +40,9 @@
  * a parameter says host).  A and B must stay alive and unchanged from
  * mad_build_tables until mad_destroy or the next mad_build_tables: sampling
  * and rescoring read them.  The library owns its tables, hash and scratch,
- * allocated stream-ordered on the stream of mad_build_tables.
+ * allocated stream-ordered on the stream of mad_build_tables.  CUDA graphs
+ * that captured calls on a context hold addresses of these: they must not be
+ * replayed after the next mad_build_tables or mad_pipeline_plan on it.
  *
  * Errors: every call returns a status and never aborts.  Device-side
  * failures (hash probe limit, bad index) set a sticky flag that the next

@@ -237,7 +237,7 @@ mad_status alloc_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* B, 
     ctx->A = *A;
     ctx->B = *B;
     ctx->sampled = 0;
-    ctx->x_empty = ctx->x_overflow = ctx->x_pass_captured = false;
+    ctx->x_empty = ctx->x_overflow = ctx->x_captured = ctx->x_pass_captured = false;
     if (ctx->regioned)
       ctx->hcap = ctx->hcap_alloc = hash_region_bound((uint64_t)ctx->m, s_max) + ctx->hov;
     return MAD_OK;
@@ -252,7 +252,7 @@ mad_status alloc_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* B, 
   ctx->n = B->cols;
   ctx->s_max = s_max;
   ctx->sampled = 0;
-  ctx->x_empty = ctx->x_overflow = ctx->x_pass_captured = false;
+  ctx->x_empty = ctx->x_overflow = ctx->x_captured = ctx->x_pass_captured = false;
   mad_status rs = MAD_OK;
   if (!dense) {
     int64_t na = 0, nb = 0;

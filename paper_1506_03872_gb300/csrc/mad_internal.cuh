@@ -173,7 +173,8 @@ struct mad_ctx {
   uint64_t nnz_a = 0, nnz_b = 0;
   uint64_t s_max = 0, sampled = 0;
   // What is known of X when a call is enqueued; replays of captured calls may
-  // change X unseen, so each is stated on its safe side.
+  // change X unseen, so each is stated on its safe side (a table build ends the
+  // life of graphs captured before it: mad.h).
   //   x_empty: cleared by a call that ran, nothing added since.
   //   x_overflow: X may have been written whole by the region builder, with keys
   //     in the overflow table, where adding calls do not look (fold_overflow).

@@ -626,3 +626,36 @@ def test_keys_past_their_group_are_folded_back(m, s, scale, factor):
         st = mad.mad_stats(c.ctx)
         assert st["device_error"] == 0 and st["distinct"] == len(ok) == cnt
         assert np.array_equal(keys, ok) and np.array_equal(vals, 2 * ov)
+
+
+def test_a_table_build_ends_what_captured_calls_meant():
+    """mad_sample of the whole budget builds X region by region unless a
+    captured call of these tables may add to it: a context that captured one
+    does so again once its tables are built again, and gives the same X."""
+    import paper_1506_03872_gb300 as mad
+    m, d, n, s = 700, 40, 3001, 50_000
+    A, B = _inputs(99, m, d, n)
+    tA, tB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    (ok, ov), _ = _oracle_x(A, B, 0, s, 17)
+
+    def sampled(c):
+        mad.mad_reset_hash(c.ctx)
+        before = mad.mad_stats(c.ctx)["launches"]
+        mad.mad_sample(c.ctx, s, 17)
+        launches = mad.mad_stats(c.ctx)["launches"] - before
+        keys, vals, cnt = _export_sorted(mad, c.ctx, s + 1)
+        assert cnt == len(ok) and np.array_equal(keys, ok) and np.array_equal(vals, ov)
+        return launches
+
+    with mad.Context() as c:
+        c.build(mad.dense(tA), mad.dense(tB), s, keep=(tA, tB))
+        built = sampled(c)
+        mad.mad_reset_hash(c.ctx)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            mad.mad_sample(c.ctx, s // 2, 17)
+        assert sampled(c) < built          # key by key
+        c.build(mad.dense(tA), mad.dense(tB), s, keep=(tA, tB))
+        assert sampled(c) == built
+        del g
