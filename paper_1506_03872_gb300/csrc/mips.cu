@@ -372,9 +372,12 @@ struct Kept {
 // Step 2: part u - ubase of query unit_q[u].  The table is open addressing
 // with linear probing over 32-bit columns; the sums are 64-bit (two 32-bit
 // shared atomics, the low word's carry into the high word).  When it fills up
-// (a statistical rarity, or a batch whose parts are capped at kMaxParts) the
-// part is taken in 2, 4, ... slices of another mix of j, each slice's kept
-// columns competing with those of the slices before.
+// (a statistical rarity, or every part of a batch whose parts are capped at
+// kMaxParts) the part is taken in 2, 4, ... slices of another mix of j, each
+// slice's kept columns competing with those of the slices before.  Once one
+// record has found no slot, the others are left: with each of them looking for a
+// free slot through the whole table, one query of 8e7 diamonds on 4e7 items took
+// 627 ms, 35 so.
 //
 // The part's records lie in one run per chunk of the query: the runs' offsets are
 // scanned (kGroup chunks at a time) and the records dealt out evenly, four of a
@@ -472,6 +475,7 @@ k_mips_parts(const MipsQuery* __restrict__ queries, const uint32_t* __restrict__
         uint32_t slot = fmix32(v.x) & mask;
         int probes = 1;
         for (; probes < slots; ++probes) {
+          if ((probes & 63) == 0 && *(volatile uint32_t*)&s_full) break;
           slot = (slot + 1) & mask;
           const uint32_t cur = atomicCAS(keys + slot, kNoKey, v.x);
           if (cur == kNoKey || cur == v.x) {
@@ -484,7 +488,10 @@ k_mips_parts(const MipsQuery* __restrict__ queries, const uint32_t* __restrict__
       };
       int waiting = 0;   // of the warp
       for (uint32_t g0 = 0; g0 < nch; g0 += kGroup) {
-        if (nch > (uint32_t)kGroup) in_group = scan_group(g0);
+        if (nch > (uint32_t)kGroup) {
+          if (g0 && __syncthreads_or((int)s_full)) break;
+          in_group = scan_group(g0);
+        }
         const int runs = (int)(nch - g0 < (uint32_t)kGroup ? nch - g0 : (uint32_t)kGroup);
         const uint2* __restrict__ r = rec + mq.rec + (unsigned long long)g0 * chunk;
         // A warp's records: an even share of them, in a row.
@@ -492,6 +499,7 @@ k_mips_parts(const MipsQuery* __restrict__ queries, const uint32_t* __restrict__
         const uint32_t end = min(in_group, (warp + 1) * share);
         int run = 0;   // the last run that starts at or before the lane's record
         for (uint32_t base = warp * share; base < end; base += 32 * kAhead) {
+          if (__any_sync(0xFFFFFFFFu, *(volatile uint32_t*)&s_full)) break;
           uint2 v[kAhead];
 #pragma unroll
           for (int a = 0; a < kAhead; ++a) {

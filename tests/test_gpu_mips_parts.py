@@ -136,3 +136,33 @@ def test_many_parts_of_long_items():
     assert got[0][0].tolist() == [t, t]
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+def test_a_full_table_costs_passes_over_the_records_not_over_itself():
+    """Tables of 0.3 slots a record fill up at two or three levels, and the part
+    is read again for each slice: at most some ten times the records, where a
+    record that searched the full table for a slot would cost a thousand steps."""
+    import paper_1506_03872_gb300 as mad
+    s_q = np.full(61, 50_000, np.uint64)
+    Q, B = _items(12, 20, 50_021, len(s_q))
+    tQ, tB = torch.from_numpy(Q).cuda(), torch.from_numpy(B).cuda()
+    best, got = [], []
+    for factor in (1.5, 0.3):
+        out, cand = mad.new_pairs(61 * 5), mad.new_pairs(61 * 100)
+        nout = torch.zeros(61, dtype=torch.int32, device="cuda")
+        with mad.Context() as c:
+            mad.mad_debug_set_hash_layout(c.ctx, factor)
+            mad.mad_mips_items(c.ctx, mad.dense(tB), 1 << 17)
+            mad.mad_mips_plan(c.ctx, s_q, 100, 5)
+            ms = []
+            for _ in range(8):
+                e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                e0.record()
+                mad.mad_mips_run(c.ctx, mad.dense(tQ), 5, out, nout, cand)
+                e1.record()
+                torch.cuda.synchronize()
+                ms.append(e0.elapsed_time(e1))
+            best.append(min(ms))
+            got.append((out, cand, nout))
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+    assert best[1] < 12 * best[0], best
