@@ -961,8 +961,9 @@ mad_status select_from_hash(mad_ctx* ctx, const SelectWs& ws, uint64_t K, uint64
 
 // Dense inputs: the threshold from a sample (as in select_hash_dev), the exact
 // number of items at or above it, of positive keys and the table's scalars in one
-// read-back; the list is sized for a few times K and grown when more passed, and
-// the exact histogram runs only when fewer than K did.  (1e7 diamonds, t' =
+// read-back; the list is sized for a few times K (a long one for the keys there
+// are, after one more read-back) and grown when more passed, and the exact
+// histogram runs only when fewer than K did.  (1e7 diamonds, t' =
 // 1e4: mad_topk 227 -> 184 us, of the plain search's 94 us 30 less.)
 mad_status topk_dense(mad_ctx* ctx, uint64_t K, mad_pair* out, uint64_t* n_sel, DevScalars* hs,
                       cudaStream_t st) {
@@ -972,6 +973,11 @@ mad_status topk_dense(mad_ctx* ctx, uint64_t K, mad_pair* out, uint64_t* n_sel, 
   uint64_t cap = K < (1ull << 40) ? 4 * K : bound;
   cap = cap < (1u << 16) ? (1u << 16) : cap;
   cap = cap < bound ? cap : bound;
+  if (cap > (1ull << 20)) {   // 75 MB of lists
+    const mad_status rs = read_device_scalars(ctx, hs, st);
+    if (rs != MAD_OK) return rs;
+    cap = cap < hs->new_keys ? cap : (hs->new_keys ? hs->new_keys : 1);
+  }
   unsigned long long* host = (unsigned long long*)ctx->pinned;   // count, max, positive, theta
   unsigned long long theta = 0;
   SelectWs ws;

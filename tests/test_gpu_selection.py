@@ -80,3 +80,30 @@ def test_bounded_rescore_equals_the_whole_one(kind, ta, tb, d):
                 top, nt = mad.mad_rescore(c.ctx, cand, len(q), t)
                 assert nw == len(q) and nt == t
                 assert torch.equal(top, whole[:t])
+
+
+def test_a_long_candidate_list_is_sized_by_the_keys_there_are():
+    """t' above the number of keys of X: the selection's lists (three of 24
+    bytes an item and the sorted one) hold those keys, not X's slots (three
+    and more per diamond of the budget)."""
+    import paper_1506_03872_gb300 as mad
+    rng = _rng(8)
+    m, d, n, s = 20_000, 20, 3001, 1 << 22
+    tA = torch.from_numpy(rng.standard_normal((m, d)).astype(np.float32)).cuda()
+    tB = torch.from_numpy(rng.standard_normal((d, n)).astype(np.float32)).cuda()
+    out = mad.new_pairs(s)
+    with mad.Context() as c:
+        c.build(mad.dense(tA), mad.dense(tB), s, keep=(tA, tB))
+        mad.mad_sample(c.ctx, s, 3)
+        st = mad.mad_stats(c.ctx)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        _, cnt = mad.mad_topk(c.ctx, s, out)
+        used = free - torch.cuda.mem_get_info()[0]
+        keys, vals, nx = mad.mad_export_x(c.ctx, cap=s)
+    x = vals[:nx]
+    assert st["distinct"] == nx and cnt == int((x > 0).sum())
+    got = out[:cnt, 1]
+    assert torch.equal(got, torch.sort(x[x > 0], descending=True).values)
+    lists = 3 * 24 * nx + 24 * (1 << (nx - 1).bit_length())
+    assert used <= lists + (64 << 20), (used, lists)
