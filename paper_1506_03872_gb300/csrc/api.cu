@@ -151,11 +151,39 @@ mad_status clear_hash(mad_ctx* ctx, cudaStream_t st) {
   if (rs != MAD_OK) return rs;
   cudaMemsetAsync(&ctx->sc->inserted, 0, 5 * sizeof(unsigned long long), st);
   ctx->sampled = 0;
-  if (!stream_capturing(st)) {   // (a captured one clears X when it is replayed)
+  if (stream_capturing(st)) {   // (X is cleared when it is replayed)
+    ctx->x_held = true;
+  } else {
     ctx->x_empty = true;
     ctx->x_overflow = ctx->x_pass_captured;
+    ctx->x_added = 0;
   }
   return cuda_status(cudaGetLastError());
+}
+
+// X of 0/1 inputs moved to a table of ctx->x_wide slots (asynchronous).  Without
+// the memory for it X stays where it is, and says so if it fills up.
+mad_status widen_x(mad_ctx* ctx, cudaStream_t st) {
+  unsigned long long* const keys = ctx->hkeys;
+  long long* const vals = ctx->hvals;
+  const uint64_t slots = ctx->hcap;
+  decltype(ctx->hkeys) wide_keys = nullptr;
+  decltype(ctx->hvals) wide_vals = nullptr;
+  if (alloc(ctx, wide_keys, ctx->x_wide, st) != MAD_OK ||
+      alloc(ctx, wide_vals, ctx->x_wide, st) != MAD_OK) {
+    free_async(wide_keys, st);
+    return MAD_OK;
+  }
+  ctx->hkeys = wide_keys;
+  ctx->hvals = wide_vals;
+  ctx->hcap = ctx->hcap_alloc = ctx->x_wide;
+  mad_status rs = clear_x_slots(ctx, st);
+  cudaMemsetAsync(&ctx->sc->new_keys, 0, sizeof(unsigned long long), st);
+  if (rs == MAD_OK)
+    rs = accumulate_pairs(ctx, (const uint64_t*)keys, (const int64_t*)vals, slots, st);
+  cudaFreeAsync(keys, st);
+  cudaFreeAsync(vals, st);
+  return rs;
 }
 
 }  // namespace
@@ -237,7 +265,7 @@ mad_status alloc_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* B, 
     ctx->A = *A;
     ctx->B = *B;
     ctx->sampled = 0;
-    ctx->x_empty = ctx->x_overflow = ctx->x_captured = ctx->x_pass_captured = false;
+    ctx->x_empty = ctx->x_overflow = ctx->x_captured = ctx->x_pass_captured = ctx->x_held = false;
     if (ctx->regioned)
       ctx->hcap = ctx->hcap_alloc = hash_region_bound((uint64_t)ctx->m, s_max) + ctx->hov;
     return MAD_OK;
@@ -252,7 +280,8 @@ mad_status alloc_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix* B, 
   ctx->n = B->cols;
   ctx->s_max = s_max;
   ctx->sampled = 0;
-  ctx->x_empty = ctx->x_overflow = ctx->x_captured = ctx->x_pass_captured = false;
+  ctx->x_empty = ctx->x_overflow = ctx->x_captured = ctx->x_pass_captured = ctx->x_held = false;
+  ctx->x_wide = ctx->x_added = 0;
   mad_status rs = MAD_OK;
   if (!dense) {
     int64_t na = 0, nb = 0;
@@ -566,6 +595,12 @@ mad_status mad_build_tables(mad_ctx* ctx, const mad_matrix* A, const mad_matrix*
                                  per * (double)s_max / 0.6);
     uint64_t cap = 1024;
     while ((double)cap < want && cap < (1ull << 40)) cap <<= 1;
+    // Pairs that mad_accumulate adds (partial X of other runs) may be more than
+    // the budget's own: X then grows to a sixteenth of a load.
+    ctx->x_wide = cap;
+    while ((double)ctx->x_wide < std::min(4.0 * want, per * (double)s_max / 0.6) &&
+           ctx->x_wide < (1ull << 40))
+      ctx->x_wide <<= 1;
     ctx->hcap = ctx->hcap_alloc = cap;
     if ((rs = alloc(ctx, ctx->hkeys, cap, st)) != MAD_OK) return rs;
     if ((rs = alloc(ctx, ctx->hvals, cap, st)) != MAD_OK) return rs;
@@ -589,6 +624,7 @@ mad_status mad_sample(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first_di
   cudaStream_t st = (cudaStream_t)stream;
   const bool captured = stream_capturing(st);
   ctx->x_captured |= captured;
+  ctx->x_held |= captured;
   const bool fresh = s == ctx->s_max && ctx->sampled == 0 && ctx->x_empty &&
                      ctx->region_factor == 1.5f && ctx->hov_request == 0 &&
                      !(ctx->flags & (MAD_WEDGE | MAD_ALIAS)) && x_builder_applies(ctx, s) &&
@@ -776,6 +812,14 @@ mad_status mad_accumulate(mad_ctx* ctx, const uint64_t* keys_dev, const int64_t*
   cudaStream_t st = (cudaStream_t)stream;
   const bool captured = stream_capturing(st);
   ctx->x_captured |= captured;
+  ctx->x_held |= captured;
+  // (A quarter of the slots holds the budget's own keys.)
+  ctx->x_added = ctx->x_added + n < n ? UINT64_MAX : ctx->x_added + n;
+  if (!ctx->x_held && ctx->x_wide > ctx->hcap &&
+      (double)ctx->x_added > 0.35 * (double)ctx->hcap) {
+    const mad_status rs = widen_x(ctx, st);
+    if (rs != MAD_OK) return rs;
+  }
   if (ctx->x_overflow || captured) {   // (X may have been built whole again before a replay)
     const mad_status rs = fold_overflow(ctx, st);
     if (rs != MAD_OK) return rs;

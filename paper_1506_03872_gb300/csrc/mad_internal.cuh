@@ -181,7 +181,11 @@ struct mad_ctx {
   //   x_captured: a captured call adds to X when it is replayed.
   //   x_pass_captured: a captured pass writes X whole when it is replayed.
   bool x_empty = false, x_overflow = false;
-  bool x_captured = false, x_pass_captured = false;
+  //   x_held: a captured call holds X's addresses.
+  bool x_captured = false, x_pass_captured = false, x_held = false;
+  // 0/1 inputs: the slots X grows to when pairs added to it would fill it (0:
+  // it does not grow), and the pairs added since it was cleared.
+  uint64_t x_wide = 0, x_added = 0;
   int e1 = 0, f = 0;
   unsigned long long t1_total = 0;
   // Owned device memory.

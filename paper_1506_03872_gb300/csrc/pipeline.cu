@@ -119,7 +119,9 @@ mad_status enqueue_pass(mad_ctx* ctx, uint64_t seed, mad_pair* out_dev, uint32_t
   ctx->sampled = ctx->pipe_s;
   ctx->x_empty = false;
   ctx->x_overflow |= fresh;
-  ctx->x_pass_captured |= fresh && stream_capturing(st);
+  const bool captured = stream_capturing(st);
+  ctx->x_held |= captured;
+  ctx->x_pass_captured |= fresh && captured;
   ctx->built = true;
   // Alg. 3: Omega_t' (its length min(t', compacted) on the device) ...
   if (long_sel)

@@ -101,3 +101,53 @@ def test_select_pairs_orders_and_filters():
         assert n == 2
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("name", ["chung_lu_small", "bipartite_binary"])
+@pytest.mark.parametrize("first", [0, 30_000])
+def test_binary_x_takes_more_pairs_than_its_budget_draws(name, first):
+    """Partial X of other runs merged into a 0/1 context: the table, sized for
+    the context's own diamonds, grows before the added pairs fill it."""
+    import paper_1506_03872_gb300 as mad
+    s = 60_000
+    c = Case(name, s_max=s)
+    try:
+        ctx = c.ctx.ctx
+        if first:
+            mad.mad_sample(ctx, first, 5)
+        own_k, own_v = _x_sorted(mad, ctx, s + 1)
+        cap = mad.mad_stats(ctx)["hash_capacity"]
+        rng = np.random.Generator(np.random.PCG64(1))
+        flat = rng.permutation(c.m * c.n)
+        i, j = flat // c.n, flat % c.n
+        if c.flags & 2:
+            i, j = i[i < j], j[i < j]
+        n = s   # (what s_max / 0.6 slots hold)
+        assert n > cap or name == "bipartite_binary"
+        k = (i[:n].astype(np.uint64) << np.uint64(32)) | j[:n].astype(np.uint64)
+        v = rng.integers(1, 9, n)
+        for a in range(0, n, n // 3 + 1):   # in three calls
+            b = a + n // 3 + 1
+            mad.mad_accumulate(ctx, torch.from_numpy(k[a:b].view(np.int64).copy()).cuda(),
+                               torch.from_numpy(v[a:b].copy()).cuda())
+        want = dict(zip(own_k.tolist(), own_v.tolist()))
+        for key, val in zip(k.tolist(), v.tolist()):
+            want[key] = want.get(key, 0) + val
+        gk, gv = _x_sorted(mad, ctx, 4 * cap)
+        wk = np.array(sorted(want), dtype=np.uint64)
+        assert np.array_equal(gk, wk)
+        assert np.array_equal(gv, np.array([want[x] for x in wk.tolist()]))
+        st = mad.mad_stats(ctx)
+        assert st["device_error"] == 0 and st["distinct"] == len(wk)
+        top, nt = mad.mad_topk(ctx, 50)
+        assert nt == 50
+        # The grown table serves the next run as the first one did.
+        mad.mad_reset_hash(ctx)
+        mad.mad_sample(ctx, s, 9)
+        o = c.oracle
+        assert o.sample(s, 9) == 0
+        ok, ov = o.x()
+        gk, gv = _x_sorted(mad, ctx, s + 1)
+        assert np.array_equal(gk, ok) and np.array_equal(gv, ov)
+    finally:
+        c.close()
