@@ -25,6 +25,9 @@ SPACE = {
     "blocks_per_sm": (0, 2, 3),
     "select_threads": (128, 256, 512),
 }
+# What the stored shapes were timed on: changed with the kernels that the four
+# parameters shape, so that times of others are not found.
+KERNELS = "records+parts"
 DEFAULT = {"region_lg": 1, "chunk_mult": 8, "blocks_per_sm": 0, "select_threads": 256}
 
 
@@ -35,12 +38,12 @@ def cache_path() -> str:
 
 
 def shape_key(d: int, n: int, s_q, tprime: int, t: int) -> str:
-    """Device, item matrix shape and a summary of the batch (query count,
-    budget range and total rounded to two significant digits)."""
+    """Kernels, device, item matrix shape and a summary of the batch (query
+    count, budget range and total rounded to two significant digits)."""
     import torch
     s = np.asarray(s_q, dtype=np.float64)
     dev = torch.cuda.get_device_name() if torch.cuda.is_available() else "cpu"
-    return (f"{dev}|d={d}|n={n}|nq={len(s)}|s=[{int(s.min())},{int(s.max())}]"
+    return (f"{KERNELS}|{dev}|d={d}|n={n}|nq={len(s)}|s=[{int(s.min())},{int(s.max())}]"
             f"|sum={float(f'{s.sum():.2g}')}|tp={tprime}|t={t}")
 
 
