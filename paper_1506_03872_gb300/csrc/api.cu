@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "mad_internal.cuh"
@@ -49,6 +50,46 @@ mad_status ensure_scratch(mad_ctx* ctx, size_t bytes, cudaStream_t st) {
 using namespace mad;
 
 namespace {
+
+// Pages of pinned host memory for read-backs.  Page-locking and releasing one took
+// 300 of the 500 us that creating and destroying a context took, so a few
+// released ones are kept for the next contexts of the process (any thread, any
+// device); the others are given back at once.
+constexpr size_t kPinnedBytes = 4096;
+constexpr int kPinnedKept = 16;
+struct PinnedPages {
+  std::mutex lock;
+  void* page[kPinnedKept];
+  int n = 0;
+} pinned_pages;
+
+cudaError_t pinned_take(void** out) {
+  for (;;) {
+    *out = nullptr;
+    {
+      std::lock_guard<std::mutex> hold(pinned_pages.lock);
+      if (pinned_pages.n > 0) *out = pinned_pages.page[--pinned_pages.n];
+    }
+    if (!*out) return cudaHostAlloc(out, kPinnedBytes, cudaHostAllocPortable);
+    // (a device reset since has taken the kept pages with it)
+    cudaPointerAttributes at = {};
+    if (cudaPointerGetAttributes(&at, *out) == cudaSuccess && at.type == cudaMemoryTypeHost)
+      return cudaSuccess;
+    cudaGetLastError();
+  }
+}
+
+void pinned_give(void* page) {
+  if (!page) return;
+  {
+    std::lock_guard<std::mutex> hold(pinned_pages.lock);
+    if (pinned_pages.n < kPinnedKept) {
+      pinned_pages.page[pinned_pages.n++] = page;
+      return;
+    }
+  }
+  cudaFreeHost(page);
+}
 
 int ceil_log2(uint64_t x) {
   int e = 0;
@@ -433,11 +474,14 @@ mad_status mad_create(mad_ctx** out, uint32_t flags) {
     uint64_t keep = UINT64_MAX;
     e = cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
   }
-  if (e == cudaSuccess) e = cudaMalloc((void**)&ctx->sc, sizeof(DevScalars));
-  if (e == cudaSuccess) e = cudaMemset(ctx->sc, 0, sizeof(DevScalars));
-  if (e == cudaSuccess) e = cudaMalloc(&ctx->bound_state, bound_state_bytes());
-  if (e == cudaSuccess) e = cudaMemset(ctx->bound_state, 0, bound_state_bytes());
-  if (e == cudaSuccess) e = cudaMallocHost(&ctx->pinned, 4096);
+  // The scalars, and the bounds' state behind them.
+  constexpr size_t sc_bytes = (sizeof(DevScalars) + 255) & ~(size_t)255;
+  if (e == cudaSuccess) e = cudaMalloc((void**)&ctx->sc, sc_bytes + bound_state_bytes());
+  if (e == cudaSuccess) {
+    ctx->bound_state = (char*)ctx->sc + sc_bytes;
+    e = cudaMemset(ctx->sc, 0, sc_bytes + bound_state_bytes());
+  }
+  if (e == cudaSuccess) e = pinned_take(&ctx->pinned);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork2, cudaEventDisableTiming);
@@ -447,8 +491,7 @@ mad_status mad_create(mad_ctx** out, uint32_t flags) {
     if (ctx->ev_fork2) cudaEventDestroy(ctx->ev_fork2);
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->side) cudaStreamDestroy(ctx->side);
-    if (ctx->pinned) cudaFreeHost(ctx->pinned);
-    if (ctx->bound_state) cudaFree(ctx->bound_state);
+    pinned_give(ctx->pinned);
     if (ctx->sc) cudaFree(ctx->sc);
     if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
     delete ctx;
@@ -471,8 +514,7 @@ void mad_destroy(mad_ctx* ctx) {
   free_tables(ctx, 0);
   if (ctx->scratch) cudaFreeAsync(ctx->scratch, 0);
   cudaStreamSynchronize(0);
-  cudaFreeHost(ctx->pinned);
-  cudaFree(ctx->bound_state);
+  pinned_give(ctx->pinned);
   cudaFree(ctx->sc);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
   if (ctx->ev_fork2) cudaEventDestroy(ctx->ev_fork2);

@@ -271,7 +271,7 @@ struct mad_ctx {
   float region_factor = 1.5f;
   uint64_t hov_request = 0;
   mad::DevScalars* sc = nullptr;
-  void* bound_state = nullptr;      // bounds of mad_rescore (rescore_bounded)
+  void* bound_state = nullptr;      // bounds of mad_rescore (rescore_bounded), behind sc
   void* pinned = nullptr;           // 4 KB of pinned host memory for read-backs
   // The shape whose tables are allocated (dense tables without the optional
   // ones): a rebuild of the same shape keeps them.

@@ -175,3 +175,30 @@ def test_candidates_outside_the_matrices_are_reported(ncand, t, inside):
         c.build(mad.dense(A), mad.dense(B), 1024, keep=(A, B))
         got, ng = mad.mad_rescore(c.ctx, good, ncand, t)
         assert ng == nw == t and torch.equal(got, want)
+
+
+def test_contexts_are_cheap_to_make_and_their_read_backs_their_own():
+    """A context per request: creating and destroying one page-locks nothing
+    once a page is there (some 200 us; 500 with it), and the pages that
+    contexts alive at once read back through are different ones."""
+    import time
+
+    import paper_1506_03872_gb300 as mad
+    A, B = _dense_inputs()
+    mad.mad_destroy(mad.mad_create(0))
+    took = []
+    for _ in range(50):
+        t0 = time.perf_counter()
+        mad.mad_destroy(mad.mad_create(0))
+        took.append(time.perf_counter() - t0)
+    assert min(took) < 350e-6, min(took)
+    totals = []
+    for _ in range(2):
+        live = [mad.Context() for _ in range(20)]   # (more than are kept)
+        for q, c in enumerate(live):
+            c.build(mad.dense(A[:100 + q]), mad.dense(B), 1000, keep=(A, B))
+            mad.mad_sample(c.ctx, 1000, q)
+        totals.append([(mad.mad_topk(c.ctx, 10)[1], mad.mad_stats(c.ctx)["t1_total"]) for c in live])
+        for c in live:
+            c.close()
+    assert totals[0] == totals[1] and len({t for _, t in totals[0]}) == 20
