@@ -270,6 +270,9 @@ struct mad_ctx {
   // dense hash.
   float region_factor = 1.5f;
   uint64_t hov_request = 0;
+  // Kernels of sorting, building X and selecting that have opted in to their
+  // shared memory on this context's device.
+  bool sort_smem = false, image_smem = false, select_smem = false;
   mad::DevScalars* sc = nullptr;
   void* bound_state = nullptr;      // bounds of mad_rescore (rescore_bounded), behind sc
   void* pinned = nullptr;           // 4 KB of pinned host memory for read-backs

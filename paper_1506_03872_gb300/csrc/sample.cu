@@ -1196,13 +1196,12 @@ mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first, 
   const int blocks = sort_blocks();
   const int bits = sort_bits(ctx->m);
   const int coarse = bits < kCoarseBits ? bits : kCoarseBits, fine = bits - coarse;
-  static bool sort_attr = false;
-  if (!sort_attr) {
+  if (!ctx->sort_smem) {
     cudaFuncSetAttribute(k_sort_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sizeof(SortTile));
     cudaFuncSetAttribute(k_sort_fine, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(kFineStage * sizeof(uint32_t)));
-    sort_attr = true;
+    ctx->sort_smem = true;
   }
   const uint64_t batch = s < kSortBatch ? s : kSortBatch;
   // An empty X filled by one batch, keys owned by their drawn row: the
@@ -1213,12 +1212,11 @@ mad_status sample_impl(mad_ctx* ctx, uint64_t s, uint64_t seed, uint64_t first, 
   const size_t image_smem =
       (size_t)(kImageSlots + kSpill) * ((narrow ? sizeof(uint32_t) : sizeof(unsigned long long)) +
                              sizeof(unsigned long long));
-  static bool image_attr = false;
-  if (build_x && !image_attr) {
+  if (build_x && !ctx->image_smem) {
     const int wide_smem = (int)(2 * (size_t)(kImageSlots + kSpill) * sizeof(unsigned long long));
     cudaFuncSetAttribute(k_build_x<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide_smem);
     cudaFuncSetAttribute(k_build_x<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide_smem);
-    image_attr = true;
+    ctx->image_smem = true;
   }
   mad_status rs = ensure_scratch(ctx, sample_scratch_bytes(ctx, s), st);
   if (rs != MAD_OK) return rs;

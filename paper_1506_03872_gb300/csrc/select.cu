@@ -1329,11 +1329,10 @@ void block_select_dev(mad_ctx* ctx, const Item* in, uint64_t cap, uint64_t K,
                       const unsigned long long* n_dev, bool sorted, Item* tile_sorted,
                       uint32_t* pos, Item* out, unsigned int* gate, unsigned int* over_err,
                       cudaStream_t st) {
-  static bool attr = false;
   const size_t smem = (size_t)kBlockSel * sizeof(unsigned long long);
-  if (!attr) {
+  if (!ctx->select_smem) {
     cudaFuncSetAttribute(k_block_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = true;
+    ctx->select_smem = true;
   }
   if (sorted && (K > (uint64_t)kTile || cap <= (uint64_t)kTile)) {
     // Too many for k_rank_sort, or a list short enough to be ranked at once.
