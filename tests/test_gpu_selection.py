@@ -107,3 +107,24 @@ def test_a_long_candidate_list_is_sized_by_the_keys_there_are():
     assert torch.equal(got, torch.sort(x[x > 0], descending=True).values)
     lists = 3 * 24 * nx + 24 * (1 << (nx - 1).bit_length())
     assert used <= lists + (64 << 20), (used, lists)
+
+
+@pytest.mark.parametrize("ld,first", [(100, 0), (104, 0), (128, 4), (102, 0), (104, 2), (101, 1)])
+def test_bounded_rescore_of_rows_in_a_wider_matrix(ld, first):
+    """A leading dimension above d, rows on 16-byte boundaries or not."""
+    import paper_1506_03872_gb300 as mad
+    rng = _rng(ld + first)
+    m, d, n, ncand, t = 700, 100, 900, 50_000, 300
+    wide = torch.from_numpy(rng.standard_normal(m * ld + first + 8).astype(np.float32)).cuda()
+    tA = wide[first:].as_strided((m, d), (ld, 1))
+    tB = torch.from_numpy(rng.standard_normal((d, n)).astype(np.float32)).cuda()
+    q = rng.permutation(m * n)[:ncand]
+    cand = mad.encode_pairs(q // n, q % n, np.arange(1, ncand + 1))
+    with mad.Context() as c:
+        c.build(mad.dense(tA), mad.dense(tB), 1024, keep=(wide, tB))
+        whole, nw = mad.mad_rescore(c.ctx, cand, ncand, ncand)
+        top, nt = mad.mad_rescore(c.ctx, cand, ncand, t)
+    assert nw == ncand and nt == t and torch.equal(top, whole[:t])
+    A64, B64 = tA.double().cpu().numpy(), tB.double().cpu().numpy()
+    gi, gj, _, gc = mad.decode_pairs(top, t)
+    assert np.allclose(gc, np.einsum("ij,ji->i", A64[gi], B64[:, gj]), rtol=0, atol=1e-11)

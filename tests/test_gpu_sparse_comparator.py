@@ -157,3 +157,18 @@ def test_zero_product_and_errors():
         with pytest.raises(mad.MadError) as e:
             mad.mad_sparse_topt(c.ctx, MA, MB, 5, options=2)
         assert e.value.status == 1
+
+
+@pytest.mark.parametrize("n", [1_638_400, 1_638_401, 2_000_003])
+def test_more_columns_than_the_shared_bitmap(n):
+    """B restricted to its selected columns through the bitmap in L2 where the
+    columns' bits do not fit shared memory (1,638,400 do)."""
+    rng = _rng(n)
+    m, d = 300, 200
+    rpA, ciA = _csr(rng.random((m, d)) < 0.2)
+    heavy = rng.choice(n, 400, replace=False)
+    heavy[:2] = 0, n - 1
+    cols = [np.union1d(heavy[rng.random(400) < 0.6], rng.integers(0, n, 2000)) for _ in range(d)]
+    rpB = np.concatenate([[0], np.cumsum([len(c) for c in cols])]).astype(np.int64)
+    ciB = np.concatenate(cols).astype(np.int32)
+    _check(*_run(rpA, ciA, (m, d), rpB, ciB, (d, n), 0, 700))
