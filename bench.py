@@ -44,9 +44,9 @@ SAMPLER_SOURCES = ["paper_1506_03872_gb300/csrc/sample.cu",
 # 4-byte diamond index read in row order and the 16-byte (key, increment)
 # record written.
 DENSE_DRAW_BYTES = 32 * 5 + 4 + 16
-# 0/1 draw kernel (k_sample, draws and inserts): the final entry of the T1
-# search, row i's bounds, the T2 guide entries and the T2 window, the column
-# indices of k and k', row k's bounds, b_kj's index and the closure filter's
+# 0/1 draw kernel (k_sample_rows, draws and inserts): the final entry of the T1
+# search, row i's descriptor, the T2 guide entries and the T2 window, the column
+# indices of k and k', row k's descriptor, b_kj's index and the closure filter's
 # word (the exact closure search of the ~1 % of diamonds the filter passes
 # is left out); the hash read-modify-write of closed diamonds is added per
 # inserted diamond (2 sectors read and written).
@@ -604,8 +604,8 @@ def run_ours(args):
     elif phase_k is not None:
         draw_ms = float(phase_k[:, 1].mean())
         if w.csr:
-            rooflines["k_sample"] = _roof(
-                "k_sample", 32 * SPARSE_DRAW_SECTORS * s + HASH_RMW_BYTES * int(stats["inserted"]),
+            rooflines["k_sample_rows"] = _roof(
+                "k_sample_rows", 32 * SPARSE_DRAW_SECTORS * s + HASH_RMW_BYTES * int(stats["inserted"]),
                 draw_ms, peak, peak_kind, s, sectors=SPARSE_DRAW_SECTORS * s,
                 probe=(probes or {}).get("gather"))
         else:
@@ -929,8 +929,9 @@ def chung_lu_leg(args, dev, stream, flush, peak, peak_kind):
         probes = run_probes(mad, dev, stream, gather_bytes=sparse_table_bytes(w),
                             atomic_bytes=16 * int(st["hash_capacity"]))
         leg["probes"] = probes
-        r = _roof("k_sample", 32 * SPARSE_DRAW_SECTORS * w.s + HASH_RMW_BYTES * int(st["inserted"]),
-                  draw_ms, peak, peak_kind, w.s, sectors=SPARSE_DRAW_SECTORS * w.s,
+        r = _roof("k_sample_rows",
+                  32 * SPARSE_DRAW_SECTORS * w.s + HASH_RMW_BYTES * int(st["inserted"]), draw_ms,
+                  peak, peak_kind, w.s, sectors=SPARSE_DRAW_SECTORS * w.s,
                   probe=probes.get("gather"))
         ins_rate = int(st["inserted"]) / (draw_ms / 1e3)
         r["inserts_per_s"] = round(ins_rate, 1)

@@ -194,8 +194,11 @@ void mad_destroy(mad_ctx* ctx);
 const char* mad_strerror(mad_status status);
 
 /* Hash capacity in slots for the next mad_build_tables (a power of two,
- * >= 1024), or 0 for the default: the smallest power of two >= s_max / 0.6.
- * Each slot is 16 bytes. */
+ * >= 1024), or 0 for the default: dense inputs get home regions for s_max
+ * diamonds (up to 3 s_max + 4 m slots); 0/1 inputs a power of two of at most
+ * about s_max / 0.3 slots, from the share of diamonds that add to X in a pilot
+ * run: a quarter load, which mad_accumulate lets grow to a sixteenth (not
+ * while a captured call holds X's addresses).  Each slot is 16 bytes. */
 mad_status mad_set_hash_capacity(mad_ctx* ctx, uint64_t slots);
 
 /* Alg. 2 weight line and the cumulative tables of Sec. 4.2.
@@ -261,9 +264,9 @@ mad_status mad_rescore(mad_ctx* ctx, const mad_pair* cand_dev, uint32_t ncand, u
  * entries, a full overflow table of the hash; 0/1 inputs: a full hash) go
  * to the device error word.  X after a
  * run (read by mad_export_x, mad_topk, mad_rescore) is the X of the step-wise
- * calls, laid out differently: for dense non-Gram inputs the home regions
- * are built whole and keys that do not fit go to an overflow table after
- * them.  The run samples all s diamonds the plan allows, so a further
+ * calls: for dense non-Gram inputs the home regions are built whole and keys
+ * that find no place go to an overflow table after them, until mad_accumulate
+ * moves them back.  The run samples all s diamonds the plan allows, so a further
  * mad_sample needs mad_reset_hash first (MAD_ERR_OVERFLOW otherwise).
  *
  * mad_pipeline_status: synchronises, refreshes the host-side table scalars
@@ -468,8 +471,8 @@ mad_status mad_probe_atomics(void* table_dev, uint64_t bytes, uint64_t count, ui
  * sampling adds diamonds: X of the keys this rank owns, merged from every
  * rank's partials after mad_reset_hash.  Keys must belong to the
  * context's shape (row < m, column < n, unordered under MAD_GRAM); the
- * hash must hold them (MAD_ERR_HASH_FULL from the next mad_topk otherwise).
- * Asynchronous.
+ * hash must hold them (MAD_ERR_HASH_FULL from the next mad_topk otherwise;
+ * that of 0/1 inputs grows: see mad_set_hash_capacity).  Asynchronous.
  *
  * mad_select_pairs: the min(K, #{x > 0}) pairs of pairs_dev (n, device)
  * with the largest x, ties broken by smaller (i, j), sorted by (x desc, i
@@ -483,7 +486,7 @@ mad_status mad_accumulate(mad_ctx* ctx, const uint64_t* keys_dev, const int64_t*
 mad_status mad_select_pairs(mad_ctx* ctx, const mad_pair* pairs_dev, uint64_t n, uint32_t K,
                             mad_pair* out_dev, uint32_t* n_out_host, mad_stream stream);
 
-/* Counters and table scalars (synchronises the device). *//* Counters and table scalars (synchronises the device). */
+/* Counters and table scalars (synchronises the device). */
 mad_status mad_stats(mad_ctx* ctx, mad_stats_t* out);
 
 /* ---- Diagnostics (used by the parity tests; not on the hot path) ------- */
@@ -504,10 +507,11 @@ mad_status mad_debug_draws(mad_ctx* ctx, uint64_t seed, uint64_t first, uint64_t
  * up to a power of two.  Regions too small for their keys send them to the
  * overflow table in the fused pass (mad_pipeline_run); a full overflow
  * table is reported as MAD_ERR_HASH_FULL by mad_pipeline_status.  The
- * step-wise mad_sample probes the regions as one table and reports
- * MAD_ERR_HASH_FULL past its probe limit.  For batched queries region_factor
- * scales the tables of a query's parts (1.5 slots per record), and a nonzero
- * overflow_slots makes mad_mips_items build the guides of long item tables.
+ * step-wise mad_sample of such a layout adds key by key, probing the regions
+ * as one table, and reports MAD_ERR_HASH_FULL past its probe limit.  For
+ * batched queries region_factor scales the tables of a query's parts (1.5
+ * slots per record), and a nonzero overflow_slots makes mad_mips_items build
+ * the guides of long item tables; neither changes a result.
  * MAD_ERR_ARG outside these ranges. */
 mad_status mad_debug_set_hash_layout(mad_ctx* ctx, float region_factor, uint64_t overflow_slots);
 

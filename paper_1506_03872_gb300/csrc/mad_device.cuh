@@ -460,7 +460,8 @@ __host__ __device__ __forceinline__ unsigned long long bucket_floor(uint32_t b) 
 
 // Bloom filter for the 0/1 closure test: the entry (a, b) sets five bits in
 // one 64-bit word, two in its low half and three in its high half.  Word and
-// bits come from two 32-bit mixes of the pair (a 64-bit mix of the pair and a
+// bits come from two 32-bit mixes of the pair, its halves first spread by 2^32
+// over the golden ratio and two of xxHash32's primes (Collet) (a 64-bit mix of the pair and a
 // second one for the bits took about a fifth of the sampler's instructions).
 // A clear bit proves the entry absent; a set filter sends the test to the
 // exact search.

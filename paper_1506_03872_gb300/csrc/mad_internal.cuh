@@ -261,7 +261,7 @@ struct mad_ctx {
   long long* hvals = nullptr;
   // Dense inputs: row i's home region is [hreg[i], hreg[i+1]) (m + 2
   // offsets; hreg[m] is the end of the regions, followed by an overflow
-  // table of hov slots that only the fused pass's region builder fills;
+  // table of hov slots that only the region builder fills (k_build_x);
   // hreg[m+1] = hreg[m] + hov is the end of X).
   unsigned long long* hreg = nullptr;
   bool regioned = false;
@@ -449,7 +449,7 @@ constexpr uint64_t kDevSelectCap = 1ull << 17;
 size_t dev_select_state_bytes();
 // Omega_t' from the hash whose extent is *hcap_dev slots (at most
 // ctx->hcap): the positive x at or above a log-bucket threshold (estimated
-// from one 4-slot group in 8, the exact histogram as a gated fallback) are
+// from one 4-slot group in 16, the exact histogram as a gated fallback) are
 // compacted into list (kDevSelectCap entries, count at *count), then the K
 // largest go to out, in no particular order when one block selects them
 // (lists up to 16384 items), else sorted.  count[1..2] are gate words.

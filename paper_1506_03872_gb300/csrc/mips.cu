@@ -381,7 +381,7 @@ struct Kept {
 //
 // The part's records lie in one run per chunk of the query: the runs' offsets are
 // scanned (kGroup chunks at a time) and the records dealt out evenly, four of a
-// lane read at a time.  Bound by the instructions of the inserts (55 % of the issue
+// lane read at a time.  Bound by the instructions of the inserts (62 % of the issue
 // slots with the loads' latency hidden): a warp that probes until the last of its
 // records is placed takes eight to ten steps for two on average, so a record whose
 // first slot is taken (a third of them) waits in the warp's queue until 32

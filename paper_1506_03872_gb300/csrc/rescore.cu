@@ -78,7 +78,7 @@ k_rescore_dense(const mad_pair* __restrict__ cand, unsigned long long ncand_max,
 // four bits) that holds the t-th largest L.  The candidates that stay (about 1.1
 // t) get the same FP64 sums in the same order as k_rescore_dense's.
 // 1e5 of 200000 x 50000 pairs, d = 100, t = 1000: 163 us of FP64 products
-// became 48 us of bounds and 11 us of products (mad_rescore 287 -> 134 us, with
+// became 27 us of bounds and 11 us of products (mad_rescore 287 -> 114 us, with
 // the selection working on the 1,100 kept).
 //
 // The bound: a sum of d <= 1024 products in 32 lane partials and five folds

@@ -157,7 +157,7 @@ k_sample(const SampleParams p_, unsigned long long seed, unsigned long long firs
 //
 // Bound by random sectors (about ten a diamond: T1's guide, the row, its guide
 // and window of T2, the two columns, the row of B, its column, the filter
-// word), at 53 % of DRAM's rate, 61 % of L2's and 64 % of L1's at once, so it
+// word), at 54 % of DRAM's rate, 64 % of L2's and 66 % of L1's at once, so it
 // wants every warp the SM holds (32 registers).  Five arrays' worth of row data
 // in one 16-byte load, a cheaper filter mix and T2 guides of about four entries
 // a bucket took 1e8 diamonds on the graph of 1e6 nodes from 6.12 to 4.62 ms
@@ -467,10 +467,10 @@ k_sort_fine(const DevScalars* __restrict__ sc, const uint32_t* __restrict__ rec,
 // q] and vals[s + q] (Sec. 3.2.3).  k_insert adds them to X.
 //
 // The draws are draw_given_row's, written out for dense inputs of one type.
-// Issue slots and L1 bind it together (54 % and 62 % of their rates, 680
-// instructions a diamond before, DRAM 23 %): without the branches on input
-// kinds and with 32-bit totals multiplied as such the fused pass went from 930
-// to 907 us.  TB in 64-byte blocks, as the batched queries draw, is slower here
+// Load latency binds it, with issue slots and L1 at 53 % and 63 % of their rates
+// and DRAM at 17 % (560 instructions a diamond): without the branches on input
+// kinds and with 32-bit totals multiplied as such (680 instructions before) the
+// fused pass went from 930 to 907 us.  TB in 64-byte blocks, as the batched queries draw, is slower here
 // (972 us: TB and its guides are in L2, and a block reads twice their bytes),
 // and so are 7 or 8 blocks per SM (935 us).
 template <typename TBV>

@@ -42,7 +42,8 @@ constexpr uint32_t kSpWindowMax = 24576;       // labels per shared window (96 K
 // Rows and columns of the pilot: its pairs have to hold t large counts, so its
 // side grows with sqrt(t).  16 sqrt(t) measured best between 8 and 64 (2048 at
 // t = 1000, the size it always had) on graphs of 2e4 to 1e6 nodes: 1e6 nodes, t
-// = 1000: 1224, 1070, 1093, 1098 and 1193 us at 8, 16, 24, 32 and 64.
+// = 1000: 1224, 1070, 1093, 1098 and 1193 us at 8, 16, 24, 32 and 64 (measured
+// side by side).
 uint32_t pilot_size(uint32_t t) {
   const double want = 16.0 * std::sqrt((double)t);
   return want < 256.0 ? 256u : want > 2048.0 ? 2048u : (uint32_t)want;
@@ -342,8 +343,8 @@ __global__ void __launch_bounds__(kSpBlock) k_spgemm_rowblock_topk(SpRowParams p
       // entry's filtered row inside the window (32 searches side by side), then
       // the warp goes through the 32 parts in pieces of up to 32 labels, four
       // pieces in flight.  A warp per entry in turn waited for four dependent
-      // loads on each (main pass on 1e6 nodes 865 us, now 576; with 512
-      // threads a row instead of 256, 480).
+      // loads on each (main pass on 1e6 nodes 865 us, then 576; with 512
+      // threads a row instead of 256, 480; issue slots 86 % taken).
       const uint32_t alen = (uint32_t)(a1 - a0);
       for (uint32_t q0 = 0; q0 < alen; q0 += 32 * kSpWarps) {
         uint32_t start = 0, len = 0;
