@@ -543,7 +543,11 @@ const unsigned long long* rescore_bounded(mad_ctx* ctx, void* state, const mad_p
                                           uint64_t ncand, uint64_t t, Item* items, double* cvals,
                                           cudaStream_t st,
                                           const unsigned long long* n_dev = nullptr);
+// group: rescore_group_bytes of the caller's, in place of the context's buffer.
 mad_status rescore_items(mad_ctx* ctx, const mad_pair* cand, uint64_t ncand, Item* items,
-                         double* cvals, cudaStream_t st, const unsigned long long* n_dev = nullptr);
+                         double* cvals, cudaStream_t st, const unsigned long long* n_dev = nullptr,
+                         void* group = nullptr);
+// Bytes in which 0/1 Gram candidates are grouped by hub (0 for other inputs).
+size_t rescore_group_bytes(const mad_ctx* ctx, uint64_t ncand);
 
 }  // namespace mad

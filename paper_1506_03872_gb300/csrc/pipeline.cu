@@ -32,6 +32,7 @@ struct PipeBufs {
   void* state;                  // selection state of Omega_t'
   unsigned long long* count;    // compacted candidates (device length)
   void* bound;                  // bounds of the rescore (dense inputs; zeros between runs)
+  void* group;                  // grouped rescore (0/1 Gram inputs; null without)
   Item* list;                   // compacted items, list_cap
   Item* topk;                   // the K selected, unsorted (0/1 inputs), t'
   Item* sorted;                 // tile-sorted copy, kDevSelectCap
@@ -48,8 +49,10 @@ struct PipeBufs {
 
 size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// long_sel: the 0/1 pass's digit search over list_cap candidates.
-PipeBufs carve(void* base, uint64_t tprime, uint64_t t, uint64_t list_cap, bool long_sel) {
+// long_sel: the 0/1 pass's digit search over list_cap candidates.  group: bytes
+// of its grouped rescore.
+PipeBufs carve(void* base, uint64_t tprime, uint64_t t, uint64_t list_cap, bool long_sel,
+               size_t group) {
   PipeBufs b;
   char* p = (char*)base;
   size_t off = 0;
@@ -61,6 +64,8 @@ PipeBufs carve(void* base, uint64_t tprime, uint64_t t, uint64_t list_cap, bool 
   b.state = take(dev_select_state_bytes());
   b.count = (unsigned long long*)take(4 * sizeof(unsigned long long));
   b.bound = take(long_sel ? 0 : bound_state_bytes());
+  b.group = take(group);
+  if (!group) b.group = nullptr;
   b.list = (Item*)take(list_cap * sizeof(Item));
   b.topk = (Item*)take(long_sel ? tprime * sizeof(Item) : 0);
   b.sorted = (Item*)take(kDevSelectCap * sizeof(Item));
@@ -103,7 +108,8 @@ mad_status enqueue_pass(mad_ctx* ctx, uint64_t seed, mad_pair* out_dev, uint32_t
                         mad_pair* cand_dev, cudaStream_t st) {
   const bool long_sel = !ctx->dense;
   const PipeBufs b =
-      carve(ctx->pipe_buf, ctx->pipe_tprime, ctx->pipe_t, ctx->pipe_list_cap, long_sel);
+      carve(ctx->pipe_buf, ctx->pipe_tprime, ctx->pipe_t, ctx->pipe_list_cap, long_sel,
+            rescore_group_bytes(ctx, ctx->pipe_tprime));
   mad_pair* cand = cand_dev ? cand_dev : b.cand;
   mad_status rs;
   // Alg. 2: tables, an empty X, s diamonds.  Where the sampler builds the
@@ -136,8 +142,8 @@ mad_status enqueue_pass(mad_ctx* ctx, uint64_t seed, mad_pair* out_dev, uint32_t
   if (rescore_bounded_applies(ctx, ctx->pipe_tprime, ctx->pipe_t))
     scored = rescore_bounded(ctx, b.bound, cand, ctx->pipe_tprime, ctx->pipe_t, b.rs_items, b.cvals,
                              st, b.count);
-  else if ((rs = rescore_items(ctx, cand, ctx->pipe_tprime, b.rs_items, b.cvals, st, b.count)) !=
-           MAD_OK)
+  else if ((rs = rescore_items(ctx, cand, ctx->pipe_tprime, b.rs_items, b.cvals, st, b.count,
+                               b.group)) != MAD_OK)
     return rs;
   block_select_dev(ctx, b.rs_items, ctx->pipe_tprime, ctx->pipe_t, scored, true, b.rs_sorted,
                    b.rs_pos, b.rs_out, (unsigned int*)(b.count + 3), nullptr, st);
@@ -166,18 +172,17 @@ mad_status mad_pipeline_plan(mad_ctx* ctx, const mad_matrix* A, const mad_matrix
   // the Chung-Lu graph of 1e6 nodes nearly every key of X has x = 1), so the
   // 0/1 list holds every slot of the hash: it cannot overflow.
   ctx->pipe_list_cap = csr ? std::max<uint64_t>(kDevSelectCap, ctx->hcap_alloc) : kDevSelectCap;
-  const PipeBufs sizes = carve(nullptr, tprime, t, ctx->pipe_list_cap, csr);
+  const size_t group = rescore_group_bytes(ctx, tprime);
+  const PipeBufs sizes = carve(nullptr, tprime, t, ctx->pipe_list_cap, csr, group);
   if ((rs = pool_malloc(ctx, &ctx->pipe_buf, sizes.bytes, st)) != MAD_OK) return rs;
   if (!csr)
-    cudaMemsetAsync(carve(ctx->pipe_buf, tprime, t, ctx->pipe_list_cap, csr).bound, 0,
+    cudaMemsetAsync(carve(ctx->pipe_buf, tprime, t, ctx->pipe_list_cap, csr, group).bound, 0,
                     bound_state_bytes(), st);
   // The scratch every launch of a run needs, owned by the pass.
   size_t scratch = csr ? csr_build_scratch_bytes(ctx) : dense_build_scratch_bytes(ctx);
   if (sample_scratch_bytes(ctx, s) > scratch) scratch = sample_scratch_bytes(ctx, s);
   if ((rs = pool_malloc(ctx, &ctx->pipe_scratch, scratch, st)) != MAD_OK) return rs;
   ctx->pipe_scratch_bytes = scratch;
-  // The rescoring's grouping buffer (0/1 Gram inputs) for t' candidates.
-  if ((rs = rescore_reserve(ctx, tprime, st)) != MAD_OK) return rs;
   ctx->pipe = true;
   ctx->pipe_s = s;
   ctx->pipe_tprime = tprime;

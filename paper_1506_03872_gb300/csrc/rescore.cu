@@ -633,10 +633,11 @@ int rescore_bitmap_grid(size_t smem) {
   return sms * per_sm;
 }
 
-mad_status rescore_gram_grouped(mad_ctx* ctx, const mad_pair* cand, uint64_t ncand, Item* items,
-                                double* cvals, cudaStream_t st, const unsigned long long* n_dev) {
+mad_status rescore_gram_grouped(mad_ctx* ctx, void* group, const mad_pair* cand, uint64_t ncand,
+                                Item* items, double* cvals, cudaStream_t st,
+                                const unsigned long long* n_dev) {
   const RgLayout L = rg_layout(ctx->m, ncand);
-  char* base = (char*)ctx->rg_buf;
+  char* base = (char*)group;
   uint32_t* cnt = (uint32_t*)(base + L.cnt);
   uint32_t* off = (uint32_t*)(base + L.off);
   uint32_t* part = (uint32_t*)(base + L.part);
@@ -718,6 +719,10 @@ mad_status rescore_reserve(mad_ctx* ctx, uint64_t ncand, cudaStream_t st) {
   return MAD_OK;
 }
 
+size_t rescore_group_bytes(const mad_ctx* ctx, uint64_t ncand) {
+  return gram_bitmap_applies(ctx) ? rg_layout(ctx->m, ncand).bytes : 0;
+}
+
 size_t bound_state_bytes() { return sizeof(BoundState); }
 
 // Below a few thousand candidates, or with a t near their number, the bounds
@@ -740,10 +745,12 @@ const unsigned long long* rescore_bounded(mad_ctx* ctx, void* state, const mad_p
 }
 
 mad_status rescore_items(mad_ctx* ctx, const mad_pair* cand, uint64_t ncand, Item* items,
-                         double* cvals, cudaStream_t st, const unsigned long long* n_dev) {
+                         double* cvals, cudaStream_t st, const unsigned long long* n_dev,
+                         void* group) {
   if (ncand == 0) return MAD_OK;
-  if (gram_bitmap_applies(ctx) && ctx->rg_buf && ctx->rg_cap >= ncand)
-    return rescore_gram_grouped(ctx, cand, ncand, items, cvals, st, n_dev);
+  if (!group && ctx->rg_cap >= ncand) group = ctx->rg_buf;
+  if (gram_bitmap_applies(ctx) && group)
+    return rescore_gram_grouped(ctx, group, cand, ncand, items, cvals, st, n_dev);
   if (ctx->integer && (ctx->flags & MAD_GRAM)) {
     const unsigned long long blocks = (ncand * 32 + 255) / 256;
     k_rescore_gram_binary<<<(unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, st>>>(

@@ -659,3 +659,47 @@ def test_a_table_build_ends_what_captured_calls_meant():
         c.build(mad.dense(tA), mad.dense(tB), s, keep=(tA, tB))
         assert sampled(c) == built
         del g
+
+
+def test_binary_replays_beside_eager_rescoring():
+    """The same for 0/1 Gram inputs, whose candidates are grouped by hub: the
+    pass's own grouping is untouched by a mad_rescore of more candidates than
+    it has, before or beside a replay."""
+    import paper_1506_03872_gb300 as mad
+    ra, ca, sa, rb, cb, sb, flags, MA, MB = _csr_case("chung_lu")
+    s, tprime, t, ncand = 400_000, 1000, 20, 60_000
+    keep = [torch.from_numpy(x).cuda() for x in (ra, ca)]
+    Am = mad.csr(keep[0], keep[1], sa)
+    rng = _rng(100)
+    i, j = rng.integers(0, sa[0], 3 * ncand), rng.integers(0, sa[0], 3 * ncand)
+    u = np.unique((np.minimum(i, j) << 32 | np.maximum(i, j))[i != j])[:ncand]
+    pairs = mad.encode_pairs(u >> 32, u & 0xFFFFFFFF, np.arange(1, len(u) + 1))
+    side = torch.cuda.Stream()
+    with mad.Context(flags) as c:
+        mad.mad_pipeline_plan(c.ctx, Am, Am, s, tprime, t)
+        out, cand = mad.new_pairs(t), mad.new_pairs(tprime)
+        counts = torch.zeros(2, dtype=torch.int32, device="cuda")
+        mad.mad_pipeline_run(c.ctx, 51, out, counts, cand)
+        torch.cuda.synchronize()
+        mad.mad_pipeline_status(c.ctx)
+        want, wc = out.clone(), counts.clone()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            mad.mad_pipeline_run(c.ctx, 51, out, counts, cand)
+        top, nt = mad.mad_rescore(c.ctx, pairs, len(u), t)
+        top = top.clone()
+        assert nt == t
+        o = oracle.Oracle(MA, MB, flags, s)
+        tk, tc = oracle.topt((u >> 32).astype(np.uint64) << np.uint64(32)
+                             | (u & 0xFFFFFFFF).astype(np.uint64),
+                             o.rescore(u.astype(np.uint64)), t)
+        gi, gj, _, gc = mad.decode_pairs(top, t)
+        assert np.array_equal(mad.keys_of(gi, gj), tk) and np.array_equal(gc, tc)
+        for _ in range(50):
+            with torch.cuda.stream(side):
+                g.replay()
+            for _ in range(2):
+                got, ng = mad.mad_rescore(c.ctx, pairs, len(u), t)
+                assert ng == nt and torch.equal(got[:ng], top[:nt])
+            side.synchronize()
+            assert torch.equal(counts, wc) and torch.equal(out, want)
