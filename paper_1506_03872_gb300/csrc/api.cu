@@ -28,7 +28,10 @@ mad_status pool_malloc(mad_ctx* ctx, void** p, size_t bytes, cudaStream_t st) {
   *p = nullptr;
   if (ctx->fault_oom_at > 0 && ++ctx->allocs >= ctx->fault_oom_at) return MAD_ERR_OOM;
   const mad_status rs = cuda_status(cudaMallocFromPoolAsync(p, bytes, ctx->pool, st));
-  if (rs != MAD_OK) *p = nullptr;
+  if (rs != MAD_OK) {
+    *p = nullptr;
+    cudaGetLastError();   // (reported here; calls that go on without it launch cleanly)
+  }
   return rs;
 }
 

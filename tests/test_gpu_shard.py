@@ -151,3 +151,40 @@ def test_binary_x_takes_more_pairs_than_its_budget_draws(name, first):
         assert np.array_equal(gk, ok) and np.array_equal(gv, ov)
     finally:
         c.close()
+
+
+def test_binary_x_without_memory_to_grow(monkeypatch):
+    """The growth is a service, not a need: where its memory is refused, pairs
+    that the table holds are added all the same, and a table that fills up is
+    reported."""
+    import paper_1506_03872_gb300 as mad
+    c = None
+    for n in range(1, 100):
+        monkeypatch.setenv("MAD_FAULT", f"oom:{n}")
+        try:
+            c = Case("chung_lu_small", s_max=60_000)   # (its allocations succeed; the next fails)
+            break
+        except mad.MadError as e:
+            assert e.status == mad.MAD_ERR_OOM
+    monkeypatch.delenv("MAD_FAULT")
+    try:
+        ctx = c.ctx.ctx
+        cap = mad.mad_stats(ctx)["hash_capacity"]
+        rng = np.random.Generator(np.random.PCG64(2))
+        flat = rng.permutation(c.m * c.m)
+        i, j = flat // c.m, flat % c.m
+        i, j = i[i < j], j[i < j]
+        k = (i.astype(np.uint64) << np.uint64(32)) | j.astype(np.uint64)
+        n = cap // 2
+        mad.mad_accumulate(ctx, torch.from_numpy(k[:n].view(np.int64).copy()).cuda(),
+                           torch.ones(n, dtype=torch.int64, device="cuda"))
+        st = mad.mad_stats(ctx)
+        assert st["hash_capacity"] == cap and st["distinct"] == n and st["device_error"] == 0
+        rest = k[n:2 * cap]
+        mad.mad_accumulate(ctx, torch.from_numpy(rest.view(np.int64).copy()).cuda(),
+                           torch.ones(len(rest), dtype=torch.int64, device="cuda"))
+        with pytest.raises(mad.MadError) as e:
+            mad.mad_topk(ctx, 10)
+        assert e.value.status == mad.MAD_ERR_HASH_FULL
+    finally:
+        c.close()
